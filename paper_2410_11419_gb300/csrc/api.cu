@@ -149,8 +149,10 @@ Workspace plan_workspace(int n, int width, int height, size_t cap) {
   L.tile_order[0] = P.take(4 * (size_t)L.ntiles);
   L.tile_order[1] = P.take(4 * (size_t)L.ntiles);
   const size_t items = shadow_seg_items(L.ntiles, cap);
-  L.seg_lvl = P.take(4 * (1025 + 3));
+  L.seg_lvl = P.take(4 * (1025 + 5));
   L.seg_flag = P.take(4 * items);
+  L.seg_desc = P.take(16 * items);
+  L.seg_lists = P.take(8 * items);
   L.seg_pub = P.take(4 * 256 * items);
   L.rank_flags = P.take(2 * N);
   L.shade = P.take(16 * N);

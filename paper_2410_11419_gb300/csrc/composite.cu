@@ -8,6 +8,7 @@
 // records).
 #include "gs3_internal.cuh"
 #include "splat_eval.cuh"
+#include "f32x2.cuh"
 
 namespace gs3 {
 namespace {
@@ -24,34 +25,42 @@ namespace {
 // Work is split into segments of a tile's list: segment s holds receivers
 // [R_s, R_s+1) (kSegLen entries; the last takes the rest) and needs the
 // occluders [C_s, C_s+1) on top of the product A(C_s) that every ray carries
-// into it, with C_s = K(R_s).  One warp takes one segment at a time from a
-// ticket counter, in segment-major order (every tile's first segment, then
-// every tile's second, ...), and:
-//   1. computes each of its 256 rays' product Q over its occluder range (a
-//      ray drops out once the product can no longer stay above the stop);
-//   2. takes A(C_s) from the segment before it (published by that warp; a
-//      bounded wait) and publishes A(C_s+1) = A(C_s) Q for the next one;
-//   3. walks its receivers in order with the products P = A(C_s) q, q the
-//      running product of the range's occluders, summing (beta P, beta) per
-//      receiver into the (tile, Gaussian) partials.
-// Step 1 runs before the wait, so the segments of a long list run side by
-// side and only the cheap step 2 is chained.  When A(C_s) is already
-// published as the warp starts, step 1 skips the rays that are stopped.
+// into it, with C_s = K(R_s).  Persistent warps take one segment at a time
+// from a ticket counter, in three kernels:
+//   K6a  computes each of the 256 rays' product Q over the occluder range,
+//        takes A(C_s) from the segment before it (published by that warp; a
+//        bounded wait) and publishes A(C_s+1) = A(C_s) Q for the next one.  Q
+//        comes before the wait, so the segments of a long list run side by
+//        side and only the last step is chained.
+//   K6b  walks the receivers of the segments that some ray enters open, with
+//        the products P = A(C_s) q, q the running product of the range's
+//        occluders, summing (beta P, beta) per receiver into the (tile,
+//        Gaussian) partials.
+//   K6c  adds up beta alone in the segments that every ray enters stopped.
 //
-// Ray stop: a ray takes occluders only while its product P = A(C_s) q stays
-// >= kShadowStop; the occluder that takes P below it is the ray's last, and
-// P stays frozen for the rest of that segment's receivers.  A(C_s+1) of a ray
-// that stopped is published as 0 (the receivers of later segments see 0; an
-// exact product there is below kShadowStop as well).  The publication and
-// the walk agree on where a ray stops: both multiply the same factors in the
-// same order and compare round(A(C_s) q) with the stop, which is monotone in
-// q.  Thread layout as in the splat evaluation: lane l owns column l & 15,
-// rows (l >> 4) + 2 i, i = 0..7, which is ray 32 i + l of the tile.
+// Ray stop: a ray takes occluders only while its product P stays >=
+// kShadowStop; the occluder that takes it below is the ray's last, and the
+// receivers behind it see 0 (an exact product there is below kShadowStop as
+// well).  K6a decides which segment a ray stops in (it publishes 0 from there
+// on) and that segment's K6b records where: at the occluder whose factor takes
+// P below the stop or, should the two products round to different sides of
+// it, at the end of the range.  Thread layout as in the splat evaluation:
+// lane l owns column l & 15, rows (l >> 4) + 2 i, i = 0..7, which is ray
+// 32 i + l of the tile.
+//
+// Bound: issue slots and the FMA pipe (every pixel test is a power, an ex2 and
+// a select).  So rays go in pairs through the packed FP32 instructions, an
+// occluder updates P alone (a retired ray holds -0.0, which no factor changes
+// and an unsigned minimum passes over, so no pixel needs a test of its own),
+// and receivers and occluders come from one merged list, staged 32 at a time.
+// Object workload (300k Gaussians, 800 x 800, 12.8 M light entries): K6a 0.377
+// -> 0.272 ms, K6b 0.784 -> 0.453 ms, K6c 0.326 -> 0.172 ms (entries picked
+// by their Gaussian's flags before their records are read, and only of
+// Gaussians with a positive numerator), reduction 0.034 -> 0.013 ms; at 1 M and
+// 1024 x 1024 K6a 1.095 -> 0.758, K6b 2.119 -> 1.122, K6c 2.081 -> 0.896 ms.
 // ---------------------------------------------------------------------------
 constexpr int kSegWarps = 4;        // independent warps per block
-constexpr int kRecv = 32;           // receivers staged at a time
 constexpr int kOccWin = 32;         // occluder window
-constexpr int kRedGroup = 16;       // receivers whose per-lane sums are reduced together
 constexpr int kPx = 8;              // rays per lane
 constexpr int kSegSpin = 1 << 20;   // polls of a predecessor's publication before giving up
 
@@ -65,6 +74,10 @@ struct ShadowParams {
   const uint32_t* tile_order;  // tiles by decreasing segment count
   const uint32_t* lvl_off;     // [kSegLevels + 1]: first work item of each segment level
   uint32_t* ticket;            // [3] work counters of K6a, K6b and K6c (zeroed per frame)
+  uint32_t* counts;            // [2] items in open_list and dead_list (zeroed per frame)
+  uint4* desc;                 // [item]: tile and kSegLast, first and past-the-last receiver, preceding item
+  uint32_t* open_list;         // items some ray enters open (K6b's), in no particular order
+  uint32_t* dead_list;         // items every ray enters stopped (K6c's)
   float* pub_a;                // [item][256]: A(C_s+1) published by item
   uint32_t* pub_flag;          // [item]: 0 not yet, 1 published, 2 published and every ray stopped
   uint8_t* pass_mask;  // per list entry: halves with a passing pixel, 0x3 rows 0-7, 0xC rows 8-15
@@ -72,27 +85,38 @@ struct ShadowParams {
   float* light_final;     // per light pixel: the product where the ray ended
   uint32_t* light_stop;   // per light pixel: 1 + index of the occluder that stopped it, or kNoStop
   uint32_t* status;
-  uint8_t* live_rank;  // per light rank: 1 if an entry of it lies in a segment with an open ray (K6b)
-  uint8_t* den_found;  // per light rank: 1 once K6c found a passing pixel of a Gaussian with no such entry
+  uchar2* rank_flags;  // per light rank: (some receiver's sum beta P > 0, some pixel known to pass)
   int W, H, gx;
   float amax;
 };
 
-struct ShadowSmem {  // one warp's
-  float ain[kPx * 32];     // A(C_s) of the segment's rays (ray 32 i + lane)
-  uint32_t xlim[kPx * 32]; // 1 + the occluder after which a ray stopped in this segment, or 0
-  float4 r0[kRecv], r1[kRecv];
-  uint32_t rk[kRecv], rslot[kRecv];
-  float4 o0[kOccWin], o1[kOccWin];
-  float2 red[kRedGroup][33];  // per receiver of the group, per lane: (num, den); padded row
+constexpr uint32_t kSegLast = 0x80000000u;  // desc.x: the tile's last segment
+constexpr uint32_t kNoItem = 0xFFFFFFFFu;   // desc.w: the tile's first segment
+constexpr int kRowPad = 17;                 // a receiver's row of 16 lane sums, padded
+
+// Entries staged for a warp's rays, the terms that pair up duplicated so that
+// they load as packed operands.
+struct StagedEntries {
+  float4 yc[32];   // -y, -y, c, c
+  float4 xart[32]; // x, a, r, threshold
+  float2 gb[32];   // -gamma, halves (as bits)
 };
 
-// one list entry, staged: make_entry's record plus the halves its box and
-// ellipse both reach (in e1.w)
-__device__ __forceinline__ void stage_entry(const ShadowParams& p, uint32_t idx, float ox, float oy, float4& e0,
-                                            float4& e1) {
-  make_entry(p.rrec[p.list[idx]], ox, oy, e0, e1);
-  e1.w = __uint_as_float(__float_as_uint(e1.w) & ellipse_halves(e0, e1));
+struct ShadowSmem {  // one warp's
+  StagedEntries e;
+  f32x2 red[32][kRowPad];  // per receiver of the batch, per lane pair: (num, den)
+};
+
+// Stages one entry in slot t: make_entry's record, and the halves its box
+// and ellipse both reach, which are returned.
+__device__ __forceinline__ uint32_t stage_entry(const SplatRec& q, float ox, float oy, StagedEntries& E, int t) {
+  float4 e0, e1;
+  make_entry(q, ox, oy, e0, e1);
+  const uint32_t bits = __float_as_uint(e1.w) & ellipse_halves(e0, e1);
+  E.yc[t] = make_float4(-e0.y, -e0.y, e0.w, e0.w);
+  E.xart[t] = make_float4(e0.x, e0.z, e1.x, e1.y);
+  E.gb[t] = make_float2(-e1.z, __uint_as_float(bits));
+  return bits;
 }
 
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* a) {
@@ -104,227 +128,117 @@ __device__ __forceinline__ void st_release(uint32_t* a, uint32_t v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(a), "r"(v) : "memory");
 }
 
-// A receiver's four rays of one half: den += beta and num += beta a_i at the
-// rays where it passes (power2 >= thr), beta = 2^power2.  Predicated, no branch.
-template <bool WITH_NUM, int H>
-__device__ __forceinline__ void recv_half(const float (&ly)[kPx], const float (&a)[kPx], float y, float c, float v,
-                                          float sx, float thr, float& num, float& den) {
+// beta of one pixel: 2^pw where it passes (pw >= thr), else 0
+__device__ __forceinline__ float beta_of(float pw, float thr) { return pw >= thr ? ex2(pw) : 0.f; }
+
+// (beta, beta) of two pixels from their packed powers
+__device__ __forceinline__ f32x2 beta2_of(f32x2 pw, float thr) {
+  return pk2(beta_of(lo2(pw), thr), beta_of(hi2(pw), thr));
+}
+
+// An entry's terms that a lane's rays share (one column): with dy = ly - y,
+// power2 = fma(dy, fma(c, dy, v), sx), the arithmetic of splat_eval.cuh.
+struct ColTerms {
+  f32x2 ny, c, v, s;
+  float thr;
+};
+__device__ __forceinline__ ColTerms col_terms(float lx, const StagedEntries& E, int t) {
+  const ulonglong2 yc = *reinterpret_cast<const ulonglong2*>(&E.yc[t]);
+  const float4 q = E.xart[t];
+  const float dx = lx - q.x;
+  return {yc.x, yc.y, dup2(q.z * dx), dup2((q.y * dx) * dx), q.w};
+}
+__device__ __forceinline__ f32x2 beta2_at(const ColTerms& e, f32x2 ly) {
+  const f32x2 dy = add2(ly, e.ny);
+  return beta2_of(fma2(dy, fma2(e.c, dy, e.v), e.s), e.thr);
+}
+
+// A receiver's four rays of one half: den += beta and num += beta P.
+template <int H>
+__device__ __forceinline__ void recv_half(const f32x2 (&ly)[kPx / 2], const f32x2 (&P)[kPx / 2], const ColTerms& e,
+                                          f32x2& num, f32x2& den) {
 #pragma unroll
-  for (int qq = 0; qq < 4; ++qq) {
-    const int i = 4 * H + qq;
-    const float dy = ly[i] - y;
-    const float pw = fmaf(dy, fmaf(c, dy, v), sx);
-    if (WITH_NUM)
-      asm("{\n\t.reg .pred p;\n\t.reg .f32 b;\n\t"
-          "setp.ge.f32 p, %2, %3;\n\t"
-          "@p ex2.approx.ftz.f32 b, %2;\n\t"
-          "@p add.rn.f32 %1, %1, b;\n\t"
-          "@p fma.rn.f32 %0, b, %4, %0;\n\t}"
-          : "+f"(num), "+f"(den) : "f"(pw), "f"(thr), "f"(a[i]));
-    else
-      asm("{\n\t.reg .pred p;\n\t.reg .f32 b;\n\t"
-          "setp.ge.f32 p, %1, %2;\n\t"
-          "@p ex2.approx.ftz.f32 b, %1;\n\t"
-          "@p add.rn.f32 %0, %0, b;\n\t}"
-          : "+f"(den) : "f"(pw), "f"(thr));
+  for (int q = 2 * H; q < 2 * H + 2; ++q) {
+    const f32x2 b = beta2_at(e, ly[q]);
+    den = add2(den, b);
+    num = fma2(b, P[q], num);
   }
 }
 
-// An occluder on four rays of one half, each still taking occluders
-// (A q >= stop): q *= max(omin, 1 - gamma 2^power2) where it passes, then
-// P = A q.  Returns bit qq set for the rays whose P fell below the stop here.
-template <int I>
-__device__ __forceinline__ uint32_t occ_ray(const float (&ly)[kPx], uint32_t ain, float (&q)[kPx], float (&P)[kPx],
-                                            float y, float c, float v, float sx, float thr, float ngamma,
-                                            float omin) {
-  const float dy = ly[I] - y;
-  const float pw = fmaf(dy, fmaf(c, dy, v), sx);
-  uint32_t x;
-  // ain: shared-memory address of the lane's A(C_s) of ray 0; ray I at + 128 I
-  asm("{\n\t.reg .pred a, p, c;\n\t.reg .f32 b, f, e;\n\t"
-      "setp.ge.f32 a, %1, %7;\n\t"           // still taking occluders
-      "setp.ge.and.f32 p, %3, %4, a;\n\t"    // and this one passes
-      "@p ex2.approx.ftz.f32 b, %3;\n\t"
-      "@p ld.shared.f32 e, [%8+%9];\n\t"
-      "@p fma.rn.f32 f, %5, b, 0f3F800000;\n\t"
-      "@p max.f32 f, f, %6;\n\t"
-      "@p mul.rn.f32 %0, %0, f;\n\t"
-      "@p mul.rn.f32 %1, e, %0;\n\t"
-      "setp.lt.and.f32 c, %1, %7, p;\n\t"    // its last one
-      "selp.u32 %2, 1, 0, c;\n\t}"
-      : "+f"(q[I]), "+f"(P[I]), "=r"(x)
-      : "f"(pw), "f"(thr), "f"(ngamma), "f"(omin), "f"(kShadowStop), "r"(ain), "n"(128 * I));
-  return x << I;
+// An occluder on four rays of one half: P *= max(omin, 1 - gamma beta), which
+// is P itself where it does not pass.
+template <int H>
+__device__ __forceinline__ void occ_half(const f32x2 (&ly)[kPx / 2], f32x2 (&P)[kPx / 2], const ColTerms& e,
+                                         float ngamma, float omin) {
+#pragma unroll
+  for (int q = 2 * H; q < 2 * H + 2; ++q) {
+    const f32x2 f = fma2(dup2(ngamma), beta2_at(e, ly[q]), dup2(1.f));
+    P[q] = mul2(P[q], pk2(fmaxf(lo2(f), omin), fmaxf(hi2(f), omin)));
+  }
 }
 
-template <int H>
-__device__ __forceinline__ uint32_t occ_half(const float (&ly)[kPx], uint32_t ain, float (&q)[kPx], float (&P)[kPx],
-                                             float y, float c, float v, float sx, float thr, float ngamma,
-                                             float omin) {
-  return occ_ray<4 * H + 0>(ly, ain, q, P, y, c, v, sx, thr, ngamma, omin) |
-         occ_ray<4 * H + 1>(ly, ain, q, P, y, c, v, sx, thr, ngamma, omin) |
-         occ_ray<4 * H + 2>(ly, ain, q, P, y, c, v, sx, thr, ngamma, omin) |
-         occ_ray<4 * H + 3>(ly, ain, q, P, y, c, v, sx, thr, ngamma, omin);
+// The lane's rays in pairs: the row offset of ray i (row (lane >> 4) + 2 i),
+// far away where the ray is not in the image
+__device__ __forceinline__ void lane_rows(int lane, int rows_in, f32x2 (&ly)[kPx / 2]) {
+#pragma unroll
+  for (int q = 0; q < kPx / 2; ++q) {
+    const float y = (float)(lane >> 4) + 4 * q + 0.5f;
+    ly[q] = pk2(2 * q < rows_in ? y : 1.0e6f, 2 * q + 1 < rows_in ? y + 2.f : 1.0e6f);
+  }
 }
 
 // halves (0x3, 0xC) with a ray whose product is still >= the stop
-__device__ __forceinline__ uint32_t live_halves(const float (&P)[kPx]) {
-  bool h0 = false, h1 = false;
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    h0 |= P[i] >= kShadowStop;
-    h1 |= P[4 + i] >= kShadowStop;
-  }
+__device__ __forceinline__ uint32_t live_halves(const f32x2 (&P)[kPx / 2]) {
+  const bool h0 = fmaxf(fmaxf(lo2(P[0]), hi2(P[0])), fmaxf(lo2(P[1]), hi2(P[1]))) >= kShadowStop;
+  const bool h1 = fmaxf(fmaxf(lo2(P[2]), hi2(P[2])), fmaxf(lo2(P[3]), hi2(P[3]))) >= kShadowStop;
   return (__any_sync(0xffffffffu, h0) ? 0x3u : 0u) | (__any_sync(0xffffffffu, h1) ? 0xCu : 0u);
 }
 
-// The per-warp state of one segment (item) of the shadow composite.
-struct SegState {
-  int lane, tx, ty, s;
-  float lx, ox, oy, omin;
-  uint32_t C1;
-  uint32_t k, wb, we;  // next occluder; staged occluder window [wb, we)
-  uint32_t live;       // halves with a ray still taking occluders
-  size_t pix0;         // the lane's first pixel
-};
-
-// Walks occluders up to kend (exclusive), staging windows of the range as it
-// goes; a ray whose product falls below the stop records where it ended.
-__device__ __forceinline__ void walk_to(const ShadowParams& p, ShadowSmem& S, SegState& st, uint32_t kend,
-                                        const float (&ly)[kPx], uint32_t ain, float (&q)[kPx], float (&P)[kPx]) {
-  while (st.live && st.k < kend) {
-    if (st.k == st.we) {
-      __syncwarp();
-      st.wb = st.k;
-      st.we = min(st.k + (uint32_t)kOccWin, st.C1);
-      for (uint32_t t = st.lane; t < st.we - st.wb; t += 32)
-        stage_entry(p, st.wb + t, st.ox, st.oy, S.o0[t], S.o1[t]);
-      __syncwarp();
-    }
-    const uint32_t stop_at = min(kend, st.we);
-    for (; st.k < stop_at; ++st.k) {
-      const int t = (int)(st.k - st.wb);
-      const float4 o1 = S.o1[t];
-      const uint32_t bits = __float_as_uint(o1.w) & st.live;
-      if (!bits) continue;
-      const float4 o0 = S.o0[t];
-      const float dx = st.lx - o0.x;
-      const float sx = (o0.z * dx) * dx, v = o1.x * dx;
-      uint32_t crossed = 0u;
-      if (bits & 0x3u) crossed = occ_half<0>(ly, ain, q, P, o0.y, o0.w, v, sx, o1.y, -o1.z, st.omin);
-      if (bits & 0xCu) crossed |= occ_half<1>(ly, ain, q, P, o0.y, o0.w, v, sx, o1.y, -o1.z, st.omin);
-      if (crossed) {  // rare: the ray's last occluder (its product stays frozen from here)
-#pragma unroll
-        for (int i = 0; i < kPx; ++i)
-          if (crossed & (1u << i)) S.xlim[32 * i + st.lane] = st.k + 1;
-      }
-    }
-    st.live = live_halves(P);
-  }
-  if (!st.live) st.k = max(st.k, kend);
-}
-
-// Stages receivers [rb, rb + rc) of the segment into shared memory.
-__device__ __forceinline__ void stage_receivers(const ShadowParams& p, ShadowSmem& S, const SegState& st, uint32_t rb,
-                                                int rc) {
-  __syncwarp();  // the previous batch is consumed
-  for (int t = st.lane; t < rc; t += 32) {
-    const uint32_t rank = p.list[rb + t];
-    const SplatRec qr = p.rrec[rank];
-    float4 e0, e1;
-    make_entry(qr, st.ox, st.oy, e0, e1);
-    e1.w = __uint_as_float(__float_as_uint(e1.w) & ellipse_halves(e0, e1));
-    S.r0[t] = e0;
-    S.r1[t] = e1;
-    S.rk[t] = p.kbound[rb + t];
-    S.rslot[t] = p.off[rank] + (uint32_t)((st.ty - qr.r.y) * (qr.r.z - qr.r.x + 1) + (st.tx - qr.r.x));
-    p.live_rank[rank] = 1;
-  }
-  __syncwarp();
-}
-
-// Receiver jj of the batch at rb: its per-lane (num, den) to a row, its pass
-// halves to pass_mask; every kRedGroup receivers (and at the batch's end)
-// lane t < 16 adds num of receiver j0 + t over the 32 lanes, lane 16 + t its
-// den, in lane order, into the (tile, Gaussian) partial.
-__device__ __forceinline__ void finish_receiver(const ShadowParams& p, ShadowSmem& S, int lane, uint32_t rb, int jj,
-                                                int rc, float num, float den0, float den1) {
-  const uint32_t bits = (__any_sync(0xffffffffu, den0 > 0.f) ? 0x3u : 0u) |
-                        (__any_sync(0xffffffffu, den1 > 0.f) ? 0xCu : 0u);
-  S.red[jj % kRedGroup][lane] = make_float2(num, den0 + den1);
-  if (lane == 0) p.pass_mask[rb + jj] = (uint8_t)bits;
-  if (jj % kRedGroup == kRedGroup - 1 || jj == rc - 1) {
-    __syncwarp();
-    const int j0 = jj - jj % kRedGroup;
-    const int t = lane & 15, c = lane >> 4;
-    if (j0 + t <= jj) {
-      const float* row = reinterpret_cast<const float*>(S.red[t]) + c;
-      float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll
-      for (int l = 0; l < 32; l += 4) {
-        a0 += row[2 * l]; a1 += row[2 * l + 2]; a2 += row[2 * l + 4]; a3 += row[2 * l + 6];
-      }
-      reinterpret_cast<float*>(p.partial)[2 * (size_t)S.rslot[j0 + t] + c] = (a0 + a1) + (a2 + a3);
-    }
-    __syncwarp();  // the group's rows are free again
-  }
+// The smallest product among the lane's rays, as bits: a retired ray holds
+// -0.0, whose bits are above every positive product's.
+__device__ __forceinline__ uint32_t min_bits(const f32x2 (&P)[kPx / 2]) {
+  uint32_t m = __vimin3_u32((uint32_t)P[0], (uint32_t)(P[0] >> 32), (uint32_t)P[1]);
+  m = __vimin3_u32(m, (uint32_t)(P[1] >> 32), (uint32_t)P[2]);
+  m = __vimin3_u32(m, (uint32_t)(P[2] >> 32), (uint32_t)P[3]);
+  return min(m, (uint32_t)(P[3] >> 32));
 }
 
 // A(C_s) of the lane's rays: 1 / 0 (in / outside the image) for a tile's
 // first segment, else the predecessor's publication (read from L2: it was
 // written on another SM); flag 2 publishes that every ray stopped.
-__device__ __forceinline__ void load_entering(const ShadowParams& p, int s, uint32_t wpred, uint32_t flag, int lane,
-                                              int rows_in, float (&A)[kPx]) {
+__device__ __forceinline__ void load_entering(const ShadowParams& p, bool first, uint32_t wpred, uint32_t flag, int lane,
+                                              int rows_in, f32x2 (&A)[kPx / 2]) {
+  auto one = [&](int i) {
+    return first ? (i < rows_in ? 1.f : 0.f)
+                 : (flag == 2u ? 0.f : __ldcg(p.pub_a + (size_t)wpred * 256 + 32 * i + lane));
+  };
 #pragma unroll
-  for (int i = 0; i < kPx; ++i)
-    A[i] = s == 0 ? (i < rows_in ? 1.f : 0.f)
-                  : (flag == 2u ? 0.f : __ldcg(p.pub_a + (size_t)wpred * 256 + 32 * i + lane));
+  for (int q = 0; q < kPx / 2; ++q) A[q] = pk2(one(2 * q), one(2 * q + 1));
 }
 
-__device__ __forceinline__ bool all_stopped(const float (&A)[kPx]) {
-  bool any = false;
-#pragma unroll
-  for (int i = 0; i < kPx; ++i) any |= A[i] >= kShadowStop;
-  return !__any_sync(0xffffffffu, any);
-}
-
-// den + 2^pw where pw >= thr (predicated, no branch)
-__device__ __forceinline__ float recv_den(float pw, float thr, float den) {
-  asm("{\n\t.reg .pred p;\n\t.reg .f32 b;\n\t"
-      "setp.ge.f32 p, %1, %2;\n\t"
-      "@p ex2.approx.ftz.f32 b, %1;\n\t"
-      "@p add.rn.f32 %0, %0, b;\n\t}"
-      : "+f"(den) : "f"(pw), "f"(thr));
-  return den;
-}
-
-// The segment a work item names: its level s (segment index) and tile, the
-// levels being prefixes of the tile order.
+// The segment a work item names.
 struct SegItem {
-  int s, tile, tx, ty, rows_in;
+  int tx, ty, rows_in;
   uint32_t R0, R1, C0, C1, wpred;
-  bool last;
+  bool first, last;
 };
 
 __device__ __forceinline__ SegItem seg_item(const ShadowParams& p, uint32_t w, int lane) {
+  const uint4 d = p.desc[w];
   SegItem it;
-  int lo = 0, hi = kSegLevels;  // largest s with lvl_off[s] <= w
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (p.lvl_off[mid] <= w) lo = mid; else hi = mid;
+  const int tile = (int)(d.x & ~kSegLast);
+  it.last = (d.x & kSegLast) != 0u;
+  it.first = d.w == kNoItem;
+  it.tx = tile % p.gx;
+  it.ty = tile / p.gx;
+  it.R0 = d.y;
+  it.R1 = d.z;
+  it.wpred = d.w;
+  it.C0 = it.C1 = it.R0;
+  if (it.R1 > it.R0) {  // an empty tile has one segment without entries
+    it.C0 = p.kbound[it.R0];
+    it.C1 = p.kbound[it.last ? it.R1 - 1 : it.R1];
   }
-  it.s = lo;
-  const uint32_t pos = w - p.lvl_off[lo];
-  it.tile = (int)p.tile_order[pos];
-  it.tx = it.tile % p.gx;
-  it.ty = it.tile / p.gx;
-  const uint32_t b = p.tile_start[it.tile], e = p.tile_start[it.tile + 1];
-  it.last = (uint32_t)lo == seg_count(e - b) - 1;
-  it.R0 = b + (uint32_t)lo * kSegLen;
-  it.R1 = it.last ? e : it.R0 + kSegLen;
-  it.C0 = e > b ? p.kbound[it.R0] : b;
-  it.C1 = e > b ? (it.last ? p.kbound[e - 1] : p.kbound[it.R1]) : b;
-  it.wpred = lo > 0 ? p.lvl_off[lo - 1] + pos : 0u;
   // ray i of the lane is row (lane >> 4) + 2 i: rows below the image hold no ray
   const int lxi = lane & 15, lyi = lane >> 4;
   it.rows_in = it.tx * kTile + lxi < p.W ? min(kPx, (p.H - it.ty * kTile - lyi + 1) / 2) : 0;
@@ -340,129 +254,110 @@ __device__ __forceinline__ bool next_item(uint32_t* ticket, uint32_t total, int 
 }
 
 // K6a: A(C_s+1) of every segment but a tile's last, chained from A(C_s).
-// Step 1 (the range's products Q) runs before the chain is known, so the
-// segments of a list run side by side and only the combination is chained.
-__device__ __forceinline__ void chain_item(const ShadowParams& p, uint32_t w, ShadowSmem& S, int lane) {
-  const int lxi = lane & 15, lyi = lane >> 4;
-  const float lx = lxi + 0.5f, omin = 1.f - p.amax;
-  const uint32_t ain = (uint32_t)__cvta_generic_to_shared(&S.ain[lane]);
-
-    const SegItem it = seg_item(p, w, lane);
-    if (it.last) return;  // nothing follows it
-    const float ox = (float)(it.tx * kTile), oy = (float)(it.ty * kTile);
-    float ly[kPx];
+__device__ __forceinline__ void chain_item(const ShadowParams& p, uint32_t w, StagedEntries& S, int lane) {
+  const float lx = (lane & 15) + 0.5f, omin = 1.f - p.amax;
+  const SegItem it = seg_item(p, w, lane);
+  if (it.last) return;  // nothing follows it
+  const float ox = (float)(it.tx * kTile), oy = (float)(it.ty * kTile);
+  f32x2 ly[kPx / 2];
+  lane_rows(lane, it.rows_in, ly);
+  // A(C_s): known now for the first segment, or when the predecessor
+  // published already; until then A = 1 stands in (A <= 1)
+  uint32_t flag = 1u;
+  if (!it.first && lane == 0) flag = ld_acquire(p.pub_flag + it.wpred);
+  flag = __shfl_sync(0xffffffffu, flag, 0);
+  __syncwarp();  // orders every lane's reads after lane 0's acquire
+  bool known = flag != 0u;
+  f32x2 A[kPx / 2];
+  load_entering(p, it.first || !known, it.wpred, flag, lane, it.rows_in, A);
+  // the range's products Q; once no ray's A Q stays at the stop the rest of
+  // the range changes nothing (each ray stops in it either way)
+  f32x2 Q[kPx / 2];
 #pragma unroll
-    for (int i = 0; i < kPx; ++i) ly[i] = i < it.rows_in ? lyi + 2 * i + 0.5f : 1.0e6f;
-    // A(C_s): known now for the first segment, or when the predecessor
-    // published already; until then A = 1 stands in (A <= 1)
-    uint32_t flag = 1u;
-    if (it.s > 0 && lane == 0) flag = ld_acquire(p.pub_flag + it.wpred);
-    flag = __shfl_sync(0xffffffffu, flag, 0);
-    __syncwarp();  // orders every lane's reads after lane 0's acquire
-    bool known = flag != 0u;
-    float A[kPx];
-    if (known) {
-      load_entering(p, it.s, it.wpred, flag, lane, it.rows_in, A);
-    } else {
-#pragma unroll
-      for (int i = 0; i < kPx; ++i) A[i] = i < it.rows_in ? 1.f : 0.f;
-    }
-    const bool dead = known && all_stopped(A);
-    // the range's products Q; a ray drops out once A Q < stop (it stops
-    // either way); the product so far is the same whichever A stood in
-    float Q[kPx], PQ[kPx];
-#pragma unroll
-    for (int i = 0; i < kPx; ++i) {
-      Q[i] = 1.f;
-      PQ[i] = A[i] >= kShadowStop ? A[i] : 0.f;
-    }
-    if (!dead) {
-      __syncwarp();
-#pragma unroll
-      for (int i = 0; i < kPx; ++i) S.ain[32 * i + lane] = A[i];
-      uint32_t live = live_halves(PQ);
-      for (uint32_t wb = it.C0; wb < it.C1 && live; wb += kOccWin) {
-        if (!known) {  // the predecessor may have published meanwhile
-          uint32_t fl = 0u;
-          if (lane == 0) fl = ld_acquire(p.pub_flag + it.wpred);
-          fl = __shfl_sync(0xffffffffu, fl, 0);
-          __syncwarp();
-          if (fl != 0u) {
-            known = true;
-            load_entering(p, it.s, it.wpred, fl, lane, it.rows_in, A);
-#pragma unroll
-            for (int i = 0; i < kPx; ++i) {
-              S.ain[32 * i + lane] = A[i];
-              PQ[i] = A[i] >= kShadowStop ? A[i] * Q[i] : 0.f;
-            }
-            live = live_halves(PQ);
-            if (!live) break;
-          }
-        }
-        const int wc = (int)min((uint32_t)kOccWin, it.C1 - wb);
-        __syncwarp();
-        for (int t = lane; t < wc; t += 32) stage_entry(p, wb + t, ox, oy, S.o0[t], S.o1[t]);
-        __syncwarp();
-        for (int t = 0; t < wc; ++t) {
-          const float4 o1 = S.o1[t];
-          const uint32_t bits = __float_as_uint(o1.w) & live;
-          if (!bits) continue;
-          const float4 o0 = S.o0[t];
-          const float dx = lx - o0.x;
-          const float sx = (o0.z * dx) * dx, v = o1.x * dx;
-          if (bits & 0x3u) occ_half<0>(ly, ain, Q, PQ, o0.y, o0.w, v, sx, o1.y, -o1.z, omin);
-          if (bits & 0xCu) occ_half<1>(ly, ain, Q, PQ, o0.y, o0.w, v, sx, o1.y, -o1.z, omin);
-        }
-        live = live_halves(PQ);
-      }
-    }
-    // A(C_s) from the predecessor (bounded wait), then A(C_s+1) for the successor
-    if (!known) {
+  for (int q = 0; q < kPx / 2; ++q) Q[q] = dup2(1.f);
+  uint32_t live = live_halves(A);
+  for (uint32_t wb = it.C0; wb < it.C1 && live; wb += kOccWin) {
+    if (!known) {  // the predecessor may have published meanwhile
       uint32_t fl = 0u;
-      if (lane == 0) {
-        int spins = 0;
-        while ((fl = ld_acquire(p.pub_flag + it.wpred)) == 0u) {
-          if (++spins > kSegSpin) {
-            atomicCAS(p.status, 0u, (uint32_t)GS3_ERR_TIMEOUT);
-            fl = 2u;  // give up: the frame is reported invalid, the warp finishes
-            break;
-          }
-          __nanosleep(64);
-        }
-      }
+      if (lane == 0) fl = ld_acquire(p.pub_flag + it.wpred);
       fl = __shfl_sync(0xffffffffu, fl, 0);
       __syncwarp();
-      load_entering(p, it.s, it.wpred, fl, lane, it.rows_in, A);
-    }
-    const bool dead_in = all_stopped(A);
-    bool any = false;
-#pragma unroll
-    for (int i = 0; i < kPx; ++i) {
-      float a = 0.f;
-      if (A[i] >= kShadowStop) {
-        a = A[i] * Q[i];
-        if (!(a >= kShadowStop)) a = 0.f;  // the ray stops in this range
+      if (fl != 0u) {
+        known = true;
+        load_entering(p, false, it.wpred, fl, lane, it.rows_in, A);
       }
-      any |= a != 0.f;
-      if (!dead_in) p.pub_a[(size_t)w * 256 + 32 * i + lane] = a;
     }
-    const bool any_out = __any_sync(0xffffffffu, any);
-    __threadfence();  // every lane's products before the flag
+    f32x2 AQ[kPx / 2];
+#pragma unroll
+    for (int q = 0; q < kPx / 2; ++q) AQ[q] = mul2(A[q], Q[q]);
+    live = live_halves(AQ);
+    if (!live) break;
+    const int wc = (int)min((uint32_t)kOccWin, it.C1 - wb);
     __syncwarp();
-    if (lane == 0) st_release(p.pub_flag + w, any_out ? 1u : 2u);
+    if (lane < wc) stage_entry(p.rrec[p.list[wb + lane]], ox, oy, S, lane);
+    __syncwarp();
+    for (int t = 0; t < wc; ++t) {
+      const float2 gb = S.gb[t];
+      const uint32_t bits = __float_as_uint(gb.y) & live;
+      if (!bits) continue;
+      const ColTerms e = col_terms(lx, S, t);
+      if (bits & 0x3u) occ_half<0>(ly, Q, e, gb.x, omin);
+      if (bits & 0xCu) occ_half<1>(ly, Q, e, gb.x, omin);
+    }
   }
+  // A(C_s) from the predecessor (bounded wait), then A(C_s+1) for the successor
+  if (!known) {
+    uint32_t fl = 0u;
+    if (lane == 0) {
+      int spins = 0;
+      while ((fl = ld_acquire(p.pub_flag + it.wpred)) == 0u) {
+        if (++spins > kSegSpin) {
+          atomicCAS(p.status, 0u, (uint32_t)GS3_ERR_TIMEOUT);
+          fl = 2u;  // give up: the frame is reported invalid, the warp finishes
+          break;
+        }
+        __nanosleep(64);
+      }
+    }
+    fl = __shfl_sync(0xffffffffu, fl, 0);
+    __syncwarp();
+    load_entering(p, false, it.wpred, fl, lane, it.rows_in, A);
+  }
+  const bool dead_in = live_halves(A) == 0u;
+  bool any = false;
+#pragma unroll
+  for (int q = 0; q < kPx / 2; ++q) {
+    const f32x2 AQ = mul2(A[q], Q[q]);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float a = h ? hi2(AQ) : lo2(AQ);
+      if (!(a >= kShadowStop)) a = 0.f;  // the ray stopped in this range or before it
+      any |= a != 0.f;
+      if (!dead_in) p.pub_a[(size_t)w * 256 + 64 * q + 32 * h + lane] = a;
+    }
+  }
+  const bool any_out = __any_sync(0xffffffffu, any);
+  __threadfence();  // every lane's products before the flag
+  __syncwarp();
+  if (lane == 0) st_release(p.pub_flag + w, any_out ? 1u : 2u);
+}
 
 // The work items of a batch of frames: the tickets run over every frame's
-// items in turn; locate() maps a ticket to its frame and the frame's item.
-__device__ __forceinline__ uint32_t batch_items(const ShadowParams* reqs, int nreq) {
+// items in turn; locate() maps a ticket to its frame and the frame's item
+// (or, for K6b and K6c, its place in the frame's list of such items).
+enum { kAllItems = 0, kOpenItems = 1, kDeadItems = 2 };
+__device__ __forceinline__ uint32_t item_count(const ShadowParams& p, int kind) {
+  return kind == kAllItems ? p.lvl_off[kSegLevels] : p.counts[kind - 1];
+}
+__device__ __forceinline__ uint32_t batch_items(const ShadowParams* reqs, int nreq, int kind) {
   uint32_t t = 0;
-  for (int r = 0; r < nreq; ++r) t += reqs[r].lvl_off[kSegLevels];
+  for (int r = 0; r < nreq; ++r) t += item_count(reqs[r], kind);
   return t;
 }
-__device__ __forceinline__ int locate(const ShadowParams* reqs, int nreq, uint32_t& w) {
+__device__ __forceinline__ int locate(const ShadowParams* reqs, int nreq, int kind, uint32_t& w) {
   int r = 0;
   for (; r < nreq - 1; ++r) {
-    const uint32_t t = reqs[r].lvl_off[kSegLevels];
+    const uint32_t t = item_count(reqs[r], kind);
     if (w < t) break;
     w -= t;
   }
@@ -470,18 +365,19 @@ __device__ __forceinline__ int locate(const ShadowParams* reqs, int nreq, uint32
 }
 
 // One frame (p) or a batch of nreq frames (reqs, in device memory; p is the
-// first, whose tickets the batch shares).
+// first, whose tickets the batch shares).  5 blocks per SM: 0.272 ms against
+// 0.279 at 4, 0.287 at 6 and 0.314 at 8.
 template <bool BATCH>
-__global__ void __launch_bounds__(kSegWarps * 32, 4) k_shadow_chain(const ShadowParams p, const ShadowParams* reqs,
+__global__ void __launch_bounds__(kSegWarps * 32, 5) k_shadow_chain(const ShadowParams p, const ShadowParams* reqs,
                                                                     int nreq) {
-  __shared__ ShadowSmem smem[kSegWarps];
-  ShadowSmem& S = smem[threadIdx.x >> 5];
+  __shared__ StagedEntries smem[kSegWarps];
+  StagedEntries& S = smem[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
-  const uint32_t total = BATCH ? batch_items(reqs, nreq) : p.lvl_off[kSegLevels];
+  const uint32_t total = BATCH ? batch_items(reqs, nreq, kAllItems) : item_count(p, kAllItems);
   uint32_t w;
   while (next_item(p.ticket, total, lane, w)) {
     if (BATCH) {
-      const int r = locate(reqs, nreq, w);
+      const int r = locate(reqs, nreq, kAllItems, w);
       chain_item(reqs[r], w, S, lane);
     } else {
       chain_item(p, w, S, lane);
@@ -489,60 +385,53 @@ __global__ void __launch_bounds__(kSegWarps * 32, 4) k_shadow_chain(const Shadow
   }
 }
 
-// The light tile of the pixel nearest a splat's centre (k_dead_probe's
-// pixel), or all ones off the image.
-__device__ __forceinline__ uint32_t probe_tile(const SplatRec& q, int W, int H, int gx) {
-  const float cx = q.a.x + q.b.w, cy = q.a.y + q.c.x;
-  if (!(cx >= 0.f && cy >= 0.f && cx < (float)W && cy < (float)H)) return 0xFFFFFFFFu;
-  return (uint32_t)(((int)cy / kTile) * gx + (int)cx / kTile);
-}
-
 // K6c: the receivers of the segments every ray of which stopped before the
 // segment (A(C_s) = 0 throughout, as K6a published).  The products are 0,
 // so a receiver needs only its beta sum over the tile, which depends on no
-// other entry.  A warp stages up to kDeadBatch receivers, lists their
-// (receiver, half) units (the halves their box and ellipse reach), and each
-// lane walks the 16 x 8 pixels of one unit at a time, with the power
-// arithmetic of the ray layout (pixel centres x + 0.5, y + 0.5); the two
-// halves of a receiver are then added in a fixed order.
-// A Gaussian none of whose entries lies in a segment with an open ray (K6b
-// marked those) has a zero numerator everywhere, so its shadow value is 0 if
-// any of its pixels passes and 1 otherwise: the beta sum only has to be
-// known to be positive.  Once that is known (den_found: k_dead_probe found
-// its pixel nearest the centre passing, or one of its units here found a
-// passing pixel), its entries are skipped (partial (0, 0), no pass halves)
-// except the one of the probe tile, which is evaluated in full, so the sum
-// stays positive.  Which other entries are skipped depends on timing; T
-// does not, and the backward takes nothing from such a Gaussian (its
-// products and T are 0).
+// other entry, and only if its Gaussian's numerator is not 0: K6b marked the
+// Gaussians with a positive one (rank_flags.x).  Of any other Gaussian the
+// shadow value is 0 if some pixel passes and 1 if none does, so its entries
+// are needed only until one is known to pass (rank_flags.y: K6b or
+// k_dead_probe found one, or a unit here did), and its partials are neither
+// written nor read.  A warp takes a segment, picks the entries it needs from
+// their flags (before it reads any record), stages up to kDeadBatch of them,
+// lists their (receiver, half) units (the halves their box and ellipse
+// reach), and each lane walks the 16 x 8 pixels of one unit at a time, with
+// the power arithmetic of the ray layout (pixel centres x + 0.5, y + 0.5);
+// the two halves of a receiver are then added in a fixed order.  Which
+// entries of an unmarked Gaussian are evaluated depends on timing; T does not.
 constexpr int kDeadBatch = 128;
 constexpr int kDeadWarps = 4;
+constexpr int kDeadScan = 256;  // entries whose flags are read at a time
 
 struct DeadSmem {  // one warp's
   float4 e0[kDeadBatch], e1[kDeadBatch];
   float den[2][kDeadBatch];
   uint32_t slot[kDeadBatch];      // the receiver's partial slot
-  uint32_t rank[kDeadBatch];      // its depth rank, bit 31 set if K6b saw it
+  uint32_t rank[kDeadScan];       // needed entries: depth rank, bit 31 set if K6b marked it
+  uint8_t at[kDeadScan];          // and their places among the entries read
   uint16_t unit[2 * kDeadBatch];  // receiver (bits 0-7) and half (bit 8) of each unit
 };
 
 // The beta sum of one receiver entry over the 16 x 8 pixels of half h of an
-// interior tile, column by column.
+// interior tile, column by column, pixel pairs in packed registers.
 __device__ __forceinline__ float dead_half(const float4 e0, const float4 e1, int h) {
-  float dy[8];
+  f32x2 dy[4];
   const float y0 = 8.f * h + 0.5f;
 #pragma unroll
-  for (int y = 0; y < 8; ++y) dy[y] = (y0 + (float)y) - e0.y;
-  float den = 0.f, fx = 0.5f;
+  for (int q = 0; q < 4; ++q) dy[q] = pk2((y0 + 2.f * q) - e0.y, (y0 + 2.f * q + 1.f) - e0.y);
+  const f32x2 c = dup2(e0.w);
+  f32x2 den = 0ull;
+  float fx = 0.5f;
 #pragma unroll 1
   for (int x = 0; x < kTile; ++x) {
     const float dx = fx - e0.x;
     fx += 1.f;
-    const float sx = (e0.z * dx) * dx, v = e1.x * dx;
+    const f32x2 sx = dup2((e0.z * dx) * dx), v = dup2(e1.x * dx);
 #pragma unroll
-    for (int y = 0; y < 8; ++y) den = recv_den(fmaf(dy[y], fmaf(e0.w, dy[y], v), sx), e1.y, den);
+    for (int q = 0; q < 4; ++q) den = add2(den, beta2_of(fma2(dy[q], fma2(c, dy[q], v), sx), e1.y));
   }
-  return den;
+  return lo2(den) + hi2(den);
 }
 
 // the same over the pixels of half h that lie inside the image (edge tiles)
@@ -555,7 +444,7 @@ __device__ __forceinline__ float dead_half_edge(const float4 e0, const float4 e1
     float fy = 8.f * h + 0.5f;
     for (int y = 8 * h; y < y1; ++y, fy += 1.f) {
       const float dy = fy - e0.y;
-      den = recv_den(fmaf(dy, fmaf(e0.w, dy, v), sx), e1.y, den);
+      den += beta_of(fmaf(dy, fmaf(e0.w, dy, v), sx), e1.y);
     }
   }
   return den;
@@ -563,92 +452,110 @@ __device__ __forceinline__ float dead_half_edge(const float4 e0, const float4 e1
 
 __device__ __forceinline__ void dead_item(const ShadowParams& p, uint32_t w, DeadSmem& D, int lane) {
 
-    int lo = 0, hi = kSegLevels;  // the item's level: largest s with lvl_off[s] <= w
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (p.lvl_off[mid] <= w) lo = mid; else hi = mid;
-    }
-    if (lo == 0) return;  // a tile's first segment starts with every ray open
-    const uint32_t pos = w - p.lvl_off[lo];
-    if (__ldcg(p.pub_flag + p.lvl_off[lo - 1] + pos) != 2u) return;  // not stopped: K6b's
-    const int tile = (int)p.tile_order[pos];
+    const uint4 d = p.desc[w];
+    const int tile = (int)(d.x & ~kSegLast);
     const int tx = tile % p.gx, ty = tile / p.gx;
     const float ox = (float)(tx * kTile), oy = (float)(ty * kTile);
-    const uint32_t b = p.tile_start[tile], e = p.tile_start[tile + 1];
-    const bool last = (uint32_t)lo == seg_count(e - b) - 1;
-    const uint32_t R0 = b + (uint32_t)lo * kSegLen, R1 = last ? e : R0 + kSegLen;
+    const uint32_t R0 = d.y, R1 = d.z;
     const int ncol = min(kTile, p.W - tx * kTile), nrow = min(kTile, p.H - ty * kTile);
     const bool interior = ncol == kTile && nrow == kTile;
-    for (uint32_t rb = R0; rb < R1; rb += kDeadBatch) {
-      const int rc = (int)min((uint32_t)kDeadBatch, R1 - rb);
-      // stage the receivers; list the units of half 0, then of half 1
-      __syncwarp();
-      int n0 = 0, n1 = 0;
-      uint32_t box[kDeadBatch / 32];
+    const uint32_t below = (1u << lane) - 1u;
+    for (uint32_t rs = R0; rs < R1; rs += kDeadScan) {
+      // the entries needed, from their Gaussians' flags
+      uint32_t rank[kDeadScan / 32];
+      uchar2 fl[kDeadScan / 32];
 #pragma unroll
-      for (int c = 0; c < kDeadBatch / 32; ++c) {
-        const int t = 32 * c + lane;
-        box[c] = 0u;
-        if (t < rc) {
-          const uint32_t rank = p.list[rb + t];
-          const SplatRec q = p.rrec[rank];
-          const bool live = p.live_rank[rank] != 0;
-          float4 e0, e1;
-          make_entry(q, ox, oy, e0, e1);
-          // skipped: a Gaussian with no open-ray entry whose den is known positive,
-          // except in its probe tile (whose entry keeps den > 0 in the sum)
-          const bool skip = !live && __ldcg(p.den_found + rank) != 0 &&
-                            probe_tile(q, p.W, p.H, p.gx) != (uint32_t)(ty * p.gx + tx);
-          box[c] = skip ? 0u : __float_as_uint(e1.w) & ellipse_halves(e0, e1);
-          D.e0[t] = e0;
-          D.e1[t] = e1;
-          D.slot[t] = p.off[rank] + (uint32_t)((ty - q.r.y) * (q.r.z - q.r.x + 1) + (tx - q.r.x));
-          D.rank[t] = rank | (live ? 0x80000000u : 0u);
+      for (int c = 0; c < kDeadScan / 32; ++c) {
+        const uint32_t i = rs + 32 * c + lane;
+        rank[c] = i < R1 ? p.list[i] : 0u;
+      }
+#pragma unroll
+      for (int c = 0; c < kDeadScan / 32; ++c) {
+        // the second flag may be set meanwhile: read past the L1
+        const uint16_t f = __ldcg(reinterpret_cast<const uint16_t*>(p.rank_flags) + rank[c]);
+        fl[c] = make_uchar2((uint8_t)f, (uint8_t)(f >> 8));
+      }
+      int nq = 0;
+      __syncwarp();
+#pragma unroll
+      for (int c = 0; c < kDeadScan / 32; ++c) {
+        const uint32_t i = rs + 32 * c + lane;
+        const bool need = i < R1 && (fl[c].x || !fl[c].y);
+        const uint32_t m = __ballot_sync(0xffffffffu, need);
+        if (need) {
+          D.rank[nq + __popc(m & below)] = rank[c] | (fl[c].x ? 0x80000000u : 0u);
+          D.at[nq + __popc(m & below)] = (uint8_t)(32 * c + lane);
+        } else if (i < R1) {
+          p.pass_mask[i] = 0;
         }
-        n0 += __popc(__ballot_sync(0xffffffffu, (box[c] & 0x3u) != 0u));
-        n1 += __popc(__ballot_sync(0xffffffffu, (box[c] & 0xCu) != 0u));
+        nq += __popc(m);
       }
-      int b0 = 0, b1 = n0;  // next unit slot of each half
+      __syncwarp();
+      for (int q0 = 0; q0 < nq; q0 += kDeadBatch) {
+        const int rc = min(kDeadBatch, nq - q0);
+        // stage the receivers; list the units of half 0, then of half 1
+        int n0 = 0, n1 = 0;
+        uint32_t box[kDeadBatch / 32];
 #pragma unroll
-      for (int c = 0; c < kDeadBatch / 32; ++c) {
-        const int t = 32 * c + lane;
-        const uint32_t m0 = __ballot_sync(0xffffffffu, (box[c] & 0x3u) != 0u);
-        const uint32_t m1 = __ballot_sync(0xffffffffu, (box[c] & 0xCu) != 0u);
-        const uint32_t below = (1u << lane) - 1u;
-        if (box[c] & 0x3u) D.unit[b0 + __popc(m0 & below)] = (uint16_t)t;
-        if (box[c] & 0xCu) D.unit[b1 + __popc(m1 & below)] = (uint16_t)(t | 0x100);
-        b0 += __popc(m0);
-        b1 += __popc(m1);
-        if (t < rc) D.den[0][t] = D.den[1][t] = 0.f;
-      }
-      __syncwarp();
-      const int nu = n0 + n1;
-      for (int u = lane; u < nu; u += 32) {
-        const int code = D.unit[u];
-        const int t = code & 0xFF, h = code >> 8;
-        const float4 e0 = D.e0[t], e1 = D.e1[t];
-        D.den[h][t] = interior ? dead_half(e0, e1, h) : dead_half_edge(e0, e1, h, ncol, nrow);
-      }
-      __syncwarp();
-      for (int t = lane; t < rc; t += 32) {
-        const float d0 = D.den[0][t], d1 = D.den[1][t];
-        const uint32_t rk = D.rank[t];
-        p.partial[D.slot[t]] = make_float2(0.f, d0 + d1);
-        p.pass_mask[rb + t] = (uint8_t)((d0 > 0.f ? 0x3u : 0u) | (d1 > 0.f ? 0xCu : 0u));
-        if (d0 + d1 > 0.f && !(rk >> 31)) __stcg(p.den_found + rk, (uint8_t)1);
+        for (int c = 0; c < kDeadBatch / 32; ++c) {
+          const int t = 32 * c + lane;
+          box[c] = 0u;
+          if (t < rc) {
+            const uint32_t r = D.rank[q0 + t] & 0x7FFFFFFFu;
+            const SplatRec q = p.rrec[r];
+            float4 e0, e1;
+            make_entry(q, ox, oy, e0, e1);
+            box[c] = __float_as_uint(e1.w) & ellipse_halves(e0, e1);
+            D.e0[t] = e0;
+            D.e1[t] = e1;
+            D.slot[t] = p.off[r] + (uint32_t)((ty - q.r.y) * (q.r.z - q.r.x + 1) + (tx - q.r.x));
+          }
+          n0 += __popc(__ballot_sync(0xffffffffu, (box[c] & 0x3u) != 0u));
+          n1 += __popc(__ballot_sync(0xffffffffu, (box[c] & 0xCu) != 0u));
+        }
+        int b0 = 0, b1 = n0;  // next unit slot of each half
+#pragma unroll
+        for (int c = 0; c < kDeadBatch / 32; ++c) {
+          const int t = 32 * c + lane;
+          const uint32_t m0 = __ballot_sync(0xffffffffu, (box[c] & 0x3u) != 0u);
+          const uint32_t m1 = __ballot_sync(0xffffffffu, (box[c] & 0xCu) != 0u);
+          if (box[c] & 0x3u) D.unit[b0 + __popc(m0 & below)] = (uint16_t)t;
+          if (box[c] & 0xCu) D.unit[b1 + __popc(m1 & below)] = (uint16_t)(t | 0x100);
+          b0 += __popc(m0);
+          b1 += __popc(m1);
+          if (t < rc) D.den[0][t] = D.den[1][t] = 0.f;
+        }
+        __syncwarp();
+        const int nu = n0 + n1;
+        for (int u = lane; u < nu; u += 32) {
+          const int code = D.unit[u];
+          const int t = code & 0xFF, h = code >> 8;
+          const float4 e0 = D.e0[t], e1 = D.e1[t];
+          D.den[h][t] = interior ? dead_half(e0, e1, h) : dead_half_edge(e0, e1, h, ncol, nrow);
+        }
+        __syncwarp();
+        for (int t = lane; t < rc; t += 32) {
+          const float d0 = D.den[0][t], d1 = D.den[1][t];
+          const uint32_t r = D.rank[q0 + t];
+          const bool live = (r >> 31) != 0u;
+          if (live) p.partial[D.slot[t]] = make_float2(0.f, d0 + d1);
+          else if (d0 + d1 > 0.f) reinterpret_cast<volatile uchar2*>(p.rank_flags)[r].y = 1;
+          p.pass_mask[rs + D.at[q0 + t]] = live ? (uint8_t)((d0 > 0.f ? 0x3u : 0u) | (d1 > 0.f ? 0xCu : 0u)) : 0;
+        }
+        __syncwarp();
       }
     }
   }
 
-// Before K6c: a Gaussian none of whose entries K6b saw has its pixel nearest
-// the splat centre tested with K6c's exact arithmetic (the entry of that
-// tile, the pixel's power against the threshold); if it passes, den > 0 is
-// known and K6c can skip every entry of the Gaussian.  Only a pixel that K6c
-// itself would evaluate counts: inside the image, in a tile of the
-// Gaussian's rectangle, in a half its box and ellipse reach.
+// Before K6c: a Gaussian of which K6b found neither a positive numerator nor
+// a passing pixel has its pixel nearest the splat centre tested with K6c's
+// exact arithmetic (the entry of that tile, the pixel's power against the
+// threshold); if it passes, K6c can skip every entry of the Gaussian.  Only a
+// pixel that K6c itself would evaluate counts: inside the image, in a tile of
+// the Gaussian's rectangle, in a half its box and ellipse reach.
 __global__ void k_dead_probe(const ShadowParams p, int n) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= n || p.live_rank[r]) return;
+  if (r >= n || p.rank_flags[r].x || p.rank_flags[r].y) return;
   const SplatRec q = p.rrec[r];
   if (q.r.x < 0) return;  // not in the light view
   const float cx = q.a.x + q.b.w, cy = q.a.y + q.c.x;
@@ -665,7 +572,7 @@ __global__ void k_dead_probe(const ShadowParams p, int n) {
   const float sx = (e0.z * dx) * dx, v = e1.x * dx;
   const float dy = ((8.f * h + 0.5f) + (float)(y & 7)) - e0.y;
   const float pw = fmaf(dy, fmaf(e0.w, dy, v), sx);
-  if (pw >= e1.y) p.den_found[r] = 1;
+  if (pw >= e1.y) p.rank_flags[r].y = 1;
 }
 
 template <bool BATCH>
@@ -674,124 +581,172 @@ __global__ void __launch_bounds__(kDeadWarps * 32, 7) k_shadow_dead(const Shadow
   __shared__ DeadSmem smem[kDeadWarps];
   DeadSmem& D = smem[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
-  const uint32_t total = BATCH ? batch_items(reqs, nreq) : p.lvl_off[kSegLevels];
+  const uint32_t total = BATCH ? batch_items(reqs, nreq, kDeadItems) : item_count(p, kDeadItems);
   uint32_t w;
   while (next_item(p.ticket + 2, total, lane, w)) {
     if (BATCH) {
-      const int r = locate(reqs, nreq, w);
-      dead_item(reqs[r], w, D, lane);
+      const int r = locate(reqs, nreq, kDeadItems, w);
+      dead_item(reqs[r], reqs[r].dead_list[w], D, lane);
     } else {
-      dead_item(p, w, D, lane);
+      dead_item(p, p.dead_list[w], D, lane);
     }
   }
 }
 
-// K6b: the receivers of every segment, with the products P = A(C_s) q, q the
-// running product of the range's occluders; A(C_s) comes from K6a.
+// K6b: the receivers of a segment that some ray enters open, with the
+// products P = A(C_s) times the running product of the range's occluders.
+// The occluders of the range and the receivers are merged into one sequence
+// (occluder k before receiver j where k < K(j)) and taken 32 at a time: the
+// place of receiver j is (j - R0) + (K(j) - C0), the other places are the
+// occluders', so each lane finds and stages one entry of the batch; the warp
+// then walks the 32 entries.  A receiver's per-lane sums go to a row of shared
+// memory; after the walk the lane that staged it adds up the row (in a fixed
+// order) and writes its partial.
 __device__ __forceinline__ void live_item(const ShadowParams& p, uint32_t w, ShadowSmem& S, int lane) {
-  SegState st;
-  st.lane = lane;
   const int lxi = lane & 15, lyi = lane >> 4;
-  st.lx = lxi + 0.5f;
-  st.omin = 1.f - p.amax;
-  const uint32_t ain = (uint32_t)__cvta_generic_to_shared(&S.ain[lane]);
-
-    const SegItem it = seg_item(p, w, lane);
-    st.s = it.s;
-    st.tx = it.tx;
-    st.ty = it.ty;
-    st.ox = (float)(it.tx * kTile);
-    st.oy = (float)(it.ty * kTile);
-    st.C1 = it.C1;
-    float ly[kPx];
+  const float lx = lxi + 0.5f, omin = 1.f - p.amax;
+  const SegItem it = seg_item(p, w, lane);
+  const float ox = (float)(it.tx * kTile), oy = (float)(it.ty * kTile);
+  f32x2 ly[kPx / 2];
+  lane_rows(lane, it.rows_in, ly);
+  // A(C_s) and A(C_s+1), as K6a published them
+  const uint32_t fl_in = it.first ? 1u : __ldcg(p.pub_flag + it.wpred);
+  const uint32_t fl_out = it.last ? 1u : __ldcg(p.pub_flag + w);
+  f32x2 P[kPx / 2];
+  load_entering(p, it.first, it.wpred, fl_in, lane, it.rows_in, P);
+  uint32_t live = live_halves(P);
+  // where a ray ended is recorded by the segment K6a has it stop in, or by
+  // the tile's last one (ends: the lane's rays that this segment records)
+  uint32_t ends = 0u;
 #pragma unroll
-    for (int i = 0; i < kPx; ++i) ly[i] = i < it.rows_in ? lyi + 2 * i + 0.5f : 1.0e6f;
-    // A(C_s) and A(C_s+1), as K6a published them
-    uint32_t fl_in = it.s == 0 ? 1u : __ldcg(p.pub_flag + it.wpred);
-    uint32_t fl_out = it.last ? 1u : __ldcg(p.pub_flag + w);
-    float P[kPx];
-    load_entering(p, it.s, it.wpred, fl_in, lane, it.rows_in, P);
-    const bool dead = all_stopped(P);
-    if (dead) return;  // K6c takes it
-    // rays the publication has stop in this range (they must reach their stop)
-    bool pending = false;
-    float q[kPx];
-    __syncwarp();
-#pragma unroll
-    for (int i = 0; i < kPx; ++i) {
-      q[i] = 1.f;
-      S.ain[32 * i + lane] = P[i];
-      S.xlim[32 * i + lane] = 0u;
-      if (P[i] >= kShadowStop && !it.last) {
-        const float out = fl_out == 2u ? 0.f : __ldcg(p.pub_a + (size_t)w * 256 + 32 * i + lane);
-        pending |= out == 0.f;
-      }
-      if (!(P[i] >= kShadowStop)) P[i] = 0.f;
-    }
-    __syncwarp();
-    st.live = live_halves(P);
-    st.k = st.wb = st.we = it.C0;
-    st.pix0 = (size_t)(it.ty * kTile + lyi) * p.W + it.tx * kTile + lxi;
-    // one pseudo-receiver past the last: the rest of the range, for rays that
-    // stop in it after the last receiver
-    const bool tail = __any_sync(0xffffffffu, pending);
-    for (uint32_t rb = it.R0; rb < it.R1 || (tail && rb == it.R1); rb += kRecv) {
-      const int rc = (int)min((uint32_t)kRecv, it.R1 - min(rb, it.R1));
-      if (rc > 0) stage_receivers(p, S, st, rb, rc);
-      const int steps = rc + (tail && rb + kRecv >= it.R1 ? 1 : 0);
-      for (int jj = 0; jj < steps; ++jj) {
-        const bool real = jj < rc;
-        if (st.live) walk_to(p, S, st, real ? S.rk[jj] : st.C1, ly, ain, q, P);
-        if (!real) break;
-        const float4 r1 = S.r1[jj];
-        const uint32_t box = __float_as_uint(r1.w);
-        float den0 = 0.f, den1 = 0.f, num = 0.f;
-        if (box) {
-          const float4 r0 = S.r0[jj];
-          const float dx = st.lx - r0.x;
-          const float sx = (r0.z * dx) * dx, v = r1.x * dx;
-          if (box & 0x3u) recv_half<true, 0>(ly, P, r0.y, r0.w, v, sx, r1.y, num, den0);
-          if (box & 0xCu) recv_half<true, 1>(ly, P, r0.y, r0.w, v, sx, r1.y, num, den1);
-        }
-        finish_receiver(p, S, lane, rb, jj, rc, num, den0, den1);
-      }
-    }
-    // where each ray ended (the backward starts from it): rays that stopped in
-    // this segment, and those that ran through every segment without
-    // stopping, written by the tile's last segment
-    __syncwarp();
-#pragma unroll
-    for (int i = 0; i < kPx; ++i) {
-      const uint32_t lim = S.xlim[32 * i + lane];
-      if (lim != 0u || (it.last && i < it.rows_in && P[i] >= kShadowStop)) {
-        p.light_final[st.pix0 + (size_t)2 * i * p.W] = P[i];
-        p.light_stop[st.pix0 + (size_t)2 * i * p.W] = lim != 0u ? lim : kNoStop;
-      }
-    }
+  for (int i = 0; i < kPx; ++i) {
+    const float a = i & 1 ? hi2(P[i / 2]) : lo2(P[i / 2]);
+    bool end = a >= kShadowStop;
+    if (end && !it.last && fl_out != 2u) end = __ldcg(p.pub_a + (size_t)w * 256 + 32 * i + lane) == 0.f;
+    ends |= end ? 1u << i : 0u;
   }
+#pragma unroll
+  for (int q = 0; q < kPx / 2; ++q)  // rays that are stopped or outside the image hold -0.0
+    P[q] = pk2(lo2(P[q]) >= kShadowStop ? lo2(P[q]) : -0.f, hi2(P[q]) >= kShadowStop ? hi2(P[q]) : -0.f);
+  const size_t pix0 = (size_t)(it.ty * kTile + lyi) * p.W + it.tx * kTile + lxi;
+  auto record = [&](int i, float a, uint32_t lim) {  // ray i ended with product a; it took the occluders below lim
+    p.light_final[pix0 + (size_t)2 * i * p.W] = a;
+    p.light_stop[pix0 + (size_t)2 * i * p.W] = lim;
+  };
+  // occluders past the last receiver's are walked only for rays that stop in
+  // the rest of the range
+  const bool tail = !it.last && __any_sync(0xffffffffu, ends != 0u);
+  uint32_t j = it.R0, k = it.C0;
+  uint32_t kend = it.R1 > it.R0 ? (tail ? it.C1 : p.kbound[it.R1 - 1]) : it.C0;
+  for (;;) {
+    if (!live) kend = k;  // no ray takes occluders any more
+    const uint32_t left = (it.R1 - j) + (kend - k);
+    if (left == 0u) break;
+    const int nops = (int)min(32u, left);
+    // the receivers' places among the batch's 32
+    uint32_t pos = 32u;
+    if (j + lane < it.R1) pos = live ? lane + (p.kbound[j + lane] - k) : (uint32_t)lane;
+    const uint32_t M = __reduce_or_sync(0xffffffffu, pos < 32u ? 1u << pos : 0u);
+    const int nrecv = __popc(M), mine = __popc(M & ((1u << lane) - 1u));
+    const bool is_recv = (M >> lane) & 1u;
+    uint32_t rank = 0u, slot = 0u;
+    __syncwarp();  // the previous batch is consumed
+    if (lane < nops) {
+      const uint32_t idx = is_recv ? j + mine : k + (lane - mine);
+      rank = p.list[idx];
+      const SplatRec q = p.rrec[rank];
+      const uint32_t bits = stage_entry(q, ox, oy, S.e, lane);
+      if (is_recv) {
+        slot = p.off[rank] + (uint32_t)((it.ty - q.r.y) * (q.r.z - q.r.x + 1) + (it.tx - q.r.x));
+        p.pass_mask[idx] = (uint8_t)bits;
+      }
+    }
+    __syncwarp();
+    int row = 0;
+    for (int t = 0; t < nops; ++t) {
+      const float2 gb = S.e.gb[t];
+      const uint32_t bits = __float_as_uint(gb.y);
+      if ((M >> t) & 1u) {
+        f32x2 num = 0ull, den = 0ull;
+        if (bits) {
+          const ColTerms e = col_terms(lx, S.e, t);
+          if (bits & 0x3u) recv_half<0>(ly, P, e, num, den);
+          if (bits & 0xCu) recv_half<1>(ly, P, e, num, den);
+        }
+        const float n1 = lo2(num) + hi2(num), d1 = lo2(den) + hi2(den);
+        const float n2 = __shfl_xor_sync(0xffffffffu, n1, 16), d2 = __shfl_xor_sync(0xffffffffu, d1, 16);
+        S.red[row][lxi] = pk2(n1 + n2, d1 + d2);  // lanes l and l + 16 hold the same sums
+        ++row;
+      } else {
+        const uint32_t b = bits & live;
+        if (!b) continue;
+        const ColTerms e = col_terms(lx, S.e, t);
+        if (b & 0x3u) occ_half<0>(ly, P, e, gb.x, omin);
+        if (b & 0xCu) occ_half<1>(ly, P, e, gb.x, omin);
+        // the occluder that takes a ray's product below the stop is its last:
+        // P becomes -0.0, where it stays, and the receivers behind see 0
+        if (min_bits(P) < __float_as_uint(kShadowStop)) {
+          const uint32_t lim = k + (uint32_t)(t - row) + 1u;
+#pragma unroll
+          for (int i = 0; i < kPx; ++i) {
+            const float a = i & 1 ? hi2(P[i / 2]) : lo2(P[i / 2]);
+            if (__float_as_uint(a) < __float_as_uint(kShadowStop)) {
+              if (ends & (1u << i)) record(i, a, lim);
+              ends &= ~(1u << i);
+              P[i / 2] = i & 1 ? pk2(lo2(P[i / 2]), -0.f) : pk2(-0.f, hi2(P[i / 2]));
+            }
+          }
+        }
+      }
+    }
+    __syncwarp();
+    if (is_recv && lane < nops) {
+      f32x2 s0 = S.red[mine][0], s1 = S.red[mine][1];
+#pragma unroll
+      for (int c = 2; c < 16; c += 2) {
+        s0 = add2(s0, S.red[mine][c]);
+        s1 = add2(s1, S.red[mine][c + 1]);
+      }
+      const f32x2 nd = add2(s0, s1);
+      p.partial[slot] = make_float2(lo2(nd), hi2(nd));
+      if (lo2(nd) > 0.f) p.rank_flags[rank].x = 1;
+      if (hi2(nd) > 0.f) p.rank_flags[rank].y = 1;
+    }
+    j += nrecv;
+    k += nops - nrecv;
+    live = live_halves(P);
+  }
+  // rays that end past this segment's last occluder
+#pragma unroll
+  for (int i = 0; i < kPx; ++i)
+    if (ends & (1u << i)) record(i, i & 1 ? hi2(P[i / 2]) : lo2(P[i / 2]), it.last ? kNoStop : it.C1);
+}
 
+// 6 blocks per SM (80 registers): 0.453 ms against 0.476 at 5 and 0.524 at 4
+// (object workload).
 template <bool BATCH>
-__global__ void __launch_bounds__(kSegWarps * 32, 4) k_shadow(const ShadowParams p, const ShadowParams* reqs, int nreq) {
+__global__ void __launch_bounds__(kSegWarps * 32, 6) k_shadow(const ShadowParams p, const ShadowParams* reqs, int nreq) {
   __shared__ ShadowSmem smem[kSegWarps];
   ShadowSmem& S = smem[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
-  const uint32_t total = BATCH ? batch_items(reqs, nreq) : p.lvl_off[kSegLevels];
+  const uint32_t total = BATCH ? batch_items(reqs, nreq, kOpenItems) : item_count(p, kOpenItems);
   uint32_t w;
   while (next_item(p.ticket + 1, total, lane, w)) {
     if (BATCH) {
-      const int r = locate(reqs, nreq, w);
-      live_item(reqs[r], w, S, lane);
+      const int r = locate(reqs, nreq, kOpenItems, w);
+      live_item(reqs[r], reqs[r].open_list[w], S, lane);
     } else {
-      live_item(p, w, S, lane);
+      live_item(p, p.open_list[w], S, lane);
     }
   }
 }
 
-// K(i) of entry i of a light list: the first index of i's tile list (from b)
-// whose distance is >= d_i - bias, the end of i's occluder prefix.
-__device__ __forceinline__ uint32_t occ_bound(const float* __restrict__ dl, uint32_t b, uint32_t i, float bias) {
+// K(i) of entry i of a light list: the first index of i's tile list whose
+// distance is >= d_i - bias, the end of i's occluder prefix, which lies in
+// [lo, hi] (at most i).
+__device__ __forceinline__ uint32_t occ_bound(const float* __restrict__ dl, uint32_t lo, uint32_t hi, uint32_t i,
+                                              float bias) {
   const float thr = __fsub_rn(dl[i], bias);
-  uint32_t lo = b, hi = i;
   while (lo < hi) {
     const uint32_t mid = (lo + hi) >> 1;
     if (dl[mid] < thr) lo = mid + 1; else hi = mid;
@@ -810,54 +765,69 @@ __device__ __forceinline__ int item_level(const uint32_t* lvl_off, uint32_t w) {
   return lo;
 }
 
-// K at the entries the segment plan reads (every segment's first entry and
-// every tile's last), one thread per segment, before K6a.
+// The items' descriptors, and K at the entries the segment plan reads (every
+// segment's first entry and every tile's last), one thread per segment,
+// before K6a.
 __global__ void __launch_bounds__(256) k_bound_starts(const ShadowParams p, const float* __restrict__ dl,
                                                       uint32_t* __restrict__ kb, float bias) {
   const uint32_t w = blockIdx.x * blockDim.x + threadIdx.x;
   if (w >= p.lvl_off[kSegLevels]) return;
   const int s = item_level(p.lvl_off, w);
-  const int tile = (int)p.tile_order[w - p.lvl_off[s]];
-  const uint32_t b = p.tile_start[tile], e = p.tile_start[tile + 1];
-  if (e <= b) return;
-  const uint32_t r0 = b + (uint32_t)s * kSegLen;
-  kb[r0] = occ_bound(dl, b, r0, bias);
-  if ((uint32_t)s == seg_count(e - b) - 1 && e - 1 > r0) kb[e - 1] = occ_bound(dl, b, e - 1, bias);
-}
-
-// After K6a: K of every other entry of a segment with an open ray (K6b reads
-// it per receiver), one warp per segment.  In a segment every ray enters
-// stopped no kernel takes an occluder or needs the exact bound: its entries
-// get the segment's first bound C_s (<= K(j)); the backward, which reads
-// them, takes no occluder at or past a ray's stop, and every ray stopped
-// before C_s, so any bound in [C_s, K(j)] gives it the same result.
-__global__ void __launch_bounds__(256) k_bound_rest(const ShadowParams p, const float* __restrict__ dl,
-                                                    uint32_t* __restrict__ kb, float bias) {
-  const uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (w >= p.lvl_off[kSegLevels]) return;
-  const int s = item_level(p.lvl_off, w);
   const uint32_t pos = w - p.lvl_off[s];
   const int tile = (int)p.tile_order[pos];
   const uint32_t b = p.tile_start[tile], e = p.tile_start[tile + 1];
-  if (e <= b) return;
   const bool last = (uint32_t)s == seg_count(e - b) - 1;
   const uint32_t r0 = b + (uint32_t)s * kSegLen, r1 = last ? e : r0 + kSegLen;
-  const bool open = s == 0 || __ldcg(p.pub_flag + p.lvl_off[s - 1] + pos) != 2u;
-  const uint32_t c0 = kb[r0];
-  for (uint32_t j = r0 + 1 + lane; j < r1; j += 32) {
-    if (j == e - 1) continue;  // k_bound_starts's
-    kb[j] = open ? occ_bound(dl, b, j, bias) : c0;
+  p.desc[w] = make_uint4((uint32_t)tile | (last ? kSegLast : 0u), r0, r1, s > 0 ? p.lvl_off[s - 1] + pos : kNoItem);
+  if (e <= b) return;
+  kb[r0] = occ_bound(dl, b, r0, r0, bias);
+  if (last && e - 1 > r0) kb[e - 1] = occ_bound(dl, b, e - 1, e - 1, bias);
+}
+
+// After K6a, one warp per segment: the lists of the segments with an open
+// ray (K6b's) and of those every ray enters stopped (K6c's), and K of the
+// open segments' other entries (K6b reads it per receiver), which lies
+// between the segment's first bound and the next segment's.  No kernel takes
+// an occluder for the entries of a stopped segment, so theirs stay unwritten
+// past the first.
+__global__ void __launch_bounds__(256) k_bound_rest(const ShadowParams p, const float* __restrict__ dl,
+                                                    uint32_t* __restrict__ kb, float bias) {
+  __shared__ uint32_t cnt[2], base[2];
+  const uint32_t total = p.lvl_off[kSegLevels];
+  if (blockIdx.x * 8u >= total) return;
+  const uint32_t w = blockIdx.x * 8u + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x < 2) cnt[threadIdx.x] = 0u;
+  __syncthreads();
+  uint4 d = make_uint4(0u, 0u, 0u, kNoItem);
+  int dead = -1;
+  uint32_t at = 0u;
+  if (w < total) {
+    d = p.desc[w];
+    dead = d.w != kNoItem && __ldcg(p.pub_flag + d.w) == 2u ? 1 : 0;
+    if (lane == 0) at = atomicAdd(&cnt[dead], 1u);
   }
+  __syncthreads();
+  if (threadIdx.x < 2) base[threadIdx.x] = cnt[threadIdx.x] ? atomicAdd(p.counts + threadIdx.x, cnt[threadIdx.x]) : 0u;
+  __syncthreads();
+  if (dead >= 0 && lane == 0) (dead ? p.dead_list : p.open_list)[base[dead] + at] = w;
+  if (dead != 0 || d.z <= d.y) return;
+  const bool last = (d.x & kSegLast) != 0u;
+  const uint32_t c0 = kb[d.y], c1 = kb[last ? d.z - 1 : d.z];
+  for (uint32_t j = d.y + 1 + lane; j < d.z - (last ? 1u : 0u); j += 32) kb[j] = occ_bound(dl, c0, min(c1, j), j, bias);
 }
 
 // K7: per Gaussian, sum its (tile) partials; T = num / den, or 1 when the
-// Gaussian meets no shadow ray.  Eight lanes per Gaussian rank (four per
-// warp): lane s adds partials s, s + 8, ... in order, then three shuffle
-// levels combine the eight sums in a fixed order.
+// Gaussian meets no shadow ray.  A Gaussian that K6b did not mark has a zero
+// numerator and no sum to add: T is 0 if a pixel of it passes, else 1, and
+// its den is stored as 0 (its gradients through the shadow splat are 0).
+// Eight lanes per Gaussian rank (four per warp): lane s adds partials s,
+// s + 8, ... in order, then three shuffle levels combine the eight sums in a
+// fixed order.
 __global__ void __launch_bounds__(256) k_shadow_reduce(int n, const uint32_t* __restrict__ off,
                                                        const uint32_t* __restrict__ cnt,
                                                        const float2* __restrict__ partial,
+                                                       const uchar2* __restrict__ flags,
                                                        const uint32_t* __restrict__ order,
                                                        const uint32_t* header, float* __restrict__ T,
                                                        float* __restrict__ den_out) {
@@ -865,8 +835,9 @@ __global__ void __launch_bounds__(256) k_shadow_reduce(int n, const uint32_t* __
   const int sub = threadIdx.x & 7;
   const bool valid = r < n;
   const uint32_t P = header[H_PAIRS_LIGHT];
+  const uchar2 fl = valid ? flags[r] : make_uchar2(0, 0);
   float num = 0.f, den = 0.f;
-  if (valid) {
+  if (fl.x) {
     const uint32_t o = off[r], c = cnt[r];
     if (o + c <= P) {
       for (uint32_t i = sub; i < c; i += 8) {
@@ -882,8 +853,9 @@ __global__ void __launch_bounds__(256) k_shadow_reduce(int n, const uint32_t* __
     den += __shfl_xor_sync(0xffffffffu, den, sh);
   }
   if (valid && sub == 0) {
-    T[order[r]] = den > 0.f ? num / den : 1.f;
-    den_out[order[r]] = den;
+    const uint32_t g = order[r];
+    T[g] = den > 0.f ? num / den : (fl.y ? 0.f : 1.f);
+    den_out[g] = den;
   }
 }
 
@@ -1249,6 +1221,10 @@ ShadowParams shadow_params(const FrameArgs& f) {
   p.tile_order = at<uint32_t>(ws, f.L->tile_order[1]);
   p.lvl_off = lvl;
   p.ticket = lvl + kSegLevels + 1;
+  p.counts = lvl + kSegLevels + 4;
+  p.desc = at<uint4>(ws, f.L->seg_desc);
+  p.open_list = at<uint32_t>(ws, f.L->seg_lists);
+  p.dead_list = p.open_list + shadow_seg_items(f.L->ntiles, f.L->cap);
   p.pub_a = at<float>(ws, f.L->seg_pub);
   p.pub_flag = at<uint32_t>(ws, f.L->seg_flag);
   p.list = at<uint32_t>(ws, b.tv[fin]);
@@ -1261,8 +1237,7 @@ ShadowParams shadow_params(const FrameArgs& f) {
   p.light_final = at<float>(ws, f.L->light_final);
   p.light_stop = at<uint32_t>(ws, f.L->light_stop);
   p.status = header + H_STATUS;
-  p.live_rank = at<uint8_t>(ws, f.L->rank_flags);
-  p.den_found = p.live_rank + f.L->n;
+  p.rank_flags = at<uchar2>(ws, f.L->rank_flags);
   p.W = f.L->width; p.H = f.L->height; p.gx = f.L->gx;
   p.amax = f.opts.alpha_max;
   return p;
@@ -1344,7 +1319,7 @@ void prepare_shadow_composite(const FrameArgs& f, cudaStream_t s) {
   uint32_t* kb = at<uint32_t>(ws, b.tv[1 - fin]);
   // the light tiles by segment count, and the work items of each segment level
   uint32_t* lvl = at<uint32_t>(ws, f.L->seg_lvl);
-  cudaMemsetAsync(lvl + kSegLevels + 1, 0, 12, s);  // the tickets
+  cudaMemsetAsync(lvl + kSegLevels + 1, 0, 20, s);  // the tickets and list counts
   cudaMemsetAsync(at<uint32_t>(ws, f.L->seg_flag), 0, 4 * shadow_seg_items(f.L->ntiles, f.L->cap), s);
   cudaMemsetAsync(ws + f.L->rank_flags, 0, 2 * (size_t)f.L->n, s);
   k_tile_order<<<1, 1024, 0, s>>>(at<uint32_t>(ws, b.tile_start), f.L->ntiles, at<uint32_t>(ws, f.L->tile_order[1]),
@@ -1419,7 +1394,7 @@ void launch_shadow_reduce(const FrameArgs& f, cudaStream_t s) {
   const int n = f.sc.n;
   k_shadow_reduce<<<(n * 8 + 255) / 256, 256, 0, s>>>(
       n, at<uint32_t>(ws, b.off), at<uint32_t>(ws, b.cnt), at<float2>(ws, f.L->partial),
-      at<uint32_t>(ws, b.sv[1]), at<uint32_t>(ws, f.L->header), at<float>(ws, f.L->T),
+      at<uchar2>(ws, f.L->rank_flags), at<uint32_t>(ws, b.sv[1]), at<uint32_t>(ws, f.L->header), at<float>(ws, f.L->T),
       at<float>(ws, f.L->shadow_den));
   count_launch();
 }

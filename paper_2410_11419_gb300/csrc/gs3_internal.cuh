@@ -82,10 +82,12 @@ struct Workspace {
   size_t light_stop = 0;   // u32[HW] 1 + list index of the occluder that stopped the ray, or all ones
   size_t shadow_den = 0;   // float[N] sum of beta per Gaussian (by index)
   size_t tile_order[2] = {0, 0};  // u32[ntiles] per splat: tiles by decreasing list length (launch order)
-  size_t seg_lvl = 0;   // u32[1025 + 3]: shadow work items per segment level, then three ticket counters
+  size_t seg_lvl = 0;   // u32[1025 + 5]: shadow work items per segment level, three ticket counters, two list lengths
   size_t seg_flag = 0;  // u32[items]: shadow segment publications (0 none, 1 done, 2 done and all stopped)
+  size_t seg_desc = 0;   // uint4[items]: each shadow segment's tile, receivers and predecessor
+  size_t seg_lists = 0;  // u32[2][items]: the segments with an open ray; those every ray enters stopped
   size_t seg_pub = 0;   // float[items][256]: the products each shadow segment hands to the next
-  size_t rank_flags = 0;  // u8[2N] by light rank: has an entry in a segment with an open ray; a dead unit passed
+  size_t rank_flags = 0;  // uchar2[N] by light rank: a receiver of it saw some light; a pixel of it is known to pass
   int n = 0, width = 0, height = 0, gx = 0, gy = 0, ntiles = 0;
   size_t cap = 0;
   int nb_n = 0;     // radix blocks over N
