@@ -427,7 +427,7 @@ gs3_status gs3_server_destroy(gs3_server *server);
  * middle of a frame.  It is the per-splat depth sort of gs3_render (stable
  * ascending order of 32-bit keys, the FP32 depth or light-distance bits) with
  * its scratch in a file-scope device array of GS3_STATIC_SORT_MAX_KEYS keys
- * (about 12.3 MB), which every GPU that loads the library holds until exit.
+ * (about 13.6 MB), which every GPU that loads the library holds until exit.
  *   keys:      device, uint32[n], read only
  *   order_out: device, uint32[n], caller-owned; receives the permutation
  *              order_out[r] = position of the r-th smallest key (ties in
@@ -445,7 +445,7 @@ gs3_status gs3_server_destroy(gs3_server *server);
  * array: calls whose
  * work overlaps on the GPU (other streams, other host threads) race and must
  * be serialised by the caller.  Nothing in the array needs to start at zero:
- * each pass overwrites all scratch it reads. */
+ * each call clears or overwrites all scratch it reads. */
 #define GS3_STATIC_SORT_MAX_KEYS 1048576u
 gs3_status gs3_depth_order_static(const uint32_t *keys, uint32_t n, uint32_t *order_out, void *stream);
 

@@ -14,8 +14,6 @@ namespace gs3 {
 constexpr int kTile = 16;             // screen tile edge (pixels)
 constexpr int kTilePix = kTile * kTile;
 constexpr int kSortThreads = 256;     // radix-sort block size
-constexpr int kSortRounds = 16;       // items per thread per block tile
-constexpr int kSortTileItems = kSortThreads * kSortRounds;  // 4096 items per block
 constexpr int kTileSortRounds = 16;   // look-back sort of the wait self-test: items per thread per block
 constexpr int kTileSortItems = kSortThreads * kTileSortRounds;
 // Tile binning by counting (tile_bin.cu)
@@ -281,18 +279,19 @@ void device_exclusive_scan(const uint32_t* in, uint32_t* out, uint32_t n, uint32
                            uint32_t* scratch, cudaStream_t s);
 size_t scan_scratch_words(size_t n);
 
-// bytes of a look-back sort's region: u64[passes][256 * nblocks] look-back
-// words, u32 tickets[passes], u32 totals[passes][256]
-inline size_t onesweep_bytes(int nblocks, int passes) {
-  return 8ull * passes * 256 * (size_t)nblocks + 4ull * (passes + passes * 256);
+// bytes of a look-back sort's region: u64[256 * nblocks] look-back words (every
+// pass's in turn), u32 tickets[passes], u32 totals[passes][256]
+constexpr size_t onesweep_bytes(int nblocks, int passes) {
+  return 8ull * 256 * (size_t)nblocks + 4ull * (passes + passes * 256);
 }
 
-// stable LSD radix sort of n (key, value) pairs on the low 8 * passes key bits
-// (vin null: values are the input positions); the result lands in (k1, v1)
-// for an even number of passes, (k0, v0) for an odd one
-void radix_sort_pairs(const uint32_t* kin, const uint32_t* vin, uint32_t* k0, uint32_t* v0, uint32_t* k1,
-                      uint32_t* v1, uint32_t n, int passes, uint32_t* hist, uint32_t* scan_part,
-                      cudaStream_t s);
+// The stable ascending order of n <= GS3_STATIC_SORT_MAX_KEYS keys (the
+// sort's position of rank r at order[r]).  k0, v0, k1: n words each;
+// look_region: onesweep_bytes(kDepthOrderBlocks, 4) bytes; status: a word that
+// is set to GS3_ERR_TIMEOUT (from 0) if a bounded wait runs out.
+constexpr int kDepthOrderBlocks = 512;
+void depth_order(const uint32_t* keys, uint32_t n, uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* order,
+                 unsigned char* look_region, uint32_t* status, cudaStream_t s);
 
 // false when [ptr, ptr + bytes) provably leaves ptr's device allocation
 bool device_range_ok(const void* ptr, size_t bytes);
