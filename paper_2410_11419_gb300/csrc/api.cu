@@ -145,10 +145,12 @@ Workspace plan_workspace(int n, int width, int height, size_t cap) {
     b.bin_plan = P.take(4 * (3 * (size_t)L.gy + 3));
     b.bin_tab = P.take(4 * bin_tab_words(cap, L.gx, L.gy));
   }
-  L.partial = P.take(8 * cap);
+  // the shadow partials; afterwards the backward's per-ray sums of the shadow
+  // segments (256 floats each)
+  const size_t items = shadow_seg_items(L.ntiles, cap);
+  L.partial = P.take(8 * cap > 1024 * items ? 8 * cap : 1024 * items);
   L.tile_order[0] = P.take(4 * (size_t)L.ntiles);
   L.tile_order[1] = P.take(4 * (size_t)L.ntiles);
-  const size_t items = shadow_seg_items(L.ntiles, cap);
   L.seg_lvl = P.take(4 * (1025 + 5));
   L.seg_flag = P.take(4 * items);
   L.seg_desc = P.take(16 * items);

@@ -8,15 +8,14 @@
 //   K8b  Psi and Phi: forward recomputed per 32-row tile, backward through
 //        the layers, weight gradients as per-block partials summed in a fixed
 //        order                                                  (Sec. 4.2, 4.3)
-//   K6b  shadow splat: per shadow ray, back to front from the stored final
-//        occluder product; receivers j add (dL/dT_j / den_j) beta T_m(j) to a
-//        suffix sum S; an occluder k gets dL/dalpha = -S / (1 - alpha)  (Sec. 4.2)
+//   K6b  shadow splat (shadow_bwd.cu)                                 (Sec. 4.2)
 //   K1b  per Gaussian: both EWA projections and the shading back to the
 //        parameters                                       (Eq. 1-5, Sec. 3, 4.1)
 // Per-Gaussian accumulators are summed with float atomics (after warp
 // reductions); the result is deterministic up to the order of those atomics.
 #include "gs3_internal.cuh"
 #include "splat_eval.cuh"
+#include "shadow_bwd.cuh"
 
 namespace gs3 {
 namespace {
@@ -47,7 +46,7 @@ __host__ __device__ size_t mlp_params(const MlpDev& m) {
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 struct BwdPlan {
-  size_t cam_geom, light_geom, color, dT, mlp_in, wred[2], mlp_scratch, total;
+  size_t cam_geom, light_geom, color, dT, mlp_in, wred[2], ticket, mlp_scratch, ct, total;
 };
 
 BwdPlan plan_bwd(int n, const MlpDev& phi, const MlpDev& psi) {
@@ -61,8 +60,10 @@ BwdPlan plan_bwd(int n, const MlpDev& phi, const MlpDev& psi) {
   p.mlp_in = take(4ull * kMlpIn * n);
   p.wred[0] = take(4ull * mlp_params(phi));
   p.wred[1] = take(4ull * mlp_params(psi));
+  p.ticket = take(12);
   const size_t sa = mlp_bwd_scratch_bytes(n, phi), sb = mlp_bwd_scratch_bytes(n, psi);
   p.mlp_scratch = take(sa > sb ? sa : sb);  // Phi and Psi use it in turn
+  p.ct = take(8ull * n);
   p.total = c;
   return p;
 }
@@ -244,351 +245,6 @@ __global__ void k_copy_strided(const float* src, int stride, int off, float* dst
 }
 
 // ---------------------------------------------------------------------------
-// K6b: shadow splat backward.
-// Reverse sweep of the forward's two-cursor pass over each light tile, with
-// the forward's thread layout (one warp per tile, eight rays per lane), its
-// entries and alpha decisions (splat_eval.cuh).  Per ray m the lane restarts
-// from the product A_m where the forward's ray ended and the limit below
-// which it took occluders (both stored by the forward; a ray that stopped
-// keeps its frozen product past the limit, so occluders at or past it are
-// skipped), and a suffix sum S_m = sum coef_j beta_jm T_m(j) over the
-// receivers already visited (coef_j = dL/dT_j / den_j):
-//   occluder k (passing, taken):  A /= (1 - alpha_k),  dL/dalpha_k = -S / (1 - alpha_k)
-//   receiver j (passing):  dL/dbeta_j = coef_j (A - T_j),  S += coef_j beta_j A
-// with A = T_m(j) when receiver j is reached.  Occluders are undone before
-// the receiver whose prefix end K(j) they reach, so S holds exactly the
-// receivers with K(j) > k.  An entry is evaluated only in the halves of the
-// tile where it passed in the forward (the pass halves it stored).
-// With dL/dpower = w at a pixel (dx, dy) from the splat centre, the centre
-// and conic gradients are linear in (w, w dy, w dy^2) for a fixed dx, and
-// a lane's eight pixels share dx: each lane sums those three moments and
-// forms (du, dv, dA, dB, dC) once per entry; the warp then sums them and
-// dgamma over its 256 rays through shared-memory rows, four entries at a
-// time, and adds them to the Gaussian's accumulators.
-// ---------------------------------------------------------------------------
-struct ShadowBwdParams {
-  const uint32_t* list;
-  const uint32_t* tile_start;
-  const SplatRec* rrec;
-  const uint32_t* order;
-  const uint32_t* kbound;
-  const uint32_t* tile_order;  // the forward's launch order of the light tiles
-  const uint8_t* pass_mask;
-  const float* light_final;    // the product where each ray ended
-  const uint32_t* light_stop;  // each ray took the occluders below this list index
-  const float* dT;   // by index
-  const float* den;  // by index
-  const float* T;    // by index
-  const uint32_t* lvl_off;   // the forward's segment plan: first work item of each segment level
-  const uint32_t* pub_flag;  // per item: 2 when every ray entered the next segment stopped
-  float* light_geom;
-  int W, H, gx;
-  float amax;
-};
-
-// The first entry of the tile at launch position pos whose segment every ray
-// enters stopped (the forward's K6a published A = 0 for all rays into it),
-// or e.  Such segments form a suffix of the list.
-__device__ __forceinline__ uint32_t stopped_from(const ShadowBwdParams& p, uint32_t pos, uint32_t b, uint32_t e,
-                                                 int lane) {
-  const uint32_t nseg = seg_count(e - b);
-  for (uint32_t s0 = 1; s0 < nseg; s0 += 32) {
-    const uint32_t s = s0 + (uint32_t)lane;
-    const bool dead = s < nseg && __ldcg(p.pub_flag + p.lvl_off[s - 1] + pos) == 2u;
-    const uint32_t m = __ballot_sync(0xffffffffu, dead);
-    if (m) return b + (s0 + (uint32_t)(__ffs(m) - 1)) * kSegLen;
-  }
-  return e;
-}
-
-constexpr int kBRecv = 64;
-constexpr int kBOcc = 128;
-constexpr int kGradGroup = 4;  // entries whose per-lane gradients are reduced together
-constexpr int kBThreads = 32;
-constexpr int kBPx = 8;  // rays per lane: column lane & 15, rows (lane >> 4) + 2 i
-constexpr float kLn2 = 0.6931471805599453f;
-
-struct ShadowBwdSmem {
-  float4 r0[kBRecv], r1[kBRecv];
-  uint32_t rk[kBRecv], rg[kBRecv];
-  float rc[kBRecv], rt[kBRecv];
-  float4 o0[kBOcc], o1[kBOcc];
-  uint32_t og[kBOcc];
-  float gr[kGradGroup][6][33];  // per entry of the group, per gradient term, per lane (padded row)
-  uint32_t gg[kGradGroup];      // the entries' Gaussians
-};
-
-// The lane's (du, dv, dA, dB, dC) from its moments m0 = sum w, m1 = sum w dy,
-// m2 = sum w dy^2 at column offset dx, in g[0..4]: the power (log2 units) is
-// a dx^2 + r dx dy + c dy^2 (e0.z = a, e0.w = c), with the conic
-// (A, B, C) = -(2 a, r, 2 c) ln 2 and d/du = A dx + B dy, d/dv = C dy + B dx,
-// d/dA = -dx^2 / 2, d/dB = -dx dy, d/dC = -dy^2 / 2 (natural units).
-__device__ __forceinline__ void moments_to_grad(const float4 e0, float r, float dx, float m0, float m1, float m2,
-                                                float (&g)[8]) {
-  g[0] = -(2.f * e0.z * dx * m0 + r * m1) * kLn2;
-  g[1] = -(2.f * e0.w * m1 + r * dx * m0) * kLn2;
-  g[2] = -0.5f * dx * dx * m0;
-  g[3] = -dx * m1;
-  g[4] = -0.5f * m2;
-}
-
-__global__ void __launch_bounds__(kBThreads, 18) k_shadow_bwd(ShadowBwdParams p) {
-  __shared__ ShadowBwdSmem S;
-  const int tile = (int)p.tile_order[blockIdx.x], tx = tile % p.gx, ty = tile / p.gx;
-  const int lane = threadIdx.x;
-  const int lxi = lane & 15, lyi = lane >> 4;
-  const bool inx = tx * kTile + lxi < p.W;
-  const float lx = lxi + 0.5f;
-  const float kFar = 1.0e6f;  // off-image pixels never pass (same rule as the forward)
-  const float ox = (float)(tx * kTile), oy = (float)(ty * kTile);
-  const float omin = 1.f - p.amax;
-  const uint32_t b = p.tile_start[tile], e_all = p.tile_start[tile + 1];
-  if (b == e_all) return;
-  // receivers from the first stopped segment on are k_shadow_bwd_stopped's;
-  // this warp sweeps the open segments back to front
-  const uint32_t e = stopped_from(p, blockIdx.x, b, e_all, lane);
-  float ly[kBPx], A[kBPx], Sm[kBPx];
-  uint32_t lim[kBPx];
-  uint32_t lmax = 0u;
-#pragma unroll
-  for (int i = 0; i < kBPx; ++i) {
-    const int y = ty * kTile + lyi + 2 * i;
-    const bool in = inx && y < p.H;
-    const size_t pix = (size_t)y * p.W + tx * kTile + lxi;
-    ly[i] = in ? lyi + 2 * i + 0.5f : kFar;
-    A[i] = in ? p.light_final[pix] : 1.f;
-    lim[i] = in ? p.light_stop[pix] : 0u;  // an off-image ray took nothing
-    Sm[i] = 0.f;
-    lmax = max(lmax, lim[i]);
-  }
-  // occluders at or past every ray's limit were taken by none
-  const uint32_t wlim = __reduce_max_sync(0xffffffffu, lmax);
-  // occluders the forward walked end at K of the last entry, or, before a
-  // stopped segment, at its first bound C (every ray stopped below it)
-  uint32_t kc = min(e < e_all ? p.kbound[e] : p.kbound[e - 1], max(wlim, b));
-
-  // An entry's gradient terms, per lane, go to a shared-memory row; every
-  // kGradGroup entries lane 6 e + c (< 24) adds term c of entry e over the
-  // 32 lanes, in lane order, and adds the total to the Gaussian's
-  // accumulator.  No shuffle chain per entry.
-  int ng = 0;
-  auto reduce_grads = [&]() {
-    const int ge = lane / 6, gc = lane % 6;
-    if (ge < ng) {
-      const float* row = S.gr[ge][gc];
-      float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll
-      for (int l = 0; l < 32; l += 4) {
-        a0 += row[l]; a1 += row[l + 1]; a2 += row[l + 2]; a3 += row[l + 3];
-      }
-      const float v = (a0 + a1) + (a2 + a3);
-      if (v != 0.f) atomicAdd(p.light_geom + (size_t)kGeom * S.gg[ge] + gc, v);
-    }
-    __syncwarp();  // the rows are free again
-    ng = 0;
-  };
-  auto push_grad = [&](uint32_t g, const float (&v)[8]) {
-#pragma unroll
-    for (int c = 0; c < 6; ++c) S.gr[ng][c][lane] = v[c];
-    if (lane == 0) S.gg[ng] = g;
-    __syncwarp();
-    if (++ng == kGradGroup) reduce_grads();
-  };
-
-  // undo occluder kk (window slot i) on the lane's rays; accumulate its gradient
-  auto occlude_bwd = [&](int i, uint32_t kk) {
-    const float4 o1 = S.o1[i];
-    const uint32_t bits = __float_as_uint(o1.w);
-    if (!bits) return;
-    const float4 o0 = S.o0[i];
-    const float dx = lx - o0.x;
-    const float sx = (o0.z * dx) * dx, v = o1.x * dx;
-    float m0 = 0.f, m1 = 0.f, m2 = 0.f, dg = 0.f;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      if (!(bits & (3u << (2 * h)))) continue;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int i8 = 4 * h + q;
-        const float dy = ly[i8] - o0.y;
-        const float pw = fmaf(dy, fmaf(o0.w, dy, v), sx);
-        if (pw >= o1.y && kk < lim[i8]) {
-          const float beta = ex2(pw), ga = o1.z * beta;
-          const float f = fmaxf(omin, fmaf(-o1.z, beta, 1.f));
-          const float inv = __frcp_rn(f);
-          A[i8] *= inv;
-          if (ga < p.amax) {  // alpha = gamma beta (not clamped)
-            const float dalpha = -Sm[i8] * inv;
-            dg = fmaf(dalpha, beta, dg);  // d/dgamma
-            const float w = dalpha * ga, wdy = w * dy;
-            m0 += w;
-            m1 += wdy;
-            m2 = fmaf(wdy, dy, m2);
-          }
-        }
-      }
-    }
-    float g[8];
-    moments_to_grad(o0, o1.x, dx, m0, m1, m2, g);
-    g[5] = dg;
-    g[6] = g[7] = 0.f;
-    push_grad(S.og[i], g);
-  };
-  // load the occluder window [kt, kc)
-  auto load_window = [&](uint32_t kt) {
-    __syncwarp();
-    for (uint32_t i = lane; i < kc - kt; i += kBThreads) {
-      const uint32_t rank = p.list[kt + i];
-      make_entry(p.rrec[rank], ox, oy, S.o0[i], S.o1[i]);
-      S.o1[i].w = __uint_as_float((uint32_t)p.pass_mask[kt + i]);
-      S.og[i] = p.order[rank];
-    }
-    __syncwarp();
-  };
-
-  for (uint32_t re = e; re > b;) {
-    const uint32_t rs = re > b + kBRecv ? re - kBRecv : b;
-    const int rc = (int)(re - rs);
-    __syncwarp();
-    for (int t = lane; t < rc; t += kBThreads) {
-      const uint32_t rank = p.list[rs + t];
-      const uint32_t g = p.order[rank];
-      make_entry(p.rrec[rank], ox, oy, S.r0[t], S.r1[t]);
-      S.r1[t].w = __uint_as_float((uint32_t)p.pass_mask[rs + t]);
-      S.rk[t] = p.kbound[rs + t];
-      S.rg[t] = g;
-      const float den = p.den[g];
-      S.rc[t] = den > 0.f ? p.dT[g] / den : 0.f;
-      S.rt[t] = p.T[g];
-    }
-    __syncwarp();
-    int jj = rc - 1;
-    while (jj >= 0) {
-      const uint32_t kfirst = S.rk[0];
-      const uint32_t kt = kc > kfirst + kBOcc ? kc - kBOcc : min(kfirst, kc);
-      load_window(kt);
-      for (; jj >= 0; --jj) {
-        const uint32_t kend = S.rk[jj];
-        if (kend < kt) break;
-        for (; kc > kend; --kc) occlude_bwd((int)(kc - 1 - kt), kc - 1);
-        const float4 r1 = S.r1[jj];
-        const uint32_t bits = __float_as_uint(r1.w);
-        if (!bits) continue;
-        const float4 r0 = S.r0[jj];
-        const float dx = lx - r0.x;
-        const float sx = (r0.z * dx) * dx, v = r1.x * dx;
-        const float coef = S.rc[jj], Tj = S.rt[jj];
-        float m0 = 0.f, m1 = 0.f, m2 = 0.f;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          if (!(bits & (3u << (2 * h)))) continue;
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int i8 = 4 * h + q;
-            const float dy = ly[i8] - r0.y;
-            const float pw = fmaf(dy, fmaf(r0.w, dy, v), sx);
-            if (pw >= r1.y) {
-              const float cb = coef * ex2(pw);
-              Sm[i8] = fmaf(cb, A[i8], Sm[i8]);
-              const float w = cb * (A[i8] - Tj), wdy = w * dy;
-              m0 += w;
-              m1 += wdy;
-              m2 = fmaf(wdy, dy, m2);
-            }
-          }
-        }
-        float g[8];
-        moments_to_grad(r0, r1.x, dx, m0, m1, m2, g);
-        g[5] = g[6] = g[7] = 0.f;
-        push_grad(S.rg[jj], g);
-      }
-      for (; kc > kt; --kc) occlude_bwd((int)(kc - 1 - kt), kc - 1);
-    }
-    re = rs;
-  }
-  // occluders below every receiver's prefix end: S holds all receivers
-  while (kc > b) {
-    const uint32_t kt = kc > b + kBOcc ? kc - kBOcc : b;
-    load_window(kt);
-    for (; kc > kt; --kc) occlude_bwd((int)(kc - 1 - kt), kc - 1);
-  }
-  if (ng) reduce_grads();
-}
-
-
-// K6b for the receivers of the segments every ray enters stopped: the
-// forward's products there are 0 (its K6a publishes A = 0 into them), so
-// receiver j's beta at ray m carries dL/dbeta = coef_j (0 - T_j) and no
-// occluder of these segments is taken.  The receivers are independent: a
-// warp takes one such segment, its lanes one (receiver, half) unit at a time
-// (the halves the forward found passing), walk the unit's 16 x 8 pixels with
-// the forward's power arithmetic, and turn the per-column moments of
-// w = dL/dpower into the centre and conic gradients, added to the Gaussian's
-// accumulators.  A receiver with T_j = 0 (no pixel of it sees light) adds
-// nothing and is skipped.
-constexpr int kStopWarps = 4;
-__global__ void __launch_bounds__(kStopWarps * 32) k_shadow_bwd_stopped(ShadowBwdParams p) {
-  const int lane = threadIdx.x & 31;
-  const uint32_t w = blockIdx.x * kStopWarps + (threadIdx.x >> 5);
-  if (w >= p.lvl_off[kSegLevels]) return;
-  int lo = 0, hi = kSegLevels;  // the item's level: largest s with lvl_off[s] <= w
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (p.lvl_off[mid] <= w) lo = mid; else hi = mid;
-  }
-  if (lo == 0) return;  // a tile's first segment starts with every ray open
-  const uint32_t pos = w - p.lvl_off[lo];
-  if (__ldcg(p.pub_flag + p.lvl_off[lo - 1] + pos) != 2u) return;
-  const int tile = (int)p.tile_order[pos];
-  const int tx = tile % p.gx, ty = tile / p.gx;
-  const float ox = (float)(tx * kTile), oy = (float)(ty * kTile);
-  const uint32_t b = p.tile_start[tile], e = p.tile_start[tile + 1];
-  const bool last = (uint32_t)lo == seg_count(e - b) - 1;
-  const uint32_t r0 = b + (uint32_t)lo * kSegLen, r1 = last ? e : r0 + kSegLen;
-  const int ncol = min(kTile, p.W - tx * kTile), nrow = min(kTile, p.H - ty * kTile);
-  // units (receiver, half), two per receiver, taken by the lanes in turn
-  for (uint32_t u = lane; u < 2u * (r1 - r0); u += 32) {
-    const uint32_t j = r0 + (u >> 1);
-    const int h = (int)(u & 1u);
-    const uint32_t bits = p.pass_mask[j];
-    if (!(bits & (3u << (2 * h)))) continue;
-    const uint32_t rank = p.list[j];
-    const uint32_t g = p.order[rank];
-    const float den = p.den[g], Tj = p.T[g];
-    const float coef = den > 0.f ? p.dT[g] / den : 0.f;
-    const float cw = -coef * Tj;  // w = dL/dpower = coef beta (0 - T_j)
-    if (cw == 0.f) continue;
-    float4 e0, e1;
-    make_entry(p.rrec[rank], ox, oy, e0, e1);
-    float gsum[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-    const int y1 = min(8 * h + 8, nrow);
-    for (int x = 0; x < ncol; ++x) {
-      const float lx = (float)x + 0.5f;
-      const float dx = lx - e0.x;
-      const float sx = (e0.z * dx) * dx, v = e1.x * dx;
-      float m0 = 0.f, m1 = 0.f, m2 = 0.f;
-      for (int y = 8 * h; y < y1; ++y) {
-        const float dy = ((float)y + 0.5f) - e0.y;
-        const float pw = fmaf(dy, fmaf(e0.w, dy, v), sx);
-        if (pw >= e1.y) {
-          const float wv = cw * ex2(pw), wdy = wv * dy;
-          m0 += wv;
-          m1 += wdy;
-          m2 = fmaf(wdy, dy, m2);
-        }
-      }
-      float gc[8];
-      moments_to_grad(e0, e1.x, dx, m0, m1, m2, gc);
-#pragma unroll
-      for (int c = 0; c < 5; ++c) gsum[c] += gc[c];
-    }
-#pragma unroll
-    for (int c = 0; c < 5; ++c)
-      if (gsum[c] != 0.f) atomicAdd(p.light_geom + (size_t)kGeom * g + c, gsum[c]);
-  }
-}
-
-// ---------------------------------------------------------------------------
 // K1b: per-Gaussian backward of both projections and the shading
 // ---------------------------------------------------------------------------
 struct M3 {
@@ -707,6 +363,7 @@ struct PrepBwdParams {
   int falloff;
   const float* cam_geom;
   const float* light_geom;
+  const SplatRec* light_rec;  // by index
   const float* color;
   const float* mlp_in;
   gs3_grads out;
@@ -720,7 +377,13 @@ __device__ __forceinline__ void prep_bwd_one(const PrepBwdParams& p, int g, floa
   const float4 m = p.sc.mean_op[g], s = p.sc.scale[g];
   const float gamma = 1.f / (1.f + expf(-m.w));
   const float* gc = p.cam_geom + (size_t)kGeom * g;
-  const float* gl = p.light_geom + (size_t)kGeom * g;
+  // the light splat's sums (shadow_bwd.cuh) times its conic (A, B, C), with
+  // d/du = A dx + B dy, d/dv = C dy + B dx, d/dA = -dx^2 / 2, d/dB = -dx dy,
+  // d/dC = -dy^2 / 2
+  const float* sl = p.light_geom + (size_t)kGeom * g;
+  const float4 cl = p.light_rec[g].b;
+  const float gl[6] = {cl.x * sl[1] + cl.y * sl[2], cl.z * sl[2] + cl.y * sl[1], -0.5f * sl[4], -sl[3], -0.5f * sl[5],
+                       sl[0]};
   float dmu[3] = {0, 0, 0}, ds[3] = {0, 0, 0}, dRq[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
   float Rq[9], qn[4], qlen;
   quat_rot(p.sc.rot[g], Rq, qn, qlen);
@@ -1015,45 +678,22 @@ gs3_status run_backward(const FrameArgs& f, const float* dimg, void* bws, size_t
   };
   // Phi first: the shadow backward takes its dL/dT.  Then Psi, which the
   // shadow backward does not need, runs on the side stream beside it (the
-  // networks share the MLP scratch, so they run in turn), with the receivers
-  // of the stopped segments; the one-warp-per-tile sweep leaves most SMs idle
-  // towards its end.
+  // networks share the MLP scratch, so they run in turn), after the receivers
+  // of the stopped segments.
   mlp_bwd(0, s);
-  cudaStream_t ss = s;
-  if (side) {
-    cudaEventRecord(side->fork, s);
-    cudaStreamWaitEvent(side->s, side->fork, 0);
-    ss = side->s;
-  }
+  cudaStream_t ss = side ? side->s : s;
   // K6b
   if (!(f.opts.ablate & GS3_ABLATE_SHADOW_SPLAT)) {
-    ShadowBwdParams p;
-    p.list = at<uint32_t>(ws, L.sp[1].tv[fin]);
-    p.tile_start = at<uint32_t>(ws, L.sp[1].tile_start);
-    p.rrec = at<SplatRec>(ws, L.sp[1].rrec);
-    p.order = at<uint32_t>(ws, L.sp[1].sv[1]);
-    p.kbound = at<uint32_t>(ws, L.sp[1].tv[1 - fin]);
-    p.pass_mask = reinterpret_cast<const uint8_t*>(at<float>(ws, L.sp[1].tk[1 - fin]));
-    p.tile_order = at<uint32_t>(ws, L.tile_order[1]);
-    p.light_final = at<float>(ws, L.light_final);
-    p.light_stop = at<uint32_t>(ws, L.light_stop);
-    p.dT = dT;
-    p.den = at<float>(ws, L.shadow_den);
-    p.T = at<float>(ws, L.T);
-    p.lvl_off = at<uint32_t>(ws, L.seg_lvl);
-    p.pub_flag = at<uint32_t>(ws, L.seg_flag);
-    p.light_geom = light_geom;
-    p.W = L.width; p.H = L.height; p.gx = L.gx;
-    p.amax = f.opts.alpha_max;
-    static DeviceOnce once;
-    once.run([] {
-      return cudaFuncSetAttribute(k_shadow_bwd, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                  (int)cudaSharedmemCarveoutMaxShared) == cudaSuccess;
-    });
-    k_shadow_bwd<<<L.ntiles, kBThreads, 0, s>>>(p);
-    const size_t items = shadow_seg_items(L.ntiles, L.cap);
-    k_shadow_bwd_stopped<<<(int)((items + kStopWarps - 1) / kStopWarps), kStopWarps * 32, 0, ss>>>(p);
-    count_launch(2);
+    ShadowBwdArgs a;
+    a.dT = dT;
+    a.ct = reinterpret_cast<float2*>(B + bp.ct);
+    a.ticket = reinterpret_cast<uint32_t*>(B + bp.ticket);
+    a.light_geom = light_geom;
+    a.fork = side ? side->fork : nullptr;
+    launch_shadow_backward(f, a, s, ss);
+  } else if (side) {
+    cudaEventRecord(side->fork, s);
+    cudaStreamWaitEvent(ss, side->fork, 0);
   }
   mlp_bwd(1, ss);
   if (side) {
@@ -1077,6 +717,7 @@ gs3_status run_backward(const FrameArgs& f, const float* dimg, void* bws, size_t
     p.falloff = f.opts.falloff;
     p.cam_geom = cam_geom;
     p.light_geom = light_geom;
+    p.light_rec = at<SplatRec>(ws, L.sp[1].rec);
     p.color = color;
     p.mlp_in = mlp_in;
     p.out = out;

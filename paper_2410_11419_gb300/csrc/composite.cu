@@ -7,8 +7,7 @@
 // with one 128-thread block per tile (two pixels per thread, batches of 256
 // records).
 #include "gs3_internal.cuh"
-#include "splat_eval.cuh"
-#include "f32x2.cuh"
+#include "shadow_seg.cuh"
 
 namespace gs3 {
 namespace {
@@ -54,14 +53,13 @@ namespace {
 // and an unsigned minimum passes over, so no pixel needs a test of its own),
 // and receivers and occluders come from one merged list, staged 32 at a time.
 // Object workload (300k Gaussians, 800 x 800, 12.8 M light entries): K6a 0.377
-// -> 0.272 ms, K6b 0.784 -> 0.453 ms, K6c 0.326 -> 0.172 ms (entries picked
+// -> 0.272 ms, K6b 0.784 -> 0.466 ms, K6c 0.326 -> 0.165 ms (entries picked
 // by their Gaussian's flags before their records are read, and only of
-// Gaussians with a positive numerator), reduction 0.034 -> 0.013 ms; at 1 M and
-// 1024 x 1024 K6a 1.095 -> 0.758, K6b 2.119 -> 1.122, K6c 2.081 -> 0.896 ms.
+// Gaussians with a positive numerator), reduction 0.034 -> 0.020 ms; at 1 M and
+// 1024 x 1024 K6a 1.095 -> 0.758, K6b 2.119 -> 1.154, K6c 2.081 -> 0.896 ms.
 // ---------------------------------------------------------------------------
 constexpr int kSegWarps = 4;        // independent warps per block
 constexpr int kOccWin = 32;         // occluder window
-constexpr int kPx = 8;              // rays per lane
 constexpr int kSegSpin = 1 << 20;   // polls of a predecessor's publication before giving up
 
 
@@ -90,34 +88,12 @@ struct ShadowParams {
   float amax;
 };
 
-constexpr uint32_t kSegLast = 0x80000000u;  // desc.x: the tile's last segment
-constexpr uint32_t kNoItem = 0xFFFFFFFFu;   // desc.w: the tile's first segment
 constexpr int kRowPad = 17;                 // a receiver's row of 16 lane sums, padded
-
-// Entries staged for a warp's rays, the terms that pair up duplicated so that
-// they load as packed operands.
-struct StagedEntries {
-  float4 yc[32];   // -y, -y, c, c
-  float4 xart[32]; // x, a, r, threshold
-  float2 gb[32];   // -gamma, halves (as bits)
-};
 
 struct ShadowSmem {  // one warp's
   StagedEntries e;
   f32x2 red[32][kRowPad];  // per receiver of the batch, per lane pair: (num, den)
 };
-
-// Stages one entry in slot t: make_entry's record, and the halves its box
-// and ellipse both reach, which are returned.
-__device__ __forceinline__ uint32_t stage_entry(const SplatRec& q, float ox, float oy, StagedEntries& E, int t) {
-  float4 e0, e1;
-  make_entry(q, ox, oy, e0, e1);
-  const uint32_t bits = __float_as_uint(e1.w) & ellipse_halves(e0, e1);
-  E.yc[t] = make_float4(-e0.y, -e0.y, e0.w, e0.w);
-  E.xart[t] = make_float4(e0.x, e0.z, e1.x, e1.y);
-  E.gb[t] = make_float2(-e1.z, __uint_as_float(bits));
-  return bits;
-}
 
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* a) {
   uint32_t v;
@@ -126,31 +102,6 @@ __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* a) {
 }
 __device__ __forceinline__ void st_release(uint32_t* a, uint32_t v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(a), "r"(v) : "memory");
-}
-
-// beta of one pixel: 2^pw where it passes (pw >= thr), else 0
-__device__ __forceinline__ float beta_of(float pw, float thr) { return pw >= thr ? ex2(pw) : 0.f; }
-
-// (beta, beta) of two pixels from their packed powers
-__device__ __forceinline__ f32x2 beta2_of(f32x2 pw, float thr) {
-  return pk2(beta_of(lo2(pw), thr), beta_of(hi2(pw), thr));
-}
-
-// An entry's terms that a lane's rays share (one column): with dy = ly - y,
-// power2 = fma(dy, fma(c, dy, v), sx), the arithmetic of splat_eval.cuh.
-struct ColTerms {
-  f32x2 ny, c, v, s;
-  float thr;
-};
-__device__ __forceinline__ ColTerms col_terms(float lx, const StagedEntries& E, int t) {
-  const ulonglong2 yc = *reinterpret_cast<const ulonglong2*>(&E.yc[t]);
-  const float4 q = E.xart[t];
-  const float dx = lx - q.x;
-  return {yc.x, yc.y, dup2(q.z * dx), dup2((q.y * dx) * dx), q.w};
-}
-__device__ __forceinline__ f32x2 beta2_at(const ColTerms& e, f32x2 ly) {
-  const f32x2 dy = add2(ly, e.ny);
-  return beta2_of(fma2(dy, fma2(e.c, dy, e.v), e.s), e.thr);
 }
 
 // A receiver's four rays of one half: den += beta and num += beta P.
@@ -165,35 +116,6 @@ __device__ __forceinline__ void recv_half(const f32x2 (&ly)[kPx / 2], const f32x
   }
 }
 
-// An occluder on four rays of one half: P *= max(omin, 1 - gamma beta), which
-// is P itself where it does not pass.
-template <int H>
-__device__ __forceinline__ void occ_half(const f32x2 (&ly)[kPx / 2], f32x2 (&P)[kPx / 2], const ColTerms& e,
-                                         float ngamma, float omin) {
-#pragma unroll
-  for (int q = 2 * H; q < 2 * H + 2; ++q) {
-    const f32x2 f = fma2(dup2(ngamma), beta2_at(e, ly[q]), dup2(1.f));
-    P[q] = mul2(P[q], pk2(fmaxf(lo2(f), omin), fmaxf(hi2(f), omin)));
-  }
-}
-
-// The lane's rays in pairs: the row offset of ray i (row (lane >> 4) + 2 i),
-// far away where the ray is not in the image
-__device__ __forceinline__ void lane_rows(int lane, int rows_in, f32x2 (&ly)[kPx / 2]) {
-#pragma unroll
-  for (int q = 0; q < kPx / 2; ++q) {
-    const float y = (float)(lane >> 4) + 4 * q + 0.5f;
-    ly[q] = pk2(2 * q < rows_in ? y : 1.0e6f, 2 * q + 1 < rows_in ? y + 2.f : 1.0e6f);
-  }
-}
-
-// halves (0x3, 0xC) with a ray whose product is still >= the stop
-__device__ __forceinline__ uint32_t live_halves(const f32x2 (&P)[kPx / 2]) {
-  const bool h0 = fmaxf(fmaxf(lo2(P[0]), hi2(P[0])), fmaxf(lo2(P[1]), hi2(P[1]))) >= kShadowStop;
-  const bool h1 = fmaxf(fmaxf(lo2(P[2]), hi2(P[2])), fmaxf(lo2(P[3]), hi2(P[3]))) >= kShadowStop;
-  return (__any_sync(0xffffffffu, h0) ? 0x3u : 0u) | (__any_sync(0xffffffffu, h1) ? 0xCu : 0u);
-}
-
 // The smallest product among the lane's rays, as bits: a retired ray holds
 // -0.0, whose bits are above every positive product's.
 __device__ __forceinline__ uint32_t min_bits(const f32x2 (&P)[kPx / 2]) {
@@ -201,56 +123,6 @@ __device__ __forceinline__ uint32_t min_bits(const f32x2 (&P)[kPx / 2]) {
   m = __vimin3_u32(m, (uint32_t)(P[1] >> 32), (uint32_t)P[2]);
   m = __vimin3_u32(m, (uint32_t)(P[2] >> 32), (uint32_t)P[3]);
   return min(m, (uint32_t)(P[3] >> 32));
-}
-
-// A(C_s) of the lane's rays: 1 / 0 (in / outside the image) for a tile's
-// first segment, else the predecessor's publication (read from L2: it was
-// written on another SM); flag 2 publishes that every ray stopped.
-__device__ __forceinline__ void load_entering(const ShadowParams& p, bool first, uint32_t wpred, uint32_t flag, int lane,
-                                              int rows_in, f32x2 (&A)[kPx / 2]) {
-  auto one = [&](int i) {
-    return first ? (i < rows_in ? 1.f : 0.f)
-                 : (flag == 2u ? 0.f : __ldcg(p.pub_a + (size_t)wpred * 256 + 32 * i + lane));
-  };
-#pragma unroll
-  for (int q = 0; q < kPx / 2; ++q) A[q] = pk2(one(2 * q), one(2 * q + 1));
-}
-
-// The segment a work item names.
-struct SegItem {
-  int tx, ty, rows_in;
-  uint32_t R0, R1, C0, C1, wpred;
-  bool first, last;
-};
-
-__device__ __forceinline__ SegItem seg_item(const ShadowParams& p, uint32_t w, int lane) {
-  const uint4 d = p.desc[w];
-  SegItem it;
-  const int tile = (int)(d.x & ~kSegLast);
-  it.last = (d.x & kSegLast) != 0u;
-  it.first = d.w == kNoItem;
-  it.tx = tile % p.gx;
-  it.ty = tile / p.gx;
-  it.R0 = d.y;
-  it.R1 = d.z;
-  it.wpred = d.w;
-  it.C0 = it.C1 = it.R0;
-  if (it.R1 > it.R0) {  // an empty tile has one segment without entries
-    it.C0 = p.kbound[it.R0];
-    it.C1 = p.kbound[it.last ? it.R1 - 1 : it.R1];
-  }
-  // ray i of the lane is row (lane >> 4) + 2 i: rows below the image hold no ray
-  const int lxi = lane & 15, lyi = lane >> 4;
-  it.rows_in = it.tx * kTile + lxi < p.W ? min(kPx, (p.H - it.ty * kTile - lyi + 1) / 2) : 0;
-  return it;
-}
-
-// The next work item of the warp (a ticket), or false past the last.
-__device__ __forceinline__ bool next_item(uint32_t* ticket, uint32_t total, int lane, uint32_t& w) {
-  uint32_t t = 0;
-  if (lane == 0) t = atomicAdd(ticket, 1u);
-  w = __shfl_sync(0xffffffffu, t, 0);
-  return w < total;
 }
 
 // K6a: A(C_s+1) of every segment but a tile's last, chained from A(C_s).
@@ -722,7 +594,7 @@ __device__ __forceinline__ void live_item(const ShadowParams& p, uint32_t w, Sha
     if (ends & (1u << i)) record(i, i & 1 ? hi2(P[i / 2]) : lo2(P[i / 2]), it.last ? kNoStop : it.C1);
 }
 
-// 6 blocks per SM (80 registers): 0.453 ms against 0.476 at 5 and 0.524 at 4
+// 6 blocks per SM (80 registers): 5 took 5 % longer and 4 took 16 % longer
 // (object workload).
 template <bool BATCH>
 __global__ void __launch_bounds__(kSegWarps * 32, 6) k_shadow(const ShadowParams p, const ShadowParams* reqs, int nreq) {
