@@ -4,8 +4,7 @@
 // Both composites stream a 16x16 tile's depth-ordered list through shared
 // memory as tile-relative entries (splat_eval.cuh): the shadow composite
 // over segments of the list with eight rays per lane, the camera composite
-// with one 128-thread block per tile (two pixels per thread, batches of 256
-// records).
+// with a warp per 8x8 quadrant (two pixels per lane, 32 records at a time).
 #include "gs3_internal.cuh"
 #include "shadow_seg.cuh"
 
@@ -743,7 +742,6 @@ __global__ void k_fill(float* x, int n, float v) {
 // Output: shading * shadow + residual per pixel.
 // ---------------------------------------------------------------------------
 constexpr int kCamThreads = 128;  // two pixels per thread
-constexpr int kCamRec = 256;      // records staged per batch
 
 struct CamParams {
   const uint32_t* list;
@@ -759,101 +757,237 @@ struct CamParams {
   float amax, tstop;
 };
 
-struct CamSmem {
-  float4 E0[kCamRec], E1[kCamRec], C0[kCamRec], C1[kCamRec];
+// Entries staged for a warp's quadrant, as the shadow splat's (centre relative
+// to the tile, conic times log2 e), the terms that pair up duplicated, with
+// COLS colour quadruples each; the slots past the last are filled up to a
+// whole group of G with entries that never pass.
+template <int COLS, int G>
+struct CamEntries {
+  float4 yc[32];          // -y, -y, c, c
+  float4 xart[32];        // x, a, r, threshold
+  float2 gi[32];          // gamma, place in the list (as bits)
+  float4 col[32][COLS];
+};
+
+// A thread's two pixels (one column, rows cy and cy + 4) in packed registers.
+struct CamPixels {
+  float lx;
+  f32x2 ly;  // far away where the pixel is outside the image or its ray stopped
+  f32x2 T;
+  uint32_t done;  // bit k: pixel k takes no more entries
+  uint32_t consumed[2];
+};
+
+// The weights alpha T with which entries t .. t + G - 1 enter the two pixels, 0
+// where they do not pass; T goes on behind them.  The alpha is gamma
+// 2^power2, the power's arithmetic that of the backward (power2_at).  A ray
+// stops before T would fall below tstop: it keeps its T, and its row moves
+// far away, so that nothing passes from there on.  The alphas of a group do
+// not depend on one another; only the product T is a chain.
+template <int COLS, int G>
+__device__ __forceinline__ void camera_weights(const CamEntries<COLS, G>& E, int t, float amax, float tstop,
+                                               CamPixels& px, f32x2 (&w)[G]) {
+  f32x2 alpha[G], T[G + 1];
+  T[0] = px.T;
+#pragma unroll
+  for (int i = 0; i < G; ++i) {
+    const ulonglong2 yc = *reinterpret_cast<const ulonglong2*>(&E.yc[t + i]);
+    const float4 q = E.xart[t + i];
+    const float dx = px.lx - q.x;
+    const f32x2 dy = add2(px.ly, yc.x);
+    const f32x2 pw = fma2(dy, fma2(yc.y, dy, dup2(q.z * dx)), dup2((q.y * dx) * dx));
+    const f32x2 ga = mul2(dup2(E.gi[t + i].x), beta2_of(pw, q.w));
+    alpha[i] = pk2(fminf(amax, lo2(ga)), fminf(amax, hi2(ga)));
+    T[i + 1] = mul2(T[i], fma2(alpha[i], dup2(-1.f), dup2(1.f)));
+  }
+  px.T = T[G];
+  if (fminf(lo2(T[G]), hi2(T[G])) < tstop) {  // once per ray: it stopped at an entry of this group
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      bool stopped = false;
+      float Tk = k ? hi2(T[G]) : lo2(T[G]);
+#pragma unroll
+      for (int i = 0; i < G; ++i) {
+        const float Tn = k ? hi2(T[i + 1]) : lo2(T[i + 1]);
+        if (!stopped && Tn < tstop) {
+          stopped = true;
+          Tk = k ? hi2(T[i]) : lo2(T[i]);
+          px.consumed[k] = __float_as_uint(E.gi[t + i].y);
+        }
+        if (stopped) alpha[i] = k ? pk2(lo2(alpha[i]), 0.f) : pk2(0.f, hi2(alpha[i]));
+      }
+      if (stopped) {
+        px.done |= 1u << k;
+        px.ly = k ? pk2(lo2(px.ly), 1.0e6f) : pk2(1.0e6f, hi2(px.ly));
+        px.T = k ? pk2(lo2(px.T), Tk) : pk2(Tk, hi2(px.T));
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < G; ++i) w[i] = mul2(alpha[i], T[i]);
+}
+
+struct CamTile {
+  float ox, oy;
+  uint32_t b, e, wq;
+  int px, py0;
 };
 
 // Block blk of a frame: tile tile_order[blk] (longest list first).  128
 // threads, two pixels each: warp w covers quadrant w (the 8x8 block at
 // (8 (w & 1), 8 (w >> 1))), lane l column l & 7 and rows l >> 3 and
-// (l >> 3) + 4 of it, so the two pixels share the entry's dx terms and a
-// warp skips an entry whose box and ellipse miss its quadrant.  Records are
-// staged as shadow-splat entries (centre relative to the tile, conic times
-// log2 e): the alpha is gamma 2^power2, the power's arithmetic that of the
-// backward (power2_at).
-__device__ __forceinline__ void camera_tile(const CamParams& p, int blk, CamSmem& M) {
+// (l >> 3) + 4 of it, so the two pixels share the entry's dx terms.
+__device__ __forceinline__ CamTile camera_tile_of(const CamParams& p, int blk, CamPixels& x) {
   const int tile = (int)p.tile_order[blk];
   const int tx = tile % p.gx, ty = tile / p.gx;
-  const float ox = (float)(tx * kTile), oy = (float)(ty * kTile);
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  const uint32_t wq = 1u << w;
-  const int cx = 8 * (w & 1) + (lane & 7), cy0 = 8 * (w >> 1) + (lane >> 3);
-  const int px = tx * kTile + cx, py[2] = {ty * kTile + cy0, ty * kTile + cy0 + 4};
-  const float lx = cx + 0.5f, ly0 = cy0 + 0.5f, ly1 = cy0 + 4.5f;
-  const uint32_t b = p.tile_start[tile], e = p.tile_start[tile + 1];
-  float T[2] = {1.f, 1.f}, acc[2][7];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int cx = 8 * (w & 1) + (lane & 7), cy = 8 * (w >> 1) + (lane >> 3);
+  CamTile t{(float)(tx * kTile), (float)(ty * kTile), p.tile_start[tile], p.tile_start[tile + 1], 1u << w,
+            tx * kTile + cx, ty * kTile + cy};
+  const bool in0 = t.px < p.W && t.py0 < p.H, in1 = t.px < p.W && t.py0 + 4 < p.H;
+  x.lx = cx + 0.5f;
+  x.ly = pk2(in0 ? cy + 0.5f : 1.0e6f, in1 ? cy + 4.5f : 1.0e6f);
+  x.T = dup2(1.f);
+  x.done = (in0 ? 0u : 1u) | (in1 ? 0u : 2u);
+  x.consumed[0] = x.consumed[1] = t.e - t.b;
+  return t;
+}
+
+// 16 bytes from global to shared memory, asynchronously (cp.async)
+__device__ __forceinline__ void copy16_async(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
+// Composites a quadrant's list: each warp on its own takes 32 entries at a
+// time, one per lane, keeps those whose box and ellipse reach its quadrant,
+// stages them side by side and walks them G at a time; cols(E, slot, rank)
+// starts the copies of an entry's colours, use(E, t, w) adds G weighted
+// entries.  It leaves when every pixel is done.  The next 32 entries are
+// staged, and the records and ranks of those behind them asked for, before
+// the current ones are walked.  No block barrier: a quadrant does not wait
+// for another.
+template <int COLS, int G, typename Cols, typename Use>
+__device__ __forceinline__ void camera_walk(const CamParams& p, const CamTile& t, CamPixels& x,
+                                            CamEntries<COLS, G> (&E)[2], Cols&& cols, Use&& use) {
+  const int lane = threadIdx.x & 31;
+  auto rank_at = [&](uint32_t i) { return i < t.e ? p.list[i] : 0u; };
+  struct Rec {
+    float4 a, b, c;
+  };
+  auto rec_at = [&](uint32_t r) { return Rec{p.rrec[r].a, p.rrec[r].b, p.rrec[r].c}; };
+  // entries [rb, rb + 32) into a buffer; returns how many reach the quadrant
+  auto stage = [&](CamEntries<COLS, G>& B, uint32_t rb, uint32_t rank, const Rec& rec) {
+    SplatRec q;
+    q.a = rec.a; q.b = rec.b; q.c = rec.c;
+    float4 e0, e1;
+    make_entry(q, t.ox, t.oy, e0, e1);
+    const bool hit = rb + lane < t.e && (__float_as_uint(e1.w) & ellipse_halves(e0, e1) & t.wq) != 0u;
+    const uint32_t m = __ballot_sync(0xffffffffu, hit);
+    const int n = __popc(m), slot = __popc(m & ((1u << lane) - 1u));
+    if (hit) {
+      B.yc[slot] = make_float4(-e0.y, -e0.y, e0.w, e0.w);
+      B.xart[slot] = make_float4(e0.x, e0.z, e1.x, e1.y);
+      B.gi[slot] = make_float2(e1.z, __uint_as_float(rb - t.b + lane));
+      cols(B, slot, rank);
+    } else {  // lanes without a hit fill the last group
+      const int fill = n + lane - slot;
+      if (fill < (n + G - 1) / G * G) {
+        B.yc[fill] = make_float4(0.f, 0.f, 0.f, 0.f);
+        B.xart[fill] = make_float4(0.f, 0.f, 0.f, 1.f);  // power 0, below its threshold
+        B.gi[fill] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int c = 0; c < COLS; ++c) B.col[fill][c] = make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    return n;
+  };
+  if (t.b >= t.e) return;
+  uint32_t rank = rank_at(t.b + lane);
+  Rec rec = rec_at(rank);
+  uint32_t rank2 = rank_at(t.b + 32 + lane);
+  int n = stage(E[0], t.b, rank, rec), buf = 0;
+  rank = rank2;
+  rec = rec_at(rank);
+  rank2 = rank_at(t.b + 64 + lane);
+  for (uint32_t rb = t.b; rb < t.e; rb += 32) {
+    if (__all_sync(0xffffffffu, x.done == 3u)) break;
+    int next = 0;
+    if (rb + 32 < t.e) {
+      next = stage(E[buf ^ 1], rb + 32, rank, rec);
+      rank = rank2;
+      rec = rec_at(rank);
+      rank2 = rank_at(rb + 128 + lane - 32);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncwarp();
+    for (int k = 0; k < n; k += G) {
+      f32x2 w[G];
+      camera_weights(E[buf], k, p.amax, p.tstop, x, w);
+      use(E[buf], k, w);
+    }
+    __syncwarp();  // the buffer is free again
+    n = next;
+    buf ^= 1;
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// Bound: issue slots and the FMA pipe, once a warp has independent work.
+// Object workload (443 entries per quadrant and 5,100 in its list) / 1 M at
+// 1024 x 1024: 0.400 / 0.797 ms with block-wide batches of 256 records and
+// scalar updates under branches (0.406 / 0.797 with the updates packed and
+// without branches: a warp waited on its loads and the chain of T); 0.297 /
+// 0.620 with a list per quadrant and four entries at a time; 0.255 / 0.535
+// with the next entries staged ahead.  Two entries at a time take the same
+// time, eight 5 % longer.
+constexpr int kCamGroup = 4;
+using CamSmem = CamEntries<2, kCamGroup>;
+
+__device__ __forceinline__ void camera_tile(const CamParams& p, int blk, CamSmem (*smem)[2]) {
+  CamPixels x;
+  const CamTile t = camera_tile_of(p, blk, x);
+  f32x2 acc[2][4];  // per pixel: (S r, g), (S b, Sh), (R r, g), (R b, -)
 #pragma unroll
   for (int k = 0; k < 2; ++k)
 #pragma unroll
-    for (int c = 0; c < 7; ++c) acc[k][c] = 0.f;
-  bool done[2] = {!(px < p.W && py[0] < p.H), !(px < p.W && py[1] < p.H)};
-  uint32_t consumed[2] = {0u, 0u};
-  for (uint32_t rb = b; rb < e; rb += kCamRec) {
-    if (__syncthreads_count(done[0] && done[1]) == kCamThreads) break;
-    const int rc = (int)min((uint32_t)kCamRec, e - rb);
-    for (int k = t; k < rc; k += kCamThreads) {
-      const uint32_t rank = p.list[rb + k];
-      float4 e0, e1;
-      make_entry(p.rrec[rank], ox, oy, e0, e1);
-      e1.w = __uint_as_float(__float_as_uint(e1.w) & ellipse_halves(e0, e1));
-      M.E0[k] = e0;
-      M.E1[k] = e1;
-      M.C0[k] = p.ccol[2 * rank];
-      M.C1[k] = p.ccol[2 * rank + 1];
-    }
-    __syncthreads();
-    if (!(done[0] && done[1])) {
-      // one pixel's step: false once its ray stopped here
-      auto take = [&](int k, int jj, float pw, float g) {
-        const float alpha = fminf(p.amax, g * ex2(pw));
-        const float Tn = T[k] * (1.f - alpha);
-        if (Tn < p.tstop) {
-          done[k] = true;
-          consumed[k] = rb - b + jj;
-          return;
-        }
-        const float wt = alpha * T[k];
-        const float4 c0 = M.C0[jj], c1 = M.C1[jj];
-        acc[k][0] += wt * c0.x; acc[k][1] += wt * c0.y; acc[k][2] += wt * c0.z;
-        acc[k][3] += wt * c0.w;
-        acc[k][4] += wt * c1.x; acc[k][5] += wt * c1.y; acc[k][6] += wt * c1.z;
-        T[k] = Tn;
-      };
-      // two records' powers are formed ahead of the updates (the same
-      // arithmetic, in the same order, as one record at a time)
-      for (int jj = 0; jj < rc; jj += 2) {
-        const float4 ea = M.E1[jj];
-        const bool two = jj + 1 < rc;
-        const float4 eb = two ? M.E1[jj + 1] : ea;
-        const bool ha = (__float_as_uint(ea.w) & wq) != 0u, hb = two && (__float_as_uint(eb.w) & wq) != 0u;
-        float pa0 = 0.f, pa1 = 0.f, pb0 = 0.f, pb1 = 0.f;
-        if (ha) powers2(M.E0[jj], ea.x, lx, ly0, ly1, pa0, pa1);
-        if (hb) powers2(M.E0[jj + 1], eb.x, lx, ly0, ly1, pb0, pb1);
-        if (ha) {
-          if (!done[0] && pa0 >= ea.y) take(0, jj, pa0, ea.z);
-          if (!done[1] && pa1 >= ea.y) take(1, jj, pa1, ea.z);
-        }
-        if (hb) {
-          if (!done[0] && pb0 >= eb.y) take(0, jj + 1, pb0, eb.z);
-          if (!done[1] && pb1 >= eb.y) take(1, jj + 1, pb1, eb.z);
-        }
-        if (done[0] && done[1]) break;
-      }
+    for (int c = 0; c < 4; ++c) acc[k][c] = 0ull;
+  camera_walk<2, kCamGroup>(
+      p, t, x, smem[threadIdx.x >> 5],
+      [&](CamSmem& E, int slot, uint32_t rank) {
+        copy16_async(&E.col[slot][0], &p.ccol[2 * (size_t)rank]);
+        copy16_async(&E.col[slot][1], &p.ccol[2 * (size_t)rank + 1]);
+      },
+      [&](const CamSmem& E, int k0, const f32x2 (&w)[kCamGroup]) {
 #pragma unroll
-      for (int k = 0; k < 2; ++k)
-        if (!done[k]) consumed[k] = rb - b + rc;
-    }
-  }
+        for (int i = 0; i < kCamGroup; ++i) {
+          const ulonglong2 c0 = *reinterpret_cast<const ulonglong2*>(&E.col[k0 + i][0]);
+          const ulonglong2 c1 = *reinterpret_cast<const ulonglong2*>(&E.col[k0 + i][1]);
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            const f32x2 wk = dup2(k ? hi2(w[i]) : lo2(w[i]));
+            acc[k][0] = fma2(wk, c0.x, acc[k][0]);
+            acc[k][1] = fma2(wk, c0.y, acc[k][1]);
+            acc[k][2] = fma2(wk, c1.x, acc[k][2]);
+            acc[k][3] = fma2(wk, c1.y, acc[k][3]);
+          }
+        }
+      });
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
-    if (px < p.W && py[k] < p.H) {
-      const size_t pix = (size_t)py[k] * p.W + px;
-      const float* a = acc[k];
+    const int py = t.py0 + 4 * k;
+    if (t.px < p.W && py < p.H) {
+      const size_t pix = (size_t)py * p.W + t.px;
+      const float a[8] = {lo2(acc[k][0]), hi2(acc[k][0]), lo2(acc[k][1]), hi2(acc[k][1]),
+                          lo2(acc[k][2]), hi2(acc[k][2]), lo2(acc[k][3]), 0.f};
       p.out[3 * pix + 0] = a[0] * a[3] + a[4];
       p.out[3 * pix + 1] = a[1] * a[3] + a[5];
       p.out[3 * pix + 2] = a[2] * a[3] + a[6];
-      p.final_t[pix] = T[k];
-      p.n_contrib[pix] = consumed[k];
+      p.final_t[pix] = k ? hi2(x.T) : lo2(x.T);
+      p.n_contrib[pix] = x.consumed[k];
       p.pix_aux[2 * pix] = make_float4(a[0], a[1], a[2], a[3]);
       p.pix_aux[2 * pix + 1] = make_float4(a[4], a[5], a[6], 0.f);
     }
@@ -865,7 +999,7 @@ __device__ __forceinline__ void camera_tile(const CamParams& p, int blk, CamSmem
 template <bool BATCH>
 __global__ void __launch_bounds__(kCamThreads) k_camera(const CamParams p, const CamParams* reqs, const uint32_t* tile_prefix,
                                                 int nreq) {
-  __shared__ CamSmem M;
+  __shared__ CamSmem M[kCamThreads / 32][2];
   if (BATCH) {
     int r = 0;
     while (r < nreq - 1 && blockIdx.x >= tile_prefix[r + 1]) ++r;
@@ -884,7 +1018,7 @@ __global__ void __launch_bounds__(kCamThreads) k_camera(const CamParams p, const
 // the residual R, which does not see the light, is composited once.
 // out (+)= sum_l w_l (S_l Sh_l + R).
 // ---------------------------------------------------------------------------
-constexpr int kEnvRec = 128;  // records staged per batch
+constexpr int kEnvGroup = 2;  // entries taken together
 
 struct EnvCamParams {
   CamParams c;           // the first light's workspace: camera splat, residual colours, final T
@@ -894,99 +1028,69 @@ struct EnvCamParams {
   int accumulate;  // add to out (a later group of lights)
 };
 
-struct EnvSmem {
-  float4 E0[kEnvRec], E1[kEnvRec], R[kEnvRec];
-  float4 C[kEnvRec][kMaxBatch];
-};
+using EnvSmem = CamEntries<kMaxBatch + 1, kEnvGroup>;  // colours: the lights', then R
 
 // The thread layout and entry arithmetic of camera_tile, with 4 accumulators
 // per light and pixel plus 3 for R.
 __global__ void __launch_bounds__(kCamThreads) k_camera_env(const EnvCamParams e) {
-  __shared__ EnvSmem M;
+  __shared__ EnvSmem M[kCamThreads / 32][2];
   const CamParams& p = e.c;
   const int nl = e.nl;
-  const int tile = (int)p.tile_order[blockIdx.x];
-  const int tx = tile % p.gx, ty = tile / p.gx;
-  const float ox = (float)(tx * kTile), oy = (float)(ty * kTile);
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-  const uint32_t wq = 1u << w;
-  const int cx = 8 * (w & 1) + (lane & 7), cy0 = 8 * (w >> 1) + (lane >> 3);
-  const int px = tx * kTile + cx, py[2] = {ty * kTile + cy0, ty * kTile + cy0 + 4};
-  const float lx = cx + 0.5f, ly0 = cy0 + 0.5f, ly1 = cy0 + 4.5f;
-  const uint32_t b = p.tile_start[tile], end = p.tile_start[tile + 1];
-  float T[2] = {1.f, 1.f}, R[2][3], S[2][kMaxBatch][3], Sh[2][kMaxBatch];
+  CamPixels x;
+  const CamTile t = camera_tile_of(p, (int)blockIdx.x, x);
+  f32x2 R[2][2], S[2][kMaxBatch][2];  // per pixel: (R r, g), (R b, -); per light (S r, g), (S b, Sh)
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
-    R[k][0] = R[k][1] = R[k][2] = 0.f;
+    R[k][0] = R[k][1] = 0ull;
 #pragma unroll
-    for (int l = 0; l < kMaxBatch; ++l) S[k][l][0] = S[k][l][1] = S[k][l][2] = Sh[k][l] = 0.f;
+    for (int l = 0; l < kMaxBatch; ++l) S[k][l][0] = S[k][l][1] = 0ull;
   }
-  bool done[2] = {!(px < p.W && py[0] < p.H), !(px < p.W && py[1] < p.H)};
-  uint32_t consumed[2] = {0u, 0u};
-  for (uint32_t rb = b; rb < end; rb += kEnvRec) {
-    if (__syncthreads_count(done[0] && done[1]) == kCamThreads) break;
-    const int rc = (int)min((uint32_t)kEnvRec, end - rb);
-    if (t < rc) {
-      const uint32_t rank = p.list[rb + t];
-      float4 e0, e1;
-      make_entry(p.rrec[rank], ox, oy, e0, e1);
-      e1.w = __uint_as_float(__float_as_uint(e1.w) & ellipse_halves(e0, e1));
-      M.E0[t] = e0;
-      M.E1[t] = e1;
-      M.R[t] = p.ccol[2 * rank + 1];
-      const float4* src = e.envcol + (size_t)rank * nl;
+  camera_walk<kMaxBatch + 1, kEnvGroup>(
+      p, t, x, M[threadIdx.x >> 5],
+      [&](EnvSmem& E, int slot, uint32_t rank) {
+        const float4* src = e.envcol + (size_t)rank * nl;
 #pragma unroll
-      for (int l = 0; l < kMaxBatch; ++l)
-        if (l < nl) M.C[t][l] = src[l];
-    }
-    __syncthreads();
-    if (!(done[0] && done[1])) {
-      auto take = [&](int k, int jj, float pw, float g) {
-        const float alpha = fminf(p.amax, g * ex2(pw));
-        const float Tn = T[k] * (1.f - alpha);
-        if (Tn < p.tstop) {
-          done[k] = true;
-          consumed[k] = rb - b + jj;
-          return;
-        }
-        const float wt = alpha * T[k];
+        for (int l = 0; l < kMaxBatch; ++l)
+          if (l < nl) copy16_async(&E.col[slot][l], src + l);
+        copy16_async(&E.col[slot][kMaxBatch], &p.ccol[2 * (size_t)rank + 1]);
+      },
+      [&](const EnvSmem& E, int k0, const f32x2 (&w)[kEnvGroup]) {
 #pragma unroll
-        for (int l = 0; l < kMaxBatch; ++l) {
-          if (l < nl) {
-            const float4 c = M.C[jj][l];
-            S[k][l][0] += wt * c.x; S[k][l][1] += wt * c.y; S[k][l][2] += wt * c.z;
-            Sh[k][l] += wt * c.w;
+        for (int i = 0; i < kEnvGroup; ++i) {
+          if (!__any_sync(0xffffffffu, w[i] != 0ull)) continue;
+          const f32x2 wk[2] = {dup2(lo2(w[i])), dup2(hi2(w[i]))};
+          const ulonglong2 r = *reinterpret_cast<const ulonglong2*>(&E.col[k0 + i][kMaxBatch]);
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            R[k][0] = fma2(wk[k], r.x, R[k][0]);
+            R[k][1] = fma2(wk[k], r.y, R[k][1]);
+          }
+#pragma unroll
+          for (int l = 0; l < kMaxBatch; ++l) {
+            if (l < nl) {
+              const ulonglong2 c = *reinterpret_cast<const ulonglong2*>(&E.col[k0 + i][l]);
+#pragma unroll
+              for (int k = 0; k < 2; ++k) {
+                S[k][l][0] = fma2(wk[k], c.x, S[k][l][0]);
+                S[k][l][1] = fma2(wk[k], c.y, S[k][l][1]);
+              }
+            }
           }
         }
-        const float4 r = M.R[jj];
-        R[k][0] += wt * r.x; R[k][1] += wt * r.y; R[k][2] += wt * r.z;
-        T[k] = Tn;
-      };
-      for (int jj = 0; jj < rc; ++jj) {
-        const float4 e1 = M.E1[jj];
-        if (!(__float_as_uint(e1.w) & wq)) continue;  // warp-uniform
-        float p0, p1;
-        powers2(M.E0[jj], e1.x, lx, ly0, ly1, p0, p1);
-        if (!done[0] && p0 >= e1.y) take(0, jj, p0, e1.z);
-        if (!done[1] && p1 >= e1.y) take(1, jj, p1, e1.z);
-        if (done[0] && done[1]) break;
-      }
-#pragma unroll
-      for (int k = 0; k < 2; ++k)
-        if (!done[k]) consumed[k] = rb - b + rc;
-    }
-  }
+      });
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
-    if (!(px < p.W && py[k] < p.H)) continue;
-    const size_t pix = (size_t)py[k] * p.W + px;
+    const int py = t.py0 + 4 * k;
+    if (!(t.px < p.W && py < p.H)) continue;
+    const size_t pix = (size_t)py * p.W + t.px;
     float o0 = 0.f, o1 = 0.f, o2 = 0.f;
 #pragma unroll
     for (int l = 0; l < kMaxBatch; ++l) {
       if (l < nl) {
         // the image light l's own frame gives, then its weight
-        const float i0 = S[k][l][0] * Sh[k][l] + R[k][0], i1 = S[k][l][1] * Sh[k][l] + R[k][1],
-                    i2 = S[k][l][2] * Sh[k][l] + R[k][2];
+        const float sh = hi2(S[k][l][1]);
+        const float i0 = lo2(S[k][l][0]) * sh + lo2(R[k][0]), i1 = hi2(S[k][l][0]) * sh + hi2(R[k][0]),
+                    i2 = lo2(S[k][l][1]) * sh + lo2(R[k][1]);
         o0 = fmaf(e.w[l], i0, o0);
         o1 = fmaf(e.w[l], i1, o1);
         o2 = fmaf(e.w[l], i2, o2);
@@ -1000,8 +1104,8 @@ __global__ void __launch_bounds__(kCamThreads) k_camera_env(const EnvCamParams e
     p.out[3 * pix + 0] = o0;
     p.out[3 * pix + 1] = o1;
     p.out[3 * pix + 2] = o2;
-    p.final_t[pix] = T[k];
-    p.n_contrib[pix] = consumed[k];
+    p.final_t[pix] = k ? hi2(x.T) : lo2(x.T);
+    p.n_contrib[pix] = x.consumed[k];
   }
 }
 

@@ -74,19 +74,9 @@ __device__ __forceinline__ uint32_t ellipse_halves(const float4 e0, const float4
   return m;
 }
 
-// power2 at the thread's two pixels (lx, ly0), (lx, ly1): the dx terms are shared
-__device__ __forceinline__ void powers2(const float4 e0, float r, float lx, float ly0, float ly1, float& p0,
-                                        float& p1) {
-  const float dx = lx - e0.x;
-  const float sx = (e0.z * dx) * dx, v = r * dx;
-  const float dy0 = ly0 - e0.y, dy1 = ly1 - e0.y;
-  p0 = fmaf(dy0, fmaf(e0.w, dy0, v), sx);
-  p1 = fmaf(dy1, fmaf(e0.w, dy1, v), sx);
-}
-
-// The same power2 at one pixel (lx, ly) of the tile: the camera composite
-// and its backward evaluate an entry with this arithmetic (powers2 is its
-// two-pixel form), so both take every alpha decision alike.
+// power2 at one pixel (lx, ly) of the tile: the camera composite and its
+// backward evaluate an entry with this arithmetic, so both take every alpha
+// decision alike.
 __device__ __forceinline__ float power2_at(const float4 e0, float r, float lx, float ly) {
   const float dx = lx - e0.x;
   const float sx = (e0.z * dx) * dx, v = r * dx;
@@ -95,14 +85,13 @@ __device__ __forceinline__ float power2_at(const float4 e0, float r, float lx, f
 }
 
 // A shadow ray stops taking occluders once its product A falls below
-// kShadowStop: the occluder that takes A below it is the last one applied,
-// and A stays frozen after it.  Every receiver behind the stop would see an
-// exact product in [0, kShadowStop) and sees the frozen one, also in
-// [0, kShadowStop), so each T_m(j) and every beta-weighted average of them
-// moves by less than kShadowStop.  Without the stop, FP32 products underflow
+// kShadowStop: the occluder that takes A below it is the last one applied.
+// Every receiver behind the stop would see an exact product in
+// [0, kShadowStop) and sees 0, so each T_m(j) and every beta-weighted average
+// of them moves by less than kShadowStop.  Without the stop, FP32 products underflow
 // on deep rays (thousands of passing entries through an object), and the
 // backward, which rebuilds A from the ray's final product, would rebuild 0
-// for every receiver of such a ray.  A frozen A is at least
+// for every receiver of such a ray.  The product a ray stops with is at least
 // kShadowStop (1 - alpha_max), far from the denormals.
 constexpr float kShadowStop = 0x1p-40f;
 constexpr uint32_t kNoStop = 0xFFFFFFFFu;  // the ray never stopped
