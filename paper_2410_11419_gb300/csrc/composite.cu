@@ -17,8 +17,8 @@ namespace {
 // alpha test, T_m(j) = prod (1 - alpha_k,m) over passing k with
 // d_k < d_j - bias.  The list is ordered by distance, so the occluders of j
 // form a prefix of the tile's list; its end K(j) is precomputed per entry
-// (k_bound_starts, k_bound_rest, from the distances the binning writes beside
-// the list) and is non-decreasing in j.
+// (k_bound_starts, k_bound_rest, from each Gaussian's bound among the depth
+// ranks) and is non-decreasing in j.
 //
 // Work is split into segments of a tile's list: segment s holds receivers
 // [R_s, R_s+1) (kSegLen entries; the last takes the rest) and needs the
@@ -612,15 +612,30 @@ __global__ void __launch_bounds__(kSegWarps * 32, 6) k_shadow(const ShadowParams
   }
 }
 
-// K(i) of entry i of a light list: the first index of i's tile list whose
-// distance is >= d_i - bias, the end of i's occluder prefix, which lies in
-// [lo, hi] (at most i).
-__device__ __forceinline__ uint32_t occ_bound(const float* __restrict__ dl, uint32_t lo, uint32_t hi, uint32_t i,
-                                              float bias) {
-  const float thr = __fsub_rn(dl[i], bias);
+// The ranks that shadow rank r's Gaussian are those of smaller distance:
+// bound[r] = the first rank whose distance is >= d_r - bias (at most r).  The
+// depth sort leaves the distances' bit patterns in rank order.
+__global__ void __launch_bounds__(256) k_rank_bound(const float* __restrict__ dist, uint32_t* __restrict__ bound, int n,
+                                                    float bias) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= n) return;
+  const float thr = __fsub_rn(dist[r], bias);
+  uint32_t lo = 0u, hi = (uint32_t)r;
   while (lo < hi) {
     const uint32_t mid = (lo + hi) >> 1;
-    if (dl[mid] < thr) lo = mid + 1; else hi = mid;
+    if (dist[mid] < thr) lo = mid + 1; else hi = mid;
+  }
+  bound[r] = lo;
+}
+
+// K(i) of an entry of a light list whose Gaussian's rank bound is `first`: the
+// first index of the tile's list with a rank >= first, the end of the
+// entry's occluder prefix, which lies in [lo, hi].
+__device__ __forceinline__ uint32_t occ_bound(const uint32_t* __restrict__ list, uint32_t lo, uint32_t hi,
+                                              uint32_t first) {
+  while (lo < hi) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if (list[mid] < first) lo = mid + 1; else hi = mid;
   }
   return lo;
 }
@@ -639,8 +654,8 @@ __device__ __forceinline__ int item_level(const uint32_t* lvl_off, uint32_t w) {
 // The items' descriptors, and K at the entries the segment plan reads (every
 // segment's first entry and every tile's last), one thread per segment,
 // before K6a.
-__global__ void __launch_bounds__(256) k_bound_starts(const ShadowParams p, const float* __restrict__ dl,
-                                                      uint32_t* __restrict__ kb, float bias) {
+__global__ void __launch_bounds__(256) k_bound_starts(const ShadowParams p,
+                                                      const uint32_t* __restrict__ bound, uint32_t* __restrict__ kb) {
   const uint32_t w = blockIdx.x * blockDim.x + threadIdx.x;
   if (w >= p.lvl_off[kSegLevels]) return;
   const int s = item_level(p.lvl_off, w);
@@ -651,8 +666,8 @@ __global__ void __launch_bounds__(256) k_bound_starts(const ShadowParams p, cons
   const uint32_t r0 = b + (uint32_t)s * kSegLen, r1 = last ? e : r0 + kSegLen;
   p.desc[w] = make_uint4((uint32_t)tile | (last ? kSegLast : 0u), r0, r1, s > 0 ? p.lvl_off[s - 1] + pos : kNoItem);
   if (e <= b) return;
-  kb[r0] = occ_bound(dl, b, r0, r0, bias);
-  if (last && e - 1 > r0) kb[e - 1] = occ_bound(dl, b, e - 1, e - 1, bias);
+  kb[r0] = occ_bound(p.list, b, r0, bound[p.list[r0]]);
+  if (last && e - 1 > r0) kb[e - 1] = occ_bound(p.list, b, e - 1, bound[p.list[e - 1]]);
 }
 
 // After K6a, one warp per segment: the lists of the segments with an open
@@ -661,8 +676,8 @@ __global__ void __launch_bounds__(256) k_bound_starts(const ShadowParams p, cons
 // between the segment's first bound and the next segment's.  No kernel takes
 // an occluder for the entries of a stopped segment, so theirs stay unwritten
 // past the first.
-__global__ void __launch_bounds__(256) k_bound_rest(const ShadowParams p, const float* __restrict__ dl,
-                                                    uint32_t* __restrict__ kb, float bias) {
+__global__ void __launch_bounds__(256) k_bound_rest(const ShadowParams p, const uint32_t* __restrict__ bound,
+                                                    uint32_t* __restrict__ kb) {
   __shared__ uint32_t cnt[2], base[2];
   const uint32_t total = p.lvl_off[kSegLevels];
   if (blockIdx.x * 8u >= total) return;
@@ -685,7 +700,8 @@ __global__ void __launch_bounds__(256) k_bound_rest(const ShadowParams p, const 
   if (dead != 0 || d.z <= d.y) return;
   const bool last = (d.x & kSegLast) != 0u;
   const uint32_t c0 = kb[d.y], c1 = kb[last ? d.z - 1 : d.z];
-  for (uint32_t j = d.y + 1 + lane; j < d.z - (last ? 1u : 0u); j += 32) kb[j] = occ_bound(dl, c0, min(c1, j), j, bias);
+  for (uint32_t j = d.y + 1 + lane; j < d.z - (last ? 1u : 0u); j += 32)
+    kb[j] = occ_bound(p.list, c0, min(c1, j), bound[p.list[j]]);
 }
 
 // K7: per Gaussian, sum its (tile) partials; T = num / den, or 1 when the
@@ -1208,7 +1224,7 @@ ShadowParams shadow_params(const FrameArgs& f) {
   p.rrec = at<SplatRec>(ws, b.rrec);
   p.off = at<uint32_t>(ws, b.off);
   p.kbound = at<uint32_t>(ws, b.tv[1 - fin]);
-  p.pass_mask = at<uint8_t>(ws, b.tk[1 - fin]);  // over the distances, once the occluder bounds are done
+  p.pass_mask = at<uint8_t>(ws, b.tk[1 - fin]);
   p.partial = at<float2>(ws, f.L->partial);
   p.light_final = at<float>(ws, f.L->light_final);
   p.light_stop = at<uint32_t>(ws, f.L->light_stop);
@@ -1290,8 +1306,6 @@ void prepare_shadow_composite(const FrameArgs& f, cudaStream_t s) {
   const SplatBufs& b = f.L->sp[1];
   unsigned char* ws = f.ws;
   const int fin = (f.L->ntiles <= 256 ? 1 : 2) & 1;
-  // the distance of every list entry (written by the binning) and the occluder bounds
-  float* dl = at<float>(ws, b.tk[1 - fin]);
   uint32_t* kb = at<uint32_t>(ws, b.tv[1 - fin]);
   // the light tiles by segment count, and the work items of each segment level
   uint32_t* lvl = at<uint32_t>(ws, f.L->seg_lvl);
@@ -1302,8 +1316,11 @@ void prepare_shadow_composite(const FrameArgs& f, cudaStream_t s) {
                                   kSegLen, lvl);
   // the occluder bounds the segment plan reads; the rest follow K6a
   const size_t items = shadow_seg_items(f.L->ntiles, f.L->cap);
-  k_bound_starts<<<(int)((items + 255) / 256), 256, 0, s>>>(shadow_params(f), dl, kb, f.opts.shadow_bias);
-  count_launch(2);
+  const int n = f.sc.n;
+  uint32_t* bound = at<uint32_t>(ws, b.sk[0]);  // free once the depths are sorted
+  k_rank_bound<<<(n + 255) / 256, 256, 0, s>>>(at<float>(ws, b.sk[1]), bound, n, f.opts.shadow_bias);
+  k_bound_starts<<<(int)((items + 255) / 256), 256, 0, s>>>(shadow_params(f), bound, kb);
+  count_launch(3);
 }
 
 // the occluder bounds of the open segments' other entries (after K6a)
@@ -1311,8 +1328,8 @@ void launch_bound_rest(const FrameArgs& f, const ShadowParams& p, cudaStream_t s
   const SplatBufs& b = f.L->sp[1];
   const int fin = (f.L->ntiles <= 256 ? 1 : 2) & 1;
   const size_t items = shadow_seg_items(f.L->ntiles, f.L->cap);
-  k_bound_rest<<<(int)((items * 32 + 255) / 256), 256, 0, s>>>(p, at<float>(f.ws, b.tk[1 - fin]),
-                                                               at<uint32_t>(f.ws, b.tv[1 - fin]), f.opts.shadow_bias);
+  k_bound_rest<<<(int)((items * 32 + 255) / 256), 256, 0, s>>>(p, at<uint32_t>(f.ws, b.sk[0]),
+                                                               at<uint32_t>(f.ws, b.tv[1 - fin]));
   count_launch();
 }
 

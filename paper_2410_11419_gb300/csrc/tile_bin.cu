@@ -16,14 +16,26 @@
 //            after the pairs of the rows above, which gives every tile's
 //            start and every chunk's offset in each of its tiles; k_bin_place
 //            writes the list entries.
-// Both placements take 256 items at a time, one per thread, in order.  A
-// warp's offset in bucket x is the bucket's running offset plus the items of
-// earlier warps covering x (per-warp difference arrays); inside a warp the
-// (item, bucket) pairs are dealt 32 per round in item order, and a pair's
+// Up to kScanBuckets rows or columns, each placement goes over the buckets
+// (scan_place): a warp holds 256 items, eight per lane, and for every bucket
+// it owns asks which of them cover it (a ballot per 32 items), which gives the
+// bucket's entries in item order, side by side in memory, without shared
+// memory or barriers.  That is 64 instructions per bucket and 256 items
+// whatever the spans, so past that many buckets it loses to going over the
+// (item, bucket) pairs (place_spans), about 4.6 instructions each: 256 items,
+// one per thread; a warp's offset in bucket x is the bucket's running offset
+// plus the items of earlier warps covering x (per-warp difference arrays);
+// inside a warp the pairs are dealt 32 per round in item order, and a pair's
 // rank among the round's pairs of the same bucket (match_any) is added to a
-// per-bucket counter.  Every list is therefore in rank order, the result a
+// per-bucket counter.  Either way every list is in rank order, the result a
 // stable sort of the pairs by tile would give, and no step depends on timing
 // or waits on another block.
+// Bound: the scattered 4-byte stores of the list (a bucket's run of 256 items
+// holds about 36 entries) and the ballots.  Rows + counts + placement of both
+// splats, beside the shadow composite (over the pairs, the light splat also
+// writing each entry's distance, -> over the buckets): 300k Gaussians at
+// 800 x 800 0.06 + 0.12 + 0.26 -> 0.04 + 0.08 + 0.14 ms, 1 M at 1024 x 1024
+// 0.19 + 0.54 + 1.57 -> 0.11 + 0.38 + 0.70 ms.
 #include <climits>
 
 #include "gs3_internal.cuh"
@@ -201,6 +213,39 @@ __device__ void place_spans(SpanSmem& S, int nbk, int a, int b, uint32_t v0, uin
   __syncthreads();  // S is rewritten by the next call
 }
 
+// A warp's 256 items in order, eight per lane (item 32 c + lane at c): item c
+// covers buckets lo .. lo + wid (lo = kNoSpan: none).
+constexpr int kScanBuckets = 128;
+constexpr uint32_t kNoSpan = 0x80000000u;
+struct WarpSpans {
+  uint32_t lo[8], wid[8], v0[8];
+};
+
+// Stable placement of a warp's 256 items into the buckets x = first, first +
+// step, ... < nbk, `first + step l` starting at lane l's base: an item's copy
+// for bucket x goes to out0[base + the earlier items covering x], and
+// v1 likewise to out1 if out1 is given.
+template <bool TWO>
+__device__ __forceinline__ void scan_place(const WarpSpans& S, const uint32_t (&v1)[8], int nbk, int first, int step,
+                                           uint32_t base, uint32_t* __restrict__ out0, uint32_t* __restrict__ out1,
+                                           size_t cap) {
+  const uint32_t below = (1u << (threadIdx.x & 31)) - 1u;
+  for (int x = first, l = 0; x < nbk; x += step, ++l) {
+    uint32_t at = __shfl_sync(0xffffffffu, base, l);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const bool in = (uint32_t)x - S.lo[c] <= S.wid[c];
+      const uint32_t m = __ballot_sync(0xffffffffu, in);
+      const uint32_t pos = at + (uint32_t)__popc(m & below);
+      if (in && pos < cap) {
+        out0[pos] = S.v0[c];
+        if (TWO) out1[pos] = v1[c];
+      }
+      at += (uint32_t)__popc(m);
+    }
+  }
+}
+
 // Each row's block counts scanned in place (exclusive, within the row); the
 // row's total goes to rs[y] for k_bin_plan.
 __global__ void __launch_bounds__(kBinThreads) k_bin_rowtot(uint32_t* __restrict__ row_cnt, int nb, int gy,
@@ -281,6 +326,108 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_rows(int n, const SplatRec*
   place_spans(S, gy, a, b, (uint32_t)r, span, rowseq, rowspan, cap);
 }
 
+// k_bin_rows going over the rows (gy <= kScanBuckets).
+__global__ void __launch_bounds__(kBinThreads) k_bin_rows_scan(int n, const SplatRec* __restrict__ rrec,
+                                                               const uint32_t* __restrict__ row_cnt, int nb, int gy,
+                                                               const uint32_t* __restrict__ plan,
+                                                               uint32_t* __restrict__ rowseq,
+                                                               uint32_t* __restrict__ rowspan, size_t cap) {
+  if (plan[3 * gy + 2] == 0u) return;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  WarpSpans S;
+  uint32_t span[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const int r = blockIdx.x * kBinThreads + 32 * c + lane;
+    int4 q = make_int4(-1, 0, 0, 0);
+    if (r < n) q = rrec[r].r;
+    S.lo[c] = q.x >= 0 ? (uint32_t)q.y : kNoSpan;
+    S.wid[c] = q.x >= 0 ? (uint32_t)(q.w - q.y) : 0u;
+    S.v0[c] = (uint32_t)r;
+    span[c] = (uint32_t)q.x | ((uint32_t)q.z << 16);
+  }
+  const int y = w + kBinWarps * lane;
+  const uint32_t base = y < gy ? plan[y] + row_cnt[(size_t)y * nb + blockIdx.x] : 0u;
+  scan_place<true>(S, span, gy, w, kBinWarps, base, rowseq, rowspan, cap);
+}
+
+// A chunk of at most 256 items of a row's sequence, for a warp
+__device__ __forceinline__ void load_chunk(const uint32_t* __restrict__ rowspan, uint32_t i0, uint32_t i1, int lane,
+                                           WarpSpans& S) {
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const uint32_t i = i0 + 32 * c + lane;
+    const uint32_t sp = i < i1 ? rowspan[i] : kNoSpan;
+    S.lo[c] = i < i1 ? sp & 0xFFFFu : kNoSpan;
+    S.wid[c] = i < i1 ? (sp >> 16) - (sp & 0xFFFFu) : 0u;
+  }
+}
+
+// k_bin_count going over the columns (gx <= kScanBuckets, chunks of 256).
+__global__ void __launch_bounds__(kBinThreads) k_bin_count_scan(const uint32_t* __restrict__ rowspan,
+                                                                uint32_t* __restrict__ plan, int gx, int gy,
+                                                                uint32_t* __restrict__ tab) {
+  __shared__ uint32_t pairs[2];  // the chunk's list entries, chunks in turn
+  BinPlan P(plan, gy);
+  if (*P.ok == 0u) return;
+  const uint32_t C = P.cb[gy];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (threadIdx.x < 2) pairs[threadIdx.x] = 0u;
+  __syncthreads();
+  int turn = 0;
+  for (uint32_t kg = blockIdx.x; kg < C; kg += gridDim.x, turn ^= 1) {
+    const int y = chunk_row(P.cb, gy, kg);
+    const uint32_t c0 = P.cb[y], nch = P.cb[y + 1] - c0, k = kg - c0;
+    const uint32_t i0 = P.rs[y] + 256u * k, i1 = min(P.rs[y + 1], i0 + 256u);
+    WarpSpans S;
+    load_chunk(rowspan, i0, i1, lane, S);
+    uint32_t mine = 0u, total = 0u;  // lane l keeps the count of column w + 8 l
+    for (int x = w, l = 0; x < gx; x += kBinWarps, ++l) {
+      uint32_t n = 0u;
+#pragma unroll
+      for (int c = 0; c < 8; ++c) n += (uint32_t)__popc(__ballot_sync(0xffffffffu, (uint32_t)x - S.lo[c] <= S.wid[c]));
+      if (lane == l) mine = n;
+      total += n;
+    }
+    const int x = w + kBinWarps * lane;
+    if (x < gx) tab[(size_t)c0 * gx + (size_t)x * nch + k] = mine;
+    if (lane == 0 && total) atomicAdd(&pairs[turn], total);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      if (pairs[turn]) atomicAdd(P.pairs + y, pairs[turn]);
+      pairs[turn] = 0u;  // used again after the next chunk's barrier
+    }
+  }
+}
+
+// k_bin_place going over the columns (gx <= kScanBuckets, chunks of 256).
+__global__ void __launch_bounds__(kBinThreads) k_bin_place_scan(const uint32_t* __restrict__ rowseq,
+                                                                const uint32_t* __restrict__ rowspan,
+                                                                const uint32_t* __restrict__ plan,
+                                                                const uint32_t* __restrict__ tab, int gx, int gy,
+                                                                uint32_t* __restrict__ list, size_t cap) {
+  const uint32_t* rs = plan;
+  const uint32_t* cb = plan + gy + 1;
+  if (plan[3 * gy + 2] == 0u) return;
+  const uint32_t C = cb[gy];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (uint32_t kg = blockIdx.x; kg < C; kg += gridDim.x) {
+    const int y = chunk_row(cb, gy, kg);
+    const uint32_t c0 = cb[y], nch = cb[y + 1] - c0, k = kg - c0;
+    const uint32_t i0 = rs[y] + 256u * k, i1 = min(rs[y + 1], i0 + 256u);
+    WarpSpans S;
+    load_chunk(rowspan, i0, i1, lane, S);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      const uint32_t i = i0 + 32 * c + lane;
+      S.v0[c] = i < i1 ? rowseq[i] : 0u;
+    }
+    const int x = w + kBinWarps * lane;
+    const uint32_t base = x < gx ? tab[(size_t)c0 * gx + (size_t)x * nch + k] : 0u;
+    scan_place<false>(S, S.v0, gx, w, kBinWarps, base, list, nullptr, cap);
+  }
+}
+
 // Counts per (row, column, chunk): a difference array over the columns of
 // the chunk's spans, then its running sum, at tab[cb[y] gx + x nch + k]
 // (row y's counts in (column, chunk) order); adds the chunk's list entries
@@ -350,16 +497,12 @@ __global__ void __launch_bounds__(1024) k_bin_rowscan(uint32_t* __restrict__ tab
 }
 
 // The list entries: each chunk in steps of 256 items over their columns,
-// starting at the chunk's offsets in its tiles.  With dist (the light
-// splat), each entry's distance goes beside it: the depth sort's key of rank
-// r is the FP32 bit pattern of r's light distance.
+// starting at the chunk's offsets in its tiles.
 __global__ void __launch_bounds__(kBinThreads) k_bin_place(const uint32_t* __restrict__ rowseq,
                                                            const uint32_t* __restrict__ rowspan,
                                                            const uint32_t* __restrict__ plan,
                                                            const uint32_t* __restrict__ tab, int gx, int gy,
-                                                           uint32_t ch, const uint32_t* __restrict__ rank_key,
-                                                           uint32_t* __restrict__ list, uint32_t* __restrict__ dist,
-                                                           size_t cap) {
+                                                           uint32_t ch, uint32_t* __restrict__ list, size_t cap) {
   __shared__ SpanSmem S;
   const uint32_t* rs = plan;
   const uint32_t* cb = plan + gy + 1;
@@ -374,15 +517,14 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_place(const uint32_t* __res
     for (uint32_t sub = i0; sub < i1; sub += kBinThreads) {
       const uint32_t i = sub + threadIdx.x;
       int a = 0, b = -1;
-      uint32_t r = 0, key = 0;
+      uint32_t r = 0;
       if (i < i1) {
         r = rowseq[i];
         const uint32_t sp = rowspan[i];
         a = (int)(sp & 0xFFFFu);
         b = (int)(sp >> 16);
-        if (dist) key = rank_key[r];
       }
-      place_spans(S, gx, a, b, r, key, list, dist, cap);
+      place_spans(S, gx, a, b, r, 0u, list, nullptr, cap);
     }
     __syncthreads();  // S.run is rewritten for the next chunk
   }
@@ -402,12 +544,10 @@ void launch_binning(const FrameArgs& f, int sp, cudaStream_t s) {
   // every rank's first list slot in rank order (the shadow partials' slots) and the total
   device_exclusive_scan(at<uint32_t>(ws, b.cnt), at<uint32_t>(ws, b.off), (uint32_t)n, header + h_need,
                         at<uint32_t>(ws, b.scan_part), s);
-  // the lists go where the composites and the backward read them, and for
-  // the light splat each entry's distance where the occluder bounds read it;
-  // the row sequence and spans use buffers that are free until then
+  // the lists go where the composites and the backward read them; the row
+  // sequence and spans use buffers that are free until then
   const int fin = (f.L->ntiles <= 256 ? 1 : 2) & 1;
   uint32_t* list = at<uint32_t>(ws, b.tv[fin]);
-  uint32_t* dist = sp ? at<uint32_t>(ws, b.tk[1 - fin]) : nullptr;
   uint32_t* rowseq = at<uint32_t>(ws, b.tk[fin]);
   uint32_t* rowspan = at<uint32_t>(ws, b.tv[1 - fin]);
   uint32_t* row_cnt = at<uint32_t>(ws, b.row_cnt);
@@ -416,14 +556,20 @@ void launch_binning(const FrameArgs& f, int sp, cudaStream_t s) {
   const uint32_t ch = bin_chunk(gx);
   k_bin_rowtot<<<gy, kBinThreads, 0, s>>>(row_cnt, nb, gy, plan);
   k_bin_plan<<<1, 1024, 0, s>>>(gy, ch, bin_tab_words(cap, gx, gy), gx, plan, header, h_need, h_pairs, cap);
-  k_bin_rows<<<nb, kBinThreads, 0, s>>>(n, at<SplatRec>(ws, b.rrec), row_cnt, nb, gy, plan, rowseq, rowspan, cap);
+  const SplatRec* rrec = at<SplatRec>(ws, b.rrec);
+  if (gy <= kScanBuckets)
+    k_bin_rows_scan<<<nb, kBinThreads, 0, s>>>(n, rrec, row_cnt, nb, gy, plan, rowseq, rowspan, cap);
+  else
+    k_bin_rows<<<nb, kBinThreads, 0, s>>>(n, rrec, row_cnt, nb, gy, plan, rowseq, rowspan, cap);
   const size_t chunks = cap / ch + (size_t)gy + 1;
-  int grid = device_sm_count() * 5;
+  const bool scan = gx <= kScanBuckets;  // chunks of 256 items
+  int grid = device_sm_count() * (scan ? 8 : 5);
   if ((size_t)grid > chunks) grid = (int)chunks;
-  k_bin_count<<<grid, kBinThreads, 0, s>>>(rowspan, plan, gx, gy, ch, tab);
+  if (scan) k_bin_count_scan<<<grid, kBinThreads, 0, s>>>(rowspan, plan, gx, gy, tab);
+  else k_bin_count<<<grid, kBinThreads, 0, s>>>(rowspan, plan, gx, gy, ch, tab);
   k_bin_rowscan<<<gy, 1024, 0, s>>>(tab, plan, gx, gy, at<uint32_t>(ws, b.tile_start));
-  k_bin_place<<<grid, kBinThreads, 0, s>>>(rowseq, rowspan, plan, tab, gx, gy, ch, at<uint32_t>(ws, b.sk[1]), list,
-                                           dist, cap);
+  if (scan) k_bin_place_scan<<<grid, kBinThreads, 0, s>>>(rowseq, rowspan, plan, tab, gx, gy, list, cap);
+  else k_bin_place<<<grid, kBinThreads, 0, s>>>(rowseq, rowspan, plan, tab, gx, gy, ch, list, cap);
   count_launch(6);
 }
 
