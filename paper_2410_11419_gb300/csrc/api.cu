@@ -156,6 +156,7 @@ Workspace plan_workspace(int n, int width, int height, size_t cap) {
   L.seg_desc = P.take(16 * items);
   L.seg_lists = P.take(8 * items);
   L.seg_pub = P.take(4 * 256 * items);
+  L.mlp_x3 = P.take(mlp_x3_bytes());
   L.rank_flags = P.take(2 * N);
   L.shade = P.take(16 * N);
   L.T = P.take(4 * N);

@@ -85,6 +85,7 @@ struct Workspace {
   size_t seg_desc = 0;   // uint4[items]: each shadow segment's tile, receivers and predecessor
   size_t seg_lists = 0;  // u32[2][items]: the segments with an open ray; those every ray enters stopped
   size_t seg_pub = 0;   // float[items][256]: the products each shadow segment hands to the next
+  size_t mlp_x3 = 0;    // the FP32 networks' hidden weights, packed for the tensor cores in every frame
   size_t rank_flags = 0;  // uchar2[N] by light rank: a receiver of it saw some light; a pixel of it is known to pass
   int n = 0, width = 0, height = 0, gx = 0, gy = 0, ntiles = 0;
   size_t cap = 0;
@@ -260,6 +261,12 @@ void launch_mlp(const FrameArgs& f, cudaStream_t s, bool identity_only = false, 
 void launch_phi_lights(const FrameArgs* const* f, int nl, float4* envcol, cudaStream_t s);
 void launch_phi_lights_tc(const FrameArgs* const* f, int nl, float4* envcol, const unsigned char* blob,
                           cudaStream_t s);
+// FP32 MLPs of widths 32, 64 and 128 on the tensor cores (mlp_x3.cu); the
+// packed weights of both networks take mlp_x3_bytes() of the workspace
+size_t mlp_x3_bytes();
+bool mlp_x3_supported(const MlpDev& m);
+void launch_mlp_x3(const FrameArgs& f, cudaStream_t s, int which_mask);
+void launch_phi_lights_x3(const FrameArgs* const* f, int nl, float4* envcol, cudaStream_t s);
 // BF16 / FP8 tensor-core MLPs (mlp_tc.cu)
 size_t mlp_tc_blob_bytes(const MlpDev& m, int dtype);
 size_t mlp_tc_scale_offset(const MlpDev& m, int dtype);  // FP8: (sx, sw) per hidden layer

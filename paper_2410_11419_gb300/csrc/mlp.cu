@@ -1,5 +1,7 @@
-// K8 (FP32 form): the shadow-refinement MLP Phi (Sec. 4.2) and the residual
-// MLP Psi (Sec. 4.3) over all spatial Gaussians.
+// K8 (FP32 form) for networks of width 16, and the ablations' identities: the
+// shadow-refinement MLP Phi (Sec. 4.2) and the residual MLP Psi (Sec. 4.3)
+// over all spatial Gaussians.  Widths 32, 64 and 128 go to the tensor cores
+// (mlp_x3.cu), which have no operand split for so narrow a layer that pays.
 //
 // One 256-thread block owns 64 Gaussians.  The prologue builds the inputs in
 // shared memory, feature-major:
@@ -9,8 +11,7 @@
 // Each hidden layer is a 64 x width register-tiled FP32 product against the
 // layer's weights staged in shared memory, transposed, in rows padded to
 // width + 4 floats: the staging stores of a warp (consecutive inputs k, one
-// output j) then spread over 8 banks instead of one, and the rows stay
-// 16-byte aligned for the vector loads of the product.  The output layer applies the
+// output j) then spread over 8 banks instead of one.  The output layer applies the
 // sigmoid.  Outputs go both by Gaussian index and, for the camera composite,
 // by camera depth rank.
 #include "gs3_internal.cuh"
@@ -20,6 +21,8 @@ namespace {
 
 constexpr int kRows = 64;
 constexpr int kHPad = kRows + 4;  // feature-major activations, padded rows
+constexpr int kWidth = 16;        // of the hidden layers
+constexpr int kMaxIn = 64;        // inputs of a layer (61 / 60 features)
 
 // Phi runs over the Gaussians of nl lights at once (row l n + g: Gaussian g
 // under light l); Psi, which does not see the light, over one set (nl = 1).
@@ -68,12 +71,11 @@ __device__ __forceinline__ void write_pe(float (*H)[kHPad], int base, int row, i
   sincospif(f * v2, &s, &c); H[o + 2][row] = s; H[o + 5][row] = c;
 }
 
-template <int WIDTH>
 __global__ void __launch_bounds__(256) k_mlp(MlpParams p) {
   extern __shared__ float4 smem4[];
   float* smem = reinterpret_cast<float*>(smem4);
-  float (*H)[kHPad] = reinterpret_cast<float (*)[kHPad]>(smem);  // [128][kHPad]
-  float* Ws = smem + 128 * kHPad;                                  // [din][dout]
+  float (*H)[kHPad] = reinterpret_cast<float (*)[kHPad]>(smem);  // [kMaxIn][kHPad]
+  float* Ws = smem + kMaxIn * kHPad;                               // [din][kWidth + 4]
   const int t = threadIdx.x;
   const int g0 = blockIdx.x * kRows;
   const int rows = p.n * p.nl;
@@ -117,61 +119,37 @@ __global__ void __launch_bounds__(256) k_mlp(MlpParams p) {
     }
   }
 
-  constexpr int CPT = WIDTH / 16;  // columns per thread
   const int tcol = t & 15, trow = t >> 4;
-  // output column c of thread column tcol: with 8 per thread two runs of 4
-  // (tcol 4 + c and 64 + tcol 4 + c - 4), so that 16 threads' 16-byte
-  // weight loads cover 256 contiguous bytes (no bank conflict)
-  auto out_col = [](int tc, int c) { return CPT == 8 ? (c >> 2) * 64 + tc * 4 + (c & 3) : tc * CPT + c; };
   int din = p.net.in_dim;
   const float* w = p.net.w;
   const float* bias = p.net.b;
   for (int l = 0; l < p.net.n_hidden; ++l) {
     __syncthreads();  // H complete, previous Ws no longer read
-    {
-      // W row-major (out, in): thread t takes input k = t % kp of rows
-      // j = t / kp, + 256 / kp, ... (kp = din rounded up to 64 or 128), so a
-      // warp's loads are consecutive and several are in flight
-      const int kp = din <= 64 ? 64 : 128, k = t % kp;
-      const int rows = 256 / kp;
-      if (k < din) {
-#pragma unroll 4
-        for (int j = t / kp; j < WIDTH; j += rows) Ws[k * (WIDTH + 4) + j] = w[(size_t)j * din + k];
-      }
+    for (int i = t; i < kWidth * din; i += 256) {  // W row-major (out, in)
+      const int j = i / din, k = i - j * din;
+      Ws[k * (kWidth + 4) + j] = w[i];
     }
     __syncthreads();
-    float acc[4][CPT];
+    float acc[4];
 #pragma unroll
-    for (int c = 0; c < CPT; ++c) {
-      const float bv = bias[out_col(tcol, c)];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) acc[r][c] = bv;
-    }
+    for (int r = 0; r < 4; ++r) acc[r] = bias[tcol];
     for (int k = 0; k < din; ++k) {
       const float4 a = *reinterpret_cast<const float4*>(&H[k][trow * 4]);
-      float bv[CPT];
-#pragma unroll
-      for (int c = 0; c < CPT; ++c) bv[c] = Ws[k * (WIDTH + 4) + out_col(tcol, c)];
-#pragma unroll
-      for (int c = 0; c < CPT; ++c) {
-        acc[0][c] = fmaf(a.x, bv[c], acc[0][c]);
-        acc[1][c] = fmaf(a.y, bv[c], acc[1][c]);
-        acc[2][c] = fmaf(a.z, bv[c], acc[2][c]);
-        acc[3][c] = fmaf(a.w, bv[c], acc[3][c]);
-      }
+      const float b = Ws[k * (kWidth + 4) + tcol];
+      acc[0] = fmaf(a.x, b, acc[0]);
+      acc[1] = fmaf(a.y, b, acc[1]);
+      acc[2] = fmaf(a.z, b, acc[2]);
+      acc[3] = fmaf(a.w, b, acc[3]);
     }
     __syncthreads();  // all reads of H done
     const bool leaky = p.net.act == GS3_ACT_LEAKY_RELU;
+    float v[4];
 #pragma unroll
-    for (int c = 0; c < CPT; ++c) {
-      float v[4];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) v[r] = acc[r][c] > 0.f ? acc[r][c] : (leaky ? 0.01f * acc[r][c] : 0.f);
-      *reinterpret_cast<float4*>(&H[out_col(tcol, c)][trow * 4]) = make_float4(v[0], v[1], v[2], v[3]);
-    }
-    w += (size_t)din * WIDTH;
-    bias += WIDTH;
-    din = WIDTH;
+    for (int r = 0; r < 4; ++r) v[r] = acc[r] > 0.f ? acc[r] : (leaky ? 0.01f * acc[r] : 0.f);
+    *reinterpret_cast<float4*>(&H[tcol][trow * 4]) = make_float4(v[0], v[1], v[2], v[3]);
+    w += (size_t)din * kWidth;
+    bias += kWidth;
+    din = kWidth;
   }
   // ---- output layer + sigmoid (its weights staged where the last layer's were) ----
   const int dout = p.net.out_dim;
@@ -196,24 +174,10 @@ __global__ void __launch_bounds__(256) k_mlp(MlpParams p) {
   }
 }
 
-template <int WIDTH>
-void launch_width(const MlpParams& p, cudaStream_t s) {
-  const size_t sm = (size_t)(128 * kHPad + 128 * (WIDTH + 4)) * sizeof(float);
-  static DeviceOnce once;
-  once.run([sm] {
-    return cudaFuncSetAttribute(k_mlp<WIDTH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) == cudaSuccess;
-  });
-  k_mlp<WIDTH><<<(p.n * p.nl + kRows - 1) / kRows, 256, sm, s>>>(p);
-  count_launch();
-}
-
 void launch_one(const MlpParams& p, cudaStream_t s) {
-  switch (p.net.width) {
-    case 16: launch_width<16>(p, s); break;
-    case 32: launch_width<32>(p, s); break;
-    case 64: launch_width<64>(p, s); break;
-    default: launch_width<128>(p, s); break;
-  }
+  const size_t sm = (size_t)(kMaxIn * kHPad + kMaxIn * (kWidth + 4)) * sizeof(float);
+  k_mlp<<<(p.n * p.nl + kRows - 1) / kRows, 256, sm, s>>>(p);
+  count_launch();
 }
 
 }  // namespace
@@ -234,15 +198,17 @@ void launch_mlp(const FrameArgs& f, cudaStream_t s, bool identity_only, int whic
   p.envcol = nullptr;
   p.rank_of = at<uint32_t>(f.ws, f.L->sp[0].rank_of);
 
-  p.net = f.sc.phi;
-  p.which = 0;
-  p.identity = (f.opts.ablate & GS3_ABLATE_PHI) != 0;
-  if ((which_mask & 1) && (p.identity || !identity_only)) launch_one(p, s);
-
-  p.net = f.sc.psi;
-  p.which = 1;
-  p.identity = (f.opts.ablate & GS3_ABLATE_PSI) != 0;
-  if ((which_mask & 2) && (p.identity || !identity_only)) launch_one(p, s);
+  int x3 = 0;  // networks that the tensor cores take
+  for (int w = 0; w < 2; ++w) {
+    if (!(which_mask & (1 << w))) continue;
+    p.net = w == 0 ? f.sc.phi : f.sc.psi;
+    p.which = w;
+    p.identity = (f.opts.ablate & (w == 0 ? GS3_ABLATE_PHI : GS3_ABLATE_PSI)) != 0;
+    if (!p.identity && identity_only) continue;
+    if (!p.identity && mlp_x3_supported(p.net)) x3 |= 1 << w;
+    else launch_one(p, s);
+  }
+  if (x3) launch_mlp_x3(f, s, x3);
 }
 
 void launch_phi_lights(const FrameArgs* const* f, int nl, float4* envcol, cudaStream_t s) {
@@ -266,7 +232,8 @@ void launch_phi_lights(const FrameArgs* const* f, int nl, float4* envcol, cudaSt
   p.envcol = envcol;
   p.rank_of = at<uint32_t>(f0.ws, f0.L->sp[0].rank_of);
   p.identity = (f0.opts.ablate & GS3_ABLATE_PHI) != 0;
-  launch_one(p, s);
+  if (!p.identity && mlp_x3_supported(p.net)) launch_phi_lights_x3(f, nl, envcol, s);
+  else launch_one(p, s);
 }
 
 }  // namespace gs3
