@@ -16,11 +16,12 @@
 #include "gs3_internal.cuh"
 #include "splat_eval.cuh"
 #include "shadow_bwd.cuh"
+#include "f32x2.cuh"
 
 namespace gs3 {
 namespace {
 
-constexpr int kGeom = 8;    // du, dv, dA, dB, dC, dgamma
+constexpr int kGeom = 8;    // dgamma, sums of w dx, w dy, w dx dy, w dx^2, w dy^2
 constexpr int kColor = 8;   // dshade rgb, dT', dres rgb
 constexpr int kMlpIn = 24;  // Phi: dmu 3, dwi 3, dl 6; Psi: dmu 3, dwo 3, dl 6
 
@@ -68,40 +69,32 @@ BwdPlan plan_bwd(int n, const MlpDev& phi, const MlpDev& psi) {
   return p;
 }
 
-// pixel offset, power and alpha of a splat record at a pixel centre
-struct Eval {
-  float dx, dy, beta, alpha;
-  bool pass, clamped;
-};
-// A camera-splat entry (make_entry, tile-relative) at the tile pixel centre
-// (lx, ly), with the forward composite's arithmetic (power2_at): pass,
-// beta = 2^power2, alpha = min(amax, gamma beta); (dx, dy) = pixel - centre.
-__device__ __forceinline__ Eval eval_entry(const float4 e0, const float4 e1, float lx, float ly, float amax) {
-  Eval r;
-  r.dx = lx - e0.x;
-  r.dy = ly - e0.y;
-  const float pw = power2_at(e0, e1.x, lx, ly);
-  r.pass = pw >= e1.y;
-  r.beta = r.pass ? ex2(pw) : 0.f;
-  const float ga = e1.z * r.beta;
-  r.clamped = ga >= amax;
-  r.alpha = fminf(amax, ga);
-  return r;
-}
-
-// dL/dpower -> (du, dv, dA, dB, dC)
-__device__ __forceinline__ void power_grad(const SplatRec& q, const Eval& e, float dpow, float* g) {
-  const float A = q.b.x, B = q.b.y, C = q.b.z;
-  g[0] = (A * e.dx + B * e.dy) * dpow;
-  g[1] = (C * e.dy + B * e.dx) * dpow;
-  g[2] = -0.5f * e.dx * e.dx * dpow;
-  g[3] = -e.dx * e.dy * dpow;
-  g[4] = -0.5f * e.dy * e.dy * dpow;
-}
-
 // ---------------------------------------------------------------------------
-// K9b: camera composite backward
+// K9b: camera composite backward.
+// Per pixel, back to front over the entries the forward's ray took, T
+// recovered by division from its final value.  With (gr, gg, gb) = dL/d(image),
+// an entry of colours c (shading, T', residual) has
+//   G      = Sh (g . c_shade) + (g . S) c_T' + g . c_res
+//   dalpha = T G - D / (1 - alpha),  D = the sum of w G over the entries behind it
+// and its colours get w Sh g, w (g . S) and w g (w = alpha T).  Geometry as in
+// the shadow splat's backward (shadow_bwd.cu): only the sums of
+// t = dalpha beta (dL/dgamma) and of gamma t times dx, dy, dx dy, dx^2, dy^2 are
+// accumulated; k_prep_bwd applies the conic.
+//
+// A warp takes one half (16 x 8) of a tile on its own: lane l column l & 15 and
+// rows (l >> 4) + 2 i, i = 0..3, so that a lane adds four pixels before the
+// warp adds its lanes.  The pixel pairs go through packed FP32 instructions;
+// the next 32 entries are staged (those whose box and ellipse reach the half)
+// while the current ones are walked, as in the forward.  The 14 terms of four
+// entries are added over the 32 lanes through shared-memory rows.
+// Bound: issue slots.  Object workload (300k Gaussians, 800 x 800): 1.24 ms with
+// a pixel per thread and a 16-shuffle butterfly per entry and warp, 0.57 ms so
+// (0.58 at 4 blocks per SM, 0.62 at 5).
 // ---------------------------------------------------------------------------
+constexpr int kCbWarps = 4;  // independent warps per block
+constexpr int kCbRows = 4;   // entries whose lane sums are added together
+constexpr int kCbTerms = 7;  // pairs of terms per entry
+
 struct CamBwdParams {
   const uint32_t* list;
   const uint32_t* tile_start;
@@ -113,130 +106,241 @@ struct CamBwdParams {
   const uint32_t* n_contrib;
   const float4* pix_aux;
   const float* dimg;
-  float* cam_geom;
+  float* cam_geom;  // [N][8] by index: dL/dgamma, sums of w dx, w dy, w dx dy, w dx^2, w dy^2
   float* color;
-  int W, H, gx;
+  int W, H, gx, ntiles;
   float amax;
 };
 
-// Sums v[0..15] over the warp with one transposing butterfly (16 shuffles):
-// each level sends the half of the remaining values that the partner lane
-// keeps.  Lane L ends with the total of value
-// 8 ((L >> 4) & 1) + 4 ((L >> 3) & 1) + 2 ((L >> 2) & 1) + ((L >> 1) & 1).
-__device__ __forceinline__ float warp_sum16(const float (&v)[16], int lane) {
-  float a8[8], a4[4], a2[2];
-  const bool h16 = (lane & 16) != 0, h8 = (lane & 8) != 0, h4 = (lane & 4) != 0, h2 = (lane & 2) != 0;
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-    a8[i] = (h16 ? v[8 + i] : v[i]) + __shfl_xor_sync(0xffffffffu, h16 ? v[i] : v[8 + i], 16);
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-    a4[i] = (h8 ? a8[4 + i] : a8[i]) + __shfl_xor_sync(0xffffffffu, h8 ? a8[i] : a8[4 + i], 8);
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-    a2[i] = (h4 ? a4[2 + i] : a4[i]) + __shfl_xor_sync(0xffffffffu, h4 ? a4[i] : a4[2 + i], 4);
-  float x = (h2 ? a2[1] : a2[0]) + __shfl_xor_sync(0xffffffffu, h2 ? a2[0] : a2[1], 2);
-  return x + __shfl_xor_sync(0xffffffffu, x, 1);
+struct CamBwdStage {
+  float4 yc[32];    // -y, -y, c, c
+  float4 xart[32];  // x, a, r, threshold
+  float2 gi[32];    // gamma, place in the list (as bits)
+  float4 c0[32], c1[32];
+  uint32_t g[32];   // Gaussian
+};
+struct CamBwdSmem {  // one warp's
+  CamBwdStage e[2];
+  f32x2 rows[kCbTerms][kCbRows][33];  // per term pair, entry and lane
+  float row_gamma[kCbRows];
+  uint32_t row_g[kCbRows];
+};
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
 }
 
-__global__ void __launch_bounds__(256) k_camera_bwd(CamBwdParams p) {
-  __shared__ SplatRec R[256];
-  __shared__ float4 E0[256], E1[256], C0[256], C1[256];
-  __shared__ uint32_t G[256];
-  __shared__ int s_max;
-  const int tile = (int)p.tile_order[blockIdx.x], tx = tile % p.gx, ty = tile / p.gx, t = threadIdx.x;
-  // warps 2q and 2q + 1 take quadrant q of the tile (the 8x8 block at
-  // (8 (q & 1), 8 (q >> 1))), so a warp skips an entry whose alpha box misses it
-  const int q4 = t >> 6, qi = t & 63;
-  const uint32_t qbit = 1u << q4;
-  const int cx = 8 * (q4 & 1) + (qi & 7), cy = 8 * (q4 >> 1) + (qi >> 3);
-  const int px = tx * kTile + cx, py = ty * kTile + cy;
-  const bool inside = px < p.W && py < p.H;
+__global__ void __launch_bounds__(kCbWarps * 32, 3) k_camera_bwd(CamBwdParams p) {
+  __shared__ CamBwdSmem smem[kCbWarps];
+  CamBwdSmem& B = smem[threadIdx.x >> 5];
+  const int lane = threadIdx.x & 31;
+  const uint32_t unit = blockIdx.x * kCbWarps + (threadIdx.x >> 5);  // (tile in launch order, half)
+  if (unit >= 2u * (uint32_t)p.ntiles) return;
+  const int tile = (int)p.tile_order[unit >> 1], half = (int)(unit & 1u);
+  const int tx = tile % p.gx, ty = tile / p.gx;
+  const uint32_t hbits = 3u << (2 * half);
   const float ox = (float)(tx * kTile), oy = (float)(ty * kTile);
-  const float lx = (float)cx + 0.5f, ly = (float)cy + 0.5f;
+  const int cx = lane & 15, cy = 8 * half + (lane >> 4);
+  const int px = tx * kTile + cx;
+  const float lx = cx + 0.5f;
   const uint32_t b = p.tile_start[tile];
-  const size_t pix = (size_t)py * p.W + px;
-  uint32_t nc = 0;
-  float T = 1.f, g7[7] = {0, 0, 0, 0, 0, 0, 0};
-  if (inside) {
-    nc = p.n_contrib[pix];
-    T = p.final_t[pix];
-    const float4 s = p.pix_aux[2 * pix], r = p.pix_aux[2 * pix + 1];
-    const float gr = p.dimg[3 * pix], gg = p.dimg[3 * pix + 1], gb = p.dimg[3 * pix + 2];
-    g7[0] = gr * s.w; g7[1] = gg * s.w; g7[2] = gb * s.w;
-    g7[3] = gr * s.x + gg * s.y + gb * s.z;
-    g7[4] = gr; g7[5] = gg; g7[6] = gb;
-    (void)r;
-  }
-  if (t == 0) s_max = 0;
-  __syncthreads();
-  atomicMax(&s_max, (int)nc);
-  __syncthreads();
-  const uint32_t end = min(b + (uint32_t)s_max, p.tile_start[tile + 1]);
-  float B7[7] = {0, 0, 0, 0, 0, 0, 0};
-  for (uint32_t hi = end; hi > b; ) {
-    const uint32_t lo = hi > b + 256 ? hi - 256 : b;
-    const int cnt = (int)(hi - lo);
-    __syncthreads();
-    if (t < cnt) {
-      const uint32_t rank = p.list[lo + t];
-      const SplatRec q = p.rrec[rank];
-      R[t] = q;
-      float4 e0, e1;
-      make_entry(q, ox, oy, e0, e1);
-      e1.w = __uint_as_float(__float_as_uint(e1.w) & ellipse_halves(e0, e1));  // as the forward culls
-      E0[t] = e0;
-      E1[t] = e1;
-      C0[t] = p.ccol[2 * rank];
-      C1[t] = p.ccol[2 * rank + 1];
-      G[t] = p.order[rank];
-    }
-    __syncthreads();
-    for (int jj = cnt - 1; jj >= 0; --jj) {
-      if (!(__float_as_uint(E1[jj].w) & qbit)) continue;  // warp-uniform: the forward skipped it here too
-      const uint32_t i = lo + jj;
-      const bool active = inside && (i - b) < nc;
-      float gv[16];
+  // per pixel pair q (rows 4 q and 4 q + 2 of the lane): row (far away until the
+  // sweep reaches the pixel's last entry), T, D, dL/d(image), Sh, g . S
+  f32x2 ly[2], T[2], D[2], gr[2], gg[2], gb[2], sh[2], gs[2];
+  uint32_t nc[4], next = 0u;
 #pragma unroll
-      for (int k = 0; k < 16; ++k) gv[k] = 0.f;
-      bool contrib = false;
-      if (active) {
-        const SplatRec q = R[jj];
-        const Eval ev = eval_entry(E0[jj], E1[jj], lx, ly, p.amax);
-        if (ev.pass) {
-          contrib = true;
-          T = T / (1.f - ev.alpha);
-          const float w = ev.alpha * T;
-          const float c[7] = {C0[jj].x, C0[jj].y, C0[jj].z, C0[jj].w, C1[jj].x, C1[jj].y, C1[jj].z};
-          float dalpha = 0.f;
-          const float inv = 1.f / (1.f - ev.alpha);
+  for (int q = 0; q < 2; ++q) {
+    float t2[2], r2[2], g2[2], b2[2], h2[2], s2[2];
 #pragma unroll
-          for (int k = 0; k < 7; ++k) {
-            gv[6 + k] = w * g7[k];
-            dalpha += g7[k] * (c[k] * T - B7[k] * inv);
-            B7[k] += w * c[k];
-          }
-          if (!ev.clamped) {
-            gv[5] = dalpha * ev.beta;
-            power_grad(q, ev, dalpha * ev.alpha, gv);
-          }
-        }
+    for (int h = 0; h < 2; ++h) {
+      const int py = ty * kTile + cy + 4 * q + 2 * h;
+      nc[2 * q + h] = 0u;
+      t2[h] = 1.f;
+      r2[h] = g2[h] = b2[h] = h2[h] = s2[h] = 0.f;
+      if (px < p.W && py < p.H) {
+        const size_t pix = (size_t)py * p.W + px;
+        nc[2 * q + h] = p.n_contrib[pix];
+        t2[h] = p.final_t[pix];
+        const float4 s = p.pix_aux[2 * pix];
+        r2[h] = p.dimg[3 * pix]; g2[h] = p.dimg[3 * pix + 1]; b2[h] = p.dimg[3 * pix + 2];
+        h2[h] = s.w;
+        s2[h] = r2[h] * s.x + g2[h] * s.y + b2[h] * s.z;
       }
-      if (__any_sync(0xffffffffu, contrib)) {
-        // geometry terms 0-5 and colour terms 6-12 in one butterfly; lane pair
-        // (2 k', 2 k' + 1) holds term k', and the even lane adds it
-        const int lane = t & 31;
-        const float v = warp_sum16(gv, lane);
-        const int k = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
-        if ((lane & 1) == 0 && k < 13 && v != 0.f) {
-          const uint32_t g = G[jj];
-          if (k < 6) atomicAdd(p.cam_geom + (size_t)kGeom * g + k, v);
-          else atomicAdd(p.color + (size_t)kColor * g + (k - 6), v);
-        }
+      next = max(next, nc[2 * q + h]);
+    }
+    ly[q] = dup2(1.0e6f);
+    D[q] = 0ull;
+    T[q] = pk2(t2[0], t2[1]);
+    gr[q] = pk2(r2[0], r2[1]); gg[q] = pk2(g2[0], g2[1]); gb[q] = pk2(b2[0], b2[1]);
+    sh[q] = pk2(h2[0], h2[1]); gs[q] = pk2(s2[0], s2[1]);
+  }
+  const uint32_t end = __reduce_max_sync(0xffffffffu, next);  // entries some pixel of the half took
+
+  int nrow = 0;
+  auto flush = [&]() {
+    __syncwarp();
+    const int r = lane & 3, c = lane >> 2;
+    if (r < nrow && c < kCbTerms) {
+      const f32x2* row = B.rows[c][r];
+      f32x2 s0 = row[0], s1 = row[1];
+#pragma unroll
+      for (int l = 2; l < 32; l += 2) {
+        s0 = add2(s0, row[l]);
+        s1 = add2(s1, row[l + 1]);
+      }
+      const f32x2 s = add2(s0, s1);
+      float x = lo2(s), y = hi2(s);
+      const size_t g = B.row_g[r];
+      if (c < 3) {
+        const float gamma = B.row_gamma[r];
+        if (c > 0) x *= gamma;  // the first term is dL/dgamma itself
+        y *= gamma;
+      }
+      if (x != 0.f || y != 0.f) {
+        float* dst = c < 3 ? p.cam_geom + kGeom * g + 2 * c : p.color + kColor * g + 2 * (c - 3);
+        asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(dst), "f"(x), "f"(y) : "memory");
       }
     }
-    hi = lo;
+    __syncwarp();  // the rows are free again
+    nrow = 0;
+  };
+
+  // entries below hi, last first: lane l takes entry hi - 1 - l
+  auto rank_at = [&](uint32_t hi) { return hi > (uint32_t)lane ? p.list[b + hi - 1 - lane] : 0u; };
+  struct Rec {
+    float4 a, b, c;
+  };
+  auto rec_at = [&](uint32_t r) { return Rec{p.rrec[r].a, p.rrec[r].b, p.rrec[r].c}; };
+  auto stage = [&](CamBwdStage& E, uint32_t hi, uint32_t rank, const Rec& rec) {
+    SplatRec q;
+    q.a = rec.a; q.b = rec.b; q.c = rec.c;
+    float4 e0, e1;
+    make_entry(q, ox, oy, e0, e1);
+    // the halves (and no fewer) that the forward's quadrants lie in
+    const bool hit = hi > (uint32_t)lane && (__float_as_uint(e1.w) & ellipse_halves(e0, e1) & hbits) != 0u;
+    const uint32_t m = __ballot_sync(0xffffffffu, hit);
+    const int slot = __popc(m & ((1u << lane) - 1u));
+    if (hit) {
+      E.yc[slot] = make_float4(-e0.y, -e0.y, e0.w, e0.w);
+      E.xart[slot] = make_float4(e0.x, e0.z, e1.x, e1.y);
+      E.gi[slot] = make_float2(e1.z, __uint_as_float(hi - 1 - lane));
+      cp_async16(&E.c0[slot], p.ccol + 2 * (size_t)rank);
+      cp_async16(&E.c1[slot], p.ccol + 2 * (size_t)rank + 1);
+      cp_async4(&E.g[slot], p.order + rank);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    return __popc(m);
+  };
+  auto below = [](uint32_t hi, uint32_t d) { return hi > d ? hi - d : 0u; };
+
+  uint32_t rank = rank_at(end);
+  Rec rec = rec_at(rank);
+  uint32_t rank2 = rank_at(below(end, 32));
+  int n = stage(B.e[0], end, rank, rec), buf = 0;
+  rank = rank2;
+  rec = rec_at(rank);
+  rank2 = rank_at(below(end, 64));
+  for (uint32_t hi = end; hi > 0; hi = below(hi, 32)) {
+    int n2 = 0;
+    if (hi > 32) {
+      n2 = stage(B.e[buf ^ 1], hi - 32, rank, rec);
+      rank = rank2;
+      rec = rec_at(rank);
+      rank2 = rank_at(below(hi, 96));
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    __syncwarp();
+    const CamBwdStage& E = B.e[buf];
+    for (int t = 0; t < n; ++t) {
+      const float2 gi = E.gi[t];
+      const uint32_t idx = __float_as_uint(gi.y);
+      if (idx < next) {  // pixels whose last entry this is, or lies ahead: once per pixel
+        next = 0u;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float y = (float)(cy + 2 * i) + 0.5f;
+          if (idx < nc[i]) {
+            ly[i / 2] = i & 1 ? pk2(lo2(ly[i / 2]), y) : pk2(y, hi2(ly[i / 2]));
+            nc[i] = 0u;
+          }
+          next = max(next, nc[i]);
+        }
+      }
+      const ulonglong2 yc = *reinterpret_cast<const ulonglong2*>(&E.yc[t]);
+      const float4 qx = E.xart[t], c0 = E.c0[t], c1 = E.c1[t];
+      const float dx = lx - qx.x;
+      const f32x2 v = dup2(qx.z * dx), sx = dup2((qx.y * dx) * dx);
+      const bool clampable = !(gi.x * 1.00001f < p.amax);
+      f32x2 m0 = 0ull, m1 = 0ull, m2 = 0ull, k0 = 0ull, k1 = 0ull, k2 = 0ull, k3 = 0ull, k4 = 0ull, k5 = 0ull, k6 = 0ull;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const f32x2 dy = add2(ly[q], yc.x);
+        const f32x2 pw = fma2(dy, fma2(yc.y, dy, v), sx);
+        f32x2 beta = pk2(lo2(pw) >= qx.w ? ex2(lo2(pw)) : 0.f, hi2(pw) >= qx.w ? ex2(hi2(pw)) : 0.f);
+        f32x2 alpha = mul2(dup2(gi.x), beta);
+        if (clampable) {  // the same for the warp: alpha = alpha_max passes no gradient to the geometry
+          const float a0 = lo2(alpha), a1 = hi2(alpha);
+          beta = pk2(a0 < p.amax ? lo2(beta) : 0.f, a1 < p.amax ? hi2(beta) : 0.f);
+          alpha = pk2(fminf(p.amax, a0), fminf(p.amax, a1));
+        }
+        const f32x2 om = fma2(alpha, dup2(-1.f), dup2(1.f));
+        float ia, ib;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ia) : "f"(lo2(om)));
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ib) : "f"(hi2(om)));
+        f32x2 inv = pk2(ia, ib);  // one Newton step: within an ulp, and exactly 1 for alpha = 0
+        inv = fma2(inv, fma2(pk2(-lo2(om), -hi2(om)), inv, dup2(1.f)), inv);
+        T[q] = mul2(T[q], inv);
+        const f32x2 w = mul2(alpha, T[q]);
+        f32x2 G = mul2(gr[q], dup2(c0.x));
+        G = fma2(gg[q], dup2(c0.y), G);
+        G = mul2(sh[q], fma2(gb[q], dup2(c0.z), G));
+        G = fma2(gs[q], dup2(c0.w), G);
+        G = fma2(gr[q], dup2(c1.x), G);
+        G = fma2(gg[q], dup2(c1.y), G);
+        G = fma2(gb[q], dup2(c1.z), G);
+        const f32x2 dalpha = fma2(T[q], G, mul2(mul2(inv, dup2(-1.f)), D[q]));
+        D[q] = fma2(w, G, D[q]);
+        const f32x2 ws = mul2(w, sh[q]);
+        k0 = fma2(ws, gr[q], k0);
+        k1 = fma2(ws, gg[q], k1);
+        k2 = fma2(ws, gb[q], k2);
+        k3 = fma2(w, gs[q], k3);
+        k4 = fma2(w, gr[q], k4);
+        k5 = fma2(w, gg[q], k5);
+        k6 = fma2(w, gb[q], k6);
+        const f32x2 tt = mul2(dalpha, beta), td = mul2(tt, dy);
+        m0 = add2(m0, tt);
+        m1 = add2(m1, td);
+        m2 = fma2(td, dy, m2);
+      }
+      auto sum = [](f32x2 x) { return lo2(x) + hi2(x); };
+      const float s0 = sum(m0), s1 = sum(m1), x1 = s0 * dx;
+      B.rows[0][nrow][lane] = pk2(s0, x1);
+      B.rows[1][nrow][lane] = pk2(s1, s1 * dx);
+      B.rows[2][nrow][lane] = pk2(x1 * dx, sum(m2));
+      B.rows[3][nrow][lane] = pk2(sum(k0), sum(k1));
+      B.rows[4][nrow][lane] = pk2(sum(k2), sum(k3));
+      B.rows[5][nrow][lane] = pk2(sum(k4), sum(k5));
+      B.rows[6][nrow][lane] = pk2(sum(k6), 0.f);
+      if (lane == 0) {
+        B.row_gamma[nrow] = gi.x;
+        B.row_g[nrow] = E.g[t];
+      }
+      if (++nrow == kCbRows) flush();
+    }
+    __syncwarp();  // the buffer is free again
+    n = n2;
+    buf ^= 1;
   }
+  if (nrow) flush();
+  asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 __global__ void k_copy_strided(const float* src, int stride, int off, float* dst, int n) {
@@ -363,7 +467,7 @@ struct PrepBwdParams {
   int falloff;
   const float* cam_geom;
   const float* light_geom;
-  const SplatRec* light_rec;  // by index
+  const SplatRec *cam_rec, *light_rec;  // by index
   const float* color;
   const float* mlp_in;
   gs3_grads out;
@@ -376,14 +480,20 @@ __device__ __forceinline__ void prep_bwd_one(const PrepBwdParams& p, int g, floa
   const int n = p.sc.n;
   const float4 m = p.sc.mean_op[g], s = p.sc.scale[g];
   const float gamma = 1.f / (1.f + expf(-m.w));
-  const float* gc = p.cam_geom + (size_t)kGeom * g;
-  // the light splat's sums (shadow_bwd.cuh) times its conic (A, B, C), with
-  // d/du = A dx + B dy, d/dv = C dy + B dx, d/dA = -dx^2 / 2, d/dB = -dx dy,
-  // d/dC = -dy^2 / 2
-  const float* sl = p.light_geom + (size_t)kGeom * g;
-  const float4 cl = p.light_rec[g].b;
-  const float gl[6] = {cl.x * sl[1] + cl.y * sl[2], cl.z * sl[2] + cl.y * sl[1], -0.5f * sl[4], -sl[3], -0.5f * sl[5],
-                       sl[0]};
+  // a splat's sums of w dx, ... (K9b, shadow_bwd.cuh) times its conic (A, B, C),
+  // with d/du = A dx + B dy, d/dv = C dy + B dx, d/dA = -dx^2 / 2,
+  // d/dB = -dx dy, d/dC = -dy^2 / 2: (du, dv, dA, dB, dC, dgamma)
+  float gc[6], gl[6];
+  auto geometry = [&](const float* sum, const float4 c, float* out) {
+    out[0] = c.x * sum[1] + c.y * sum[2];
+    out[1] = c.z * sum[2] + c.y * sum[1];
+    out[2] = -0.5f * sum[4];
+    out[3] = -sum[3];
+    out[4] = -0.5f * sum[5];
+    out[5] = sum[0];
+  };
+  geometry(p.cam_geom + (size_t)kGeom * g, p.cam_rec[g].b, gc);
+  geometry(p.light_geom + (size_t)kGeom * g, p.light_rec[g].b, gl);
   float dmu[3] = {0, 0, 0}, ds[3] = {0, 0, 0}, dRq[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
   float Rq[9], qn[4], qlen;
   quat_rot(p.sc.rot[g], Rq, qn, qlen);
@@ -637,9 +747,9 @@ gs3_status run_backward(const FrameArgs& f, const float* dimg, void* bws, size_t
     p.dimg = dimg;
     p.cam_geom = cam_geom;
     p.color = color;
-    p.W = L.width; p.H = L.height; p.gx = L.gx;
+    p.W = L.width; p.H = L.height; p.gx = L.gx; p.ntiles = L.ntiles;
     p.amax = f.opts.alpha_max;
-    k_camera_bwd<<<L.ntiles, 256, 0, s>>>(p);
+    k_camera_bwd<<<(2 * L.ntiles + kCbWarps - 1) / kCbWarps, kCbWarps * 32, 0, s>>>(p);
     count_launch();
   }
   // K8b: one network's backward, then its weight gradients in fixed block order
@@ -717,6 +827,7 @@ gs3_status run_backward(const FrameArgs& f, const float* dimg, void* bws, size_t
     p.falloff = f.opts.falloff;
     p.cam_geom = cam_geom;
     p.light_geom = light_geom;
+    p.cam_rec = at<SplatRec>(ws, L.sp[0].rec);
     p.light_rec = at<SplatRec>(ws, L.sp[1].rec);
     p.color = color;
     p.mlp_in = mlp_in;
