@@ -1,6 +1,6 @@
 // K1: per-Gaussian preparation, fused for both splats.
 //
-// One thread per spatial Gaussian reads its structure-of-arrays parameters
+// A thread per spatial Gaussian and part reads the structure-of-arrays parameters
 // (coalesced float4 loads) and writes
 //   - the camera splat record and FP32 view-depth key          (Sec. 3, Eq. 1)
 //   - the light splat record and FP32 light-distance key       (Sec. 4.2)
@@ -67,12 +67,17 @@ struct View {
   float ortho;  // > 0: orthographic with this many pixels per world unit
 };
 
-__device__ void accurate_geometry(const float4 m, const float Rq[9], const float sv[3], const View& v,
-                                  float lowpass, float gamma, float amin, SplatRec& rec);
+// A view's FP32 values in FP64 (converted once, not per Gaussian)
+struct ViewD {
+  double R[9], t[3], fx, fy, cx, cy, ortho;
+};
+
+__device__ void accurate_geometry(const float4 m, const double (&md)[3], const float Rq[9], const float sv[3],
+                                  const View& v, const ViewD& d, float lowpass, float gamma, float amin, SplatRec& rec);
 
 // FP32 recipe: returns false when culled; fills the record otherwise.
-__device__ bool project_rn(const float4 m, const float4 s, const float4 q, const View& v,
-                           const gs3_render_opts& o, int gx, int gy, const float* pL, float gamma,
+__device__ bool project_rn(const float4 m, const double (&md)[3], const float4 s, const float4 q, const View& v,
+                           const ViewD& vd, const gs3_render_opts& o, int gx, int gy, const float* pL, float gamma,
                            float nl_amin, SplatRec& rec) {
   const float* R = v.R;
   float tx = A_(dot3_rn(R[0], R[1], R[2], m.x, m.y, m.z), v.t[0]);
@@ -177,7 +182,7 @@ __device__ bool project_rn(const float4 m, const float4 s, const float4 q, const
   } else {
     depth = tz;
   }
-  accurate_geometry(m, Rq, sv, v, o.lowpass, gamma, o.alpha_min, rec);
+  accurate_geometry(m, md, Rq, sv, v, vd, o.lowpass, gamma, o.alpha_min, rec);
   rec.a.w = depth;
   return true;
 }
@@ -197,16 +202,35 @@ __device__ __forceinline__ float minor_fma(float a, float b, float c, float d) {
   return f + e;
 }
 
-__device__ void accurate_geometry(const float4 m, const float Rq[9], const float sv[3], const View& v,
-                                  float lowpass, float gamma, float amin, SplatRec& rec) {
+// 1 / x in FP64 from the FP32 reciprocal by two Newton steps (2^-23 -> 2^-45
+// -> rounding); x lies in the FP32 range, away from its ends.
+__device__ __forceinline__ double rcp_f64(double x) {
+  double y = (double)__frcp_rn((float)x);
+  y = fma(y, fma(-x, y, 1.0), y);
+  return fma(y, fma(-x, y, 1.0), y);
+}
+
+__device__ void accurate_geometry(const float4 m, const double (&md)[3], const float Rq[9], const float sv[3],
+                                  const View& v, const ViewD& d, float lowpass, float gamma, float amin,
+                                  SplatRec& rec) {
   const float* R = v.R;
-  const double tx = (double)R[0] * m.x + (double)R[1] * m.y + (double)R[2] * m.z + (double)v.t[0];
-  const double ty = (double)R[3] * m.x + (double)R[4] * m.y + (double)R[5] * m.z + (double)v.t[1];
-  const double tz = (double)R[6] * m.x + (double)R[7] * m.y + (double)R[8] * m.z + (double)v.t[2];
+  const double tx = fma(d.R[0], md[0], fma(d.R[1], md[1], fma(d.R[2], md[2], d.t[0])));
+  const double ty = fma(d.R[3], md[0], fma(d.R[4], md[1], fma(d.R[5], md[2], d.t[1])));
   const bool ortho = v.ortho > 0.f;
-  const double itz = 1.0 / tz;
-  const double u = ortho ? (double)v.ortho * tx + (double)v.cx : (double)v.fx * (tx * itz) + (double)v.cx;
-  const double vv = ortho ? (double)v.ortho * ty + (double)v.cy : (double)v.fy * (ty * itz) + (double)v.cy;
+  double u, vv;
+  float fz = 0.f, xz = 0.f, yz = 0.f;
+  if (ortho) {
+    u = fma(d.ortho, tx, d.cx);
+    vv = fma(d.ortho, ty, d.cy);
+  } else {
+    const double tz = fma(d.R[6], md[0], fma(d.R[7], md[1], fma(d.R[8], md[2], d.t[2])));
+    const double itz = rcp_f64(tz), qx = tx * itz, qy = ty * itz;
+    u = fma(d.fx, qx, d.cx);
+    vv = fma(d.fy, qy, d.cy);
+    fz = (float)tz;
+    xz = (float)qx;
+    yz = (float)qy;
+  }
   const float uh = (float)u, vh = (float)vv;
   const float ul = (float)(u - (double)uh), vl = (float)(vv - (double)vh);
   float T0[3], T1[3];
@@ -217,7 +241,6 @@ __device__ void accurate_geometry(const float4 m, const float Rq[9], const float
       T1[k] = v.ortho * R[3 + k];
     }
   } else {
-    const float fz = (float)tz, xz = (float)(tx * itz), yz = (float)(ty * itz);
     const float j00 = v.fx / fz, j02 = -v.fx * xz / fz;
     const float j11 = v.fy / fz, j12 = -v.fy * yz / fz;
 #pragma unroll
@@ -290,6 +313,7 @@ __device__ __forceinline__ float angular_gaussian(float hx, float hy, float hz, 
 struct PrepParams {
   SceneDev sc;
   View cam;
+  ViewD camd;
   gs3_light light;
   float4 lh;  // homogeneous light (light_h)
   float nl_amin;  // -ln(alpha_min) as FP32, from double precision on the host
@@ -297,7 +321,7 @@ struct PrepParams {
   float intensity;
   gs3_render_opts o;
   int gx, gy;
-  int sp0;  // first splat projected: 0 camera and light, 1 light only
+  int part0;  // first part: 0 both splats and the shading, 1 the light splat and the shading
   uint32_t* key[2];
   SplatRec* rec[2];
   int4* rect[2];
@@ -305,39 +329,58 @@ struct PrepParams {
   uint32_t* header;
 };
 
-__global__ void __launch_bounds__(256) k_prep(PrepParams p) {
+// Bound: FP64 (the positions; the chip has 2 FP64 lanes per SM and cycle) and
+// latency.  300k Gaussians, K = 8: one thread for both projections and the
+// shading, every FP32 value converted to FP64 where it is used, took 0.106 ms
+// at 24 warps per SM; a thread per part, values converted once per view or on
+// the host, at 48 warps 0.063 ms (1 M: 0.283 -> 0.186; 1000 Gaussians: 17 -> 6
+// us).  10 blocks per SM (no spills): 0.066, 8: 0.071.
+constexpr int kPrepThreads = 128;
+// The blocks take the parts in turn: 0 and 1 the splats (camera, light), 2 the
+// shading (p.part0: the first part launched), so that one's FP64 and another's
+// loads run side by side.
+__global__ void __launch_bounds__(kPrepThreads, 12) k_prep(const __grid_constant__ PrepParams p) {
   __shared__ float sR[9], st[3], sortho;
-  if (threadIdx.x == 0) {
-    sortho = light_view_any_rn(p.light, p.o.target, p.cam.W, p.cam.H, sR, st);
-    if (blockIdx.x == 0) {
-      float* hv = reinterpret_cast<float*>(p.header + H_LIGHT_VIEW);
-      for (int i = 0; i < 9; ++i) hv[i] = sR[i];
-      for (int i = 0; i < 3; ++i) hv[9 + i] = st[i];
-      reinterpret_cast<float*>(p.header)[H_LIGHT_ORTHO] = sortho;
+  __shared__ ViewD slv;
+  const int parts = 3 - p.part0, part = p.part0 + (int)blockIdx.x % parts, block = (int)blockIdx.x / parts;
+  if (part == 1) {
+    if (threadIdx.x == 0) {
+      sortho = light_view_any_rn(p.light, p.o.target, p.cam.W, p.cam.H, sR, st);
+      for (int i = 0; i < 9; ++i) slv.R[i] = (double)sR[i];
+      for (int i = 0; i < 3; ++i) slv.t[i] = (double)st[i];
+      slv.fx = p.camd.fx; slv.fy = p.camd.fy; slv.cx = p.camd.cx; slv.cy = p.camd.cy;
+      slv.ortho = (double)sortho;
+      if (block == 0) {
+        float* hv = reinterpret_cast<float*>(p.header + H_LIGHT_VIEW);
+        for (int i = 0; i < 9; ++i) hv[i] = sR[i];
+        for (int i = 0; i < 3; ++i) hv[9 + i] = st[i];
+        reinterpret_cast<float*>(p.header)[H_LIGHT_ORTHO] = sortho;
+      }
     }
+    __syncthreads();
   }
-  __syncthreads();
-  const int g = blockIdx.x * blockDim.x + threadIdx.x;
+  const int g = block * kPrepThreads + (int)threadIdx.x;
   if (g >= p.sc.n) return;
   const int n = p.sc.n;
   const float4 m = p.sc.mean_op[g];
-  const float4 s = p.sc.scale[g];
-  const float4 q = p.sc.rot[g];
-  const float gamma = 1.f / (1.f + expf(-m.w));
-
-  View lv = p.cam;
-#pragma unroll
-  for (int i = 0; i < 9; ++i) lv.R[i] = sR[i];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) lv.t[i] = st[i];
-  lv.ortho = sortho;
-
-#pragma unroll
-  for (int sp = 0; sp < 2; ++sp) {
-    if (sp < p.sp0) continue;
+  if (part < 2) {
+    const float4 s = p.sc.scale[g];
+    const float4 q = p.sc.rot[g];
+    const float gamma = 1.f / (1.f + expf(-m.w));
+    const double md[3] = {(double)m.x, (double)m.y, (double)m.z};
     SplatRec rec;
-    bool vis = project_rn(m, s, q, sp ? lv : p.cam, p.o, p.gx, p.gy, sp ? p.light.pos : nullptr, gamma,
-                          p.nl_amin, rec);
+    bool vis;
+    if (part == 0) {
+      vis = project_rn(m, md, s, q, p.cam, p.camd, p.o, p.gx, p.gy, nullptr, gamma, p.nl_amin, rec);
+    } else {
+      View lv = p.cam;
+#pragma unroll
+      for (int i = 0; i < 9; ++i) lv.R[i] = sR[i];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) lv.t[i] = st[i];
+      lv.ortho = sortho;
+      vis = project_rn(m, md, s, q, lv, slv, p.o, p.gx, p.gy, p.light.pos, gamma, p.nl_amin, rec);
+    }
     if (!vis) {
       rec.a = make_float4(0.f, 0.f, 0.f, 0.f);
       rec.b = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -345,9 +388,10 @@ __global__ void __launch_bounds__(256) k_prep(PrepParams p) {
       rec.r = make_int4(-1, -1, -2, -2);
     }
     rec.a.z = gamma;
-    p.key[sp][g] = vis ? __float_as_uint(rec.a.w) : 0xFFFFFFFFu;
-    p.rec[sp][g] = rec;
-    p.rect[sp][g] = rec.r;
+    p.key[part][g] = vis ? __float_as_uint(rec.a.w) : 0xFFFFFFFFu;
+    p.rec[part][g] = rec;
+    p.rect[part][g] = rec.r;
+    return;
   }
 
   // ---- shading colour (Sec. 4.1); omega_i = normalize(L.xyz - L.w mu) ----
@@ -398,7 +442,7 @@ __global__ void __launch_bounds__(256) k_prep(PrepParams p) {
 
 void launch_prep(const FrameArgs& f, cudaStream_t s, bool light_only) {
   PrepParams p;
-  p.sp0 = light_only ? 1 : 0;
+  p.part0 = light_only ? 1 : 0;
   p.sc = f.sc;
   for (int i = 0; i < 9; ++i) p.cam.R[i] = f.cam.R[i];
   for (int i = 0; i < 3; ++i) { p.cam.t[i] = f.cam.t[i]; p.cam_pos[i] = f.cam.pos[i]; }
@@ -408,6 +452,10 @@ void launch_prep(const FrameArgs& f, cudaStream_t s, bool light_only) {
   p.nl_amin = (float)(-log((double)f.opts.alpha_min));
   p.cam.fx = f.cam.fx; p.cam.fy = f.cam.fy; p.cam.cx = f.cam.cx; p.cam.cy = f.cam.cy;
   p.cam.W = f.cam.width; p.cam.H = f.cam.height;
+  for (int i = 0; i < 9; ++i) p.camd.R[i] = p.cam.R[i];
+  for (int i = 0; i < 3; ++i) p.camd.t[i] = p.cam.t[i];
+  p.camd.fx = p.cam.fx; p.camd.fy = p.cam.fy; p.camd.cx = p.cam.cx; p.camd.cy = p.cam.cy;
+  p.camd.ortho = 0.0;
   p.intensity = f.light.intensity;
   p.o = f.opts;
   p.gx = f.L->gx; p.gy = f.L->gy;
@@ -419,7 +467,7 @@ void launch_prep(const FrameArgs& f, cudaStream_t s, bool light_only) {
   p.shade = at<float4>(f.ws, f.L->shade);
   p.header = at<uint32_t>(f.ws, f.L->header);
   const int n = f.sc.n;
-  k_prep<<<(n + 255) / 256, 256, 0, s>>>(p);
+  k_prep<<<(unsigned)((n + kPrepThreads - 1) / kPrepThreads) * (3u - p.part0), kPrepThreads, 0, s>>>(p);
   count_launch();
 }
 
