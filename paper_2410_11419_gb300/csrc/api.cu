@@ -151,7 +151,7 @@ Workspace plan_workspace(int n, int width, int height, size_t cap) {
   L.partial = P.take(8 * cap > 1024 * items ? 8 * cap : 1024 * items);
   L.tile_order[0] = P.take(4 * (size_t)L.ntiles);
   L.tile_order[1] = P.take(4 * (size_t)L.ntiles);
-  L.seg_lvl = P.take(4 * (1025 + 5));
+  L.seg_lvl = P.take(4 * (kSegWord + 1));
   L.seg_flag = P.take(4 * items);
   L.seg_desc = P.take(16 * items);
   L.seg_lists = P.take(8 * items);

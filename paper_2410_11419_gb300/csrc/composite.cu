@@ -21,7 +21,7 @@ namespace {
 // ranks) and is non-decreasing in j.
 //
 // Work is split into segments of a tile's list: segment s holds receivers
-// [R_s, R_s+1) (kSegLen entries; the last takes the rest) and needs the
+// [R_s, R_s+1) (32 to 256 entries; the last takes the rest) and needs the
 // occluders [C_s, C_s+1) on top of the product A(C_s) that every ray carries
 // into it, with C_s = K(R_s).  Persistent warps take one segment at a time
 // from a ticket counter, in three kernels:
@@ -662,8 +662,9 @@ __global__ void __launch_bounds__(256) k_bound_starts(const ShadowParams p,
   const uint32_t pos = w - p.lvl_off[s];
   const int tile = (int)p.tile_order[pos];
   const uint32_t b = p.tile_start[tile], e = p.tile_start[tile + 1];
-  const bool last = (uint32_t)s == seg_count(e - b) - 1;
-  const uint32_t r0 = b + (uint32_t)s * kSegLen, r1 = last ? e : r0 + kSegLen;
+  const uint32_t seg = p.lvl_off[kSegWord];
+  const bool last = (uint32_t)s == seg_count(e - b, seg) - 1;
+  const uint32_t r0 = b + (uint32_t)s * seg, r1 = last ? e : r0 + seg;
   p.desc[w] = make_uint4((uint32_t)tile | (last ? kSegLast : 0u), r0, r1, s > 0 ? p.lvl_off[s - 1] + pos : kNoItem);
   if (e <= b) return;
   kb[r0] = occ_bound(p.list, b, r0, bound[p.list[r0]]);
@@ -1130,22 +1131,39 @@ __global__ void __launch_bounds__(kCamThreads) k_camera_env(const EnvCamParams e
 // (a longest-processing-time-first schedule).  One block: a counting sort on
 // a key of the list length (1024 buckets, the largest first), placed by
 // shared-memory atomics.  The key is the length in steps of 8 (longer lists
-// share the top bucket), or with seg_len > 0 the tile's number of shadow
-// segments, seg_count(length); then lvl_off[s] (s = 0..1024) also receives
-// the first work item of segment level s: the number of segments of levels
-// below s, level s holding every tile with more than s segments (a prefix of
-// the order).  The order within a bucket may vary from run to run; no result
+// share the top bucket), or with lvl_off the tile's number of shadow segments,
+// seg_count(length, seg), whose seg is chosen here; then lvl_off[s] (s =
+// 0..1024) also receives the first work item of segment level s: the number
+// of segments of levels below s, level s holding every tile with more than s
+// segments (a prefix of the order).  The order within a bucket may vary from run to run; no result
 // depends on it.
 __global__ void __launch_bounds__(1024) k_tile_order(const uint32_t* __restrict__ tile_start, int ntiles,
-                                                     uint32_t* __restrict__ order, uint32_t seg_len,
-                                                     uint32_t* __restrict__ lvl_off) {
+                                                     uint32_t* __restrict__ order, uint32_t* __restrict__ lvl_off,
+                                                     uint32_t max_items) {
   constexpr int kBuckets = 1024;
   __shared__ uint32_t cnt[kBuckets];
   __shared__ uint32_t wsum[32];
+  __shared__ uint32_t longest;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  uint32_t seg_len = 0u;
+  if (lvl_off) {
+    if (t == 0) longest = 0u;
+    __syncthreads();
+    uint32_t len = 0u;
+    for (int i = t; i < ntiles; i += blockDim.x) len = max(len, tile_start[i + 1] - tile_start[i]);
+    len = __reduce_max_sync(0xffffffffu, len);
+    if (lane == 0) atomicMax(&longest, len);
+    __syncthreads();
+    const uint32_t pairs = tile_start[ntiles];
+    seg_len = kSegMin;
+    while (seg_len < kSegLen && (pairs / seg_len > kSegTarget || (uint32_t)ntiles + pairs / seg_len + 1u > max_items ||
+                                 longest > seg_len * (uint32_t)(kSegLevels - 1)))
+      seg_len *= 2u;
+    if (t == 0) lvl_off[kSegWord] = seg_len;
+  }
   auto bucket = [&](int i) {
     const uint32_t len = tile_start[i + 1] - tile_start[i];
-    const uint32_t key = seg_len ? seg_count(len) : min(len >> 3, (uint32_t)(kBuckets - 1));
+    const uint32_t key = seg_len ? seg_count(len, seg_len) : min(len >> 3, (uint32_t)(kBuckets - 1));
     return (uint32_t)(kBuckets - 1) - key;  // largest key first
   };
   // exclusive scan of one value per thread over the block
@@ -1194,11 +1212,14 @@ __global__ void __launch_bounds__(1024) k_tile_order(const uint32_t* __restrict_
 void launch_tile_order(const FrameArgs& f, int splat, cudaStream_t s) {
   const Workspace& L = *f.L;
   uint32_t* order = at<uint32_t>(f.ws, L.tile_order[splat]);
-  k_tile_order<<<1, 1024, 0, s>>>(at<uint32_t>(f.ws, L.sp[splat].tile_start), L.ntiles, order, 0u, nullptr);
+  k_tile_order<<<1, 1024, 0, s>>>(at<uint32_t>(f.ws, L.sp[splat].tile_start), L.ntiles, order, nullptr, 0u);
   count_launch();
 }
 
-size_t shadow_seg_items(int ntiles, size_t cap) { return (size_t)ntiles + cap / kSegLen + 1; }
+size_t shadow_seg_items(int ntiles, size_t cap) {
+  const size_t few = cap / kSegMin, many = cap / kSegLen + kSegTarget;
+  return (size_t)ntiles + (few < many ? few : many) + 1;
+}
 
 namespace {
 
@@ -1313,7 +1334,7 @@ void prepare_shadow_composite(const FrameArgs& f, cudaStream_t s) {
   cudaMemsetAsync(at<uint32_t>(ws, f.L->seg_flag), 0, 4 * shadow_seg_items(f.L->ntiles, f.L->cap), s);
   cudaMemsetAsync(ws + f.L->rank_flags, 0, 2 * (size_t)f.L->n, s);
   k_tile_order<<<1, 1024, 0, s>>>(at<uint32_t>(ws, b.tile_start), f.L->ntiles, at<uint32_t>(ws, f.L->tile_order[1]),
-                                  kSegLen, lvl);
+                                  lvl, (uint32_t)shadow_seg_items(f.L->ntiles, f.L->cap));
   // the occluder bounds the segment plan reads; the rest follow K6a
   const size_t items = shadow_seg_items(f.L->ntiles, f.L->cap);
   const int n = f.sc.n;

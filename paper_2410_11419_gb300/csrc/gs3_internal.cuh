@@ -80,7 +80,7 @@ struct Workspace {
   size_t light_stop = 0;   // u32[HW] 1 + list index of the occluder that stopped the ray, or all ones
   size_t shadow_den = 0;   // float[N] sum of beta per Gaussian (by index)
   size_t tile_order[2] = {0, 0};  // u32[ntiles] per splat: tiles by decreasing list length (launch order)
-  size_t seg_lvl = 0;   // u32[1025 + 5]: shadow work items per segment level, three ticket counters, two list lengths
+  size_t seg_lvl = 0;   // u32[1025 + 6]: shadow work items per segment level, three ticket counters, two list lengths, segment length
   size_t seg_flag = 0;  // u32[items]: shadow segment publications (0 none, 1 done, 2 done and all stopped)
   size_t seg_desc = 0;   // uint4[items]: each shadow segment's tile, receivers and predecessor
   size_t seg_lists = 0;  // u32[2][items]: the segments with an open ray; those every ray enters stopped
@@ -240,13 +240,26 @@ void launch_camera_composite_batch(const FrameArgs* const* f, float* const* out,
                                    unsigned char* host, cudaStream_t s);
 // shadow composite work items (tile segments) a frame can have at most
 size_t shadow_seg_items(int ntiles, size_t cap);
-// A light tile's list is cut into segments of kSegLen entries, at most
-// kSegLevels - 1 per tile (the last takes the rest); the shadow composite and
-// its backward share the cut.
-constexpr uint32_t kSegLen = 256;
+// A light tile's list is cut into segments of seg entries, at most kSegLevels -
+// 1 per tile (the last takes the rest); the shadow composite and its backward
+// share the cut.  k_tile_order chooses seg, a power of two from kSegMin to
+// kSegLen, and leaves it at lvl_off[kSegWord]: the smallest with which the
+// frame's pairs make no more than kSegTarget segments beside one per tile and
+// no list more than kSegLevels - 1.  It depends on the frame alone: products
+// round at the cuts, and a frame gives the same bits whatever runs beside it.
+// A frame with many pairs fills the chip's 3,648 resident warps with segments
+// of kSegLen, and shorter ones only cost more starts and links of the chain;
+// with few pairs they keep more warps busy.  K6a + K6b + K6c with segments of
+// 256 / 128 / 64 / 32: 20k Gaussians at 256 x 256 0.24 / 0.14 / 0.11 / 0.12 ms
+// (backward 0.38 / 0.23 / 0.14 / 0.13), 1000 at 128 x 128 57 / 71 / 47 / 38 us.
+// With 2.4 M pairs (120k at 512 x 512) 128 still took 1 % off a frame alone, but
+// eight lights side by side (100k at 512 x 512) took 3.01 ms against 2.79.
+constexpr uint32_t kSegLen = 256, kSegMin = 32;
+constexpr uint32_t kSegTarget = 8192;
 constexpr int kSegLevels = 1024;
-__host__ __device__ inline uint32_t seg_count(uint32_t len) {
-  const uint32_t n = (len + kSegLen - 1) / kSegLen;
+constexpr int kSegWord = kSegLevels + 6;  // in the seg_lvl array
+__host__ __device__ inline uint32_t seg_count(uint32_t len, uint32_t seg) {
+  const uint32_t n = (len + seg - 1) / seg;
   return n < 1 ? 1u : (n > (uint32_t)(kSegLevels - 1) ? (uint32_t)(kSegLevels - 1) : n);
 }
 // a splat's tiles ordered longest list first (in length steps of 8), into L.tile_order[splat]

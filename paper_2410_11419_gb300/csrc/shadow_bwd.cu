@@ -35,7 +35,7 @@
 // Bound: issue slots.  Object workload (300k Gaussians, 800 x 800): 0.24 +
 // 0.02 + 0.76 ms (0.10 for the stopped segments beside them), against 2.57 ms
 // (0.31) with one warp per tile over the tile's whole list, scalar; 20k
-// Gaussians at 256 x 256, where that left 256 warps on the chip, 0.37 ms
+// Gaussians at 256 x 256, where that left 256 warps on the chip, 0.13 ms
 // against 0.84.
 #include "shadow_bwd.cuh"
 #include "shadow_seg.cuh"
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(128) k_shadow_bwd_suffix(const BwdParams p) {
   const int lane = threadIdx.x & 31;
   if (pos >= (uint32_t)p.ntiles) return;
   const int tile = (int)p.tile_order[pos];
-  const uint32_t nseg = seg_count(p.tile_start[tile + 1] - p.tile_start[tile]);
+  const uint32_t nseg = seg_count(p.tile_start[tile + 1] - p.tile_start[tile], p.lvl_off[kSegWord]);
   uint32_t nopen = nseg;
   for (uint32_t s0 = 1; s0 < nseg && nopen == nseg; s0 += 32) {
     const uint32_t s = s0 + (uint32_t)lane;
