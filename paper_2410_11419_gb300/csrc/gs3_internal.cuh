@@ -215,6 +215,8 @@ struct MlpArgs {
 };
 size_t mlp_bwd_scratch_bytes(int n, const MlpDev& m);
 void run_mlp_backward(const MlpArgs& a, void* scratch, float* wred, cudaStream_t s);
+size_t mlp_x3_bwd_scratch_bytes(int n, const MlpDev& m);  // networks of mlp_x3_supported widths
+void run_mlp_x3_backward(const MlpArgs& a, void* scratch, float* wred, cudaStream_t s);
 // side: a second stream for the parts that can overlap (null: all on s)
 gs3_status run_backward(const FrameArgs& f, const float* dimg, void* bws, size_t bws_bytes,
                         const gs3_grads& out, cudaStream_t s, SideStream* side = nullptr);

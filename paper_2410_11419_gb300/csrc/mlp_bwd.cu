@@ -1,31 +1,21 @@
-// K8b: backward of the Phi (Sec. 4.2) and Psi (Sec. 4.3) MLPs of an FP32 scene.
+// K8b, hidden widths of 16: backward of the Phi (Sec. 4.2) and Psi (Sec. 4.3)
+// MLPs of an FP32 scene (wider networks: mlp_x3_bwd.cu, which also states the
+// formulas).
 //
-// The network is x -> h_1 = act(W_1 x + b_1) -> ... -> h_L -> y = sigmoid(W_o h_L + b_o)
-// with x = encode(Gaussian) (the positional encoding of the direction and
-// the position, and the latent).  Given dL/dy per Gaussian:
-//   dz_o = dL/dy * y (1 - y)
-//   dz_L = (dz_o W_o) * act'(h_L)
-//   dz_l = (dz_{l+1} W_{l+1}) * act'(h_l),      dx = dz_1 W_1
-//   dW_l = sum_g dz_l h_{l-1}^T,  db_l = sum_g dz_l   (h_0 = x),  same for W_o
-// and dx goes back through the encoding to the Gaussian's position,
-// direction and latent.
-//
-// Every product over the Gaussians is a dense GEMM with N rows and 128 or
-// fewer columns:
-//   row GEMM (k_rowgemm_tc):  rows = Gaussians; forward recompute h_l = act(h_{l-1} W_l^T + b_l)
-//                             and the data gradients dz_{l-1} = (dz_l W_l) * act'(h_{l-1})
-//   weight GEMM (k_wgemm_tc): rows = output units, contraction over Gaussians split
-//                             across blocks (the bias sums from a ones column); per-block
-//                             partials are summed in block order, so the gradients do not
-//                             depend on scheduling.
-// Both run on the tensor cores in three-pass TF32 (about 2^-21 relative per
-// product, FP32 accumulation).  The output layer (1 or 3 units) and its
-// weight gradient run on CUDA cores in k_out_layer.  Hidden widths of 16 take
-// their weight gradients from a register-tiled FP32 SIMT kernel (k_wgemm): a
-// block owns a 128 x 128 tile of C = A B, each thread 8 x 8 of it, with the
-// contraction staged through double-buffered shared memory in chunks of 16.
-// The activations and data gradients of one network live in the backward
-// workspace (about (64 + 4 W) N floats), shared by Phi and Psi in turn.
+// Every product over the Gaussians is a GEMM of its own with N rows:
+//   row GEMM (k_rowgemm_tc): rows = Gaussians; forward recompute h_l = act(h_{l-1} W_l^T + b_l)
+//                            and the data gradients dz_{l-1} = (dz_l W_l) * act'(h_{l-1}),
+//                            on the tensor cores in three-pass TF32 (about 2^-21
+//                            relative per product, FP32 accumulation)
+//   weight GEMM (k_wgemm):   16 output units, contraction over Gaussians split
+//                            across blocks, register-tiled FP32: a block owns a
+//                            128 x 128 tile of C = A B, each thread 8 x 8 of it, with
+//                            the contraction staged through double-buffered shared
+//                            memory in chunks of 16; per-block partials are summed in
+//                            block order, so the gradients do not depend on scheduling.
+// The output layer (1 or 3 units) and its weight gradient run on CUDA cores in
+// k_out_layer.  The activations and data gradients of one network live in the
+// backward workspace (about (64 + 4 W) N floats), shared by Phi and Psi in turn.
 #include "gs3_internal.cuh"
 #include "tc_ptx.cuh"
 
@@ -131,8 +121,8 @@ __device__ __forceinline__ void gemm_tile(GemmSmem& S, const Operand& A, const O
 //   EPI_DACT:     . * act'(H[g][j])           (data gradient, H = the layer's output)
 //   EPI_NONE:     .                           (dx)
 struct RowGemm {
-  Operand A, B;
-  const unsigned char* bpack;  // tensor-core form: B pre-split into chunk tiles (tc_pack_b), or null
+  Operand A;
+  const unsigned char* bpack;  // B pre-split into chunk tiles (k_pack_b)
   int n, ncols, kdim;
   float* C;
   int ldc;
@@ -178,7 +168,7 @@ __global__ void __launch_bounds__(kGemmThreads, 2) k_wgemm(WGemm p) {
   if (t < p.nout) out[(size_t)p.nout * p.nin + t] = bsum;
 }
 
-// ---- the same GEMMs on the tensor cores, three-pass TF32 --------------------
+// ---- row GEMMs on the tensor cores, three-pass TF32 -------------------------
 // Every FP32 operand x is split into big = x with its low 13 mantissa bits
 // cleared (a TF32 value) and small = x - big (exact in FP32); a product is
 // formed as big*big' + big*small' + small*big' by tcgen05.mma kind::tf32
@@ -187,12 +177,12 @@ __global__ void __launch_bounds__(kGemmThreads, 2) k_wgemm(WGemm p) {
 // 2^-24 for an FP32 FMA.
 //
 // A CTA of 128 threads owns a 128 x npad output tile in TMEM (npad a
-// multiple of 32).  The contraction runs in chunks of kTcK elements: each
-// thread stages one row of the A chunk and one (or two) rows of the B chunk,
-// split, into K-major no-swizzle shared-memory tiles; thread 0 issues the
-// chunk's 4 K-steps x 3 passes and commits them to an mbarrier (a bounded,
-// sleeping wait); the next chunk is staged once they have completed.  Several
-// CTAs per SM overlap one CTA's staging with another's MMAs.
+// multiple of 32).  The contraction runs in chunks of kTcK elements: the
+// threads stage the A chunk, split, into K-major no-swizzle shared-memory tiles
+// and one bulk copy brings the packed B chunk; thread 0 issues the chunk's 4
+// K-steps x 3 passes and commits them to an mbarrier (a bounded, sleeping wait);
+// the next chunk is staged once they have completed.  Several CTAs per SM
+// overlap one CTA's staging with another's MMAs.
 constexpr int kTcK = 32;            // contraction elements per chunk
 constexpr int kTcRowBytes = kTcK * 4;  // bytes of a chunk row
 constexpr int kTcTile = 128;
@@ -219,102 +209,46 @@ __device__ __forceinline__ void tc_put4(const float (&v)[4], int r, int c4, unsi
   *reinterpret_cast<float4*>(small + off) = s4;
 }
 
-// A thread's share of one operand chunk (elements kk = k0 .. k0 + 31 of
-// operand rows i0 + r, r < nrows <= 128; 0 outside the operand or past kend),
-// loaded into registers ahead of the chunk that uses it.  Both access
-// patterns keep a warp's global loads on few lines and its 16-byte shared
-// stores on distinct banks:
-//   kk_rows (operand row-major in i): lane = row r = t, consecutive lanes
-//     read consecutive i (one line per load), 32 loads per thread;
-//   otherwise (row-major in kk): a warp covers 8 rows x 4 float4 per step,
-//     lane l row l & 7 and float4 l >> 3 (16-byte loads where aligned); the
-//     stores of 8 lanes fill one 128-byte core-matrix row group.
+// A thread's share of one chunk of A (elements kk = k0 .. k0 + 31 of rows
+// i0 .. i0 + 127; 0 outside the operand), loaded into registers ahead of the
+// chunk that uses it: a warp covers 8 rows x 4 float4 per step, lane l row l & 7
+// and float4 l >> 3 (16-byte loads where aligned); the 16-byte stores of 8 lanes
+// fill one 128-byte core-matrix row group.
 struct TcRegs {
   float4 v[8];
 };
 
-__device__ __forceinline__ void tc_load(const Operand& o, int i0, int nrows, int k0, int kend, TcRegs& R) {
-  const int t = threadIdx.x;
-  const int klim = min(kend, o.nk);
-  if (o.kk_rows) {
-    const int i = i0 + t;
-    const bool row_ok = t < nrows && i < o.ni;
+__device__ __forceinline__ void tc_load(const Operand& o, int i0, int k0, TcRegs& R) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool vec = (o.ld & 3) == 0 && (reinterpret_cast<uintptr_t>(o.m) & 15) == 0;
 #pragma unroll
-    for (int c4 = 0; c4 < kTcK / 4; ++c4) {
-      float v[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int kk = k0 + 4 * c4 + e;
-        v[e] = (row_ok && kk < klim) ? o.m[(size_t)kk * o.ld + i] : 0.f;
+  for (int qq = 0; qq < 8; ++qq) {
+    const int q = warp + 4 * qq;
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int i = i0 + (q >> 1) * 8 + (lane & 7), kk = k0 + 4 * ((q & 1) * 4 + (lane >> 3));
+    if (i < o.ni) {
+      const float* src = o.m + (size_t)i * o.ld + kk;
+      if (vec && kk + 4 <= o.nk) {
+        x = *reinterpret_cast<const float4*>(src);
+      } else {
+        x.x = kk < o.nk ? src[0] : 0.f;
+        x.y = kk + 1 < o.nk ? src[1] : 0.f;
+        x.z = kk + 2 < o.nk ? src[2] : 0.f;
+        x.w = kk + 3 < o.nk ? src[3] : 0.f;
       }
-      R.v[c4] = make_float4(v[0], v[1], v[2], v[3]);
     }
-  } else {
-    const int lane = t & 31, warp = t >> 5;
-    const int steps = (nrows / 8) * 2;  // (8-row group, half of the chunk's 8 float4) pairs
-    const bool vec = (o.ld & 3) == 0 && (reinterpret_cast<uintptr_t>(o.m) & 15) == 0;
-#pragma unroll
-    for (int qq = 0; qq < 8; ++qq) {
-      const int q = warp + 4 * qq;
-      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (q < steps) {
-        const int r = (q >> 1) * 8 + (lane & 7), c4 = (q & 1) * 4 + (lane >> 3);
-        const int i = i0 + r, kk = k0 + 4 * c4;
-        if (i < o.ni) {
-          const float* src = o.m + (size_t)i * o.ld + kk;
-          if (vec && kk + 4 <= klim) {
-            x = *reinterpret_cast<const float4*>(src);
-          } else {
-            x.x = kk < klim ? src[0] : 0.f;
-            x.y = kk + 1 < klim ? src[1] : 0.f;
-            x.z = kk + 2 < klim ? src[2] : 0.f;
-            x.w = kk + 3 < klim ? src[3] : 0.f;
-          }
-        }
-      }
-      R.v[qq] = x;
-    }
+    R.v[qq] = x;
   }
 }
 
-// Split a thread's loaded share into the big and small chunk tiles.  Rows
-// [128, nrows) (a weight GEMM's N past 128) hold no operand data: the ones
-// row (1 for kk < kend) or zeros.
-__device__ __forceinline__ void tc_store(const Operand& o, int nrows, int k0, int kend, int ones_row,
-                                         const TcRegs& R, unsigned char* big, unsigned char* small) {
-  const int t = threadIdx.x;
-  if (o.kk_rows) {
-    if (t < nrows) {
+// Split a thread's loaded share into the big and small chunk tiles
+__device__ __forceinline__ void tc_store(const TcRegs& R, unsigned char* big, unsigned char* small) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-      for (int c4 = 0; c4 < kTcK / 4; ++c4) {
-        float v[4] = {R.v[c4].x, R.v[c4].y, R.v[c4].z, R.v[c4].w};
-        if (t == ones_row)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) v[e] = k0 + 4 * c4 + e < kend ? 1.f : 0.f;
-        tc_put4(v, t, c4, big, small);
-      }
-    }
-    for (int r = t + kTcTile; r < nrows; r += kTcTile) {
-#pragma unroll
-      for (int c4 = 0; c4 < kTcK / 4; ++c4) {
-        float v[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) v[e] = (r == ones_row && k0 + 4 * c4 + e < kend) ? 1.f : 0.f;
-        tc_put4(v, r, c4, big, small);
-      }
-    }
-  } else {
-    const int lane = t & 31, warp = t >> 5;
-    const int steps = (nrows / 8) * 2;
-#pragma unroll
-    for (int qq = 0; qq < 8; ++qq) {
-      const int q = warp + 4 * qq;
-      if (q < steps) {
-        const int r = (q >> 1) * 8 + (lane & 7), c4 = (q & 1) * 4 + (lane >> 3);
-        const float v[4] = {R.v[qq].x, R.v[qq].y, R.v[qq].z, R.v[qq].w};
-        tc_put4(v, r, c4, big, small);
-      }
-    }
+  for (int qq = 0; qq < 8; ++qq) {
+    const int q = warp + 4 * qq;
+    const float v[4] = {R.v[qq].x, R.v[qq].y, R.v[qq].z, R.v[qq].w};
+    tc_put4(v, (q >> 1) * 8 + (lane & 7), (q & 1) * 4 + (lane >> 3), big, small);
   }
 }
 
@@ -415,7 +349,7 @@ __device__ __forceinline__ bool tc_run_chunk(const TcCta& c, uint32_t bar, uint3
 }
 
 // C[g][j] = epi(sum_kk A[g][kk] B[kk][j]) for the 128 rows of this CTA and
-// j < ncols (npad = ncols rounded up to 32); the epilogues of k_rowgemm.
+// j < ncols (npad = ncols rounded up to 32); epilogues as in RowGemm.
 template <int EPI>
 __global__ void __launch_bounds__(kTcTile) k_rowgemm_tc(RowGemm p, int npad, uint32_t* status) {
   extern __shared__ __align__(1024) unsigned char sm[];
@@ -433,30 +367,22 @@ __global__ void __launch_bounds__(kTcTile) k_rowgemm_tc(RowGemm p, int npad, uin
   const uint32_t chunk_bytes = 2u * npad * kTcRowBytes;
   uint32_t phase = 0, phase_b = 0;
   bool ok = true, b_late = false;
-  TcRegs ra, rb;
-  tc_load(p.A, i0, kTcTile, 0, p.kdim, ra);
-  if (!p.bpack) tc_load(p.B, 0, npad, 0, p.kdim, rb);
+  TcRegs ra;
+  tc_load(p.A, i0, 0, ra);
   for (int k0 = 0; k0 < p.kdim && ok; k0 += kTcK) {
-    if (p.bpack && t == 0) {  // the chunk's B tiles (big, small) by one bulk copy
+    if (t == 0) {  // the chunk's B tiles (big, small) by one bulk copy
       tc::mbar_expect_tx(tc::smem_u32(&bar_b), chunk_bytes);
       tc::bulk_g2s(tc::smem_u32(c.bb), p.bpack + (size_t)(k0 / kTcK) * chunk_bytes, chunk_bytes,
                    tc::smem_u32(&bar_b));
     }
-    tc_store(p.A, kTcTile, k0, p.kdim, -1, ra, c.ab, c.as);
-    if (!p.bpack) tc_store(p.B, npad, k0, p.kdim, -1, rb, c.bb, c.bs);
-    if (p.bpack) {  // every thread: the B tiles have landed (a bounded wait)
-      const bool b_ok = tc::mbar_wait_bounded(tc::smem_u32(&bar_b), phase_b);
-      if (!b_ok) {
-        ok = false;
-        b_late = true;
-      }
-      phase_b ^= 1u;
+    tc_store(ra, c.ab, c.as);
+    if (!tc::mbar_wait_bounded(tc::smem_u32(&bar_b), phase_b)) {  // every thread: the B tiles have landed
+      ok = false;
+      b_late = true;
     }
+    phase_b ^= 1u;
     ok = tc_run_chunk(c, tc::smem_u32(&bar), phase, idesc, k0 == 0, [&] {
-      if (k0 + kTcK < p.kdim) {  // the next chunk's loads overlap this chunk's MMAs
-        tc_load(p.A, i0, kTcTile, k0 + kTcK, p.kdim, ra);
-        if (!p.bpack) tc_load(p.B, 0, npad, k0 + kTcK, p.kdim, rb);
-      }
+      if (k0 + kTcK < p.kdim) tc_load(p.A, i0, k0 + kTcK, ra);  // overlaps this chunk's MMAs
     }) && ok;
   }
   if (ok) {
@@ -515,66 +441,6 @@ __global__ void __launch_bounds__(kTcTile) k_rowgemm_tc(RowGemm p, int npad, uin
     }
   }
   if (b_late) tc::mbar_wait_bounded(tc::smem_u32(&bar_b), phase_b ^ 1u);  // our own copy lands before we leave
-  tc_cta_end(c, ok, status);
-}
-
-// Block b: partial[b][j][k] = sum over its Gaussians g of dZ[g][j] H[g][k]
-// (j < nout <= 128, k < nin) and, from a ones column at k = nin, the bias
-// partial sum_g dZ[g][j]; the layout of k_wgemm's partials.
-__global__ void __launch_bounds__(kTcTile) k_wgemm_tc(WGemm p, int npad, uint32_t* status) {
-  extern __shared__ __align__(1024) unsigned char sm[];
-  __shared__ __align__(8) uint64_t bar;
-  __shared__ uint32_t slot;
-  const int t = threadIdx.x;
-  const int kbeg = blockIdx.x * p.rows_per_block;
-  const int kend = min(p.n, kbeg + p.rows_per_block);
-  const TcCta c = tc_cta_begin(sm, npad, &bar, &slot);
-  const uint32_t idesc = tc::idesc_tf32(kTcTile, npad);
-  uint32_t phase = 0;
-  bool ok = true;
-  TcRegs ra, rb;
-  if (kbeg < kend) {
-    tc_load(p.A, 0, kTcTile, kbeg, kend, ra);
-    tc_load(p.B, 0, npad, kbeg, kend, rb);
-  }
-  for (int k0 = kbeg; k0 < kend && ok; k0 += kTcK) {
-    tc_store(p.A, kTcTile, k0, kend, -1, ra, c.ab, c.as);
-    tc_store(p.B, npad, k0, kend, p.nin, rb, c.bb, c.bs);
-    ok = tc_run_chunk(c, tc::smem_u32(&bar), phase, idesc, k0 == kbeg, [&] {
-      if (k0 + kTcK < kend) {  // the next chunk's loads overlap this chunk's MMAs
-        tc_load(p.A, 0, kTcTile, k0 + kTcK, kend, ra);
-        tc_load(p.B, 0, npad, k0 + kTcK, kend, rb);
-      }
-    });
-  }
-  const size_t np = (size_t)p.nout * p.nin + p.nout;
-  float* out = p.part + (size_t)blockIdx.x * np;
-  if (ok && kbeg >= kend) {  // no rows: zero partials
-    for (size_t i = t; i < np; i += kTcTile) out[i] = 0.f;
-  } else if (ok) {
-    float* buf = reinterpret_cast<float*>(sm);
-    const uint32_t lane_addr = c.tmem + ((uint32_t)((t >> 5) * 32) << 16);
-    const int lane = t & 31, warp = t >> 5;
-    for (int c0 = 0; c0 < npad; c0 += 32) {
-      float v[32];
-      tc::tmem_ld32(lane_addr + (uint32_t)c0, v);
-      tc_rows_to_smem(v, buf);
-      __syncthreads();
-      for (int q = warp; q < kTcTile / 4; q += kTcTile / 32) {
-        const int j = q * 4 + (lane >> 3), k0c = c0 + 4 * (lane & 7);
-        if (j < p.nout) {
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const int k = k0c + e;
-            const float x = buf[j * kTcOutStride + 4 * (lane & 7) + e];
-            if (k < p.nin) out[(size_t)j * p.nin + k] = x;
-            else if (k == p.nin) out[(size_t)p.nout * p.nin + j] = x;
-          }
-        }
-      }
-      __syncthreads();
-    }
-  }
   tc_cta_end(c, ok, status);
 }
 
@@ -813,6 +679,7 @@ Scratch carve(void* base, int n, const MlpDev& m) {
 }  // namespace
 
 size_t mlp_bwd_scratch_bytes(int n, const MlpDev& m) {
+  if (mlp_x3_supported(m)) return mlp_x3_bwd_scratch_bytes(n, m);
   auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
   const size_t wide = (size_t)(m.width > kXdim ? m.width : kXdim);
   const size_t layer_max = (size_t)m.width * (m.width > m.in_dim ? m.width : m.in_dim) + m.width;
@@ -849,21 +716,10 @@ void launch_rowgemm_tc(const RowGemm& g, int grid, uint32_t* status, cudaStream_
   count_launch();
 }
 
-void launch_wgemm_tc(const WGemm& w, int grid, uint32_t* status, cudaStream_t s) {
-  const int npad = round32(w.nin + 1);
-  const size_t smem = tc_launch_smem(npad);
-  static DeviceOnce once;
-  once.run([] {
-    return cudaFuncSetAttribute(k_wgemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) ==
-           cudaSuccess;
-  });
-  k_wgemm_tc<<<grid, kTcTile, smem, s>>>(w, npad, status);
-  count_launch();
-}
-
 }  // namespace
 
 void run_mlp_backward(const MlpArgs& a, void* scratch, float* wred, cudaStream_t s) {
+  if (mlp_x3_supported(a.net)) return run_mlp_x3_backward(a, scratch, wred, s);
   const MlpDev& m = a.net;
   const int n = a.n, W = m.width, nh = m.n_hidden;
   Scratch S = carve(scratch, n, m);
@@ -912,7 +768,6 @@ void run_mlp_backward(const MlpArgs& a, void* scratch, float* wred, cudaStream_t
     const int din = l == 0 ? m.in_dim : W;
     RowGemm g;
     g.A = {l == 0 ? S.X : S.H + (size_t)(l - 1) * n * W, l == 0 ? kXdim : W, n, din, false};
-    g.B = {wl[l], din, W, din, false};  // B[kk][j] = W_l[j][kk]
     g.bpack = S.bpack + (size_t)(2 * l) * kPackBytes;
     g.n = n; g.ncols = W; g.kdim = din;
     g.C = S.H + (size_t)l * n * W; g.ldc = W;
@@ -937,12 +792,8 @@ void run_mlp_backward(const MlpArgs& a, void* scratch, float* wred, cudaStream_t
     w.B = {Hin, ldhin, nin, n, true};
     w.n = n; w.nout = nout; w.nin = nin; w.rows_per_block = rpb;
     w.part = S.part;
-    if (nout >= 32) {
-      launch_wgemm_tc(w, nb, a.status, s);
-    } else {  // hidden widths of 16: FP32 SIMT
-      k_wgemm<<<nb, kGemmThreads, 0, s>>>(w);
-      count_launch();
-    }
+    k_wgemm<<<nb, kGemmThreads, 0, s>>>(w);
+    count_launch();
     const size_t np = (size_t)nout * nin + nout;
     k_sum_parts<<<(int)((np + 31) / 32), kSumWarps * 32, 0, s>>>(S.part, np, nb, wred + poff[layer]);
     count_launch();
@@ -957,7 +808,6 @@ void run_mlp_backward(const MlpArgs& a, void* scratch, float* wred, cudaStream_t
     // data gradient into the layer below (dx for l = 0)
     RowGemm g;
     g.A = {S.dz[cur], W, n, W, false};
-    g.B = {wl[l], din, din, W, true};  // B[kk][j] = W_l[kk][j]
     g.bpack = S.bpack + (size_t)(2 * l + 1) * kPackBytes;
     g.n = n; g.ncols = din; g.kdim = W;
     g.C = S.dz[cur ^ 1]; g.ldc = l == 0 ? kXdim : W;

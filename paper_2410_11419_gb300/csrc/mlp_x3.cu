@@ -25,23 +25,14 @@
 // conversions between layers (a tile takes 11 us, its MMAs alone 4.3).  300k
 // Gaussians, 3 x 128: 0.18 ms per network, against 0.68 ms for register-tiled
 // FP32 FMAs (46 % of the FMA pipe).
-#include <cuda_bf16.h>
-
-#include "gs3_internal.cuh"
-#include "tc_ptx.cuh"
+#include "mlp_x3.cuh"
 
 namespace gs3 {
 namespace {
 
-using namespace tc;
+using namespace x3;
 
-constexpr int kRows = 128;
-constexpr int kEpiThreads = 256;              // two warpgroups
-constexpr int kThreads = kEpiThreads + 64;    // and the MMA and copy warps
-constexpr int kK0 = 64;                       // padded input width (61 / 60 features)
-constexpr int kChunk = 32;                    // inputs of a layer per weight chunk
-constexpr int kStages = 4;
-constexpr int kMaxHidden = 4;
+constexpr int kThreads = kEpiThreads + 64;  // and the MMA and copy warps
 
 struct X3Params {
   int n, nh, width, act;
@@ -63,8 +54,6 @@ struct X3Params {
   uint32_t* status;
 };
 
-__host__ __device__ inline uint32_t chunk_bytes(int W) { return 3u * (uint32_t)W * kChunk * 2u; }
-
 // ---- packing -----------------------------------------------------------------
 struct PackArgs {
   const float* w[2];  // Phi, Psi hidden weights
@@ -72,13 +61,6 @@ struct PackArgs {
   unsigned char* dst[2];
   int total[2];  // elements
 };
-
-__device__ __forceinline__ void split3(float x, __nv_bfloat16& h, __nv_bfloat16& m, __nv_bfloat16& l) {
-  h = __float2bfloat16_rn(x);
-  const float r = x - __bfloat162float(h);
-  m = __float2bfloat16_rn(r);
-  l = __float2bfloat16_rn(r - __bfloat162float(m));
-}
 
 // Element (layer, output row, input k) of a network's hidden layers into its
 // chunk: chunk k / 32 of the layer holds the three splits one after the other,
@@ -111,101 +93,6 @@ __global__ void __launch_bounds__(256) k_x3_pack(PackArgs a) {
 int hidden_elems(const MlpDev& m) { return m.width * kK0 + (m.n_hidden - 1) * m.width * m.width; }
 
 // ---- the networks -------------------------------------------------------------
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-
-// Whether x holds for any thread of the two warpgroups (a barrier of theirs)
-__device__ __forceinline__ bool epi_any(bool x) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.u32 p, %1, 0;\n\t"
-      "barrier.cta.red.or.pred q, 1, %2, p;\n\t"
-      "selp.u32 %0, 1, 0, q;\n\t}"
-      : "=r"(r) : "r"((uint32_t)x), "n"(kEpiThreads) : "memory");
-  return r != 0u;
-}
-
-// Eight values of row `row`, columns k0 .. k0 + 7, as three splits (16 bytes each)
-__device__ __forceinline__ void store_split8(unsigned char* A, uint32_t split_bytes, int row, int k0, int kdim,
-                                             const float* v) {
-  __nv_bfloat162 h[4], m[4], l[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    h[i] = __float22bfloat162_rn(make_float2(v[2 * i], v[2 * i + 1]));
-    const float2 hf = __bfloat1622float2(h[i]);
-    const float2 r = make_float2(v[2 * i] - hf.x, v[2 * i + 1] - hf.y);
-    m[i] = __float22bfloat162_rn(r);
-    const float2 mf = __bfloat1622float2(m[i]);
-    l[i] = __float22bfloat162_rn(make_float2(r.x - mf.x, r.y - mf.y));
-  }
-  unsigned char* p = A + canon_off(row, 2 * k0, 2 * kdim);
-  *reinterpret_cast<uint4*>(p) = *reinterpret_cast<uint4*>(h);
-  *reinterpret_cast<uint4*>(p + split_bytes) = *reinterpret_cast<uint4*>(m);
-  *reinterpret_cast<uint4*>(p + 2 * split_bytes) = *reinterpret_cast<uint4*>(l);
-}
-
-// Features [base, base + 27) of x: [v, sin(2^q pi v), cos(2^q pi v)], q < bands
-__device__ __forceinline__ void pe_bands(float* x, int base, const float (&v)[3], int bands) {
-#pragma unroll
-  for (int c = 0; c < 3; ++c) x[base + c] = v[c];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    if (q >= bands) break;
-    const float f = (float)(1 << q);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) sincospif(f * v[c], &x[base + 3 + 6 * q + c], &x[base + 6 + 6 * q + c]);
-  }
-}
-
-// Inputs 32 HALF .. 32 HALF + 31 of a row: Phi [T, PE(w_i), PE(mu), l], Psi
-// [PE(w_o), PE(mu), l], padded to 64 with zeros.
-template <int WHICH, int HALF>
-__device__ __forceinline__ void encode_half(const X3Params& p, int li, int g, unsigned char* A, uint32_t split_bytes,
-                                            int row) {
-  constexpr int b0 = WHICH == 0 ? 1 : 0;
-  float x[kK0 + 8];
-  const float4 m = p.mean_op[g];
-  const float mu[3] = {m.x, m.y, m.z};
-  if (HALF == 0) {
-    float sx, sy, sz, sw;
-    if (WHICH == 0) {
-      const float4 lh = p.light[li];
-      sx = lh.x; sy = lh.y; sz = lh.z; sw = lh.w;
-    } else {
-      sx = p.cam_pos[0]; sy = p.cam_pos[1]; sz = p.cam_pos[2]; sw = 1.f;
-    }
-    const float dx = sx - sw * m.x, dy = sy - sw * m.y, dz = sz - sw * m.z;
-    const float il = rsqrtf(dx * dx + dy * dy + dz * dz);
-    const float d[3] = {dx * il, dy * il, dz * il};
-    if (WHICH == 0) x[0] = p.T[li][g];
-    pe_bands(x, b0, d, 4);
-    pe_bands(x, b0 + 27, mu, 1);  // the first of them
-  } else {
-    pe_bands(x, b0 + 27, mu, 4);
-    const float4 l0 = p.latent[g], l1 = p.latent[p.n + g];
-    x[b0 + 54] = l0.x; x[b0 + 55] = l0.y; x[b0 + 56] = l0.z; x[b0 + 57] = l0.w;
-    x[b0 + 58] = l1.x; x[b0 + 59] = l1.y;
-#pragma unroll
-    for (int k = b0 + 60; k < kK0; ++k) x[k] = 0.f;
-  }
-#pragma unroll
-  for (int k0 = 32 * HALF; k0 < 32 * HALF + 32; k0 += 8) store_split8(A, split_bytes, row, k0, kK0, x + k0);
-}
-
 __host__ __device__ inline uint32_t x3_cols(int W) {  // TMEM: two buffers of two accumulators
   return W < 32 ? 32u : 4u * (uint32_t)W;
 }
@@ -332,8 +219,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_x3(X3Params p) {
       bool ok = true;  // the same for a warp's lanes
       const int r = ((int)blockIdx.x + it * (int)gridDim.x) * kRows + row, rc = min(r, rows - 1);
       const int li = rc / p.n, g = rc - li * p.n;
-      if (wg == 0) encode_half<WHICH, 0>(p, li, g, A, split_bytes, row);
-      else encode_half<WHICH, 1>(p, li, g, A, split_bytes, row);
+      const X3Input in = {p.n, p.mean_op, p.latent, WHICH == 0 ? p.T[li] : nullptr,
+                          WHICH == 0 ? p.light[li] : make_float4(p.cam_pos[0], p.cam_pos[1], p.cam_pos[2], 1.f)};
+      const auto put = [&](int k0, const float* x) { store_split8(A, split_bytes, row, k0, kK0, x); };
+      if (wg == 0) encode_half<WHICH, 0>(in, g, put);
+      else encode_half<WHICH, 1>(in, g, put);
       hand_on(0);
       hand_on(1);
       float acc[kOut];
@@ -346,12 +236,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_x3(X3Params p) {
         const uint32_t big = lane_addr + (uint32_t)(layer & 1) * 2u * (uint32_t)W;
         for (int c = 0; c < chunksN; ++c) {
           const int c0 = kChunk * c + 16 * wg;
-          float v[16], u[16];
-          tmem_ld16(big + (uint32_t)c0, v);
-          tmem_ld16(big + (uint32_t)(W + c0), u);
+          float v[16];
+          acc_load16(big + (uint32_t)c0, big + (uint32_t)(W + c0), v);
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
-            const float h = (v[i] + u[i]) + bsm[l * W + c0 + i];
+            const float h = v[i] + bsm[l * W + c0 + i];
             v[i] = h > 0.f ? h : (leaky ? 0.01f * h : 0.f);
           }
           if (l + 1 < nh) {
