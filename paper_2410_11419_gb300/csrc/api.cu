@@ -433,7 +433,7 @@ gs3_status render_frame(gs3_scene* scene, const gs3_camera* cam, const gs3_light
       launch_mlp(f, s);
     }
   }
-  if (stages & GS3_STAGE_CAMERA) launch_camera_composite(f, out_rgb, s);
+  if (stages & GS3_STAGE_CAMERA) launch_camera_composite(f, out_rgb, (stages & GS3_STAGE_MLP) != 0, s);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "gs3_render: launch");
   return GS3_OK;

@@ -241,6 +241,7 @@ __device__ __forceinline__ int locate(const ShadowParams* reqs, int nreq, int ki
 template <bool BATCH>
 __global__ void __launch_bounds__(kSegWarps * 32, 5) k_shadow_chain(const ShadowParams p, const ShadowParams* reqs,
                                                                     int nreq) {
+  after_previous();
   __shared__ StagedEntries smem[kSegWarps];
   StagedEntries& S = smem[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
@@ -425,6 +426,7 @@ __device__ __forceinline__ void dead_item(const ShadowParams& p, uint32_t w, Dea
 // pixel that K6c itself would evaluate counts: inside the image, in a tile of
 // the Gaussian's rectangle, in a half its box and ellipse reach.
 __global__ void k_dead_probe(const ShadowParams p, int n) {
+  after_previous();
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= n || p.rank_flags[r].x || p.rank_flags[r].y) return;
   const SplatRec q = p.rrec[r];
@@ -449,6 +451,7 @@ __global__ void k_dead_probe(const ShadowParams p, int n) {
 template <bool BATCH>
 __global__ void __launch_bounds__(kDeadWarps * 32, 7) k_shadow_dead(const ShadowParams p, const ShadowParams* reqs,
                                                                     int nreq) {
+  after_previous();
   __shared__ DeadSmem smem[kDeadWarps];
   DeadSmem& D = smem[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
@@ -597,6 +600,7 @@ __device__ __forceinline__ void live_item(const ShadowParams& p, uint32_t w, Sha
 // (object workload).
 template <bool BATCH>
 __global__ void __launch_bounds__(kSegWarps * 32, 6) k_shadow(const ShadowParams p, const ShadowParams* reqs, int nreq) {
+  after_previous();
   __shared__ ShadowSmem smem[kSegWarps];
   ShadowSmem& S = smem[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
@@ -614,11 +618,14 @@ __global__ void __launch_bounds__(kSegWarps * 32, 6) k_shadow(const ShadowParams
 
 // The ranks that shadow rank r's Gaussian are those of smaller distance:
 // bound[r] = the first rank whose distance is >= d_r - bias (at most r).  The
-// depth sort leaves the distances' bit patterns in rank order.
-__global__ void __launch_bounds__(256) k_rank_bound(const float* __restrict__ dist, uint32_t* __restrict__ bound, int n,
-                                                    float bias) {
+// depth sort leaves the distances' bit patterns in rank order.  The ranks' flags
+// are cleared on the way.
+__global__ void __launch_bounds__(256) k_rank_bound(const float* __restrict__ dist, uint32_t* __restrict__ bound,
+                                                    uchar2* __restrict__ flags, int n, float bias) {
+  after_previous();
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= n) return;
+  flags[r] = make_uchar2(0, 0);
   const float thr = __fsub_rn(dist[r], bias);
   uint32_t lo = 0u, hi = (uint32_t)r;
   while (lo < hi) {
@@ -651,13 +658,15 @@ __device__ __forceinline__ int item_level(const uint32_t* lvl_off, uint32_t w) {
   return lo;
 }
 
-// The items' descriptors, and K at the entries the segment plan reads (every
+// The items' descriptors and cleared flags, and K at the entries the segment plan reads (every
 // segment's first entry and every tile's last), one thread per segment,
 // before K6a.
 __global__ void __launch_bounds__(256) k_bound_starts(const ShadowParams p,
                                                       const uint32_t* __restrict__ bound, uint32_t* __restrict__ kb) {
+  after_previous();
   const uint32_t w = blockIdx.x * blockDim.x + threadIdx.x;
   if (w >= p.lvl_off[kSegLevels]) return;
+  p.pub_flag[w] = 0u;
   const int s = item_level(p.lvl_off, w);
   const uint32_t pos = w - p.lvl_off[s];
   const int tile = (int)p.tile_order[pos];
@@ -679,6 +688,7 @@ __global__ void __launch_bounds__(256) k_bound_starts(const ShadowParams p,
 // past the first.
 __global__ void __launch_bounds__(256) k_bound_rest(const ShadowParams p, const uint32_t* __restrict__ bound,
                                                     uint32_t* __restrict__ kb) {
+  after_previous();
   __shared__ uint32_t cnt[2], base[2];
   const uint32_t total = p.lvl_off[kSegLevels];
   if (blockIdx.x * 8u >= total) return;
@@ -719,6 +729,7 @@ __global__ void __launch_bounds__(256) k_shadow_reduce(int n, const uint32_t* __
                                                        const uint32_t* __restrict__ order,
                                                        const uint32_t* header, float* __restrict__ T,
                                                        float* __restrict__ den_out) {
+  after_previous();
   const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 3;
   const int sub = threadIdx.x & 7;
   const bool valid = r < n;
@@ -1016,6 +1027,7 @@ __device__ __forceinline__ void camera_tile(const CamParams& p, int blk, CamSmem
 template <bool BATCH>
 __global__ void __launch_bounds__(kCamThreads) k_camera(const CamParams p, const CamParams* reqs, const uint32_t* tile_prefix,
                                                 int nreq) {
+  after_previous();
   __shared__ CamSmem M[kCamThreads / 32][2];
   if (BATCH) {
     int r = 0;
@@ -1140,6 +1152,7 @@ __global__ void __launch_bounds__(kCamThreads) k_camera_env(const EnvCamParams e
 __global__ void __launch_bounds__(1024) k_tile_order(const uint32_t* __restrict__ tile_start, int ntiles,
                                                      uint32_t* __restrict__ order, uint32_t* __restrict__ lvl_off,
                                                      uint32_t max_items) {
+  after_previous();
   constexpr int kBuckets = 1024;
   __shared__ uint32_t cnt[kBuckets];
   __shared__ uint32_t wsum[32];
@@ -1160,6 +1173,7 @@ __global__ void __launch_bounds__(1024) k_tile_order(const uint32_t* __restrict_
                                  longest > seg_len * (uint32_t)(kSegLevels - 1)))
       seg_len *= 2u;
     if (t == 0) lvl_off[kSegWord] = seg_len;
+    if (t > 0 && t < (int)(kSegWord - kSegLevels)) lvl_off[kSegLevels + t] = 0u;  // the tickets and list counts
   }
   auto bucket = [&](int i) {
     const uint32_t len = tile_start[i + 1] - tile_start[i];
@@ -1212,7 +1226,7 @@ __global__ void __launch_bounds__(1024) k_tile_order(const uint32_t* __restrict_
 void launch_tile_order(const FrameArgs& f, int splat, cudaStream_t s) {
   const Workspace& L = *f.L;
   uint32_t* order = at<uint32_t>(f.ws, L.tile_order[splat]);
-  k_tile_order<<<1, 1024, 0, s>>>(at<uint32_t>(f.ws, L.sp[splat].tile_start), L.ntiles, order, nullptr, 0u);
+  launch_after(k_tile_order, 1, 1024, 0, s, at<uint32_t>(f.ws, L.sp[splat].tile_start), L.ntiles, order, nullptr, 0u);
   count_launch();
 }
 
@@ -1330,17 +1344,15 @@ void prepare_shadow_composite(const FrameArgs& f, cudaStream_t s) {
   uint32_t* kb = at<uint32_t>(ws, b.tv[1 - fin]);
   // the light tiles by segment count, and the work items of each segment level
   uint32_t* lvl = at<uint32_t>(ws, f.L->seg_lvl);
-  cudaMemsetAsync(lvl + kSegLevels + 1, 0, 20, s);  // the tickets and list counts
-  cudaMemsetAsync(at<uint32_t>(ws, f.L->seg_flag), 0, 4 * shadow_seg_items(f.L->ntiles, f.L->cap), s);
-  cudaMemsetAsync(ws + f.L->rank_flags, 0, 2 * (size_t)f.L->n, s);
-  k_tile_order<<<1, 1024, 0, s>>>(at<uint32_t>(ws, b.tile_start), f.L->ntiles, at<uint32_t>(ws, f.L->tile_order[1]),
+  launch_after(k_tile_order, 1, 1024, 0, s, at<uint32_t>(ws, b.tile_start), f.L->ntiles, at<uint32_t>(ws, f.L->tile_order[1]),
                                   lvl, (uint32_t)shadow_seg_items(f.L->ntiles, f.L->cap));
   // the occluder bounds the segment plan reads; the rest follow K6a
   const size_t items = shadow_seg_items(f.L->ntiles, f.L->cap);
   const int n = f.sc.n;
   uint32_t* bound = at<uint32_t>(ws, b.sk[0]);  // free once the depths are sorted
-  k_rank_bound<<<(n + 255) / 256, 256, 0, s>>>(at<float>(ws, b.sk[1]), bound, n, f.opts.shadow_bias);
-  k_bound_starts<<<(int)((items + 255) / 256), 256, 0, s>>>(shadow_params(f), bound, kb);
+  launch_after(k_rank_bound, (n + 255) / 256, 256, 0, s, at<float>(ws, b.sk[1]), bound,
+               at<uchar2>(ws, f.L->rank_flags), n, f.opts.shadow_bias);
+  launch_after(k_bound_starts, (int)((items + 255) / 256), 256, 0, s, shadow_params(f), bound, kb);
   count_launch(3);
 }
 
@@ -1349,7 +1361,7 @@ void launch_bound_rest(const FrameArgs& f, const ShadowParams& p, cudaStream_t s
   const SplatBufs& b = f.L->sp[1];
   const int fin = (f.L->ntiles <= 256 ? 1 : 2) & 1;
   const size_t items = shadow_seg_items(f.L->ntiles, f.L->cap);
-  k_bound_rest<<<(int)((items * 32 + 255) / 256), 256, 0, s>>>(p, at<uint32_t>(f.ws, b.sk[0]),
+  launch_after(k_bound_rest, (int)((items * 32 + 255) / 256), 256, 0, s, p, at<uint32_t>(f.ws, b.sk[0]),
                                                                at<uint32_t>(f.ws, b.tv[1 - fin]));
   count_launch();
 }
@@ -1360,11 +1372,11 @@ void launch_shadow_composite(const FrameArgs& f, cudaStream_t s) {
   const SegOccupancy o = seg_occupancy();
   const int nsm = device_sm_count();
   // persistent warps: every resident warp slot takes segments from a ticket
-  k_shadow_chain<false><<<nsm * o.chain, kSegWarps * 32, 0, s>>>(p, nullptr, 1);
+  launch_after(k_shadow_chain<false>, nsm * o.chain, kSegWarps * 32, 0, s, p, nullptr, 1);
   launch_bound_rest(f, p, s);
-  k_shadow<false><<<nsm * o.live, kSegWarps * 32, 0, s>>>(p, nullptr, 1);
-  k_dead_probe<<<(f.L->n + 255) / 256, 256, 0, s>>>(p, f.L->n);
-  k_shadow_dead<false><<<nsm * o.dead, kDeadWarps * 32, 0, s>>>(p, nullptr, 1);
+  launch_after(k_shadow<false>, nsm * o.live, kSegWarps * 32, 0, s, p, nullptr, 1);
+  launch_after(k_dead_probe, (f.L->n + 255) / 256, 256, 0, s, p, f.L->n);
+  launch_after(k_shadow_dead<false>, nsm * o.dead, kDeadWarps * 32, 0, s, p, nullptr, 1);
   count_launch(4);
 }
 
@@ -1381,7 +1393,7 @@ void launch_shadow_chain_selftest(const FrameArgs& f, cudaStream_t s) {
   const ShadowParams p = shadow_params(f);
   k_skip_first_level<<<1, 32, 0, s>>>(p.lvl_off, p.ticket);
   const SegOccupancy o = seg_occupancy();
-  k_shadow_chain<false><<<device_sm_count() * o.chain, kSegWarps * 32, 0, s>>>(p, nullptr, 1);
+  launch_after(k_shadow_chain<false>, device_sm_count() * o.chain, kSegWarps * 32, 0, s, p, nullptr, 1);
   count_launch(2);
 }
 
@@ -1396,9 +1408,9 @@ void launch_shadow_composite_batch(const FrameArgs* const* f, int n, unsigned ch
   const int nsm = device_sm_count();
   k_shadow_chain<true><<<nsm * o.chain, kSegWarps * 32, 0, s>>>(hp[0], dp, n);
   for (int r = 0; r < n; ++r) launch_bound_rest(*f[r], hp[r], s);
-  k_shadow<true><<<nsm * o.live, kSegWarps * 32, 0, s>>>(hp[0], dp, n);
-  for (int r = 0; r < n; ++r) k_dead_probe<<<(f[r]->L->n + 255) / 256, 256, 0, s>>>(hp[r], f[r]->L->n);
-  k_shadow_dead<true><<<nsm * o.dead, kDeadWarps * 32, 0, s>>>(hp[0], dp, n);
+  launch_after(k_shadow<true>, nsm * o.live, kSegWarps * 32, 0, s, hp[0], dp, n);
+  for (int r = 0; r < n; ++r) launch_after(k_dead_probe, (f[r]->L->n + 255) / 256, 256, 0, s, hp[r], f[r]->L->n);
+  launch_after(k_shadow_dead<true>, nsm * o.dead, kDeadWarps * 32, 0, s, hp[0], dp, n);
   count_launch(2 + n + 1);
 }
 
@@ -1406,8 +1418,7 @@ void launch_shadow_reduce(const FrameArgs& f, cudaStream_t s) {
   const SplatBufs& b = f.L->sp[1];
   unsigned char* ws = f.ws;
   const int n = f.sc.n;
-  k_shadow_reduce<<<(n * 8 + 255) / 256, 256, 0, s>>>(
-      n, at<uint32_t>(ws, b.off), at<uint32_t>(ws, b.cnt), at<float2>(ws, f.L->partial),
+  launch_after(k_shadow_reduce, (n * 8 + 255) / 256, 256, 0, s, n, at<uint32_t>(ws, b.off), at<uint32_t>(ws, b.cnt), at<float2>(ws, f.L->partial),
       at<uchar2>(ws, f.L->rank_flags), at<uint32_t>(ws, b.sv[1]), at<uint32_t>(ws, f.L->header), at<float>(ws, f.L->T),
       at<float>(ws, f.L->shadow_den));
   count_launch();
@@ -1421,8 +1432,10 @@ void launch_fill_shadow_one(const FrameArgs& f, cudaStream_t s) {
   count_launch();
 }
 
-void launch_camera_composite(const FrameArgs& f, float* out_rgb, cudaStream_t s) {
-  k_camera<false><<<f.L->ntiles, kCamThreads, 0, s>>>(camera_params(f, out_rgb), nullptr, nullptr, 1);
+void launch_camera_composite(const FrameArgs& f, float* out_rgb, bool after_mlp, cudaStream_t s) {
+  const CamParams p = camera_params(f, out_rgb);
+  if (after_mlp) launch_after(k_camera<false>, f.L->ntiles, kCamThreads, 0, s, p, nullptr, nullptr, 1);
+  else k_camera<false><<<f.L->ntiles, kCamThreads, 0, s>>>(p, nullptr, nullptr, 1);
   count_launch();
 }
 

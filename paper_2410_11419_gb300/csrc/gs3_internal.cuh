@@ -288,7 +288,8 @@ size_t mlp_tc_scale_offset(const MlpDev& m, int dtype);  // FP8: (sx, sw) per hi
 void pack_mlp_tc(const MlpDev& m, int dtype, const SceneDev& sc, int which, unsigned char* dst, cudaStream_t s);
 bool mlp_tc_supported(const MlpDev& m, int dtype);
 void launch_mlp_tc(const FrameArgs& f, const unsigned char* const blobs[2], cudaStream_t s, int which_mask = 3);
-void launch_camera_composite(const FrameArgs& f, float* out_rgb, cudaStream_t s);
+// after_mlp: the stream's last operation is the networks' last kernel
+void launch_camera_composite(const FrameArgs& f, float* out_rgb, bool after_mlp, cudaStream_t s);
 // camera composite of nl <= kMaxBatch lights over f0's camera splat:
 // out (+)= sum_l w[l] (S_l Sh_l + R), (S_l, Sh_l) per camera rank from envcol
 void launch_camera_env(const FrameArgs& f0, const float4* envcol, int nl, const float* w, bool accumulate,
@@ -340,6 +341,27 @@ struct DeviceOnce {
     return ok;
   }
 };
+
+// A launch whose kernel starts with after_previous(): the grid is set up while
+// the stream's previous kernel drains, and its threads wait there until that
+// kernel has finished and its writes are visible.  Used where the previous
+// operation of the stream is always a kernel.  Between two dependent kernels it
+// takes 0.8 us instead of 1.9.
+template <typename... P, typename... A>
+inline void launch_after(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Streaming multiprocessors of the current device (cudaDevAttrMultiProcessorCount),
 // looked up once per device; grid caps are multiples of it.

@@ -146,6 +146,7 @@ __global__ void __launch_bounds__(kLThreads) k_ssim_grad(const float* __restrict
                                                          const float* __restrict__ dmaps,
                                                          const double* __restrict__ part, float* __restrict__ dimg,
                                                          float* __restrict__ loss, int W, int H, float lambda) {
+  after_previous();
   __shared__ float D[3][kLH][kLRow];
   __shared__ float B[3][kLH][kLT];
   const LossTile T = loss_tile(W, H);
@@ -242,7 +243,7 @@ gs3_status run_loss(const float* img, const float* tgt, int W, int H, float lamb
   double* part = reinterpret_cast<double*>((reinterpret_cast<uintptr_t>(dm + 9 * (size_t)W * H) + 7) & ~uintptr_t(7));
   const unsigned nb = (unsigned)(3 * loss_tiles(W, H));
   k_ssim<<<nb, kLThreads, 0, s>>>(img, tgt, dm, part, W, H);
-  k_ssim_grad<<<nb, kLThreads, 0, s>>>(img, tgt, dm, part, dimg, loss, W, H, lambda);
+  launch_after(k_ssim_grad, nb, kLThreads, 0, s, img, tgt, dm, part, dimg, loss, W, H, lambda);
   count_launch(2);
   return cudaGetLastError() == cudaSuccess ? GS3_OK : GS3_ERR_CUDA;
 }

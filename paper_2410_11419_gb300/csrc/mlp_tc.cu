@@ -177,6 +177,7 @@ __device__ __forceinline__ void tmem_bias(uint32_t lane_addr, const float* b, in
 // the others encode or run their epilogues.  The weights are shared.
 template <int EB, int WHICH>
 __global__ void __launch_bounds__(kTcThreads * kTcMaxGroups, 1) k_mlp_tc(TcParams p) {
+  after_previous();
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ __align__(8) uint64_t bar_w, bar_mma[kTcMaxGroups];
   __shared__ uint32_t tmem_slot;
@@ -540,7 +541,8 @@ TcParams tc_params(const FrameArgs& f, int which, const unsigned char* blob) {
   return p;
 }
 
-void launch_tc(const TcParams& p, const MlpDev& m, int eb, cudaStream_t s) {
+// after: the stream's last operation is a kernel
+void launch_tc(const TcParams& p, const MlpDev& m, int eb, bool after, cudaStream_t s) {
   const int groups = tc_groups(m, eb);
   size_t smem = tc_smem_bytes(m, eb, groups);
   // CTAs of this kernel (of any launch) that share an SM must fit in its 512
@@ -557,7 +559,8 @@ void launch_tc(const TcParams& p, const MlpDev& m, int eb, cudaStream_t s) {
   const int ntiles = (p.n * p.nl + kTcRows - 1) / kTcRows;
   const int ctas = (ntiles + groups - 1) / groups;
   const int grid = ctas < nsm ? ctas : nsm;
-  kern<<<grid, kTcThreads * groups, smem, s>>>(p);
+  if (after) launch_after(kern, grid, kTcThreads * groups, smem, s, p);
+  else kern<<<grid, kTcThreads * groups, smem, s>>>(p);
   count_launch();
 }
 
@@ -565,11 +568,13 @@ void launch_tc(const TcParams& p, const MlpDev& m, int eb, cudaStream_t s) {
 
 void launch_mlp_tc(const FrameArgs& f, const unsigned char* const blobs[2], cudaStream_t s, int which_mask) {
   const int eb = elem_bytes(f.sc.mlp_dtype);
+  bool after = false;
   for (int which = 0; which < 2; ++which) {
     if (!(which_mask & (1 << which))) continue;
     const bool identity = (f.opts.ablate & (which == 0 ? GS3_ABLATE_PHI : GS3_ABLATE_PSI)) != 0;
     if (identity) continue;  // handled by the FP32 kernel's identity path
-    launch_tc(tc_params(f, which, blobs[which]), which == 0 ? f.sc.phi : f.sc.psi, eb, s);
+    launch_tc(tc_params(f, which, blobs[which]), which == 0 ? f.sc.phi : f.sc.psi, eb, after, s);
+    after = true;
   }
 }
 
@@ -585,7 +590,7 @@ void launch_phi_lights_tc(const FrameArgs* const* f, int nl, float4* envcol, con
   }
   p.ccol = nullptr;
   p.envcol = envcol;
-  launch_tc(p, f[0]->sc.phi, elem_bytes(f[0]->sc.mlp_dtype), s);
+  launch_tc(p, f[0]->sc.phi, elem_bytes(f[0]->sc.mlp_dtype), false, s);
 }
 
 }  // namespace gs3

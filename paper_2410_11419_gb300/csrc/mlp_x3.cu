@@ -100,6 +100,7 @@ __host__ __device__ inline uint32_t x3_act_bytes(int W) { return 3u * kRows * 2u
 
 template <int WHICH>
 __global__ void __launch_bounds__(kThreads, 1) k_mlp_x3(X3Params p) {
+  after_previous();
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ __align__(8) uint64_t bar_full[kStages], bar_empty[kStages], bar_a[4], bar_d[2];
   __shared__ uint32_t tmem_slot;
@@ -344,7 +345,7 @@ void launch_net(const X3Params& p, int which, const MlpDev& m, cudaStream_t s) {
     return ok;
   });
   const int ntiles = (p.n * p.nl + kRows - 1) / kRows, nsm = device_sm_count();
-  kern<<<ntiles < nsm ? ntiles : nsm, kThreads, smem, s>>>(p);
+  launch_after(kern, ntiles < nsm ? ntiles : nsm, kThreads, smem, s, p);
   count_launch();
 }
 

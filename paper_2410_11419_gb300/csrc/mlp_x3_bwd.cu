@@ -195,6 +195,7 @@ __device__ __forceinline__ void pe_grad(const float* d, const float (&v)[3], flo
 
 template <int WHICH>
 __global__ void __launch_bounds__(kThreads, 1) k_mlp_x3_rows(RowsParams p) {
+  after_previous();
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ __align__(8) uint64_t bar_full[kStages], bar_empty[kStages], bar_a[4], bar_d[2], bar_z, bar_s;
   __shared__ uint32_t tmem_slot;
@@ -566,6 +567,7 @@ struct WgradParams {
 };
 
 __global__ void __launch_bounds__(kWThreads, 1) k_mlp_x3_wgrad(WgradParams p) {
+  after_previous();
   extern __shared__ __align__(1024) unsigned char sm[];
   __shared__ __align__(16) __nv_bfloat16 ones[256];
   __shared__ __align__(8) uint64_t bar_full[kWStages], bar_empty[kWStages], bar_d, bar_o;
@@ -723,6 +725,7 @@ struct SumParams {
   float* red;
 };
 __global__ void __launch_bounds__(kSumWarps * 32) k_mlp_x3_sum(SumParams p) {
+  after_previous();
   __shared__ float acc[kSumWarps][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
   const bool hidden = i < p.np;
@@ -829,14 +832,14 @@ void run_mlp_x3_backward(const MlpArgs& a, void* scratch, float* wred, cudaStrea
     const int gw = w.ntiles * (kRows / kWRows) < nsm ? w.ntiles * (kRows / kWRows) : nsm;
     r.opart = opart + (size_t)no * P.op;
     w.part = wpart + (size_t)nw * P.np;
-    if (a.which == 0) k_mlp_x3_rows<0><<<gr, kThreads, smem_for_cols(rows_smem(m), 4u * wide(W)), s>>>(r);
-    else k_mlp_x3_rows<1><<<gr, kThreads, smem_for_cols(rows_smem(m), 4u * wide(W)), s>>>(r);
-    k_mlp_x3_wgrad<<<gw, kWThreads, smem_for_cols((size_t)kWStages * wstage_bytes(W), wcols(W)), s>>>(w);
+    if (a.which == 0) launch_after(k_mlp_x3_rows<0>, gr, kThreads, smem_for_cols(rows_smem(m), 4u * wide(W)), s, r);
+    else launch_after(k_mlp_x3_rows<1>, gr, kThreads, smem_for_cols(rows_smem(m), 4u * wide(W)), s, r);
+    launch_after(k_mlp_x3_wgrad, gw, kWThreads, smem_for_cols((size_t)kWStages * wstage_bytes(W), wcols(W)), s, w);
     no += gr;
     nw += gw;
   }
   const SumParams q = {wpart, opart, nw, no, P.np, P.op, W, m.in_dim, wred};
-  k_mlp_x3_sum<<<(P.np + P.op + 31) / 32, kSumWarps * 32, 0, s>>>(q);
+  launch_after(k_mlp_x3_sum, (P.np + P.op + 31) / 32, kSumWarps * 32, 0, s, q);
   count_launch(2 + 2 * P.batches);
 }
 

@@ -160,6 +160,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 6) k_shadow_bwd_sums(const Bwd
 // One warp per tile: seg_sum of each open segment becomes the sum over the
 // tile's later open segments (the open ones are a prefix of the segments).
 __global__ void __launch_bounds__(128) k_shadow_bwd_suffix(const BwdParams p) {
+  after_previous();
   const uint32_t pos = blockIdx.x * 4 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (pos >= (uint32_t)p.ntiles) return;
@@ -398,6 +399,7 @@ __device__ __forceinline__ void bwd_item(const BwdParams& p, uint32_t w, BwdSmem
 }
 
 __global__ void __launch_bounds__(kBwdWarps * 32, 4) k_shadow_bwd(const BwdParams p) {
+  after_previous();
   __shared__ BwdSmem smem[kBwdWarps];
   const int lane = threadIdx.x & 31;
   const uint32_t total = p.counts[0];
@@ -563,8 +565,8 @@ void launch_shadow_backward(const FrameArgs& f, const ShadowBwdArgs& a, cudaStre
   }
   k_shadow_bwd_stopped<<<nsm * o.stopped, kBwdWarps * 32, 0, side>>>(p);
   k_shadow_bwd_sums<<<nsm * o.sums, kBwdWarps * 32, 0, s>>>(p);
-  k_shadow_bwd_suffix<<<(L.ntiles + 3) / 4, 128, 0, s>>>(p);
-  k_shadow_bwd<<<nsm * o.open, kBwdWarps * 32, 0, s>>>(p);
+  launch_after(k_shadow_bwd_suffix, (L.ntiles + 3) / 4, 128, 0, s, p);
+  launch_after(k_shadow_bwd, nsm * o.open, kBwdWarps * 32, 0, s, p);
   count_launch(5);
 }
 

@@ -21,6 +21,7 @@ namespace {
 // block ever waits on another block.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_scan_reduce(const uint32_t* in, uint32_t n, uint32_t* part) {
+  after_previous();
   __shared__ uint32_t red[8];
   const uint32_t base = blockIdx.x * kScanItems;
   uint32_t s = 0;
@@ -41,6 +42,7 @@ __global__ void __launch_bounds__(256) k_scan_reduce(const uint32_t* in, uint32_
 
 // single block: exclusive scan of the block sums, any length
 __global__ void __launch_bounds__(1024) k_scan_part(uint32_t* part, uint32_t nb, uint32_t* total) {
+  after_previous();
   __shared__ uint32_t wsum[32];
   __shared__ uint32_t carry;
   if (threadIdx.x == 0) carry = 0;
@@ -76,6 +78,7 @@ __global__ void __launch_bounds__(1024) k_scan_part(uint32_t* part, uint32_t nb,
 
 __global__ void __launch_bounds__(256) k_scan_down(const uint32_t* in, uint32_t* out, uint32_t n,
                                                    const uint32_t* part) {
+  after_previous();
   __shared__ uint32_t sm[kScanItems];
   __shared__ uint32_t wsum[8];
   const uint32_t base = blockIdx.x * kScanItems;
@@ -211,6 +214,7 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_onesweep(
     const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
     uint32_t* __restrict__ vout, const uint32_t* n_ptr, uint32_t n_fixed, int shift,
     const uint32_t* __restrict__ totals, unsigned long long* look, uint32_t* ticket, uint32_t* header) {
+  after_previous();
   constexpr int kItems = kSortThreads * ROUNDS;
   constexpr int kWarps = kSortThreads / 32;
   extern __shared__ uint4 onesweep_raw[];
@@ -347,6 +351,7 @@ __global__ void __launch_bounds__(kBinBlock) k_reorder(int n, const uint32_t* __
                                                        uint32_t* __restrict__ rank_of, uint32_t* __restrict__ cnt,
                                                        const float4* __restrict__ shade, float4* __restrict__ ccol,
                                                        uint32_t* __restrict__ row_cnt, int gy) {
+  after_previous();
   __shared__ int d[kMaxTileAxis + 1];
   for (int y = threadIdx.x; y <= gy; y += blockDim.x) d[y] = 0;
   __syncthreads();
@@ -413,8 +418,7 @@ void onesweep_sort(const uint32_t* kin, const uint32_t* vin, uint32_t* k0, uint3
   for (int p = 0; p < passes; ++p) {
     uint32_t* ko = (p & 1) ? k1 : k0;
     uint32_t* vo = (p & 1) ? v1 : v0;
-    k_onesweep<ROUNDS><<<nblocks, kSortThreads, sizeof(OnesweepSmem<ROUNDS>), s>>>(
-        ki, vi, ko, vo, n_ptr, n_fixed, 8 * p, totals + 256 * p, look, tickets + p, header);
+    launch_after(k_onesweep<ROUNDS>, nblocks, kSortThreads, sizeof(OnesweepSmem<ROUNDS>), s, ki, vi, ko, vo, n_ptr, n_fixed, 8 * p, totals + 256 * p, look, tickets + p, header);
     ki = ko;
     vi = vo;
   }
@@ -441,9 +445,9 @@ void device_exclusive_scan(const uint32_t* in, uint32_t* out, uint32_t n, uint32
                            uint32_t* scratch, cudaStream_t s) {
   const uint32_t nb = (n + kScanItems - 1) / kScanItems;
   if (nb == 0) return;
-  k_scan_reduce<<<nb, 256, 0, s>>>(in, n, scratch);
-  k_scan_part<<<1, 1024, 0, s>>>(scratch, nb, total);
-  k_scan_down<<<nb, 256, 0, s>>>(in, out, n, scratch);
+  launch_after(k_scan_reduce, nb, 256, 0, s, in, n, scratch);
+  launch_after(k_scan_part, 1, 1024, 0, s, scratch, nb, total);
+  launch_after(k_scan_down, nb, 256, 0, s, in, out, n, scratch);
   count_launch(3);
 }
 
@@ -458,8 +462,7 @@ void launch_depth_sort(const FrameArgs& f, int sp, cudaStream_t s) {
                                      nullptr, (uint32_t)n, f.L->nb_n, 4, at<unsigned char>(ws, b.dlook),
                                      at<uint32_t>(ws, f.L->header), s);
   // 4 passes end in buffer 1: sv[1] holds the index of each depth rank
-  k_reorder<<<f.L->nb_rows, kBinBlock, 0, s>>>(
-      n, at<uint32_t>(ws, b.sv[1]), at<SplatRec>(ws, b.rec), at<SplatRec>(ws, b.rrec),
+  launch_after(k_reorder, f.L->nb_rows, kBinBlock, 0, s, n, at<uint32_t>(ws, b.sv[1]), at<SplatRec>(ws, b.rec), at<SplatRec>(ws, b.rrec),
       at<uint32_t>(ws, b.rank_of), at<uint32_t>(ws, b.cnt), at<float4>(ws, f.L->shade),
       sp == 0 ? at<float4>(ws, f.L->ccol) : nullptr, at<uint32_t>(ws, b.row_cnt), f.L->gy);
   count_launch();

@@ -250,6 +250,7 @@ __device__ __forceinline__ void scan_place(const WarpSpans& S, const uint32_t (&
 // row's total goes to rs[y] for k_bin_plan.
 __global__ void __launch_bounds__(kBinThreads) k_bin_rowtot(uint32_t* __restrict__ row_cnt, int nb, int gy,
                                                             uint32_t* __restrict__ plan) {
+  after_previous();
   __shared__ uint32_t sm[32];
   const int y = blockIdx.x;
   const uint32_t t = block_scan_inplace<kBinThreads>(row_cnt + (size_t)y * nb, (size_t)nb, 0u, sm);
@@ -261,6 +262,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_rowtot(uint32_t* __restrict
 __global__ void __launch_bounds__(1024) k_bin_plan(int gy, uint32_t ch, size_t tab_words, int gx,
                                                   uint32_t* __restrict__ plan, uint32_t* header, int h_need,
                                                   int h_pairs, size_t cap) {
+  after_previous();
   __shared__ uint32_t sm[32];
   BinPlan P(plan, gy);
   const int y = threadIdx.x, lane = y & 31, w = y >> 5;
@@ -308,6 +310,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_rows(int n, const SplatRec*
                                                           const uint32_t* __restrict__ plan,
                                                           uint32_t* __restrict__ rowseq, uint32_t* __restrict__ rowspan,
                                                           size_t cap) {
+  after_previous();
   __shared__ SpanSmem S;
   if (plan[3 * gy + 2] == 0u) return;
   for (int y = threadIdx.x; y < gy; y += kBinThreads) S.run[y] = plan[y] + row_cnt[(size_t)y * nb + blockIdx.x];
@@ -332,6 +335,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_rows_scan(int n, const Spla
                                                                const uint32_t* __restrict__ plan,
                                                                uint32_t* __restrict__ rowseq,
                                                                uint32_t* __restrict__ rowspan, size_t cap) {
+  after_previous();
   if (plan[3 * gy + 2] == 0u) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   WarpSpans S;
@@ -367,6 +371,7 @@ __device__ __forceinline__ void load_chunk(const uint32_t* __restrict__ rowspan,
 __global__ void __launch_bounds__(kBinThreads) k_bin_count_scan(const uint32_t* __restrict__ rowspan,
                                                                 uint32_t* __restrict__ plan, int gx, int gy,
                                                                 uint32_t* __restrict__ tab) {
+  after_previous();
   __shared__ uint32_t pairs[2];  // the chunk's list entries, chunks in turn
   BinPlan P(plan, gy);
   if (*P.ok == 0u) return;
@@ -406,6 +411,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_place_scan(const uint32_t* 
                                                                 const uint32_t* __restrict__ plan,
                                                                 const uint32_t* __restrict__ tab, int gx, int gy,
                                                                 uint32_t* __restrict__ list, size_t cap) {
+  after_previous();
   const uint32_t* rs = plan;
   const uint32_t* cb = plan + gy + 1;
   if (plan[3 * gy + 2] == 0u) return;
@@ -435,6 +441,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_place_scan(const uint32_t* 
 __global__ void __launch_bounds__(kBinThreads) k_bin_count(const uint32_t* __restrict__ rowspan,
                                                            uint32_t* __restrict__ plan, int gx, int gy, uint32_t ch,
                                                            uint32_t* __restrict__ tab) {
+  after_previous();
   __shared__ int d[kMaxTileAxis + 1];
   __shared__ uint32_t sm[32];
   BinPlan P(plan, gy);
@@ -476,6 +483,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_count(const uint32_t* __res
 // of its first chunk.  The last row also writes the end of the last tile.
 __global__ void __launch_bounds__(1024) k_bin_rowscan(uint32_t* __restrict__ tab, const uint32_t* __restrict__ plan,
                                                       int gx, int gy, uint32_t* __restrict__ tile_start) {
+  after_previous();
   __shared__ uint32_t sm[32];
   const int y = blockIdx.x;
   const uint32_t* cb = plan + gy + 1;
@@ -503,6 +511,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_place(const uint32_t* __res
                                                            const uint32_t* __restrict__ plan,
                                                            const uint32_t* __restrict__ tab, int gx, int gy,
                                                            uint32_t ch, uint32_t* __restrict__ list, size_t cap) {
+  after_previous();
   __shared__ SpanSmem S;
   const uint32_t* rs = plan;
   const uint32_t* cb = plan + gy + 1;
@@ -554,22 +563,22 @@ void launch_binning(const FrameArgs& f, int sp, cudaStream_t s) {
   uint32_t* plan = at<uint32_t>(ws, b.bin_plan);
   uint32_t* tab = at<uint32_t>(ws, b.bin_tab);
   const uint32_t ch = bin_chunk(gx);
-  k_bin_rowtot<<<gy, kBinThreads, 0, s>>>(row_cnt, nb, gy, plan);
-  k_bin_plan<<<1, 1024, 0, s>>>(gy, ch, bin_tab_words(cap, gx, gy), gx, plan, header, h_need, h_pairs, cap);
+  launch_after(k_bin_rowtot, gy, kBinThreads, 0, s, row_cnt, nb, gy, plan);
+  launch_after(k_bin_plan, 1, 1024, 0, s, gy, ch, bin_tab_words(cap, gx, gy), gx, plan, header, h_need, h_pairs, cap);
   const SplatRec* rrec = at<SplatRec>(ws, b.rrec);
   if (gy <= kScanBuckets)
-    k_bin_rows_scan<<<nb, kBinThreads, 0, s>>>(n, rrec, row_cnt, nb, gy, plan, rowseq, rowspan, cap);
+    launch_after(k_bin_rows_scan, nb, kBinThreads, 0, s, n, rrec, row_cnt, nb, gy, plan, rowseq, rowspan, cap);
   else
-    k_bin_rows<<<nb, kBinThreads, 0, s>>>(n, rrec, row_cnt, nb, gy, plan, rowseq, rowspan, cap);
+    launch_after(k_bin_rows, nb, kBinThreads, 0, s, n, rrec, row_cnt, nb, gy, plan, rowseq, rowspan, cap);
   const size_t chunks = cap / ch + (size_t)gy + 1;
   const bool scan = gx <= kScanBuckets;  // chunks of 256 items
   int grid = device_sm_count() * (scan ? 8 : 5);
   if ((size_t)grid > chunks) grid = (int)chunks;
-  if (scan) k_bin_count_scan<<<grid, kBinThreads, 0, s>>>(rowspan, plan, gx, gy, tab);
-  else k_bin_count<<<grid, kBinThreads, 0, s>>>(rowspan, plan, gx, gy, ch, tab);
-  k_bin_rowscan<<<gy, 1024, 0, s>>>(tab, plan, gx, gy, at<uint32_t>(ws, b.tile_start));
-  if (scan) k_bin_place_scan<<<grid, kBinThreads, 0, s>>>(rowseq, rowspan, plan, tab, gx, gy, list, cap);
-  else k_bin_place<<<grid, kBinThreads, 0, s>>>(rowseq, rowspan, plan, tab, gx, gy, ch, list, cap);
+  if (scan) launch_after(k_bin_count_scan, grid, kBinThreads, 0, s, rowspan, plan, gx, gy, tab);
+  else launch_after(k_bin_count, grid, kBinThreads, 0, s, rowspan, plan, gx, gy, ch, tab);
+  launch_after(k_bin_rowscan, gy, 1024, 0, s, tab, plan, gx, gy, at<uint32_t>(ws, b.tile_start));
+  if (scan) launch_after(k_bin_place_scan, grid, kBinThreads, 0, s, rowseq, rowspan, plan, tab, gx, gy, list, cap);
+  else launch_after(k_bin_place, grid, kBinThreads, 0, s, rowseq, rowspan, plan, tab, gx, gy, ch, list, cap);
   count_launch(6);
 }
 
