@@ -27,7 +27,6 @@ inline size_t bin_tab_words(size_t cap, int gx, int gy) {
 }
 constexpr int kDepthSortRounds = 4;   // the per-splat depth sort: 1024 keys per block
 constexpr int kDepthSortItems = kSortThreads * kDepthSortRounds;
-constexpr int kScanItems = 4096;      // items per block in the device-wide scan
 constexpr int kMaxLobes = 16;
 
 // Per-Gaussian splat record (one per splat, by Gaussian index or by rank).
@@ -56,10 +55,9 @@ struct SplatBufs {
   size_t off;           // u32[N] exclusive prefix of cnt
   size_t tk[2], tv[2];  // u32[cap] each: tv[fin] the tile lists, tk[fin] the row sequence, the rest scratch
   size_t tile_start;    // u32[ntiles + 1]
-  size_t scan_part;     // u32 partial sums of the device-wide scan
   size_t dlook;         // depth sort's look-back region, onesweep_bytes(nb_n, 4)
-  size_t row_cnt;       // u32[gy][nb_rows]: ranks per (tile row, block of kBinBlock ranks), then scanned
-  size_t bin_plan;      // u32[3 gy + 3]: row starts, chunk starts, pairs per row, capacity flag
+  size_t row_cnt;       // u32[gy + 1][nb_rows]: ranks per (tile row, block of kBinBlock ranks), and the blocks' pairs; then scanned
+  size_t bin_plan;      // u32[3 gy + 4]: row starts, chunk starts, pairs per row, capacity flag, ticket
   size_t bin_tab;       // u32[bin_tab_words]: list entries per (row, column, chunk), then scanned per row
 };
 
@@ -295,12 +293,6 @@ void launch_camera_composite(const FrameArgs& f, float* out_rgb, bool after_mlp,
 void launch_camera_env(const FrameArgs& f0, const float4* envcol, int nl, const float* w, bool accumulate,
                        float* out_rgb, cudaStream_t s);
 void launch_fill_shadow_one(const FrameArgs& f, cudaStream_t s);
-
-// exclusive scan of n u32 values (in place allowed: out may equal in);
-// the total goes to *total if non-null
-void device_exclusive_scan(const uint32_t* in, uint32_t* out, uint32_t n, uint32_t* total,
-                           uint32_t* scratch, cudaStream_t s);
-size_t scan_scratch_words(size_t n);
 
 // bytes of a look-back sort's region: u64[256 * nblocks] look-back words (every
 // pass's in turn), u32 tickets[passes], u32 totals[passes][256]

@@ -17,108 +17,6 @@ namespace gs3 {
 namespace {
 
 // ---------------------------------------------------------------------------
-// Device-wide exclusive scan: reduce, scan of block sums, down-sweep.  No
-// block ever waits on another block.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_scan_reduce(const uint32_t* in, uint32_t n, uint32_t* part) {
-  after_previous();
-  __shared__ uint32_t red[8];
-  const uint32_t base = blockIdx.x * kScanItems;
-  uint32_t s = 0;
-#pragma unroll 4
-  for (int r = 0; r < kScanItems / 256; ++r) {
-    uint32_t i = base + r * 256 + threadIdx.x;
-    if (i < n) s += in[i];
-  }
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t t = 0;
-    for (int w = 0; w < 8; ++w) t += red[w];
-    part[blockIdx.x] = t;
-  }
-}
-
-// single block: exclusive scan of the block sums, any length
-__global__ void __launch_bounds__(1024) k_scan_part(uint32_t* part, uint32_t nb, uint32_t* total) {
-  after_previous();
-  __shared__ uint32_t wsum[32];
-  __shared__ uint32_t carry;
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (uint32_t base = 0; base < nb; base += 1024) {
-    uint32_t i = base + threadIdx.x;
-    uint32_t v = i < nb ? part[i] : 0;
-    uint32_t x = v;
-    for (int o = 1; o < 32; o <<= 1) {
-      uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) wsum[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-      uint32_t w = wsum[lane];
-      for (int o = 1; o < 32; o <<= 1) {
-        uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
-        if (lane >= o) w += y;
-      }
-      wsum[lane] = w;
-    }
-    __syncthreads();
-    uint32_t incl = x + (warp ? wsum[warp - 1] : 0u);
-    if (i < nb) part[i] = carry + incl - v;
-    __syncthreads();
-    if (threadIdx.x == 1023) carry += incl;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0 && total) *total = carry;
-}
-
-__global__ void __launch_bounds__(256) k_scan_down(const uint32_t* in, uint32_t* out, uint32_t n,
-                                                   const uint32_t* part) {
-  after_previous();
-  __shared__ uint32_t sm[kScanItems];
-  __shared__ uint32_t wsum[8];
-  const uint32_t base = blockIdx.x * kScanItems;
-  for (int r = 0; r < kScanItems / 256; ++r) {
-    uint32_t i = base + r * 256 + threadIdx.x;
-    sm[r * 256 + threadIdx.x] = i < n ? in[i] : 0u;
-  }
-  __syncthreads();
-  constexpr int per = kScanItems / 256;  // 16 consecutive items per thread
-  uint32_t loc[per];
-  uint32_t s = 0;
-#pragma unroll
-  for (int j = 0; j < per; ++j) {
-    loc[j] = s;
-    s += sm[threadIdx.x * per + j];
-  }
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t x = s;
-  for (int o = 1; o < 32; o <<= 1) {
-    uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  if (lane == 31) wsum[warp] = x;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t a = 0;
-    for (int w = 0; w < 8; ++w) { uint32_t t = wsum[w]; wsum[w] = a; a += t; }
-  }
-  __syncthreads();
-  const uint32_t off = part[blockIdx.x] + wsum[warp] + (x - s);
-#pragma unroll
-  for (int j = 0; j < per; ++j) sm[threadIdx.x * per + j] = off + loc[j];
-  __syncthreads();
-  for (int r = 0; r < kScanItems / 256; ++r) {
-    uint32_t i = base + r * 256 + threadIdx.x;
-    if (i < n) out[i] = sm[r * 256 + threadIdx.x];
-  }
-}
-
-// ---------------------------------------------------------------------------
 // Stable LSD radix sort pass, 8-bit digit, u32 key + u32 value.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t load_n(const uint32_t* n_ptr, uint32_t n_fixed) {
@@ -345,34 +243,45 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_onesweep(
 // Records into depth-rank order and the tile count of each rank.  Also
 // counts, for the block's kBinBlock ranks, the ranks whose rectangle covers
 // each tile row y (a difference array over the rows, then its running sum),
-// into row_cnt[y][block].
+// into row_cnt[y][block], and adds up the block's tile counts into
+// row_cnt[gy][block].  Clears the binning's ticket (the plan's last word).
 __global__ void __launch_bounds__(kBinBlock) k_reorder(int n, const uint32_t* __restrict__ order,
                                                        const SplatRec* __restrict__ rec, SplatRec* __restrict__ rrec,
                                                        uint32_t* __restrict__ rank_of, uint32_t* __restrict__ cnt,
                                                        const float4* __restrict__ shade, float4* __restrict__ ccol,
-                                                       uint32_t* __restrict__ row_cnt, int gy) {
+                                                       uint32_t* __restrict__ row_cnt, int gy, uint32_t* __restrict__ ticket) {
   after_previous();
   __shared__ int d[kMaxTileAxis + 1];
+  __shared__ uint32_t tiles;
+  if (threadIdx.x == 0) {
+    tiles = 0u;
+    if (blockIdx.x == 0) *ticket = 0u;
+  }
   for (int y = threadIdx.x; y <= gy; y += blockDim.x) d[y] = 0;
   __syncthreads();
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   const uint32_t g = r < n ? order[r] : 0xFFFFFFFFu;
+  uint32_t c = 0u;  // the rank's tiles
   if (g < (uint32_t)n) {
     const SplatRec q = rec[g];
     rrec[r] = q;
     rank_of[g] = r;
     const bool in = q.r.x >= 0;
-    cnt[r] = in ? (uint32_t)(q.r.z - q.r.x + 1) * (uint32_t)(q.r.w - q.r.y + 1) : 0u;
+    c = in ? (uint32_t)(q.r.z - q.r.x + 1) * (uint32_t)(q.r.w - q.r.y + 1) : 0u;
+    cnt[r] = c;
     if (in) {
       atomicAdd(&d[q.r.y], 1);
       atomicAdd(&d[q.r.w + 1], -1);
     }
     if (ccol) {
-      float4 c = shade[g];
-      ccol[2 * r] = make_float4(c.x, c.y, c.z, 0.f);
+      const float4 col = shade[g];
+      ccol[2 * r] = make_float4(col.x, col.y, col.z, 0.f);
     }
   }
+  c = __reduce_add_sync(0xffffffffu, c);
+  if ((threadIdx.x & 31) == 0 && c) atomicAdd(&tiles, c);
   __syncthreads();
+  if (threadIdx.x == 32) row_cnt[(size_t)gy * gridDim.x + blockIdx.x] = tiles;
   if (threadIdx.x < 32) {
     const int lane = threadIdx.x;
     int run = 0;
@@ -427,8 +336,6 @@ void onesweep_sort(const uint32_t* kin, const uint32_t* vin, uint32_t* k0, uint3
 
 }  // namespace
 
-size_t scan_scratch_words(size_t n) { return (n + kScanItems - 1) / kScanItems + 1; }
-
 // gs3_depth_order_static: 1024 keys per block up to 512 blocks, 2048 past that
 // (GS3_STATIC_SORT_MAX_KEYS is 512 such blocks), so that a few hundred thousand
 // keys fill the chip and the look-back region stays at 1 MB.
@@ -439,16 +346,6 @@ void depth_order(const uint32_t* keys, uint32_t n, uint32_t* k0, uint32_t* v0, u
     onesweep_sort<4, 4>(keys, nullptr, k0, v0, k1, order, nullptr, n, blocks(4), 4, look_region, status, s);
   else
     onesweep_sort<8, 4>(keys, nullptr, k0, v0, k1, order, nullptr, n, blocks(8), 4, look_region, status, s);
-}
-
-void device_exclusive_scan(const uint32_t* in, uint32_t* out, uint32_t n, uint32_t* total,
-                           uint32_t* scratch, cudaStream_t s) {
-  const uint32_t nb = (n + kScanItems - 1) / kScanItems;
-  if (nb == 0) return;
-  launch_after(k_scan_reduce, nb, 256, 0, s, in, n, scratch);
-  launch_after(k_scan_part, 1, 1024, 0, s, scratch, nb, total);
-  launch_after(k_scan_down, nb, 256, 0, s, in, out, n, scratch);
-  count_launch(3);
 }
 
 void launch_depth_sort(const FrameArgs& f, int sp, cudaStream_t s) {
@@ -464,7 +361,8 @@ void launch_depth_sort(const FrameArgs& f, int sp, cudaStream_t s) {
   // 4 passes end in buffer 1: sv[1] holds the index of each depth rank
   launch_after(k_reorder, f.L->nb_rows, kBinBlock, 0, s, n, at<uint32_t>(ws, b.sv[1]), at<SplatRec>(ws, b.rec), at<SplatRec>(ws, b.rrec),
       at<uint32_t>(ws, b.rank_of), at<uint32_t>(ws, b.cnt), at<float4>(ws, f.L->shade),
-      sp == 0 ? at<float4>(ws, f.L->ccol) : nullptr, at<uint32_t>(ws, b.row_cnt), f.L->gy);
+      sp == 0 ? at<float4>(ws, f.L->ccol) : nullptr, at<uint32_t>(ws, b.row_cnt), f.L->gy,
+               at<uint32_t>(ws, b.bin_plan) + 3 * f.L->gy + 3);
   count_launch();
 }
 

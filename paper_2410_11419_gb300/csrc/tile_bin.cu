@@ -8,8 +8,8 @@
 // emitting the pairs and sorting them on the tile bits:
 //   rows     the ranks covering tile row y, for every y, in rank order, with
 //            each rank's column span beside it: the counts per (row, block
-//            of kBinBlock ranks) come from k_reorder; k_bin_rowtot scans each
-//            row's counts, k_bin_plan the row totals; k_bin_rows places;
+//            of kBinBlock ranks) come from k_reorder; k_bin_plan scans each
+//            row's counts and the row totals; k_bin_rows places;
 //   columns  each row's sequence is cut into chunks of bin_chunk(gx) items;
 //            k_bin_count counts the items per (row, column, chunk);
 //            k_bin_rowscan scans each row's counts in (column, chunk) order,
@@ -20,7 +20,7 @@
 // (scan_place): a warp holds 256 items, eight per lane, and for every bucket
 // it owns asks which of them cover it (a ballot per 32 items), which gives the
 // bucket's entries in item order, side by side in memory, without shared
-// memory or barriers.  That is 64 instructions per bucket and 256 items
+// memory or barriers (the counts come from difference arrays).  That is 64 instructions per bucket and 256 items
 // whatever the spans, so past that many buckets it loses to going over the
 // (item, bucket) pairs (place_spans), about 4.6 instructions each: 256 items,
 // one per thread; a warp's offset in bucket x is the bucket's running offset
@@ -31,11 +31,10 @@
 // stable sort of the pairs by tile would give, and no step depends on timing
 // or waits on another block.
 // Bound: the scattered 4-byte stores of the list (a bucket's run of 256 items
-// holds about 36 entries) and the ballots.  Rows + counts + placement of both
-// splats, beside the shadow composite (over the pairs, the light splat also
-// writing each entry's distance, -> over the buckets): 300k Gaussians at
-// 800 x 800 0.06 + 0.12 + 0.26 -> 0.04 + 0.08 + 0.14 ms, 1 M at 1024 x 1024
-// 0.19 + 0.54 + 1.57 -> 0.11 + 0.38 + 0.70 ms.
+// holds about 36 entries) and the ballots.  Rows + counts + placement of the
+// camera splat alone, 300k Gaussians at 800 x 800: 19 + 9 + 68 us; of both splats
+// beside the shadow composite, 1 M at 1024 x 1024: 0.13 + 0.13 + 0.83 ms, where
+// all three over the pairs take 0.19 + 0.54 + 1.57.
 #include <climits>
 
 #include "gs3_internal.cuh"
@@ -107,10 +106,11 @@ __device__ uint32_t block_sum(uint32_t x, uint32_t* sm) {
 
 // The plan words: rs[gy + 1] row starts in the row sequence, cb[gy + 1]
 // chunk starts (every row has at least one chunk), pairs[gy] list entries
-// per row, ok (the pairs fit the capacity).
+// per row, ok (the pairs fit the capacity), ticket (cleared by k_reorder).
 struct BinPlan {
-  uint32_t *rs, *cb, *pairs, *ok;
-  __device__ BinPlan(uint32_t* p, int gy) : rs(p), cb(p + gy + 1), pairs(p + 2 * gy + 2), ok(p + 3 * gy + 2) {}
+  uint32_t *rs, *cb, *pairs, *ok, *ticket;
+  __device__ BinPlan(uint32_t* p, int gy)
+      : rs(p), cb(p + gy + 1), pairs(p + 2 * gy + 2), ok(p + 3 * gy + 2), ticket(p + 3 * gy + 3) {}
 };
 
 // the row of chunk kg: the largest y with cb[y] <= kg (cb[0] = 0 <= kg < cb[gy])
@@ -246,55 +246,49 @@ __device__ __forceinline__ void scan_place(const WarpSpans& S, const uint32_t (&
   }
 }
 
-// Each row's block counts scanned in place (exclusive, within the row); the
-// row's total goes to rs[y] for k_bin_plan.
-__global__ void __launch_bounds__(kBinThreads) k_bin_rowtot(uint32_t* __restrict__ row_cnt, int nb, int gy,
-                                                            uint32_t* __restrict__ plan) {
+// Blocks y < gy: the row's block counts scanned in place (exclusive, within the
+// row), its total to rs[y]; block gy: the blocks' pairs likewise (every rank's
+// first list slot starts there).  The last block to finish makes the plan, four
+// rows per thread (gy <= 1024): row starts from the row totals, chunks per row and
+// their starts, and the capacity check.  No block waits for another.
+// Bound: launches; with the ranks' slots scanned by k_bin_rows this is one kernel
+// where a scan of all ranks, this scan and the plan were five.
+__global__ void __launch_bounds__(kBinThreads) k_bin_plan(uint32_t* __restrict__ row_cnt, int nb, int gy, uint32_t ch,
+                                                          size_t tab_words, int gx, uint32_t* __restrict__ plan,
+                                                          uint32_t* header, int h_need, int h_pairs, size_t cap) {
   after_previous();
   __shared__ uint32_t sm[32];
-  const int y = blockIdx.x;
-  const uint32_t t = block_scan_inplace<kBinThreads>(row_cnt + (size_t)y * nb, (size_t)nb, 0u, sm);
-  if (threadIdx.x == 0) plan[y] = t;
-}
-
-// One block of 1024 threads (gy <= 1024, one row per thread): row starts from
-// the row totals, chunks per row and their starts, and the capacity check.
-__global__ void __launch_bounds__(1024) k_bin_plan(int gy, uint32_t ch, size_t tab_words, int gx,
-                                                  uint32_t* __restrict__ plan, uint32_t* header, int h_need,
-                                                  int h_pairs, size_t cap) {
-  after_previous();
-  __shared__ uint32_t sm[32];
+  __shared__ uint32_t rows[kMaxTileAxis], chunks[kMaxTileAxis];
+  __shared__ bool last;
   BinPlan P(plan, gy);
-  const int y = threadIdx.x, lane = y & 31, w = y >> 5;
-  const uint32_t m = y < gy ? P.rs[y] : 0u;  // the row's total
-  const uint32_t c = (uint32_t)(((uint64_t)m + ch - 1) / ch);
-  const uint32_t nch = y < gy ? (c > 1u ? c : 1u) : 0u;
-  // exclusive prefixes of (m, nch) over the rows
-  const uint32_t im = warp_inclusive_sum(m, lane), ic = warp_inclusive_sum(nch, lane);
-  if (lane == 31) sm[w] = im;
-  __syncthreads();
-  const uint32_t wm = w == 0 ? warp_inclusive_sum(sm[lane], lane) : 0u;
-  __syncthreads();
-  if (w == 0) sm[lane] = wm;
-  __syncthreads();
-  const uint32_t rs = (w ? sm[w - 1] : 0u) + im - m, M = sm[31];
-  __syncthreads();
-  if (lane == 31) sm[w] = ic;
-  __syncthreads();
-  const uint32_t wc = w == 0 ? warp_inclusive_sum(sm[lane], lane) : 0u;
-  __syncthreads();
-  if (w == 0) sm[lane] = wc;
-  __syncthreads();
-  const uint32_t cb = (w ? sm[w - 1] : 0u) + ic - nch, C = sm[31];
-  if (y < gy) {
-    P.rs[y] = rs;
-    P.cb[y] = cb;
-    P.pairs[y] = 0u;
+  const int y = blockIdx.x, t = threadIdx.x;
+  const uint32_t total = block_scan_inplace<kBinThreads>(row_cnt + (size_t)y * nb, (size_t)nb, 0u, sm);
+  if (t == 0) {
+    if (y < gy) P.rs[y] = total;
+    else header[h_need] = total;
+    __threadfence();
+    last = atomicAdd(P.ticket, 1u) == (uint32_t)gy;
   }
-  if (y == 0) {
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int i = t; i < gy; i += kBinThreads) {
+    const uint32_t m = __ldcg(P.rs + i), c = (uint32_t)(((uint64_t)m + ch - 1) / ch);
+    rows[i] = m;
+    chunks[i] = c > 1u ? c : 1u;
+    P.pairs[i] = 0u;
+  }
+  __syncthreads();
+  const uint32_t M = block_scan_inplace<kBinThreads>(rows, (size_t)gy, 0u, sm);
+  const uint32_t C = block_scan_inplace<kBinThreads>(chunks, (size_t)gy, 0u, sm);
+  for (int i = t; i < gy; i += kBinThreads) {
+    P.rs[i] = rows[i];
+    P.cb[i] = chunks[i];
+  }
+  if (t == 0) {
     P.rs[gy] = M;
     P.cb[gy] = C;
-    const uint32_t need = header[h_need];
+    const uint32_t need = __ldcg(header + h_need);
     const bool ok = need <= cap && (size_t)C * (size_t)gx <= tab_words;
     header[h_pairs] = ok ? need : 0u;
     if (!ok) atomicCAS(&header[H_STATUS], 0u, (uint32_t)GS3_ERR_CAPACITY);
@@ -302,30 +296,43 @@ __global__ void __launch_bounds__(1024) k_bin_plan(int gy, uint32_t ch, size_t t
   }
 }
 
+__device__ __forceinline__ uint32_t tiles_of(int4 q) {
+  return q.x >= 0 ? (uint32_t)(q.z - q.x + 1) * (uint32_t)(q.w - q.y + 1) : 0u;
+}
+
 // The row sequence: the block's 256 ranks over their rows, each copy with the
 // rank's column span (x0 | x1 << 16) beside it; row y's offset for this block
-// is the row's start plus the row's counts of the blocks before.
+// is the row's start plus the row's counts of the blocks before.  Also off[r], rank r's
+// first slot among all pairs in rank order (the shadow partials' slots).
 __global__ void __launch_bounds__(kBinThreads) k_bin_rows(int n, const SplatRec* __restrict__ rrec,
                                                           const uint32_t* __restrict__ row_cnt, int nb, int gy,
                                                           const uint32_t* __restrict__ plan,
                                                           uint32_t* __restrict__ rowseq, uint32_t* __restrict__ rowspan,
-                                                          size_t cap) {
+                                                          uint32_t* __restrict__ off, size_t cap) {
   after_previous();
   __shared__ SpanSmem S;
-  if (plan[3 * gy + 2] == 0u) return;
+  __shared__ uint32_t sm[kBinWarps];
   for (int y = threadIdx.x; y < gy; y += kBinThreads) S.run[y] = plan[y] + row_cnt[(size_t)y * nb + blockIdx.x];
   const int r = blockIdx.x * kBinThreads + threadIdx.x;
   int a = 0, b = -1;
-  uint32_t span = 0;
+  uint32_t span = 0, c = 0;
   if (r < n) {
     const int4 q = rrec[r].r;
+    c = tiles_of(q);
     if (q.x >= 0) {
       a = q.y;
       b = q.w;
       span = (uint32_t)q.x | ((uint32_t)q.z << 16);
     }
   }
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint32_t inc = warp_inclusive_sum(c, lane);
+  if (lane == 31) sm[w] = inc;
   __syncthreads();
+  uint32_t slot = row_cnt[(size_t)gy * nb + blockIdx.x] + inc - c;
+  for (int k = 0; k < w; ++k) slot += sm[k];
+  if (r < n) off[r] = slot;
+  if (plan[3 * gy + 2] == 0u) return;
   place_spans(S, gy, a, b, (uint32_t)r, span, rowseq, rowspan, cap);
 }
 
@@ -334,22 +341,29 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_rows_scan(int n, const Spla
                                                                const uint32_t* __restrict__ row_cnt, int nb, int gy,
                                                                const uint32_t* __restrict__ plan,
                                                                uint32_t* __restrict__ rowseq,
-                                                               uint32_t* __restrict__ rowspan, size_t cap) {
+                                                               uint32_t* __restrict__ rowspan,
+                                                               uint32_t* __restrict__ off, size_t cap) {
   after_previous();
-  if (plan[3 * gy + 2] == 0u) return;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   WarpSpans S;
   uint32_t span[8];
+  uint32_t slot = row_cnt[(size_t)gy * nb + blockIdx.x], own = 0u;  // warp w takes the slots of ranks 32 w ..
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
     const int r = blockIdx.x * kBinThreads + 32 * c + lane;
     int4 q = make_int4(-1, 0, 0, 0);
     if (r < n) q = rrec[r].r;
+    const uint32_t tiles = tiles_of(q);
+    if (c < w) slot += __reduce_add_sync(0xffffffffu, tiles);
+    if (c == w) own = tiles;
     S.lo[c] = q.x >= 0 ? (uint32_t)q.y : kNoSpan;
     S.wid[c] = q.x >= 0 ? (uint32_t)(q.w - q.y) : 0u;
     S.v0[c] = (uint32_t)r;
     span[c] = (uint32_t)q.x | ((uint32_t)q.z << 16);
   }
+  slot += warp_inclusive_sum(own, lane) - own;
+  if (blockIdx.x * kBinThreads + 32 * w + lane < n) off[blockIdx.x * kBinThreads + 32 * w + lane] = slot;
+  if (plan[3 * gy + 2] == 0u) return;
   const int y = w + kBinWarps * lane;
   const uint32_t base = y < gy ? plan[y] + row_cnt[(size_t)y * nb + blockIdx.x] : 0u;
   scan_place<true>(S, span, gy, w, kBinWarps, base, rowseq, rowspan, cap);
@@ -367,41 +381,50 @@ __device__ __forceinline__ void load_chunk(const uint32_t* __restrict__ rowspan,
   }
 }
 
-// k_bin_count going over the columns (gx <= kScanBuckets, chunks of 256).
-__global__ void __launch_bounds__(kBinThreads) k_bin_count_scan(const uint32_t* __restrict__ rowspan,
+// k_bin_count for chunks of 256 (gx <= kScanBuckets), a warp per chunk: the
+// difference array takes two shared-memory adds per item where a ballot per 32
+// items and column took three instructions.  Camera of 300k Gaussians at
+// 800 x 800: 35 -> 9 us.
+__global__ void __launch_bounds__(kBinThreads) k_bin_count_warp(const uint32_t* __restrict__ rowspan,
                                                                 uint32_t* __restrict__ plan, int gx, int gy,
                                                                 uint32_t* __restrict__ tab) {
   after_previous();
-  __shared__ uint32_t pairs[2];  // the chunk's list entries, chunks in turn
+  __shared__ int diff[kBinWarps][kScanBuckets + 1];
   BinPlan P(plan, gy);
   if (*P.ok == 0u) return;
   const uint32_t C = P.cb[gy];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (threadIdx.x < 2) pairs[threadIdx.x] = 0u;
-  __syncthreads();
-  int turn = 0;
-  for (uint32_t kg = blockIdx.x; kg < C; kg += gridDim.x, turn ^= 1) {
+  int* d = diff[w];
+  for (uint32_t kg = blockIdx.x * kBinWarps + w; kg < C; kg += gridDim.x * kBinWarps) {
     const int y = chunk_row(P.cb, gy, kg);
     const uint32_t c0 = P.cb[y], nch = P.cb[y + 1] - c0, k = kg - c0;
     const uint32_t i0 = P.rs[y] + 256u * k, i1 = min(P.rs[y + 1], i0 + 256u);
-    WarpSpans S;
-    load_chunk(rowspan, i0, i1, lane, S);
-    uint32_t mine = 0u, total = 0u;  // lane l keeps the count of column w + 8 l
-    for (int x = w, l = 0; x < gx; x += kBinWarps, ++l) {
-      uint32_t n = 0u;
+    for (int x = lane; x <= gx; x += 32) d[x] = 0;
+    __syncwarp();
+    uint32_t total = 0u;
 #pragma unroll
-      for (int c = 0; c < 8; ++c) n += (uint32_t)__popc(__ballot_sync(0xffffffffu, (uint32_t)x - S.lo[c] <= S.wid[c]));
-      if (lane == l) mine = n;
-      total += n;
+    for (int c = 0; c < 8; ++c) {
+      const uint32_t i = i0 + 32 * c + lane;
+      if (i < i1) {
+        const uint32_t sp = rowspan[i];
+        const int x0 = (int)(sp & 0xFFFFu), x1 = (int)(sp >> 16);
+        atomicAdd(&d[x0], 1);
+        atomicAdd(&d[x1 + 1], -1);
+        total += (uint32_t)(x1 - x0 + 1);
+      }
     }
-    const int x = w + kBinWarps * lane;
-    if (x < gx) tab[(size_t)c0 * gx + (size_t)x * nch + k] = mine;
-    if (lane == 0 && total) atomicAdd(&pairs[turn], total);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      if (pairs[turn]) atomicAdd(P.pairs + y, pairs[turn]);
-      pairs[turn] = 0u;  // used again after the next chunk's barrier
+    __syncwarp();
+    uint32_t* out = tab + (size_t)c0 * gx + k;
+    uint32_t run = 0u;
+    for (int x0 = 0; x0 < gx; x0 += 32) {
+      const int x = x0 + lane;
+      const uint32_t v = warp_inclusive_sum(x < gx ? (uint32_t)d[x] : 0u, lane);
+      if (x < gx) out[(size_t)x * nch] = run + v;
+      run += __shfl_sync(0xffffffffu, v, 31);
     }
+    total = __reduce_add_sync(0xffffffffu, total);
+    if (lane == 0 && total) atomicAdd(P.pairs + y, total);
+    __syncwarp();  // d is cleared for the next chunk
   }
 }
 
@@ -550,9 +573,6 @@ void launch_binning(const FrameArgs& f, int sp, cudaStream_t s) {
   uint32_t* header = at<uint32_t>(ws, f.L->header);
   const int h_need = sp ? H_NEED_LIGHT : H_NEED_CAM;
   const int h_pairs = sp ? H_PAIRS_LIGHT : H_PAIRS_CAM;
-  // every rank's first list slot in rank order (the shadow partials' slots) and the total
-  device_exclusive_scan(at<uint32_t>(ws, b.cnt), at<uint32_t>(ws, b.off), (uint32_t)n, header + h_need,
-                        at<uint32_t>(ws, b.scan_part), s);
   // the lists go where the composites and the backward read them; the row
   // sequence and spans use buffers that are free until then
   const int fin = (f.L->ntiles <= 256 ? 1 : 2) & 1;
@@ -563,23 +583,25 @@ void launch_binning(const FrameArgs& f, int sp, cudaStream_t s) {
   uint32_t* plan = at<uint32_t>(ws, b.bin_plan);
   uint32_t* tab = at<uint32_t>(ws, b.bin_tab);
   const uint32_t ch = bin_chunk(gx);
-  launch_after(k_bin_rowtot, gy, kBinThreads, 0, s, row_cnt, nb, gy, plan);
-  launch_after(k_bin_plan, 1, 1024, 0, s, gy, ch, bin_tab_words(cap, gx, gy), gx, plan, header, h_need, h_pairs, cap);
+  launch_after(k_bin_plan, gy + 1, kBinThreads, 0, s, row_cnt, nb, gy, ch, bin_tab_words(cap, gx, gy), gx, plan, header,
+               h_need, h_pairs, cap);
+  uint32_t* off = at<uint32_t>(ws, b.off);
   const SplatRec* rrec = at<SplatRec>(ws, b.rrec);
   if (gy <= kScanBuckets)
-    launch_after(k_bin_rows_scan, nb, kBinThreads, 0, s, n, rrec, row_cnt, nb, gy, plan, rowseq, rowspan, cap);
+    launch_after(k_bin_rows_scan, nb, kBinThreads, 0, s, n, rrec, row_cnt, nb, gy, plan, rowseq, rowspan, off, cap);
   else
-    launch_after(k_bin_rows, nb, kBinThreads, 0, s, n, rrec, row_cnt, nb, gy, plan, rowseq, rowspan, cap);
+    launch_after(k_bin_rows, nb, kBinThreads, 0, s, n, rrec, row_cnt, nb, gy, plan, rowseq, rowspan, off, cap);
   const size_t chunks = cap / ch + (size_t)gy + 1;
   const bool scan = gx <= kScanBuckets;  // chunks of 256 items
   int grid = device_sm_count() * (scan ? 8 : 5);
   if ((size_t)grid > chunks) grid = (int)chunks;
-  if (scan) launch_after(k_bin_count_scan, grid, kBinThreads, 0, s, rowspan, plan, gx, gy, tab);
+  const int wgrid = (int)((chunks + kBinWarps - 1) / kBinWarps);
+  if (scan) launch_after(k_bin_count_warp, wgrid < grid ? wgrid : grid, kBinThreads, 0, s, rowspan, plan, gx, gy, tab);
   else launch_after(k_bin_count, grid, kBinThreads, 0, s, rowspan, plan, gx, gy, ch, tab);
   launch_after(k_bin_rowscan, gy, 1024, 0, s, tab, plan, gx, gy, at<uint32_t>(ws, b.tile_start));
   if (scan) launch_after(k_bin_place_scan, grid, kBinThreads, 0, s, rowseq, rowspan, plan, tab, gx, gy, list, cap);
   else launch_after(k_bin_place, grid, kBinThreads, 0, s, rowseq, rowspan, plan, tab, gx, gy, ch, list, cap);
-  count_launch(6);
+  count_launch(5);
 }
 
 }  // namespace gs3
