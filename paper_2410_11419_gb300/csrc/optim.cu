@@ -26,11 +26,20 @@ __device__ __forceinline__ void adam_one(const AdamArgs& a, float g, float& p, f
   p = fmaxf(a.lo, p - step);
 }
 
-// four consecutive elements per thread (16-byte aligned arrays)
+// four consecutive elements per thread (16-byte aligned arrays); the thread past
+// the whole groups takes the last n % 4
 __global__ void __launch_bounds__(256) k_adam4(float4* __restrict__ p, const float4* __restrict__ g,
-                                               float4* __restrict__ m, float4* __restrict__ v, size_t n4, AdamArgs a) {
+                                               float4* __restrict__ m, float4* __restrict__ v, size_t n4, int tail,
+                                               AdamArgs a) {
+  after_previous();
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n4) return;
+  if (i >= n4) {
+    if (i == n4)
+      for (int k = 0; k < tail; ++k)
+        adam_one(a, reinterpret_cast<const float*>(g + n4)[k], reinterpret_cast<float*>(p + n4)[k],
+                 reinterpret_cast<float*>(m + n4)[k], reinterpret_cast<float*>(v + n4)[k]);
+    return;
+  }
   const float4 gi = __ldcs(g + i);
   float4 pi = p[i], mi = m[i], vi = v[i];
   adam_one(a, gi.x, pi.x, mi.x, vi.x);
@@ -61,23 +70,19 @@ void launch_adam(float* p, const float* g, float* m, float* v, size_t n, float l
   const AdamArgs a{lr, b1, b2, eps, (float)c1, (float)c2, lo};
   const uintptr_t addr = reinterpret_cast<uintptr_t>(p) | reinterpret_cast<uintptr_t>(g) |
                          reinterpret_cast<uintptr_t>(m) | reinterpret_cast<uintptr_t>(v);
-  // whole groups of four with vector accesses; the rest, unaligned arrays and
-  // arrays past the grid's limit one element at a time
-  size_t done = 0;
-  if ((addr & 15) == 0 && n >= 4 && n / 4 <= (size_t)0x7FFFFFFF * 256) {
+  // groups of four with vector accesses; unaligned arrays and arrays past the
+  // grid's limit one element at a time
+  if ((addr & 15) == 0 && n / 4 < (size_t)0x7FFFFFFF * 256) {
     const size_t n4 = n / 4;
+    const int tail = (int)(n - 4 * n4);
     auto f4 = [](float* x) { return reinterpret_cast<float4*>(x); };
-    k_adam4<<<(unsigned)((n4 + 255) / 256), 256, 0, s>>>(f4(p), reinterpret_cast<const float4*>(g), f4(m), f4(v), n4, a);
-    count_launch();
-    done = 4 * n4;
+    launch_after(k_adam4, (unsigned)((n4 + (tail ? 1 : 0) + 255) / 256), 256, 0, s, f4(p),
+                 reinterpret_cast<const float4*>(g), f4(m), f4(v), n4, tail, a);
+  } else {
+    const size_t want = (n + 255) / 256, cap_blocks = (size_t)device_sm_count() * 16;
+    k_adam<<<(int)(want < cap_blocks ? want : cap_blocks), 256, 0, s>>>(p, g, m, v, n, a);
   }
-  if (done < n) {
-    const size_t want = (n - done + 255) / 256;
-    const size_t cap_blocks = (size_t)device_sm_count() * 16;
-    const int blocks = (int)(want < cap_blocks ? want : cap_blocks);
-    k_adam<<<blocks, 256, 0, s>>>(p + done, g + done, m + done, v + done, n - done, a);
-    count_launch();
-  }
+  count_launch();
 }
 
 }  // namespace gs3
