@@ -65,6 +65,19 @@ bool mlp_ok(const gs3_mlp_desc& m, int in_dim, int out_dim) {
   return m.w && m.b;
 }
 
+// The part of the SMs that Psi takes beside the light chain, whose blocks find no
+// room beside a network's: 120k FP32 at 512 x 512 take 803 us with Psi after the
+// shadow composite, 763 with it on all SMs, 744 / 752 / 797 on a half / third /
+// quarter; 300k BF16 at 800 x 800 1672, 1668, 1660 / 1667 / 1647.
+constexpr int kPsiShare = 2;
+
+// stages without the light's: both networks can start after the camera's depth sort
+bool networks_beside(uint32_t stages) {
+  const uint32_t need = GS3_STAGE_CAMERA_BIN | GS3_STAGE_MLP;
+  const uint32_t light = GS3_STAGE_LIGHT_BIN | GS3_STAGE_SHADOW_COMPOSITE | GS3_STAGE_SHADOW_REDUCE;
+  return (stages & need) == need && !(stages & light);
+}
+
 }  // namespace
 
 void set_last_error(const char* msg) { g_last_error = msg; }
@@ -312,8 +325,10 @@ gs3_status gs3_workspace_layout(int32_t n, int32_t width, int32_t height, size_t
 gs3_status gs3_render_stages(gs3_scene* scene, const gs3_camera* cam, const gs3_light* light,
                              const gs3_render_opts* opts, float* out_rgb, void* workspace, size_t ws_bytes,
                              size_t key_capacity, uint32_t stages, void* stream) {
-  // a whole frame forks its light chain onto the calling thread's side stream
-  SideStream* side = stages == GS3_STAGE_ALL ? thread_side_stream() : nullptr;
+  // a whole frame forks its light chain onto the calling thread's side stream, a
+  // view under the light of the frame before its networks
+  const bool networks = networks_beside(stages);
+  SideStream* side = stages == GS3_STAGE_ALL || networks ? thread_side_stream() : nullptr;
   return render_frame(scene, cam, light, opts, out_rgb, workspace, ws_bytes, key_capacity, stages,
                       reinterpret_cast<cudaStream_t>(stream), side);
 }
@@ -350,6 +365,14 @@ SideStream* thread_side_stream() {
   int d = 0;
   if (cudaGetDevice(&d) != cudaSuccess || d < 0 || d >= 64) return nullptr;
   return t.dev[d].create() ? &t.dev[d] : nullptr;
+}
+
+// which_mask: 1 Phi, 2 Psi; sms: the SMs they may take (0: all)
+static void launch_networks(const gs3_scene* scene, const FrameArgs& f, int which_mask, int sms, cudaStream_t s) {
+  const bool tc = scene->dev.mlp_dtype != GS3_MLP_FP32;
+  launch_mlp(f, s, /*identity_only=*/tc, which_mask, sms);
+  const unsigned char* blobs[2] = {scene->tc_blob[0], scene->tc_blob[1]};
+  if (tc) launch_mlp_tc(f, blobs, s, which_mask, sms);
 }
 
 gs3_status render_frame(gs3_scene* scene, const gs3_camera* cam, const gs3_light* light,
@@ -413,25 +436,29 @@ gs3_status render_frame(gs3_scene* scene, const gs3_camera* cam, const gs3_light
     if (no_shadow) launch_fill_shadow_one(f, sl);
     else launch_shadow_reduce(f, sl);
   }
+  // The networks need the camera's depth ranks, Phi the shadow average as well.
+  // A network that waits for nothing else in this call starts right after the
+  // camera's depth sort, under the small kernels of the binning: Psi beside the
+  // light chain, both on the side stream when the light stages are not run.
+  const bool early = (stages & GS3_STAGE_CAMERA_BIN) && (stages & GS3_STAGE_MLP);
+  const bool beside = side && networks_beside(stages);
   if (stages & GS3_STAGE_CAMERA_BIN) {
     launch_depth_sort(f, 0, s);
+    if (beside) {
+      cudaEventRecord(side->fork, s);
+      cudaStreamWaitEvent(side->s, side->fork, 0);
+      launch_networks(scene, f, 3, 0, side->s);
+      cudaEventRecord(side->join, side->s);
+    } else if (early) {
+      launch_networks(scene, f, 2, fork ? device_sm_count() / kPsiShare : 0, s);
+    }
     launch_binning(f, 0, s);
     launch_tile_order(f, 0, s);  // the camera composite's launch order
   }
-  if (fork) {
-    cudaEventRecord(side->join, sl);
-    cudaStreamWaitEvent(s, side->join, 0);
-  }
-  if (stages & GS3_STAGE_MLP) {
-    if (scene->dev.mlp_dtype != GS3_MLP_FP32) {
-      launch_mlp(f, s, /*identity_only=*/true);
-      const unsigned char* blobs[2] = {scene->tc_blob[0], scene->tc_blob[1]};
-      launch_mlp_tc(f, blobs, s);
-    } else {
-      launch_mlp(f, s);
-    }
-  }
-  if (stages & GS3_STAGE_CAMERA) launch_camera_composite(f, out_rgb, (stages & GS3_STAGE_MLP) != 0, s);
+  if (fork) cudaEventRecord(side->join, sl);
+  if (fork || beside) cudaStreamWaitEvent(s, side->join, 0);
+  if ((stages & GS3_STAGE_MLP) && !beside) launch_networks(scene, f, early ? 1 : 3, 0, s);
+  if (stages & GS3_STAGE_CAMERA) launch_camera_composite(f, out_rgb, (stages & GS3_STAGE_MLP) && !beside, s);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "gs3_render: launch");
   return GS3_OK;
@@ -470,10 +497,10 @@ void BatchStreams::destroy() {
 //   1. per frame, on its own sub-stream: header reset, shading and both
 //      projections (K1), the light binning and the shadow composite's
 //      per-frame set-up (occluder bounds, segment plan), then the camera
-//      binning, which runs beside step 2;
+//      binning and Psi, which run beside step 2;
 //   2. on `stream`: the shadow composite's three persistent segment kernels
 //      over every segment of every frame, from shared tickets;
-//   3. per frame, on its sub-stream again: the shadow reduce and the MLPs;
+//   3. per frame, on its sub-stream again: the shadow reduce and Phi;
 //   4. on `stream`: one camera composite over every frame's tiles.
 gs3_status render_batch(const BatchFrame* frames, int n, cudaStream_t s, BatchStreams& bs,
                         unsigned char* param_dev, unsigned char* param_host) {
@@ -516,6 +543,7 @@ gs3_status render_batch(const BatchFrame* frames, int n, cudaStream_t s, BatchSt
     }
     cudaEventRecord(bs.join[r], sr);
     launch_depth_sort(f[r], 0, sr);
+    launch_networks(frames[r].scene, f[r], 2, 0, sr);
     launch_binning(f[r], 0, sr);
     launch_tile_order(f[r], 0, sr);
   }
@@ -529,14 +557,7 @@ gs3_status render_batch(const BatchFrame* frames, int n, cudaStream_t s, BatchSt
     cudaStreamWaitEvent(sr, bs.fork2, 0);
     if (f[r].opts.ablate & GS3_ABLATE_SHADOW_SPLAT) launch_fill_shadow_one(f[r], sr);
     else launch_shadow_reduce(f[r], sr);
-    const gs3_scene* sc = frames[r].scene;
-    if (sc->dev.mlp_dtype != GS3_MLP_FP32) {
-      launch_mlp(f[r], sr, /*identity_only=*/true);
-      const unsigned char* blobs[2] = {sc->tc_blob[0], sc->tc_blob[1]};
-      launch_mlp_tc(f[r], blobs, sr);
-    } else {
-      launch_mlp(f[r], sr);
-    }
+    launch_networks(frames[r].scene, f[r], 1, 0, sr);
     cudaEventRecord(bs.join2[r], sr);
   }
   for (int r = 0; r < n; ++r) cudaStreamWaitEvent(s, bs.join2[r], 0);

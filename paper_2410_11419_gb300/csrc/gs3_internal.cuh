@@ -267,7 +267,8 @@ void launch_tile_order(const FrameArgs& f, int splat, cudaStream_t s);
 void launch_shadow_reduce(const FrameArgs& f, cudaStream_t s);
 // Phi and Psi of one frame; which_mask bit 0 Phi, bit 1 Psi; identity_only:
 // only the networks an ablation replaces by the identity / zero
-void launch_mlp(const FrameArgs& f, cudaStream_t s, bool identity_only = false, int which_mask = 3);
+// sms: the SMs that the tensor-core kernels may take (0: all)
+void launch_mlp(const FrameArgs& f, cudaStream_t s, bool identity_only = false, int which_mask = 3, int sms = 0);
 // Phi of nl <= kMaxBatch frames of one scene and camera (an environment
 // light's directional lights; the camera ranks of f[0]) in one launch over
 // nl N rows; (shade_l, T'_l) of camera rank r go to envcol[r nl + l]
@@ -278,14 +279,15 @@ void launch_phi_lights_tc(const FrameArgs* const* f, int nl, float4* envcol, con
 // packed weights of both networks take mlp_x3_bytes() of the workspace
 size_t mlp_x3_bytes();
 bool mlp_x3_supported(const MlpDev& m);
-void launch_mlp_x3(const FrameArgs& f, cudaStream_t s, int which_mask);
+void launch_mlp_x3(const FrameArgs& f, cudaStream_t s, int which_mask, int sms);
 void launch_phi_lights_x3(const FrameArgs* const* f, int nl, float4* envcol, cudaStream_t s);
 // BF16 / FP8 tensor-core MLPs (mlp_tc.cu)
 size_t mlp_tc_blob_bytes(const MlpDev& m, int dtype);
 size_t mlp_tc_scale_offset(const MlpDev& m, int dtype);  // FP8: (sx, sw) per hidden layer
 void pack_mlp_tc(const MlpDev& m, int dtype, const SceneDev& sc, int which, unsigned char* dst, cudaStream_t s);
 bool mlp_tc_supported(const MlpDev& m, int dtype);
-void launch_mlp_tc(const FrameArgs& f, const unsigned char* const blobs[2], cudaStream_t s, int which_mask = 3);
+void launch_mlp_tc(const FrameArgs& f, const unsigned char* const blobs[2], cudaStream_t s, int which_mask = 3,
+                   int sms = 0);
 // after_mlp: the stream's last operation is the networks' last kernel
 void launch_camera_composite(const FrameArgs& f, float* out_rgb, bool after_mlp, cudaStream_t s);
 // camera composite of nl <= kMaxBatch lights over f0's camera splat:
@@ -336,9 +338,10 @@ struct DeviceOnce {
 
 // A launch whose kernel starts with after_previous(): the grid is set up while
 // the stream's previous kernel drains, and its threads wait there until that
-// kernel has finished and its writes are visible.  Used where the previous
-// operation of the stream is always a kernel.  Between two dependent kernels it
-// takes 0.8 us instead of 1.9.
+// kernel has finished and its writes are visible (after anything but a kernel it
+// is an ordinary launch).  Between two dependent kernels it takes 0.8 us instead of
+// 1.9.  Kernels that let their successor in at once (griddepcontrol.launch_dependents)
+// cost frames 2 to 5 %: the waiting blocks hold room that the other stream's need.
 template <typename... P, typename... A>
 inline void launch_after(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A&&... args) {
   cudaLaunchAttribute attr;

@@ -182,7 +182,7 @@ void launch_one(const MlpParams& p, cudaStream_t s) {
 
 }  // namespace
 
-void launch_mlp(const FrameArgs& f, cudaStream_t s, bool identity_only, int which_mask) {
+void launch_mlp(const FrameArgs& f, cudaStream_t s, bool identity_only, int which_mask, int sms) {
   MlpParams p;
   p.n = f.sc.n;
   p.nl = 1;
@@ -208,7 +208,7 @@ void launch_mlp(const FrameArgs& f, cudaStream_t s, bool identity_only, int whic
     if (!p.identity && mlp_x3_supported(p.net)) x3 |= 1 << w;
     else launch_one(p, s);
   }
-  if (x3) launch_mlp_x3(f, s, x3);
+  if (x3) launch_mlp_x3(f, s, x3, sms);
 }
 
 void launch_phi_lights(const FrameArgs* const* f, int nl, float4* envcol, cudaStream_t s) {

@@ -542,7 +542,7 @@ TcParams tc_params(const FrameArgs& f, int which, const unsigned char* blob) {
 }
 
 // after: the stream's last operation is a kernel
-void launch_tc(const TcParams& p, const MlpDev& m, int eb, bool after, cudaStream_t s) {
+void launch_tc(const TcParams& p, const MlpDev& m, int eb, bool after, int sms, cudaStream_t s) {
   const int groups = tc_groups(m, eb);
   size_t smem = tc_smem_bytes(m, eb, groups);
   // CTAs of this kernel (of any launch) that share an SM must fit in its 512
@@ -555,7 +555,7 @@ void launch_tc(const TcParams& p, const MlpDev& m, int eb, bool after, cudaStrea
   auto kern = eb == 2 ? (p.which == 0 ? k_mlp_tc<2, 0> : k_mlp_tc<2, 1>)
                       : (p.which == 0 ? k_mlp_tc<1, 0> : k_mlp_tc<1, 1>);
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  const int nsm = device_sm_count();
+  const int nsm = sms > 0 ? sms : device_sm_count();
   const int ntiles = (p.n * p.nl + kTcRows - 1) / kTcRows;
   const int ctas = (ntiles + groups - 1) / groups;
   const int grid = ctas < nsm ? ctas : nsm;
@@ -566,14 +566,14 @@ void launch_tc(const TcParams& p, const MlpDev& m, int eb, bool after, cudaStrea
 
 }  // namespace
 
-void launch_mlp_tc(const FrameArgs& f, const unsigned char* const blobs[2], cudaStream_t s, int which_mask) {
+void launch_mlp_tc(const FrameArgs& f, const unsigned char* const blobs[2], cudaStream_t s, int which_mask, int sms) {
   const int eb = elem_bytes(f.sc.mlp_dtype);
   bool after = false;
   for (int which = 0; which < 2; ++which) {
     if (!(which_mask & (1 << which))) continue;
     const bool identity = (f.opts.ablate & (which == 0 ? GS3_ABLATE_PHI : GS3_ABLATE_PSI)) != 0;
     if (identity) continue;  // handled by the FP32 kernel's identity path
-    launch_tc(tc_params(f, which, blobs[which]), which == 0 ? f.sc.phi : f.sc.psi, eb, after, s);
+    launch_tc(tc_params(f, which, blobs[which]), which == 0 ? f.sc.phi : f.sc.psi, eb, after, sms, s);
     after = true;
   }
 }
@@ -590,7 +590,7 @@ void launch_phi_lights_tc(const FrameArgs* const* f, int nl, float4* envcol, con
   }
   p.ccol = nullptr;
   p.envcol = envcol;
-  launch_tc(p, f[0]->sc.phi, elem_bytes(f[0]->sc.mlp_dtype), false, s);
+  launch_tc(p, f[0]->sc.phi, elem_bytes(f[0]->sc.mlp_dtype), false, 0, s);
 }
 
 }  // namespace gs3

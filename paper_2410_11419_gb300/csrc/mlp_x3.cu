@@ -330,7 +330,7 @@ X3Params x3_params(const FrameArgs& f, int which) {
   return p;
 }
 
-void launch_net(const X3Params& p, int which, const MlpDev& m, cudaStream_t s) {
+void launch_net(const X3Params& p, int which, const MlpDev& m, int sms, cudaStream_t s) {
   size_t smem = x3_smem(m);
   // the CTAs that can share an SM never need more than its 512 tensor-memory columns
   const size_t per_sm = 228 * 1024, reserve = 2048;
@@ -344,7 +344,7 @@ void launch_net(const X3Params& p, int which, const MlpDev& m, cudaStream_t s) {
       ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024) == cudaSuccess;
     return ok;
   });
-  const int ntiles = (p.n * p.nl + kRows - 1) / kRows, nsm = device_sm_count();
+  const int ntiles = (p.n * p.nl + kRows - 1) / kRows, nsm = sms > 0 ? sms : device_sm_count();
   launch_after(kern, ntiles < nsm ? ntiles : nsm, kThreads, smem, s, p);
   count_launch();
 }
@@ -358,7 +358,7 @@ size_t mlp_x3_bytes() {
 
 bool mlp_x3_supported(const MlpDev& m) { return m.width == 32 || m.width == 64 || m.width == 128; }
 
-void launch_mlp_x3(const FrameArgs& f, cudaStream_t s, int which_mask) {
+void launch_mlp_x3(const FrameArgs& f, cudaStream_t s, int which_mask, int sms) {
   PackArgs a;
   int total = 0;
   for (int w = 0; w < 2; ++w) {
@@ -375,7 +375,7 @@ void launch_mlp_x3(const FrameArgs& f, cudaStream_t s, int which_mask) {
   k_x3_pack<<<(total + 255) / 256, 256, 0, s>>>(a);
   count_launch();
   for (int w = 0; w < 2; ++w)
-    if (which_mask & (1 << w)) launch_net(x3_params(f, w), w, w == 0 ? f.sc.phi : f.sc.psi, s);
+    if (which_mask & (1 << w)) launch_net(x3_params(f, w), w, w == 0 ? f.sc.phi : f.sc.psi, sms, s);
 }
 
 void launch_phi_lights_x3(const FrameArgs* const* f, int nl, float4* envcol, cudaStream_t s) {
@@ -396,7 +396,7 @@ void launch_phi_lights_x3(const FrameArgs* const* f, int nl, float4* envcol, cud
   }
   p.ccol = nullptr;
   p.envcol = envcol;
-  launch_net(p, 0, m, s);
+  launch_net(p, 0, m, 0, s);
 }
 
 }  // namespace gs3

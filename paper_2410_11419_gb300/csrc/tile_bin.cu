@@ -501,10 +501,12 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_count(const uint32_t* __res
   }
 }
 
+constexpr int kRowscanThreads = 512;  // a block of 1024 finds no room beside a networks' block
+
 // One block per row: the row's counts scanned in (column, chunk) order after
 // the list entries of the rows above; tile (y, x) starts at the scanned count
 // of its first chunk.  The last row also writes the end of the last tile.
-__global__ void __launch_bounds__(1024) k_bin_rowscan(uint32_t* __restrict__ tab, const uint32_t* __restrict__ plan,
+__global__ void __launch_bounds__(kRowscanThreads) k_bin_rowscan(uint32_t* __restrict__ tab, const uint32_t* __restrict__ plan,
                                                       int gx, int gy, uint32_t* __restrict__ tile_start) {
   after_previous();
   __shared__ uint32_t sm[32];
@@ -519,10 +521,10 @@ __global__ void __launch_bounds__(1024) k_bin_rowscan(uint32_t* __restrict__ tab
   }
   uint32_t above = 0;
   for (int t = threadIdx.x; t < y; t += blockDim.x) above += pairs[t];
-  above = block_sum<1024>(above, sm);
+  above = block_sum<kRowscanThreads>(above, sm);
   const uint32_t c0 = cb[y], nch = cb[y + 1] - c0;
   uint32_t* seg = tab + (size_t)c0 * gx;
-  const uint32_t end = block_scan_inplace<1024>(seg, (size_t)nch * gx, above, sm);
+  const uint32_t end = block_scan_inplace<kRowscanThreads>(seg, (size_t)nch * gx, above, sm);
   for (int x = threadIdx.x; x < gx; x += blockDim.x) ts[x] = seg[(size_t)x * nch];
   if (y == gy - 1 && threadIdx.x == 0) tile_start[(size_t)gx * gy] = end;
 }
@@ -598,7 +600,7 @@ void launch_binning(const FrameArgs& f, int sp, cudaStream_t s) {
   const int wgrid = (int)((chunks + kBinWarps - 1) / kBinWarps);
   if (scan) launch_after(k_bin_count_warp, wgrid < grid ? wgrid : grid, kBinThreads, 0, s, rowspan, plan, gx, gy, tab);
   else launch_after(k_bin_count, grid, kBinThreads, 0, s, rowspan, plan, gx, gy, ch, tab);
-  launch_after(k_bin_rowscan, gy, 1024, 0, s, tab, plan, gx, gy, at<uint32_t>(ws, b.tile_start));
+  launch_after(k_bin_rowscan, gy, kRowscanThreads, 0, s, tab, plan, gx, gy, at<uint32_t>(ws, b.tile_start));
   if (scan) launch_after(k_bin_place_scan, grid, kBinThreads, 0, s, rowseq, rowspan, plan, tab, gx, gy, list, cap);
   else launch_after(k_bin_place, grid, kBinThreads, 0, s, rowseq, rowspan, plan, tab, gx, gy, ch, list, cap);
   count_launch(5);

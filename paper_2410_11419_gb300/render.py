@@ -144,7 +144,7 @@ class Renderer:
         if getattr(self, "bws", None) is None:
             nb = N.gs3_backward_workspace_size(self.scene.handle)
             self.bws = torch.empty(nb, dtype=torch.uint8, device=self.ws.device)
-        grads = {f: torch.zeros_like(self.scene.t[f]) for f in self.scene.ARRAYS_DEV}
+        grads = {f: torch.empty_like(self.scene.t[f]) for f in self.scene.ARRAYS_DEV}  # all overwritten
         N.gs3_render_backward(self.scene.handle, camera_struct(cam), light_struct(light), opts,
                               dl_drgb.contiguous(), self.ws, self.cap, self.bws, grads, s.cuda_stream)
         return grads

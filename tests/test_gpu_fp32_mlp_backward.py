@@ -46,3 +46,29 @@ def test_two_batches_of_rows(gs3, oracle):
     assert len(_compare(gpu, nets)) == 4
     assert not gpu["mean_op"][:312000].any()
     assert len(_compare({"latent": gpu["latent"][0, 312000:]}, {"latent": ref["latent"][:, :4]})) == 1
+
+
+@pytest.mark.parametrize("ablate", [0, 1, 8])
+@pytest.mark.parametrize("shared", [False, True])
+def test_every_gradient_is_overwritten(gs3, ablate, shared):
+    """The caller's arrays may hold anything: the backward writes every element."""
+    import torch
+    from paper_2410_11419_gb300 import _native as N, render as R
+    scene = synth.make_scene(6, 300, 3, "ball", mlp_width=32, mlp_hidden=2)
+    if shared:
+        scene.lobe_shared = True
+        scene.lobe_rot, scene.lobe_sigma = scene.lobe_rot[:, 0].copy(), scene.lobe_sigma[:, 0].copy()
+    cam, light = synth.camera_light_pair(2, 50, 34)
+    ds, opts = R.DeviceScene(scene), R.opts_struct(ablate=ablate)
+    rd = R.Renderer(ds, 50, 34, 1 << 18)
+    dimg = torch.rand_like(rd.render(cam, light, opts))
+    first = rd.backward(cam, light, dimg, opts)
+    filled = {f: torch.full_like(ds.t[f], float("nan")) for f in N.GRAD_FIELDS}
+    N.gs3_render_backward(ds.handle, R.camera_struct(cam), R.light_struct(light), opts, dimg, rd.ws, rd.cap, rd.bws,
+                          filled, torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    rd.check()
+    for f in N.GRAD_FIELDS:
+        assert torch.isfinite(filled[f]).all(), f
+        assert torch.allclose(filled[f], first[f], rtol=1e-4, atol=1e-6 * float(first[f].abs().max() + 1e-30)), f
+    ds.close()
