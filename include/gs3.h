@@ -301,8 +301,8 @@ size_t gs3_backward_workspace_size(const gs3_scene *scene);
  *              light and options, unchanged since (it holds the forward state)
  *   bwd_ws:    device, >= gs3_backward_workspace_size bytes, caller-owned
  * The MLP gradients are those of the scene's FP32 networks evaluated at the
- * forward's inputs (their GEMMs on the tensor cores in three-pass TF32,
- * about FP32 accuracy); for a BF16 or FP8 scene the rest of the backward
+ * forward's inputs (their products on the tensor cores, the operands split
+ * into TF32 or BF16 parts, about FP32 accuracy); for a BF16 or FP8 scene the rest of the backward
  * uses the forward's reduced-precision T' and residual, so the rounding of
  * the MLP operands passes straight through.
  * Asynchronous on `stream`.  Errors: INVALID_ARG, CUDA. */

@@ -5,9 +5,9 @@
 //   K9b  camera composite, back to front per pixel from the stored final
 //        transmittance, recovering T by division (per-tile recomputation; no
 //        per-pixel lists are stored)                          (Eq. 2, Sec. 4)
-//   K8b  Psi and Phi: forward recomputed per 32-row tile, backward through
-//        the layers, weight gradients as per-block partials summed in a fixed
-//        order                                                  (Sec. 4.2, 4.3)
+//   K8b  Psi and Phi (mlp_x3_bwd.cu; widths of 16: mlp_bwd.cu): forward
+//        recomputed, backward through the layers, weight gradients as per-block
+//        partials summed in a fixed order                        (Sec. 4.2, 4.3)
 //   K6b  shadow splat (shadow_bwd.cu)                                 (Sec. 4.2)
 //   K1b  per Gaussian: both EWA projections and the shading back to the
 //        parameters                                       (Eq. 1-5, Sec. 3, 4.1)
@@ -83,7 +83,10 @@ BwdPlan plan_bwd(int n, const MlpDev& phi, const MlpDev& psi) {
 //
 // A warp takes one half (16 x 8) of a tile on its own: lane l column l & 15 and
 // rows (l >> 4) + 2 i, i = 0..3, so that a lane adds four pixels before the
-// warp adds its lanes.  The pixel pairs go through packed FP32 instructions;
+// warp adds its lanes; an image too small to fill the chip that way goes by
+// quarters (16 x 4, two pixels per lane), which halves a warp's serial walk
+// (256 x 256, 20k Gaussians: 117 -> 94 us, 105 if the entries are still picked by
+// halves).  The pixel pairs go through packed FP32 instructions;
 // the next 32 entries are staged (those whose box and ellipse reach the half)
 // while the current ones are walked, as in the forward.  The 14 terms of four
 // entries are added over the 32 lanes through shared-memory rows.
@@ -135,26 +138,28 @@ __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
                : "memory");
 }
 
+template <int NQ>
 __global__ void __launch_bounds__(kCbWarps * 32, 3) k_camera_bwd(CamBwdParams p) {
   __shared__ CamBwdSmem smem[kCbWarps];
   CamBwdSmem& B = smem[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
-  const uint32_t unit = blockIdx.x * kCbWarps + (threadIdx.x >> 5);  // (tile in launch order, half)
-  if (unit >= 2u * (uint32_t)p.ntiles) return;
-  const int tile = (int)p.tile_order[unit >> 1], half = (int)(unit & 1u);
+  constexpr uint32_t kParts = 4 / NQ;  // strips of 4 NQ rows
+  const uint32_t unit = blockIdx.x * kCbWarps + (threadIdx.x >> 5);  // (tile in launch order, strip)
+  if (unit >= kParts * (uint32_t)p.ntiles) return;
+  const int tile = (int)p.tile_order[unit / kParts], part = (int)(unit % kParts), half = part * NQ / 2;
   const int tx = tile % p.gx, ty = tile / p.gx;
   const uint32_t hbits = 3u << (2 * half);
   const float ox = (float)(tx * kTile), oy = (float)(ty * kTile);
-  const int cx = lane & 15, cy = 8 * half + (lane >> 4);
+  const int cx = lane & 15, cy = 4 * NQ * part + (lane >> 4);
   const int px = tx * kTile + cx;
   const float lx = cx + 0.5f;
   const uint32_t b = p.tile_start[tile];
   // per pixel pair q (rows 4 q and 4 q + 2 of the lane): row (far away until the
   // sweep reaches the pixel's last entry), T, D, dL/d(image), Sh, g . S
-  f32x2 ly[2], T[2], D[2], gr[2], gg[2], gb[2], sh[2], gs[2];
-  uint32_t nc[4], next = 0u;
+  f32x2 ly[NQ], T[NQ], D[NQ], gr[NQ], gg[NQ], gb[NQ], sh[NQ], gs[NQ];
+  uint32_t nc[2 * NQ], next = 0u;
 #pragma unroll
-  for (int q = 0; q < 2; ++q) {
+  for (int q = 0; q < NQ; ++q) {
     float t2[2], r2[2], g2[2], b2[2], h2[2], s2[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -179,7 +184,7 @@ __global__ void __launch_bounds__(kCbWarps * 32, 3) k_camera_bwd(CamBwdParams p)
     gr[q] = pk2(r2[0], r2[1]); gg[q] = pk2(g2[0], g2[1]); gb[q] = pk2(b2[0], b2[1]);
     sh[q] = pk2(h2[0], h2[1]); gs[q] = pk2(s2[0], s2[1]);
   }
-  const uint32_t end = __reduce_max_sync(0xffffffffu, next);  // entries some pixel of the half took
+  const uint32_t end = __reduce_max_sync(0xffffffffu, next);  // entries some pixel of the strip took
 
   int nrow = 0;
   auto flush = [&]() {
@@ -221,8 +226,11 @@ __global__ void __launch_bounds__(kCbWarps * 32, 3) k_camera_bwd(CamBwdParams p)
     q.a = rec.a; q.b = rec.b; q.c = rec.c;
     float4 e0, e1;
     make_entry(q, ox, oy, e0, e1);
-    // the halves (and no fewer) that the forward's quadrants lie in
-    const bool hit = hi > (uint32_t)lane && (__float_as_uint(e1.w) & ellipse_halves(e0, e1) & hbits) != 0u;
+    // the halves (and no fewer) that the forward's quadrants lie in, or the strip's rows
+    const uint32_t bits = __float_as_uint(e1.w) & hbits;
+    bool hit = hi > (uint32_t)lane;
+    if constexpr (NQ == 2) hit = hit && (bits & ellipse_halves(e0, e1)) != 0u;
+    else hit = hit && bits != 0u && ellipse_rows(e0, e1, (float)(4 * part), (float)(4 * part + 3));
     const uint32_t m = __ballot_sync(0xffffffffu, hit);
     const int slot = __popc(m & ((1u << lane) - 1u));
     if (hit) {
@@ -264,7 +272,7 @@ __global__ void __launch_bounds__(kCbWarps * 32, 3) k_camera_bwd(CamBwdParams p)
       if (idx < next) {  // pixels whose last entry this is, or lies ahead: once per pixel
         next = 0u;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < 2 * NQ; ++i) {
           const float y = (float)(cy + 2 * i) + 0.5f;
           if (idx < nc[i]) {
             ly[i / 2] = i & 1 ? pk2(lo2(ly[i / 2]), y) : pk2(y, hi2(ly[i / 2]));
@@ -280,7 +288,7 @@ __global__ void __launch_bounds__(kCbWarps * 32, 3) k_camera_bwd(CamBwdParams p)
       const bool clampable = !(gi.x * 1.00001f < p.amax);
       f32x2 m0 = 0ull, m1 = 0ull, m2 = 0ull, k0 = 0ull, k1 = 0ull, k2 = 0ull, k3 = 0ull, k4 = 0ull, k5 = 0ull, k6 = 0ull;
 #pragma unroll
-      for (int q = 0; q < 2; ++q) {
+      for (int q = 0; q < NQ; ++q) {
         const f32x2 dy = add2(ly[q], yc.x);
         const f32x2 pw = fma2(dy, fma2(yc.y, dy, v), sx);
         f32x2 beta = pk2(lo2(pw) >= qx.w ? ex2(lo2(pw)) : 0.f, hi2(pw) >= qx.w ? ex2(hi2(pw)) : 0.f);
@@ -749,7 +757,12 @@ gs3_status run_backward(const FrameArgs& f, const float* dimg, void* bws, size_t
     p.color = color;
     p.W = L.width; p.H = L.height; p.gx = L.gx; p.ntiles = L.ntiles;
     p.amax = f.opts.alpha_max;
-    k_camera_bwd<<<(2 * L.ntiles + kCbWarps - 1) / kCbWarps, kCbWarps * 32, 0, s>>>(p);
+    // quarter tiles while halves leave warp slots free (three blocks per SM); on every
+    // image they cost the step of 300k at 800 x 800 2 % (5.05 -> 5.14 ms)
+    if (2 * L.ntiles < 3 * kCbWarps * device_sm_count())
+      k_camera_bwd<1><<<L.ntiles, kCbWarps * 32, 0, s>>>(p);
+    else
+      k_camera_bwd<2><<<(2 * L.ntiles + kCbWarps - 1) / kCbWarps, kCbWarps * 32, 0, s>>>(p);
     count_launch();
   }
   // K8b: one network's backward, then its weight gradients in fixed block order
@@ -789,7 +802,8 @@ gs3_status run_backward(const FrameArgs& f, const float* dimg, void* bws, size_t
   // Phi first: the shadow backward takes its dL/dT.  Then Psi, which the
   // shadow backward does not need, runs on the side stream beside it (the
   // networks share the MLP scratch, so they run in turn), after the receivers
-  // of the stopped segments.
+  // of the stopped segments.  (Phi's weight gradients there too: 5.25 -> 5.34 ms
+  // for the step of 300k.)
   mlp_bwd(0, s);
   cudaStream_t ss = side ? side->s : s;
   // K6b

@@ -74,6 +74,24 @@ __device__ __forceinline__ uint32_t ellipse_halves(const float4 e0, const float4
   return m;
 }
 
+// The same for the tile's rows r0 .. r1 alone (one rectangle; as a part of
+// ellipse_halves it cost the shadow composite's staging a percent)
+__device__ __forceinline__ bool ellipse_rows(const float4 e0, const float4 e1, float r0, float r1) {
+  const float al = -e0.z, ga = -e0.w, be = -e1.x, lim = -e1.y;
+  const float X0 = 0.5f - e0.x, X1 = 15.5f - e0.x;
+  const float mx = fmaxf(X0 * X0, X1 * X1);
+  auto q = [&](float dx, float dy) { return fmaf(dx, fmaf(al, dx, be * dy), ga * dy * dy); };
+  const float Y0 = r0 + 0.5f - e0.y, Y1 = r1 + 0.5f - e0.y;
+  float best = 0.f;
+  if (!(X0 <= 0.f && X1 >= 0.f && Y0 <= 0.f && Y1 >= 0.f)) {
+    const float kx = -be / (2.f * ga), ky = -be / (2.f * al);
+    best = fminf(fminf(q(X0, fminf(fmaxf(kx * X0, Y0), Y1)), q(X1, fminf(fmaxf(kx * X1, Y0), Y1))),
+                 fminf(q(fminf(fmaxf(ky * Y0, X0), X1), Y0), q(fminf(fmaxf(ky * Y1, X0), X1), Y1)));
+  }
+  const float size = 2.f * (al * mx + ga * fmaxf(Y0 * Y0, Y1 * Y1));
+  return best <= lim + 1e-4f * (1.f + size);
+}
+
 // power2 at one pixel (lx, ly) of the tile: the camera composite and its
 // backward evaluate an entry with this arithmetic, so both take every alpha
 // decision alike.
