@@ -39,11 +39,12 @@ sys.path.insert(0, ROOT)
 # one ncu capture of the kernel, valid only while its sources are unchanged:
 # kernel -> (bytes, SHA-256 of the concatenated sources, the summary file).
 PROFILED_TRAFFIC = {
-    "k_shadow": (424.0e6, "45c857b1a605bc1fa160eec9eb2162e289e65f09948bd5de23196b2d6a110c78",
-                 "profiles/k_shadow_object_300k_800.md"),
+    "k_shadow": (298.6e6, "44791f3ec9b538f94bc4191129d5e316f2ed502a5d223325152f6f893a372066",
+                 "profiles/segments_and_networks.md"),
 }
 TRAFFIC_SOURCES = {
-    "k_shadow": ("paper_2410_11419_gb300/csrc/composite.cu", "paper_2410_11419_gb300/csrc/splat_eval.cuh"),
+    "k_shadow": ("paper_2410_11419_gb300/csrc/composite.cu", "paper_2410_11419_gb300/csrc/splat_eval.cuh",
+                 "paper_2410_11419_gb300/csrc/shadow_seg.cuh"),
 }
 
 
