@@ -782,7 +782,7 @@ def main():
                 plain["differentiation"]["bf16_forward"] = {
                     "fwd_bwd_ms": float(fb16.mean()), "bwd_ms": float(bw16.mean()),
                     "note": "BF16 MLP forward; the backward's MLP gradients are the FP32 networks' at the "
-                            "same inputs (three-pass TF32 tensor-core GEMMs)"}
+                            "same inputs (operands split into TF32 or BF16 parts on the tensor cores)"}
             # one training iteration (Sec. 4.4): render, L1 + D-SSIM loss, backward, Adam on every group
             from paper_2410_11419_gb300.train import Trainer
             del rd2
