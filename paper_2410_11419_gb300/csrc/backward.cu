@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(kCbWarps * 32, 3) k_camera_bwd(CamBwdParams p)
       }
       next = max(next, nc[2 * q + h]);
     }
-    ly[q] = dup2(1.0e6f);
+    ly[q] = dup2(kFarRow);
     D[q] = 0ull;
     T[q] = pk2(t2[0], t2[1]);
     gr[q] = pk2(r2[0], r2[1]); gg[q] = pk2(g2[0], g2[1]); gb[q] = pk2(b2[0], b2[1]);

@@ -846,7 +846,7 @@ __device__ __forceinline__ void camera_weights(const CamEntries<COLS, G>& E, int
       }
       if (stopped) {
         px.done |= 1u << k;
-        px.ly = k ? pk2(lo2(px.ly), 1.0e6f) : pk2(1.0e6f, hi2(px.ly));
+        px.ly = k ? pk2(lo2(px.ly), kFarRow) : pk2(kFarRow, hi2(px.ly));
         px.T = k ? pk2(lo2(px.T), Tk) : pk2(Tk, hi2(px.T));
       }
     }
@@ -874,7 +874,7 @@ __device__ __forceinline__ CamTile camera_tile_of(const CamParams& p, int blk, C
             tx * kTile + cx, ty * kTile + cy};
   const bool in0 = t.px < p.W && t.py0 < p.H, in1 = t.px < p.W && t.py0 + 4 < p.H;
   x.lx = cx + 0.5f;
-  x.ly = pk2(in0 ? cy + 0.5f : 1.0e6f, in1 ? cy + 4.5f : 1.0e6f);
+  x.ly = pk2(in0 ? cy + 0.5f : kFarRow, in1 ? cy + 4.5f : kFarRow);
   x.T = dup2(1.f);
   x.done = (in0 ? 0u : 1u) | (in1 ? 0u : 2u);
   x.consumed[0] = x.consumed[1] = t.e - t.b;

@@ -428,7 +428,7 @@ __device__ __forceinline__ void stopped_unit(const BwdParams& p, uint32_t idx, i
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int y = 8 * h + 2 * q;  // rows below the image lie far away
-    dy[q] = pk2((y < nrow ? (float)y + 0.5f : 1.0e6f) - e0.y, (y + 1 < nrow ? (float)y + 1.5f : 1.0e6f) - e0.y);
+    dy[q] = pk2((y < nrow ? (float)y + 0.5f : kFarRow) - e0.y, (y + 1 < nrow ? (float)y + 1.5f : kFarRow) - e0.y);
   }
   const f32x2 c = dup2(e0.w);
   float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f, s4 = 0.f;  // beta dx, beta dy, beta dx dy, beta dx^2, beta dy^2

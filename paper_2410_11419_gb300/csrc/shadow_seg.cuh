@@ -76,7 +76,7 @@ __device__ __forceinline__ void lane_rows(int lane, int rows_in, f32x2 (&ly)[kPx
 #pragma unroll
   for (int q = 0; q < kPx / 2; ++q) {
     const float y = (float)(lane >> 4) + 4 * q + 0.5f;
-    ly[q] = pk2(2 * q < rows_in ? y : 1.0e6f, 2 * q + 1 < rows_in ? y + 2.f : 1.0e6f);
+    ly[q] = pk2(2 * q < rows_in ? y : kFarRow, 2 * q + 1 < rows_in ? y + 2.f : kFarRow);
   }
 }
 

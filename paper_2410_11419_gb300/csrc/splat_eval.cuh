@@ -102,6 +102,13 @@ __device__ __forceinline__ float power2_at(const float4 e0, float r, float lx, f
   return fmaf(dy, fmaf(e0.w, dy, v), sx);
 }
 
+// The row of a pixel that takes no entry (outside the image, its ray stopped or
+// not yet reached): the power there is below every threshold, so the packed
+// walks need no test per pixel.  Far enough for deviations of up to 3e17 pixels
+// (at 1e6 rows a splat of 3e5 pixels passed); finite, as the backward's moments
+// multiply it by a zero weight.
+constexpr float kFarRow = 1.0e18f;
+
 // A shadow ray stops taking occluders once its product A falls below
 // kShadowStop: the occluder that takes A below it is the last one applied.
 // Every receiver behind the stop would see an exact product in
