@@ -61,7 +61,7 @@ BwdPlan plan_bwd(int n, const MlpDev& phi, const MlpDev& psi) {
   p.mlp_in = take(4ull * kMlpIn * n);
   p.wred[0] = take(4ull * mlp_params(phi));
   p.wred[1] = take(4ull * mlp_params(psi));
-  p.ticket = take(12);
+  p.ticket = take(16);
   const size_t sa = mlp_bwd_scratch_bytes(n, phi), sb = mlp_bwd_scratch_bytes(n, psi);
   p.mlp_scratch = take(sa > sb ? sa : sb);  // Phi and Psi use it in turn
   p.ct = take(8ull * n);
@@ -111,6 +111,7 @@ struct CamBwdParams {
   const float* dimg;
   float* cam_geom;  // [N][8] by index: dL/dgamma, sums of w dx, w dy, w dx dy, w dx^2, w dy^2
   float* color;
+  const uint32_t* nonfinite;  // some colour is infinite or not a number
   int W, H, gx, ntiles;
   float amax;
 };
@@ -138,14 +139,13 @@ __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
                : "memory");
 }
 
-template <int NQ>
-__global__ void __launch_bounds__(kCbWarps * 32, 3) k_camera_bwd(CamBwdParams p) {
-  __shared__ CamBwdSmem smem[kCbWarps];
-  CamBwdSmem& B = smem[threadIdx.x >> 5];
+// MASK: a colour or a pixel's gradient is infinite or not a number, so that a
+// zero weight does not cancel it: a pixel adds only the entries it takes.  Without
+// MASK, false if a pixel asks for it (nothing is added then).
+template <int NQ, bool MASK>
+__device__ __forceinline__ bool camera_bwd_strip(const CamBwdParams& p, CamBwdSmem& B, uint32_t unit) {
   const int lane = threadIdx.x & 31;
   constexpr uint32_t kParts = 4 / NQ;  // strips of 4 NQ rows
-  const uint32_t unit = blockIdx.x * kCbWarps + (threadIdx.x >> 5);  // (tile in launch order, strip)
-  if (unit >= kParts * (uint32_t)p.ntiles) return;
   const int tile = (int)p.tile_order[unit / kParts], part = (int)(unit % kParts), half = part * NQ / 2;
   const int tx = tile % p.gx, ty = tile / p.gx;
   const uint32_t hbits = 3u << (2 * half);
@@ -158,6 +158,7 @@ __global__ void __launch_bounds__(kCbWarps * 32, 3) k_camera_bwd(CamBwdParams p)
   // sweep reaches the pixel's last entry), T, D, dL/d(image), Sh, g . S
   f32x2 ly[NQ], T[NQ], D[NQ], gr[NQ], gg[NQ], gb[NQ], sh[NQ], gs[NQ];
   uint32_t nc[2 * NQ], next = 0u;
+  float sum_in = 0.f;
 #pragma unroll
   for (int q = 0; q < NQ; ++q) {
     float t2[2], r2[2], g2[2], b2[2], h2[2], s2[2];
@@ -175,6 +176,7 @@ __global__ void __launch_bounds__(kCbWarps * 32, 3) k_camera_bwd(CamBwdParams p)
         r2[h] = p.dimg[3 * pix]; g2[h] = p.dimg[3 * pix + 1]; b2[h] = p.dimg[3 * pix + 2];
         h2[h] = s.w;
         s2[h] = r2[h] * s.x + g2[h] * s.y + b2[h] * s.z;
+        sum_in += ((r2[h] + g2[h]) + (b2[h] + h2[h])) + s2[h];
       }
       next = max(next, nc[2 * q + h]);
     }
@@ -184,6 +186,7 @@ __global__ void __launch_bounds__(kCbWarps * 32, 3) k_camera_bwd(CamBwdParams p)
     gr[q] = pk2(r2[0], r2[1]); gg[q] = pk2(g2[0], g2[1]); gb[q] = pk2(b2[0], b2[1]);
     sh[q] = pk2(h2[0], h2[1]); gs[q] = pk2(s2[0], s2[1]);
   }
+  if (!MASK && __any_sync(0xffffffffu, non_finite(sum_in))) return false;
   const uint32_t end = __reduce_max_sync(0xffffffffu, next);  // entries some pixel of the strip took
 
   int nrow = 0;
@@ -298,6 +301,7 @@ __global__ void __launch_bounds__(kCbWarps * 32, 3) k_camera_bwd(CamBwdParams p)
           beta = pk2(a0 < p.amax ? lo2(beta) : 0.f, a1 < p.amax ? hi2(beta) : 0.f);
           alpha = pk2(fminf(p.amax, a0), fminf(p.amax, a1));
         }
+        auto taken = [&](f32x2 v) { return MASK ? pk2(lo2(alpha) != 0.f ? lo2(v) : 0.f, hi2(alpha) != 0.f ? hi2(v) : 0.f) : v; };
         const f32x2 om = fma2(alpha, dup2(-1.f), dup2(1.f));
         float ia, ib;
         asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ia) : "f"(lo2(om)));
@@ -312,18 +316,20 @@ __global__ void __launch_bounds__(kCbWarps * 32, 3) k_camera_bwd(CamBwdParams p)
         G = fma2(gs[q], dup2(c0.w), G);
         G = fma2(gr[q], dup2(c1.x), G);
         G = fma2(gg[q], dup2(c1.y), G);
-        G = fma2(gb[q], dup2(c1.z), G);
+        G = taken(fma2(gb[q], dup2(c1.z), G));
         const f32x2 dalpha = fma2(T[q], G, mul2(mul2(inv, dup2(-1.f)), D[q]));
         D[q] = fma2(w, G, D[q]);
-        const f32x2 ws = mul2(w, sh[q]);
-        k0 = fma2(ws, gr[q], k0);
-        k1 = fma2(ws, gg[q], k1);
-        k2 = fma2(ws, gb[q], k2);
-        k3 = fma2(w, gs[q], k3);
-        k4 = fma2(w, gr[q], k4);
-        k5 = fma2(w, gg[q], k5);
-        k6 = fma2(w, gb[q], k6);
-        const f32x2 tt = mul2(dalpha, beta), td = mul2(tt, dy);
+        const f32x2 ws = taken(mul2(w, sh[q])), r = taken(gr[q]), g = taken(gg[q]), b = taken(gb[q]);
+        k0 = fma2(ws, r, k0);
+        k1 = fma2(ws, g, k1);
+        k2 = fma2(ws, b, k2);
+        k3 = fma2(w, taken(gs[q]), k3);
+        k4 = fma2(w, r, k4);
+        k5 = fma2(w, g, k5);
+        k6 = fma2(w, b, k6);
+        f32x2 tt = mul2(dalpha, beta);
+        if (MASK) tt = pk2(lo2(beta) != 0.f ? lo2(tt) : 0.f, hi2(beta) != 0.f ? hi2(tt) : 0.f);
+        const f32x2 td = mul2(tt, dy);
         m0 = add2(m0, tt);
         m1 = add2(m1, td);
         m2 = fma2(td, dy, m2);
@@ -349,6 +355,22 @@ __global__ void __launch_bounds__(kCbWarps * 32, 3) k_camera_bwd(CamBwdParams p)
   }
   if (nrow) flush();
   asm volatile("cp.async.wait_all;" ::: "memory");
+  return true;
+}
+
+// (a call, which leaves the other form as it is without this one)
+template <int NQ>
+__device__ __noinline__ void camera_bwd_strip_masked(const CamBwdParams& p, CamBwdSmem& B, uint32_t unit) {
+  camera_bwd_strip<NQ, true>(p, B, unit);
+}
+
+template <int NQ>
+__global__ void __launch_bounds__(kCbWarps * 32, 4) k_camera_bwd(const __grid_constant__ CamBwdParams p) {
+  __shared__ CamBwdSmem smem[kCbWarps];
+  CamBwdSmem& B = smem[threadIdx.x >> 5];
+  const uint32_t unit = blockIdx.x * kCbWarps + (threadIdx.x >> 5);  // (tile in launch order, strip)
+  if (unit >= 4 / NQ * (uint32_t)p.ntiles) return;
+  if (*p.nonfinite || !camera_bwd_strip<NQ, false>(p, B, unit)) camera_bwd_strip_masked<NQ>(p, B, unit);
 }
 
 __global__ void k_copy_strided(const float* src, int stride, int off, float* dst, int n) {
@@ -755,6 +777,7 @@ gs3_status run_backward(const FrameArgs& f, const float* dimg, void* bws, size_t
     p.dimg = dimg;
     p.cam_geom = cam_geom;
     p.color = color;
+    p.nonfinite = at<uint32_t>(ws, L.header) + H_NONFINITE;
     p.W = L.width; p.H = L.height; p.gx = L.gx; p.ntiles = L.ntiles;
     p.amax = f.opts.alpha_max;
     // quarter tiles while halves leave warp slots free (three blocks per SM); on every

@@ -781,6 +781,7 @@ struct CamParams {
   float* final_t;
   uint32_t* n_contrib;
   float4* pix_aux;
+  const uint32_t* nonfinite;  // some colour is infinite or not a number
   int W, H, gx;
   float amax, tstop;
 };
@@ -975,6 +976,9 @@ __device__ __forceinline__ void camera_walk(const CamParams& p, const CamTile& t
 constexpr int kCamGroup = 4;
 using CamSmem = CamEntries<2, kCamGroup>;
 
+// MASK: the frame has colours that a zero weight does not cancel, so a pixel
+// adds only the entries it takes (their weights are positive).
+template <bool MASK>
 __device__ __forceinline__ void camera_tile(const CamParams& p, int blk, CamSmem (*smem)[2]) {
   CamPixels x;
   const CamTile t = camera_tile_of(p, blk, x);
@@ -997,6 +1001,7 @@ __device__ __forceinline__ void camera_tile(const CamParams& p, int blk, CamSmem
 #pragma unroll
           for (int k = 0; k < 2; ++k) {
             const f32x2 wk = dup2(k ? hi2(w[i]) : lo2(w[i]));
+            if (MASK && lo2(wk) == 0.f) continue;
             acc[k][0] = fma2(wk, c0.x, acc[k][0]);
             acc[k][1] = fma2(wk, c0.y, acc[k][1]);
             acc[k][2] = fma2(wk, c1.x, acc[k][2]);
@@ -1024,17 +1029,25 @@ __device__ __forceinline__ void camera_tile(const CamParams& p, int blk, CamSmem
 
 // One frame (p), or a batch of nreq frames (reqs in device memory) whose
 // tiles follow one another: frame r owns blocks [tile_prefix[r], tile_prefix[r + 1]).
+// (a call, which leaves the other form as it is without this one)
+__device__ __noinline__ void camera_tile_masked(const CamParams& p, int blk, CamSmem (*smem)[2]) {
+  camera_tile<true>(p, blk, smem);
+}
+
 template <bool BATCH>
-__global__ void __launch_bounds__(kCamThreads) k_camera(const CamParams p, const CamParams* reqs, const uint32_t* tile_prefix,
+__global__ void __launch_bounds__(kCamThreads) k_camera(const __grid_constant__ CamParams p, const CamParams* reqs, const uint32_t* tile_prefix,
                                                 int nreq) {
   after_previous();
   __shared__ CamSmem M[kCamThreads / 32][2];
   if (BATCH) {
     int r = 0;
     while (r < nreq - 1 && blockIdx.x >= tile_prefix[r + 1]) ++r;
-    camera_tile(reqs[r], (int)(blockIdx.x - tile_prefix[r]), M);
+    const int blk = (int)(blockIdx.x - tile_prefix[r]);
+    if (*reqs[r].nonfinite) camera_tile_masked(reqs[r], blk, M);
+    else camera_tile<false>(reqs[r], blk, M);
   } else {
-    camera_tile(p, (int)blockIdx.x, M);
+    if (*p.nonfinite) camera_tile_masked(p, (int)blockIdx.x, M);
+    else camera_tile<false>(p, (int)blockIdx.x, M);
   }
 }
 
@@ -1061,8 +1074,8 @@ using EnvSmem = CamEntries<kMaxBatch + 1, kEnvGroup>;  // colours: the lights', 
 
 // The thread layout and entry arithmetic of camera_tile, with 4 accumulators
 // per light and pixel plus 3 for R.
-__global__ void __launch_bounds__(kCamThreads) k_camera_env(const EnvCamParams e) {
-  __shared__ EnvSmem M[kCamThreads / 32][2];
+template <bool MASK>
+__device__ __forceinline__ void camera_env_tile(const EnvCamParams& e, EnvSmem (*M)[2]) {
   const CamParams& p = e.c;
   const int nl = e.nl;
   CamPixels x;
@@ -1091,6 +1104,7 @@ __global__ void __launch_bounds__(kCamThreads) k_camera_env(const EnvCamParams e
           const ulonglong2 r = *reinterpret_cast<const ulonglong2*>(&E.col[k0 + i][kMaxBatch]);
 #pragma unroll
           for (int k = 0; k < 2; ++k) {
+            if (MASK && lo2(wk[k]) == 0.f) continue;
             R[k][0] = fma2(wk[k], r.x, R[k][0]);
             R[k][1] = fma2(wk[k], r.y, R[k][1]);
           }
@@ -1100,6 +1114,7 @@ __global__ void __launch_bounds__(kCamThreads) k_camera_env(const EnvCamParams e
               const ulonglong2 c = *reinterpret_cast<const ulonglong2*>(&E.col[k0 + i][l]);
 #pragma unroll
               for (int k = 0; k < 2; ++k) {
+                if (MASK && lo2(wk[k]) == 0.f) continue;
                 S[k][l][0] = fma2(wk[k], c.x, S[k][l][0]);
                 S[k][l][1] = fma2(wk[k], c.y, S[k][l][1]);
               }
@@ -1136,6 +1151,17 @@ __global__ void __launch_bounds__(kCamThreads) k_camera_env(const EnvCamParams e
     p.final_t[pix] = k ? hi2(x.T) : lo2(x.T);
     p.n_contrib[pix] = x.consumed[k];
   }
+}
+
+// (a call, which leaves the other form as it is without this one)
+__device__ __noinline__ void camera_env_tile_masked(const EnvCamParams& e, EnvSmem (*M)[2]) {
+  camera_env_tile<true>(e, M);
+}
+
+__global__ void __launch_bounds__(kCamThreads) k_camera_env(const __grid_constant__ EnvCamParams e) {
+  __shared__ EnvSmem M[kCamThreads / 32][2];
+  if (*e.c.nonfinite) camera_env_tile_masked(e, M);
+  else camera_env_tile<false>(e, M);
 }
 
 // Launch order of a splat's tiles: longest list first, so that the last
@@ -1283,6 +1309,7 @@ CamParams camera_params(const FrameArgs& f, float* out_rgb) {
   p.final_t = at<float>(ws, f.L->final_t);
   p.n_contrib = at<uint32_t>(ws, f.L->n_contrib);
   p.pix_aux = at<float4>(ws, f.L->pix_aux);
+  p.nonfinite = at<uint32_t>(ws, f.L->header) + H_NONFINITE;
   p.W = f.L->width; p.H = f.L->height; p.gx = f.L->gx;
   p.amax = f.opts.alpha_max; p.tstop = f.opts.t_stop;
   p.tile_order = at<uint32_t>(ws, f.L->tile_order[0]);  // from the camera binning stage

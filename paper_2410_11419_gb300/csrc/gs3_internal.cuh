@@ -104,7 +104,14 @@ const char* light_problem(const gs3_light& l, const gs3_render_opts& o);
 enum { H_STATUS = 0, H_PAIRS_CAM = 1, H_PAIRS_LIGHT = 2, H_NEED_CAM = 3, H_NEED_LIGHT = 4,
        H_LIGHT_VIEW = 8, H_LIGHT_ORTHO = 20,
        H_RESET_WORDS = 24,  // words a render resets; the rest survive across renders
-       H_ENV = 24 };        // environment render: status, pairs cam/light, needed cam/light
+       H_ENV = 24,          // environment render: status, pairs cam/light, needed cam/light
+       // A colour that is infinite or not a number went to the camera composite since the
+       // camera's splats were last projected: the camera composite and its backward then
+       // keep it from the pixels that do not take it (their products with its zero
+       // weight are not numbers).  Every kernel that writes a colour reports it.
+       H_NONFINITE = 32 };
+
+__device__ __forceinline__ bool non_finite(float x) { return !(fabsf(x) <= 3.402823466e38f); }
 
 // The light in homogeneous form (x, y, z, w): a point light (pos, 1) or a
 // directional light (dir / |dir|, 0).  omega_i = normalize(L.xyz - L.w mu)

@@ -39,6 +39,7 @@ struct MlpParams {
   float4 light[kMaxBatch];         // homogeneous light per light (light_h)
   float cam_pos[3];
   float* res_idx;    // Psi: float4 residual [N] (as floats)
+  uint32_t* nonfinite;
   float4* ccol;      // camera colours by rank: Phi T' into .w of [2r] (nl = 1), Psi residual into [2r + 1]
   float4* envcol;    // non-null (Phi): (shade_l, T'_l) at [r nl + l] instead of ccol
   const uint32_t* rank_of;
@@ -51,8 +52,10 @@ __device__ __forceinline__ void put_phi(const MlpParams& p, int l, int g, uint32
   if (p.envcol) {
     const float4 c = p.shade[l][g];
     p.envcol[(size_t)r * p.nl + l] = make_float4(c.x, c.y, c.z, y);
+    if (non_finite(c.x + c.y + c.z + y)) *p.nonfinite = 1u;
   } else {
     p.ccol[2 * r].w = y;
+    if (non_finite(y)) *p.nonfinite = 1u;
   }
 }
 
@@ -169,6 +172,7 @@ __global__ void __launch_bounds__(256) k_mlp(MlpParams p) {
       } else {
         p.res_idx[4 * g + o] = y;
         reinterpret_cast<float*>(&p.ccol[2 * r + 1])[o] = y;
+        if (non_finite(y)) *p.nonfinite = 1u;
       }
     }
   }
@@ -196,6 +200,7 @@ void launch_mlp(const FrameArgs& f, cudaStream_t s, bool identity_only, int whic
   p.res_idx = at<float>(f.ws, f.L->res);
   p.ccol = at<float4>(f.ws, f.L->ccol);
   p.envcol = nullptr;
+  p.nonfinite = at<uint32_t>(f.ws, f.L->header) + H_NONFINITE;
   p.rank_of = at<uint32_t>(f.ws, f.L->sp[0].rank_of);
 
   int x3 = 0;  // networks that the tensor cores take
@@ -230,6 +235,7 @@ void launch_phi_lights(const FrameArgs* const* f, int nl, float4* envcol, cudaSt
   p.res_idx = nullptr;
   p.ccol = nullptr;
   p.envcol = envcol;
+  p.nonfinite = at<uint32_t>(f0.ws, f0.L->header) + H_NONFINITE;
   p.rank_of = at<uint32_t>(f0.ws, f0.L->sp[0].rank_of);
   p.identity = (f0.opts.ablate & GS3_ABLATE_PHI) != 0;
   if (!p.identity && mlp_x3_supported(p.net)) launch_phi_lights_x3(f, nl, envcol, s);

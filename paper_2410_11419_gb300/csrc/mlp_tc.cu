@@ -75,7 +75,7 @@ struct TcParams {
   float4* ccol;    // camera colours by rank (nl = 1)
   float4* envcol;  // non-null (Phi): (shade_l, T'_l) at [r nl + l] instead of ccol
   const uint32_t* rank_of;
-  uint32_t* status;
+  uint32_t *status, *nonfinite;
 };
 
 // [v, sin(2^q pi v), cos(2^q pi v)], q = 0..3.  Band 0 is evaluated; each
@@ -311,8 +311,10 @@ __global__ void __launch_bounds__(kTcThreads * kTcMaxGroups, 1) k_mlp_tc(TcParam
         if (p.envcol) {
           const float4 c = p.shade[li][g];
           p.envcol[(size_t)r * p.nl + li] = make_float4(c.x, c.y, c.z, y);
+          if (non_finite(c.x + c.y + c.z + y)) *p.nonfinite = 1u;
         } else {
           p.ccol[2 * r].w = y;
+          if (non_finite(y)) *p.nonfinite = 1u;
         }
       } else {
         float4 y;
@@ -322,6 +324,7 @@ __global__ void __launch_bounds__(kTcThreads * kTcMaxGroups, 1) k_mlp_tc(TcParam
         y.w = 0.f;
         reinterpret_cast<float4*>(p.out[0])[g] = y;
         p.ccol[2 * r + 1] = y;
+        if (non_finite(y.x + y.y + y.z)) *p.nonfinite = 1u;
       }
     }
   }
@@ -538,6 +541,7 @@ TcParams tc_params(const FrameArgs& f, int which, const unsigned char* blob) {
   p.envcol = nullptr;
   p.rank_of = at<uint32_t>(f.ws, f.L->sp[0].rank_of);
   p.status = at<uint32_t>(f.ws, f.L->header) + H_STATUS;
+  p.nonfinite = at<uint32_t>(f.ws, f.L->header) + H_NONFINITE;
   return p;
 }
 

@@ -51,7 +51,7 @@ struct X3Params {
   float4* ccol;    // camera colours by rank (nl = 1)
   float4* envcol;  // non-null (Phi): (shade_l, T'_l) at [r nl + l] instead of ccol
   const uint32_t* rank_of;
-  uint32_t* status;
+  uint32_t *status, *nonfinite;
 };
 
 // ---- packing -----------------------------------------------------------------
@@ -275,13 +275,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_x3(X3Params p) {
           if (p.envcol) {
             const float4 c = p.shade[li][g];
             p.envcol[(size_t)rk * p.nl + li] = make_float4(c.x, c.y, c.z, y[0]);
+            if (non_finite(c.x + c.y + c.z + y[0])) *p.nonfinite = 1u;
           } else {
             p.ccol[2 * rk].w = y[0];
+            if (non_finite(y[0])) *p.nonfinite = 1u;
           }
         } else {
           const float4 res = make_float4(y[0], y[1], y[2], 0.f);
           reinterpret_cast<float4*>(p.out[0])[g] = res;
           p.ccol[2 * rk + 1] = res;
+          if (non_finite(y[0] + y[1] + y[2])) *p.nonfinite = 1u;
         }
       }
       // the next tile's partial sums wait for this read
@@ -327,6 +330,7 @@ X3Params x3_params(const FrameArgs& f, int which) {
   p.envcol = nullptr;
   p.rank_of = at<uint32_t>(f.ws, f.L->sp[0].rank_of);
   p.status = at<uint32_t>(f.ws, f.L->header) + H_STATUS;
+  p.nonfinite = at<uint32_t>(f.ws, f.L->header) + H_NONFINITE;
   return p;
 }
 

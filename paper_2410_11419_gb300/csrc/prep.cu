@@ -343,6 +343,7 @@ __global__ void __launch_bounds__(kPrepThreads, 12) k_prep(const __grid_constant
   __shared__ float sR[9], st[3], sortho;
   __shared__ ViewD slv;
   const int parts = 3 - p.part0, part = p.part0 + (int)blockIdx.x % parts, block = (int)blockIdx.x / parts;
+  if (part == 0 && block == 0 && threadIdx.x == 0) p.header[H_NONFINITE] = 0u;
   if (part == 1) {
     if (threadIdx.x == 0) {
       sortho = light_view_any_rn(p.light, p.o.target, p.cam.W, p.cam.H, sR, st);

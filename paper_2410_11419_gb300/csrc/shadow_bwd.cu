@@ -65,19 +65,21 @@ struct BwdParams {
   const uint32_t* light_stop;
   const float2* ct;    // by light rank: (coef_j, T_j)
   float* seg_sum;      // [item][256]: a segment's own sum per ray, then the later segments'
-  uint32_t* ticket;    // [3]
+  uint32_t* ticket;    // [4]: three tickets, and whether some coef_j is infinite or not a number
   float* light_geom;   // [N][8] by index: dL/dgamma, sums of w dx, w dy, w dx dy, w dx^2, w dy^2
   int W, H, gx, ntiles;
   float amax;
 };
 
 __global__ void k_bwd_coef(const uint32_t* __restrict__ order, const float* __restrict__ dT,
-                           const float* __restrict__ den, const float* __restrict__ T, float2* __restrict__ ct, int n) {
+                           const float* __restrict__ den, const float* __restrict__ T, float2* __restrict__ ct, uint32_t* nonfinite, int n) {
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= n) return;
   const uint32_t g = order[r];
   const float d = den[g];
-  ct[r] = make_float2(d > 0.f ? dT[g] / d : 0.f, T[g]);
+  const float c = d > 0.f ? dT[g] / d : 0.f;
+  ct[r] = make_float2(c, T[g]);
+  if (non_finite(c)) *nonfinite = 1u;
 }
 
 __device__ __forceinline__ void red_add2(float* p, float x, float y) {
@@ -90,6 +92,14 @@ struct SumSmem {  // one warp's
   float coef[32];
 };
 
+// x where b is not 0, else 0.  With MASK (here and below) a coefficient is
+// infinite or not a number, and a pixel that does not pass must not see it.
+template <bool MASK>
+__device__ __forceinline__ f32x2 where_passing(f32x2 b, f32x2 x) {
+  return MASK ? pk2(lo2(b) != 0.f ? lo2(x) : 0.f, hi2(b) != 0.f ? hi2(x) : 0.f) : x;
+}
+
+template <bool MASK>
 __device__ __forceinline__ void sum_item(const BwdParams& p, uint32_t w, SumSmem& S, int lane) {
   const SegItem it = seg_item(p, w, lane);
   if (it.first) return;
@@ -133,7 +143,10 @@ __device__ __forceinline__ void sum_item(const BwdParams& p, uint32_t w, SumSmem
         const f32x2 c = dup2(S.coef[t]);
 #pragma unroll
         for (int q = 0; q < kPx / 2; ++q)
-          if (bits & (q < 2 ? 0x3u : 0xCu)) sum[q] = fma2(mul2(c, beta2_at(e, ly[q])), P[q], sum[q]);
+          if (bits & (q < 2 ? 0x3u : 0xCu)) {
+            const f32x2 b = beta2_at(e, ly[q]);
+            sum[q] = fma2(where_passing<MASK>(b, mul2(c, b)), P[q], sum[q]);
+          }
       } else {
         if (bits & 0x3u) occ_half<0>(ly, P, e, gb.x, omin);
         if (bits & 0xCu) occ_half<1>(ly, P, e, gb.x, omin);
@@ -149,12 +162,21 @@ __device__ __forceinline__ void sum_item(const BwdParams& p, uint32_t w, SumSmem
   }
 }
 
-__global__ void __launch_bounds__(kBwdWarps * 32, 6) k_shadow_bwd_sums(const BwdParams p) {
+// (the masked forms are calls, which leaves the others as they are without them)
+__device__ __noinline__ void sum_item_masked(const BwdParams& p, uint32_t w, SumSmem& S, int lane) {
+  sum_item<true>(p, w, S, lane);
+}
+
+__global__ void __launch_bounds__(kBwdWarps * 32, 6) k_shadow_bwd_sums(const __grid_constant__ BwdParams p) {
   __shared__ SumSmem smem[kBwdWarps];
   const int lane = threadIdx.x & 31;
   const uint32_t total = p.counts[0];
+  const bool mask = p.ticket[3] != 0u;
   uint32_t w;
-  while (next_item(p.ticket, total, lane, w)) sum_item(p, p.open_list[w], smem[threadIdx.x >> 5], lane);
+  while (next_item(p.ticket, total, lane, w)) {
+    if (mask) sum_item_masked(p, p.open_list[w], smem[threadIdx.x >> 5], lane);
+    else sum_item<false>(p, p.open_list[w], smem[threadIdx.x >> 5], lane);
+  }
 }
 
 // One warp per tile: seg_sum of each open segment becomes the sum over the
@@ -208,13 +230,14 @@ struct Moments {
 };
 
 // A receiver's four rays of one half
-template <int H>
+template <int H, bool MASK>
 __device__ __forceinline__ void recv_bwd(const f32x2 (&ly)[kPx / 2], const f32x2 (&A)[kPx / 2], f32x2 (&S)[kPx / 2],
                                          const ColTerms& e, f32x2 coef, f32x2 nT, Moments& m) {
 #pragma unroll
   for (int q = 2 * H; q < 2 * H + 2; ++q) {
     const f32x2 dy = add2(ly[q], e.ny);
-    const f32x2 cb = mul2(coef, beta2_of(fma2(dy, fma2(e.c, dy, e.v), e.s), e.thr));
+    const f32x2 b = beta2_of(fma2(dy, fma2(e.c, dy, e.v), e.s), e.thr);
+    const f32x2 cb = where_passing<MASK>(b, mul2(coef, b));
     S[q] = fma2(cb, A[q], S[q]);
     const f32x2 w = mul2(cb, add2(A[q], nT)), wd = mul2(w, dy);
     m.m0 = add2(m.m0, w);
@@ -226,7 +249,7 @@ __device__ __forceinline__ void recv_bwd(const f32x2 (&ly)[kPx / 2], const f32x2
 // Undoing an occluder on four rays of one half; the moments are those of
 // S beta / (1 - alpha) (its factor -gamma is applied to their sums).  CLAMP:
 // gamma may reach alpha_max, where alpha is clamped and passes no gradient.
-template <int H, bool CLAMP>
+template <int H, bool CLAMP, bool MASK>
 __device__ __forceinline__ void occ_bwd(const f32x2 (&ly)[kPx / 2], f32x2 (&A)[kPx / 2], const f32x2 (&S)[kPx / 2],
                                         const ColTerms& e, float ngamma, float amax, Moments& m) {
 #pragma unroll
@@ -240,13 +263,14 @@ __device__ __forceinline__ void occ_bwd(const f32x2 (&ly)[kPx / 2], f32x2 (&A)[k
     }
     const f32x2 inv = rcp2(f);
     A[q] = mul2(A[q], inv);
-    const f32x2 w = mul2(mul2(S[q], inv), b), wd = mul2(w, dy);
+    const f32x2 w = where_passing<MASK>(b, mul2(mul2(S[q], inv), b)), wd = mul2(w, dy);
     m.m0 = add2(m.m0, w);
     m.m1 = add2(m.m1, wd);
     m.m2 = fma2(wd, dy, m.m2);
   }
 }
 
+template <bool MASK>
 __device__ __forceinline__ void bwd_item(const BwdParams& p, uint32_t w, BwdSmem& B, int lane) {
   const SegItem it = seg_item(p, w, lane);
   if (it.R1 <= it.R0) return;
@@ -360,8 +384,8 @@ __device__ __forceinline__ void bwd_item(const BwdParams& p, uint32_t w, BwdSmem
         if (!bits) continue;
         const ColTerms e = col_terms(lx, B.e, t);
         const float2 ct = B.ct[t];
-        if (bits & 0x3u) recv_bwd<0>(ly, A, S, e, dup2(ct.x), dup2(-ct.y), m);
-        if (bits & 0xCu) recv_bwd<1>(ly, A, S, e, dup2(ct.x), dup2(-ct.y), m);
+        if (bits & 0x3u) recv_bwd<0, MASK>(ly, A, S, e, dup2(ct.x), dup2(-ct.y), m);
+        if (bits & 0xCu) recv_bwd<1, MASK>(ly, A, S, e, dup2(ct.x), dup2(-ct.y), m);
       } else {
         const uint32_t kk = k - 1u - (uint32_t)(t - __popc(M & ((1u << t) - 1u)));
         if (next == kk + 1u) {  // rays that ended at this occluder: once per ray
@@ -383,11 +407,11 @@ __device__ __forceinline__ void bwd_item(const BwdParams& p, uint32_t w, BwdSmem
         if (!bits) continue;
         const ColTerms e = col_terms(lx, B.e, t);
         if (-gb.x * 1.00001f < p.amax) {  // gamma beta stays below alpha_max (beta <= 1 up to rounding)
-          if (bits & 0x3u) occ_bwd<0, false>(ly, A, S, e, gb.x, p.amax, m);
-          if (bits & 0xCu) occ_bwd<1, false>(ly, A, S, e, gb.x, p.amax, m);
+          if (bits & 0x3u) occ_bwd<0, false, MASK>(ly, A, S, e, gb.x, p.amax, m);
+          if (bits & 0xCu) occ_bwd<1, false, MASK>(ly, A, S, e, gb.x, p.amax, m);
         } else {
-          if (bits & 0x3u) occ_bwd<0, true>(ly, A, S, e, gb.x, p.amax, m);
-          if (bits & 0xCu) occ_bwd<1, true>(ly, A, S, e, gb.x, p.amax, m);
+          if (bits & 0x3u) occ_bwd<0, true, MASK>(ly, A, S, e, gb.x, p.amax, m);
+          if (bits & 0xCu) occ_bwd<1, true, MASK>(ly, A, S, e, gb.x, p.amax, m);
         }
       }
       push(t, m, lx - B.e.xart[t].x);
@@ -398,13 +422,21 @@ __device__ __forceinline__ void bwd_item(const BwdParams& p, uint32_t w, BwdSmem
   }
 }
 
-__global__ void __launch_bounds__(kBwdWarps * 32, 4) k_shadow_bwd(const BwdParams p) {
+__device__ __noinline__ void bwd_item_masked(const BwdParams& p, uint32_t w, BwdSmem& B, int lane) {
+  bwd_item<true>(p, w, B, lane);
+}
+
+__global__ void __launch_bounds__(kBwdWarps * 32, 4) k_shadow_bwd(const __grid_constant__ BwdParams p) {
   after_previous();
   __shared__ BwdSmem smem[kBwdWarps];
   const int lane = threadIdx.x & 31;
   const uint32_t total = p.counts[0];
   uint32_t w;
-  while (next_item(p.ticket + 1, total, lane, w)) bwd_item(p, p.open_list[w], smem[threadIdx.x >> 5], lane);
+  const bool mask = p.ticket[3] != 0u;
+  while (next_item(p.ticket + 1, total, lane, w)) {
+    if (mask) bwd_item_masked(p, p.open_list[w], smem[threadIdx.x >> 5], lane);
+    else bwd_item<false>(p, p.open_list[w], smem[threadIdx.x >> 5], lane);
+  }
 }
 
 // ---- stopped segments ---------------------------------------------------------
@@ -558,7 +590,7 @@ void launch_shadow_backward(const FrameArgs& f, const ShadowBwdArgs& a, cudaStre
   p.amax = f.opts.alpha_max;
   const BwdOccupancy o = bwd_occupancy();
   const int nsm = device_sm_count();
-  k_bwd_coef<<<(n + 255) / 256, 256, 0, s>>>(p.order, a.dT, at<float>(ws, L.shadow_den), at<float>(ws, L.T), a.ct, n);
+  k_bwd_coef<<<(n + 255) / 256, 256, 0, s>>>(p.order, a.dT, at<float>(ws, L.shadow_den), at<float>(ws, L.T), a.ct, a.ticket + 3, n);
   if (side != s) {
     cudaEventRecord(a.fork, s);
     cudaStreamWaitEvent(side, a.fork, 0);

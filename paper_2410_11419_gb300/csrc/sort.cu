@@ -351,7 +351,8 @@ __global__ void __launch_bounds__(kBinBlock) k_reorder(int n, const uint32_t* __
                                                        const SplatRec* __restrict__ rec, SplatRec* __restrict__ rrec,
                                                        uint32_t* __restrict__ rank_of, uint32_t* __restrict__ cnt,
                                                        const float4* __restrict__ shade, float4* __restrict__ ccol,
-                                                       uint32_t* __restrict__ row_cnt, int gy, uint32_t* __restrict__ ticket) {
+                                                       uint32_t* __restrict__ row_cnt, int gy, uint32_t* __restrict__ ticket,
+                                                       uint32_t* nonfinite) {
   after_previous();
   __shared__ int d[kMaxTileAxis + 1];
   __shared__ uint32_t tiles;
@@ -378,6 +379,7 @@ __global__ void __launch_bounds__(kBinBlock) k_reorder(int n, const uint32_t* __
     if (ccol) {
       const float4 col = shade[g];
       ccol[2 * r] = make_float4(col.x, col.y, col.z, 0.f);
+      if (non_finite(col.x + col.y + col.z)) *nonfinite = 1u;
     }
   }
   c = __reduce_add_sync(0xffffffffu, c);
@@ -470,7 +472,7 @@ void launch_depth_sort(const FrameArgs& f, int sp, cudaStream_t s) {
   launch_after(k_reorder, f.L->nb_rows, kBinBlock, 0, s, n, at<uint32_t>(ws, b.sv[1]), at<SplatRec>(ws, b.rec), at<SplatRec>(ws, b.rrec),
       at<uint32_t>(ws, b.rank_of), at<uint32_t>(ws, b.cnt), at<float4>(ws, f.L->shade),
       sp == 0 ? at<float4>(ws, f.L->ccol) : nullptr, at<uint32_t>(ws, b.row_cnt), f.L->gy,
-               at<uint32_t>(ws, b.bin_plan) + 3 * f.L->gy + 3);
+               at<uint32_t>(ws, b.bin_plan) + 3 * f.L->gy + 3, at<uint32_t>(ws, f.L->header) + H_NONFINITE);
   count_launch();
 }
 
