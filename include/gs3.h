@@ -445,9 +445,25 @@ gs3_status gs3_server_destroy(gs3_server *server);
  * array: calls whose
  * work overlaps on the GPU (other streams, other host threads) race and must
  * be serialised by the caller.  Nothing in the array needs to start at zero:
- * each call clears or overwrites all scratch it reads. */
+ * each call clears or overwrites all scratch it reads.
+ * The sort's blocks wait for one another's counts, with a bound.  If a wait runs
+ * out (GS3_ERR_TIMEOUT: the device made no progress for about a second), order_out
+ * is not a permutation and the call, which is asynchronous, has still returned
+ * GS3_OK: gs3_depth_order_static_status tells. */
 #define GS3_STATIC_SORT_MAX_KEYS 1048576u
 gs3_status gs3_depth_order_static(const uint32_t *keys, uint32_t n, uint32_t *order_out, void *stream);
+
+/* Synchronises `stream` and writes to *status_out (host) the outcome of the last
+ * gs3_depth_order_static with n > 0 on the current device: GS3_OK or
+ * GS3_ERR_TIMEOUT.  Errors: INVALID_ARG, CUDA. */
+gs3_status gs3_depth_order_static_status(uint32_t *status_out, void *stream);
+
+/* Self-test of that report: a static sort of n zero keys (4096 < n <=
+ * GS3_STATIC_SORT_MAX_KEYS) whose first pass waits for words that no block writes,
+ * gives up after its poll bound and records GS3_ERR_TIMEOUT.  Allocates and frees
+ * the keys, synchronises the device, and writes the status (read back as above) to
+ * *status_out. */
+gs3_status gs3_selftest_depth_order_timeout(uint32_t n, uint32_t *status_out);
 
 /* ---- Self-test of the bounded device waits ------------------------------
  * Not an operation of the paper: a check that a device-side wait which can

@@ -158,6 +158,8 @@ SIGNATURES = {
     "gs3_server_reset_counters": (C.c_int, [_SERVER_P]),
     "gs3_server_destroy": (C.c_int, [_SERVER_P]),
     "gs3_depth_order_static": (C.c_int, [C.c_void_p, C.c_uint32, C.c_void_p, C.c_void_p]),
+    "gs3_depth_order_static_status": (C.c_int, [C.POINTER(C.c_uint32), C.c_void_p]),
+    "gs3_selftest_depth_order_timeout": (C.c_int, [C.c_uint32, C.POINTER(C.c_uint32)]),
     "gs3_selftest_wait_timeout": (C.c_int, [C.c_uint32, C.POINTER(C.c_uint32)]),
     "gs3_selftest_shadow_wait": (C.c_int, [_SCENE_P, C.POINTER(gs3_camera), C.POINTER(gs3_light),
                                            C.POINTER(gs3_render_opts), C.c_void_p, C.c_size_t, C.c_size_t,
@@ -363,6 +365,20 @@ GS3_STATIC_SORT_MAX_KEYS = 1048576
 def gs3_depth_order_static(keys, n: int, order_out, stream: int) -> None:
     _check(lib().gs3_depth_order_static(_ptr(keys), n, _ptr(order_out), stream),
            "gs3_depth_order_static")
+
+
+def gs3_depth_order_static_status(stream: int) -> int:
+    """GS3_OK or GS3_ERR_TIMEOUT: the outcome of the current device's last static sort (synchronises)."""
+    out = C.c_uint32(0)
+    _check(lib().gs3_depth_order_static_status(C.byref(out), stream), "gs3_depth_order_static_status")
+    return out.value
+
+
+def gs3_selftest_depth_order_timeout(n: int) -> int:
+    """Status of a static sort whose first pass waits in vain (GS3_ERR_TIMEOUT)."""
+    out = C.c_uint32(0)
+    _check(lib().gs3_selftest_depth_order_timeout(n, C.byref(out)), "gs3_selftest_depth_order_timeout")
+    return out.value
 
 
 def gs3_selftest_wait_timeout(n: int) -> int:

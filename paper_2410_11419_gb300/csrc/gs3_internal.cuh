@@ -310,12 +310,14 @@ constexpr size_t onesweep_bytes(int nblocks, int passes) {
 }
 
 // The stable ascending order of n <= GS3_STATIC_SORT_MAX_KEYS keys (the
-// sort's position of rank r at order[r]).  k0, v0, k1: n words each;
-// look_region: onesweep_bytes(kDepthOrderBlocks, 4) bytes; status: a word that
-// is set to GS3_ERR_TIMEOUT (from 0) if a bounded wait runs out.
+// sort's position of rank r at order[r]).  k0, v0, k1: n words each; front:
+// kOrderFront bytes, of which the first word becomes GS3_OK or, if a bounded wait
+// runs out, GS3_ERR_TIMEOUT, then a look-back region of
+// onesweep_bytes(kDepthOrderBlocks, 4) bytes.  first_ticket: see onesweep_sort.
 constexpr int kDepthOrderBlocks = 512;
+constexpr size_t kOrderFront = 256;  // the look-back words stay on 128-byte lines (300k keys: 49 us, 55 off them)
 void depth_order(const uint32_t* keys, uint32_t n, uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* order,
-                 unsigned char* look_region, uint32_t* status, cudaStream_t s);
+                 unsigned char* front, cudaStream_t s, int first_ticket = 0);
 
 // false when [ptr, ptr + bytes) provably leaves ptr's device allocation
 bool device_range_ok(const void* ptr, size_t bytes);

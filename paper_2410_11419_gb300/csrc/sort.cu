@@ -240,15 +240,18 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_onesweep(
 // ---------------------------------------------------------------------------
 // The whole depth sort of at most kSmallSort keys by one block: the four passes
 // of k_onesweep with the keys in registers and shared memory between them, and
-// no look-back.  Warp w holds the 32 R consecutive keys from 32 R w on.
+// no look-back.  Warp w holds the 32 R consecutive keys from 32 R w on.  It waits for
+// nothing, and sets *status (if given) to 0.
 // Bound: the passes' chains of barriers.  1000 / 4000 keys: 9 / 19 us, against 21 / 23
 // in six launches (4096: 19.3 against 22.8); past that several blocks gain.
 constexpr int kSmallSort = 4096;
 constexpr int kSmallThreads = 512;
 __global__ void __launch_bounds__(kSmallThreads) k_sort_small(const uint32_t* __restrict__ kin,
                                                               uint32_t* __restrict__ kout,
-                                                              uint32_t* __restrict__ vout, uint32_t n) {
+                                                              uint32_t* __restrict__ vout, uint32_t n,
+                                                              uint32_t* status) {
   after_previous();
+  if (status && threadIdx.x == 0) *status = 0u;
   constexpr int kWarps = kSmallThreads / 32, kRounds = kSmallSort / kSmallThreads;
   __shared__ uint32_t key[kSmallSort];
   __shared__ uint16_t val[kSmallSort];
@@ -409,12 +412,16 @@ __global__ void __launch_bounds__(kBinBlock) k_reorder(int n, const uint32_t* __
 // odd passes (k1, v1), each reading the previous pass's output (pass 0 reads
 // (kin, vin)).  look_region: onesweep_bytes(nblocks, PASSES) bytes, zeroed here.
 // Up to kSmallSort keys: one launch of k_sort_small, whose output is (k1, v1).
+// own_status: the kOrderFront bytes before look_region belong to the sort and start
+// with `header`, the word for its status, which is cleared as well.  first_ticket: of
+// the first pass (past 0: a self-test, its waits run out).
 template <int ROUNDS, int PASSES>
 void onesweep_sort(const uint32_t* kin, const uint32_t* vin, uint32_t* k0, uint32_t* v0, uint32_t* k1,
                    uint32_t* v1, const uint32_t* n_ptr, uint32_t n_fixed, int nblocks, int passes,
-                   unsigned char* look_region, uint32_t* header, cudaStream_t s) {
+                   unsigned char* look_region, uint32_t* header, cudaStream_t s, bool own_status = false,
+                   int first_ticket = 0) {
   if (!n_ptr && !vin && n_fixed <= kSmallSort && passes == 4) {
-    launch_after(k_sort_small, 1, kSmallThreads, 0, s, kin, k1, v1, n_fixed);
+    launch_after(k_sort_small, 1, kSmallThreads, 0, s, kin, k1, v1, n_fixed, own_status ? header : nullptr);
     count_launch();
     return;
   }
@@ -426,7 +433,9 @@ void onesweep_sort(const uint32_t* kin, const uint32_t* vin, uint32_t* k0, uint3
   unsigned long long* look = reinterpret_cast<unsigned long long*>(look_region);
   uint32_t* tickets = reinterpret_cast<uint32_t*>(look + 256 * (size_t)nblocks);
   uint32_t* totals = tickets + PASSES;
-  cudaMemsetAsync(look_region, 0, onesweep_bytes(nblocks, PASSES), s);
+  const size_t front = own_status ? kOrderFront : 0;
+  cudaMemsetAsync(look_region - front, 0, front + onesweep_bytes(nblocks, PASSES), s);
+  if (first_ticket) cudaMemsetAsync(tickets, first_ticket, 1, s);
   const int tb_cap = device_sm_count() * 4;
   int tb = n_ptr ? tb_cap : (int)((n_fixed + 1023) / 1024);
   if (tb < 1) tb = 1;
@@ -450,12 +459,14 @@ void onesweep_sort(const uint32_t* kin, const uint32_t* vin, uint32_t* k0, uint3
 // (GS3_STATIC_SORT_MAX_KEYS is 512 such blocks), so that a few hundred thousand
 // keys fill the chip and the look-back region stays at 1 MB.
 void depth_order(const uint32_t* keys, uint32_t n, uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* order,
-                 unsigned char* look_region, uint32_t* status, cudaStream_t s) {
+                 unsigned char* front, cudaStream_t s, int first_ticket) {
+  unsigned char* look = front + kOrderFront;
+  uint32_t* status = reinterpret_cast<uint32_t*>(front);
   auto blocks = [&](int rounds) { return (int)((n + kSortThreads * rounds - 1) / (kSortThreads * rounds)); };
   if (blocks(4) <= kDepthOrderBlocks)
-    onesweep_sort<4, 4>(keys, nullptr, k0, v0, k1, order, nullptr, n, blocks(4), 4, look_region, status, s);
+    onesweep_sort<4, 4>(keys, nullptr, k0, v0, k1, order, nullptr, n, blocks(4), 4, look, status, s, true, first_ticket);
   else
-    onesweep_sort<8, 4>(keys, nullptr, k0, v0, k1, order, nullptr, n, blocks(8), 4, look_region, status, s);
+    onesweep_sort<8, 4>(keys, nullptr, k0, v0, k1, order, nullptr, n, blocks(8), 4, look, status, s, true, first_ticket);
 }
 
 void launch_depth_sort(const FrameArgs& f, int sp, cudaStream_t s) {
