@@ -91,8 +91,8 @@ BwdPlan plan_bwd(int n, const MlpDev& phi, const MlpDev& psi) {
 // while the current ones are walked, as in the forward.  The 14 terms of four
 // entries are added over the 32 lanes through shared-memory rows.
 // Bound: issue slots.  Object workload (300k Gaussians, 800 x 800): 1.24 ms with
-// a pixel per thread and a 16-shuffle butterfly per entry and warp, 0.57 ms so
-// (0.58 at 4 blocks per SM, 0.62 at 5).
+// a pixel per thread and a 16-shuffle butterfly per entry and warp, 0.60 ms so
+// (0.57 with T times the reciprocal in place of a rounded quotient).
 // ---------------------------------------------------------------------------
 constexpr int kCbWarps = 4;  // independent warps per block
 constexpr int kCbRows = 4;   // entries whose lane sums are added together
@@ -306,9 +306,15 @@ __device__ __forceinline__ bool camera_bwd_strip(const CamBwdParams& p, CamBwdSm
         float ia, ib;
         asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ia) : "f"(lo2(om)));
         asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(ib) : "f"(hi2(om)));
-        f32x2 inv = pk2(ia, ib);  // one Newton step: within an ulp, and exactly 1 for alpha = 0
-        inv = fma2(inv, fma2(pk2(-lo2(om), -hi2(om)), inv, dup2(1.f)), inv);
-        T[q] = mul2(T[q], inv);
+        // the reciprocal by a Newton step (exactly 1 for alpha = 0), and with it the
+        // quotient T / (1 - alpha), corrected by its remainder, which rounds it as a
+        // division does (Markstein 1990): T times the reciprocal repeats the
+        // reciprocal's rounding at every entry of that alpha
+        const f32x2 nom = pk2(-lo2(om), -hi2(om));
+        f32x2 inv = pk2(ia, ib);
+        inv = fma2(inv, fma2(nom, inv, dup2(1.f)), inv);
+        const f32x2 quot = mul2(T[q], inv);
+        T[q] = fma2(fma2(nom, quot, T[q]), inv, quot);
         const f32x2 w = mul2(alpha, T[q]);
         f32x2 G = mul2(gr[q], dup2(c0.x));
         G = fma2(gg[q], dup2(c0.y), G);
@@ -319,14 +325,14 @@ __device__ __forceinline__ bool camera_bwd_strip(const CamBwdParams& p, CamBwdSm
         G = taken(fma2(gb[q], dup2(c1.z), G));
         const f32x2 dalpha = fma2(T[q], G, mul2(mul2(inv, dup2(-1.f)), D[q]));
         D[q] = fma2(w, G, D[q]);
-        const f32x2 ws = taken(mul2(w, sh[q])), r = taken(gr[q]), g = taken(gg[q]), b = taken(gb[q]);
-        k0 = fma2(ws, r, k0);
-        k1 = fma2(ws, g, k1);
-        k2 = fma2(ws, b, k2);
+        const f32x2 ws = taken(mul2(w, sh[q])), pr = taken(gr[q]), pg = taken(gg[q]), pb = taken(gb[q]);
+        k0 = fma2(ws, pr, k0);
+        k1 = fma2(ws, pg, k1);
+        k2 = fma2(ws, pb, k2);
         k3 = fma2(w, taken(gs[q]), k3);
-        k4 = fma2(w, r, k4);
-        k5 = fma2(w, g, k5);
-        k6 = fma2(w, b, k6);
+        k4 = fma2(w, pr, k4);
+        k5 = fma2(w, pg, k5);
+        k6 = fma2(w, pb, k6);
         f32x2 tt = mul2(dalpha, beta);
         if (MASK) tt = pk2(lo2(beta) != 0.f ? lo2(tt) : 0.f, hi2(beta) != 0.f ? hi2(tt) : 0.f);
         const f32x2 td = mul2(tt, dy);
