@@ -156,17 +156,19 @@ Workspace plan_workspace(int n, int width, int height, size_t cap) {
     b.bin_plan = P.take(4 * (3 * (size_t)L.gy + 4));
     b.bin_tab = P.take(4 * bin_tab_words(cap, L.gx, L.gy));
   }
-  // the shadow partials; afterwards the backward's per-ray sums of the shadow
-  // segments (256 floats each)
-  const size_t items = shadow_seg_items(L.ntiles, cap);
-  L.partial = P.take(8 * cap > 1024 * items ? 8 * cap : 1024 * items);
+  const size_t items = shadow_seg_items(L.ntiles, cap), links = shadow_seg_links(L.ntiles, cap);
+  L.partial = P.take(8 * cap);
   L.tile_order[0] = P.take(4 * (size_t)L.ntiles);
   L.tile_order[1] = P.take(4 * (size_t)L.ntiles);
   L.seg_lvl = P.take(4 * (kSegWord + 1));
   L.seg_flag = P.take(4 * items);
   L.seg_desc = P.take(16 * items);
   L.seg_lists = P.take(8 * items);
-  L.seg_pub = P.take(4 * 256 * items);
+  L.seg_pub = P.take(1024 * links);
+  // the backward's sums lie where the camera binning's row sequence was, which
+  // nothing reads past that stage, if they fit (from about 2 M pairs on)
+  const size_t scratch = L.sp[0].tv[0] - L.sp[0].tk[0];
+  L.seg_sum = 1024 * links <= scratch ? L.sp[0].tk[0] : P.take(1024 * links);
   L.mlp_x3 = P.take(mlp_x3_bytes());
   L.rank_flags = P.take(2 * N);
   L.shade = P.take(16 * N);

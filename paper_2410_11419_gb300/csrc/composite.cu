@@ -75,7 +75,7 @@ struct ShadowParams {
   uint4* desc;                 // [item]: tile and kSegLast, first and past-the-last receiver, preceding item
   uint32_t* open_list;         // items some ray enters open (K6b's), in no particular order
   uint32_t* dead_list;         // items every ray enters stopped (K6c's)
-  float* pub_a;                // [item][256]: A(C_s+1) published by item
+  float* pub_a;                // [link_slot][256]: A(C_s+1) published by an item
   uint32_t* pub_flag;          // [item]: 0 not yet, 1 published, 2 published and every ray stopped
   uint8_t* pass_mask;  // per list entry: halves with a passing pixel, 0x3 rows 0-7, 0xC rows 8-15
   float2* partial;
@@ -125,7 +125,7 @@ __device__ __forceinline__ uint32_t min_bits(const f32x2 (&P)[kPx / 2]) {
 }
 
 // K6a: A(C_s+1) of every segment but a tile's last, chained from A(C_s).
-__device__ __forceinline__ void chain_item(const ShadowParams& p, uint32_t w, StagedEntries& S, int lane) {
+__device__ __forceinline__ void chain_item(const ShadowParams& p, const Links& link_slot, uint32_t w, StagedEntries& S, int lane) {
   const float lx = (lane & 15) + 0.5f, omin = 1.f - p.amax;
   const SegItem it = seg_item(p, w, lane);
   if (it.last) return;  // nothing follows it
@@ -140,7 +140,7 @@ __device__ __forceinline__ void chain_item(const ShadowParams& p, uint32_t w, St
   __syncwarp();  // orders every lane's reads after lane 0's acquire
   bool known = flag != 0u;
   f32x2 A[kPx / 2];
-  load_entering(p, it.first || !known, it.wpred, flag, lane, it.rows_in, A);
+  load_entering(p, link_slot, it.first || !known, it.wpred, flag, lane, it.rows_in, A);
   // the range's products Q; once no ray's A Q stays at the stop the rest of
   // the range changes nothing (each ray stops in it either way)
   f32x2 Q[kPx / 2];
@@ -155,7 +155,7 @@ __device__ __forceinline__ void chain_item(const ShadowParams& p, uint32_t w, St
       __syncwarp();
       if (fl != 0u) {
         known = true;
-        load_entering(p, false, it.wpred, fl, lane, it.rows_in, A);
+        load_entering(p, link_slot, false, it.wpred, fl, lane, it.rows_in, A);
       }
     }
     f32x2 AQ[kPx / 2];
@@ -192,10 +192,11 @@ __device__ __forceinline__ void chain_item(const ShadowParams& p, uint32_t w, St
     }
     fl = __shfl_sync(0xffffffffu, fl, 0);
     __syncwarp();
-    load_entering(p, false, it.wpred, fl, lane, it.rows_in, A);
+    load_entering(p, link_slot, false, it.wpred, fl, lane, it.rows_in, A);
   }
   const bool dead_in = live_halves(A) == 0u;
   bool any = false;
+  float* out = p.pub_a + link_slot(w) + lane;
 #pragma unroll
   for (int q = 0; q < kPx / 2; ++q) {
     const f32x2 AQ = mul2(A[q], Q[q]);
@@ -204,7 +205,7 @@ __device__ __forceinline__ void chain_item(const ShadowParams& p, uint32_t w, St
       float a = h ? hi2(AQ) : lo2(AQ);
       if (!(a >= kShadowStop)) a = 0.f;  // the ray stopped in this range or before it
       any |= a != 0.f;
-      if (!dead_in) p.pub_a[(size_t)w * 256 + 64 * q + 32 * h + lane] = a;
+      if (!dead_in) out[64 * q + 32 * h] = a;
     }
   }
   const bool any_out = __any_sync(0xffffffffu, any);
@@ -246,13 +247,14 @@ __global__ void __launch_bounds__(kSegWarps * 32, 5) k_shadow_chain(const Shadow
   StagedEntries& S = smem[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
   const uint32_t total = BATCH ? batch_items(reqs, nreq, kAllItems) : item_count(p, kAllItems);
+  const Links links = frame_links(p.lvl_off);
   uint32_t w;
   while (next_item(p.ticket, total, lane, w)) {
     if (BATCH) {
       const int r = locate(reqs, nreq, kAllItems, w);
-      chain_item(reqs[r], w, S, lane);
+      chain_item(reqs[r], frame_links(reqs[r].lvl_off), w, S, lane);
     } else {
-      chain_item(p, w, S, lane);
+      chain_item(p, links, w, S, lane);
     }
   }
 }
@@ -476,7 +478,7 @@ __global__ void __launch_bounds__(kDeadWarps * 32, 7) k_shadow_dead(const Shadow
 // then walks the 32 entries.  A receiver's per-lane sums go to a row of shared
 // memory; after the walk the lane that staged it adds up the row (in a fixed
 // order) and writes its partial.
-__device__ __forceinline__ void live_item(const ShadowParams& p, uint32_t w, ShadowSmem& S, int lane) {
+__device__ __forceinline__ void live_item(const ShadowParams& p, const Links& link_slot, uint32_t w, ShadowSmem& S, int lane) {
   const int lxi = lane & 15, lyi = lane >> 4;
   const float lx = lxi + 0.5f, omin = 1.f - p.amax;
   const SegItem it = seg_item(p, w, lane);
@@ -487,16 +489,17 @@ __device__ __forceinline__ void live_item(const ShadowParams& p, uint32_t w, Sha
   const uint32_t fl_in = it.first ? 1u : __ldcg(p.pub_flag + it.wpred);
   const uint32_t fl_out = it.last ? 1u : __ldcg(p.pub_flag + w);
   f32x2 P[kPx / 2];
-  load_entering(p, it.first, it.wpred, fl_in, lane, it.rows_in, P);
+  load_entering(p, link_slot, it.first, it.wpred, fl_in, lane, it.rows_in, P);
   uint32_t live = live_halves(P);
   // where a ray ended is recorded by the segment K6a has it stop in, or by
   // the tile's last one (ends: the lane's rays that this segment records)
   uint32_t ends = 0u;
+  const float* handed_on = p.pub_a + (it.last ? 0 : link_slot(w)) + lane;
 #pragma unroll
   for (int i = 0; i < kPx; ++i) {
     const float a = i & 1 ? hi2(P[i / 2]) : lo2(P[i / 2]);
     bool end = a >= kShadowStop;
-    if (end && !it.last && fl_out != 2u) end = __ldcg(p.pub_a + (size_t)w * 256 + 32 * i + lane) == 0.f;
+    if (end && !it.last && fl_out != 2u) end = __ldcg(handed_on + 32 * i) == 0.f;
     ends |= end ? 1u << i : 0u;
   }
 #pragma unroll
@@ -605,13 +608,14 @@ __global__ void __launch_bounds__(kSegWarps * 32, 6) k_shadow(const ShadowParams
   ShadowSmem& S = smem[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
   const uint32_t total = BATCH ? batch_items(reqs, nreq, kOpenItems) : item_count(p, kOpenItems);
+  const Links links = frame_links(p.lvl_off);
   uint32_t w;
   while (next_item(p.ticket + 1, total, lane, w)) {
     if (BATCH) {
       const int r = locate(reqs, nreq, kOpenItems, w);
-      live_item(reqs[r], reqs[r].open_list[w], S, lane);
+      live_item(reqs[r], frame_links(reqs[r].lvl_off), reqs[r].open_list[w], S, lane);
     } else {
-      live_item(p, p.open_list[w], S, lane);
+      live_item(p, links, p.open_list[w], S, lane);
     }
   }
 }
@@ -1256,9 +1260,16 @@ void launch_tile_order(const FrameArgs& f, int splat, cudaStream_t s) {
   count_launch();
 }
 
-size_t shadow_seg_items(int ntiles, size_t cap) {
-  const size_t few = cap / kSegMin, many = cap / kSegLen + kSegTarget;
-  return (size_t)ntiles + (few < many ? few : many) + 1;
+// Segments past each tile's first: no more than pairs / seg, for the seg that
+// k_tile_order chooses (kSegTarget of them, or seg is kSegLen).
+static size_t later_segments(size_t cap) {
+  const size_t few = cap / kSegMin, many = cap / kSegLen > kSegTarget ? cap / kSegLen : kSegTarget;
+  return (few < many ? few : many) + 1;
+}
+size_t shadow_seg_items(int ntiles, size_t cap) { return (size_t)ntiles + later_segments(cap); }
+size_t shadow_seg_links(int ntiles, size_t cap) {
+  const size_t later = later_segments(cap), firsts = (size_t)ntiles < later ? (size_t)ntiles : later;
+  return firsts + later;
 }
 
 namespace {

@@ -82,7 +82,8 @@ struct Workspace {
   size_t seg_flag = 0;  // u32[items]: shadow segment publications (0 none, 1 done, 2 done and all stopped)
   size_t seg_desc = 0;   // uint4[items]: each shadow segment's tile, receivers and predecessor
   size_t seg_lists = 0;  // u32[2][items]: the segments with an open ray; those every ray enters stopped
-  size_t seg_pub = 0;   // float[items][256]: the products each shadow segment hands to the next
+  size_t seg_pub = 0;   // float[links][256]: the products each shadow segment hands to the next
+  size_t seg_sum = 0;   // float[links][256]: the backward's per-ray sums over the later segments
   size_t mlp_x3 = 0;    // the FP32 networks' hidden weights, packed for the tensor cores in every frame
   size_t rank_flags = 0;  // uchar2[N] by light rank: a receiver of it saw some light; a pixel of it is known to pass
   int n = 0, width = 0, height = 0, gx = 0, gy = 0, ntiles = 0;
@@ -247,6 +248,8 @@ void launch_camera_composite_batch(const FrameArgs* const* f, float* const* out,
                                    unsigned char* host, cudaStream_t s);
 // shadow composite work items (tile segments) a frame can have at most
 size_t shadow_seg_items(int ntiles, size_t cap);
+// those of tiles with more than one, which alone hand products on (link_slot)
+size_t shadow_seg_links(int ntiles, size_t cap);
 // A light tile's list is cut into segments of seg entries, at most kSegLevels -
 // 1 per tile (the last takes the rest); the shadow composite and its backward
 // share the cut.  k_tile_order chooses seg, a power of two from kSegMin to

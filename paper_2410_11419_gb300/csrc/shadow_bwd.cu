@@ -64,7 +64,7 @@ struct BwdParams {
   const float* light_final;
   const uint32_t* light_stop;
   const float2* ct;    // by light rank: (coef_j, T_j)
-  float* seg_sum;      // [item][256]: a segment's own sum per ray, then the later segments'
+  float* seg_sum;      // [link_slot][256]: a segment's own sum per ray, then the later segments'
   uint32_t* ticket;    // [4]: three tickets, and whether some coef_j is infinite or not a number
   float* light_geom;   // [N][8] by index: dL/dgamma, sums of w dx, w dy, w dx dy, w dx^2, w dy^2
   int W, H, gx, ntiles;
@@ -100,14 +100,14 @@ __device__ __forceinline__ f32x2 where_passing(f32x2 b, f32x2 x) {
 }
 
 template <bool MASK>
-__device__ __forceinline__ void sum_item(const BwdParams& p, uint32_t w, SumSmem& S, int lane) {
+__device__ __forceinline__ void sum_item(const BwdParams& p, const Links& link_slot, uint32_t w, SumSmem& S, int lane) {
   const SegItem it = seg_item(p, w, lane);
   if (it.first) return;
   const float lx = (lane & 15) + 0.5f, omin = 1.f - p.amax;
   const float ox = (float)(it.tx * kTile), oy = (float)(it.ty * kTile);
   f32x2 ly[kPx / 2], P[kPx / 2], sum[kPx / 2];
   lane_rows(lane, it.rows_in, ly);
-  load_entering(p, false, it.wpred, __ldcg(p.pub_flag + it.wpred), lane, it.rows_in, P);
+  load_entering(p, link_slot, false, it.wpred, __ldcg(p.pub_flag + it.wpred), lane, it.rows_in, P);
 #pragma unroll
   for (int q = 0; q < kPx / 2; ++q) sum[q] = 0ull;
   uint32_t j = it.R0, k = it.C0;
@@ -155,16 +155,17 @@ __device__ __forceinline__ void sum_item(const BwdParams& p, uint32_t w, SumSmem
     j += nrecv;
     k += nops - nrecv;
   }
+  float* out = p.seg_sum + link_slot(w) + lane;
 #pragma unroll
   for (int q = 0; q < kPx / 2; ++q) {
-    p.seg_sum[(size_t)w * 256 + 64 * q + lane] = lo2(sum[q]);
-    p.seg_sum[(size_t)w * 256 + 64 * q + 32 + lane] = hi2(sum[q]);
+    out[64 * q] = lo2(sum[q]);
+    out[64 * q + 32] = hi2(sum[q]);
   }
 }
 
 // (the masked forms are calls, which leaves the others as they are without them)
-__device__ __noinline__ void sum_item_masked(const BwdParams& p, uint32_t w, SumSmem& S, int lane) {
-  sum_item<true>(p, w, S, lane);
+__device__ __noinline__ void sum_item_masked(const BwdParams& p, const Links& link_slot, uint32_t w, SumSmem& S, int lane) {
+  sum_item<true>(p, link_slot, w, S, lane);
 }
 
 __global__ void __launch_bounds__(kBwdWarps * 32, 6) k_shadow_bwd_sums(const __grid_constant__ BwdParams p) {
@@ -172,10 +173,11 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 6) k_shadow_bwd_sums(const __g
   const int lane = threadIdx.x & 31;
   const uint32_t total = p.counts[0];
   const bool mask = p.ticket[3] != 0u;
+  const Links links = frame_links(p.lvl_off);
   uint32_t w;
   while (next_item(p.ticket, total, lane, w)) {
-    if (mask) sum_item_masked(p, p.open_list[w], smem[threadIdx.x >> 5], lane);
-    else sum_item<false>(p, p.open_list[w], smem[threadIdx.x >> 5], lane);
+    if (mask) sum_item_masked(p, links, p.open_list[w], smem[threadIdx.x >> 5], lane);
+    else sum_item<false>(p, links, p.open_list[w], smem[threadIdx.x >> 5], lane);
   }
 }
 
@@ -188,6 +190,7 @@ __global__ void __launch_bounds__(128) k_shadow_bwd_suffix(const BwdParams p) {
   if (pos >= (uint32_t)p.ntiles) return;
   const int tile = (int)p.tile_order[pos];
   const uint32_t nseg = seg_count(p.tile_start[tile + 1] - p.tile_start[tile], p.lvl_off[kSegWord]);
+  if (nseg < 2u) return;
   uint32_t nopen = nseg;
   for (uint32_t s0 = 1; s0 < nseg && nopen == nseg; s0 += 32) {
     const uint32_t s = s0 + (uint32_t)lane;
@@ -195,9 +198,10 @@ __global__ void __launch_bounds__(128) k_shadow_bwd_suffix(const BwdParams p) {
     const uint32_t m = __ballot_sync(0xffffffffu, dead);
     if (m) nopen = s0 + (uint32_t)(__ffs(m) - 1);
   }
+  const Links link_slot = frame_links(p.lvl_off);
   float4 acc[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
   for (uint32_t s = nopen; s-- > 0;) {
-    float4* v = reinterpret_cast<float4*>(p.seg_sum + (size_t)(p.lvl_off[s] + pos) * 256) + 2 * lane;
+    float4* v = reinterpret_cast<float4*>(p.seg_sum + link_slot(p.lvl_off[s] + pos)) + 2 * lane;
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       const float4 own = s > 0 ? v[i] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -271,7 +275,7 @@ __device__ __forceinline__ void occ_bwd(const f32x2 (&ly)[kPx / 2], f32x2 (&A)[k
 }
 
 template <bool MASK>
-__device__ __forceinline__ void bwd_item(const BwdParams& p, uint32_t w, BwdSmem& B, int lane) {
+__device__ __forceinline__ void bwd_item(const BwdParams& p, const Links& link_slot, uint32_t w, BwdSmem& B, int lane) {
   const SegItem it = seg_item(p, w, lane);
   if (it.R1 <= it.R0) return;
   const int lxi = lane & 15, lyi = lane >> 4;
@@ -280,17 +284,19 @@ __device__ __forceinline__ void bwd_item(const BwdParams& p, uint32_t w, BwdSmem
   const size_t pix0 = (size_t)(it.ty * kTile + lyi) * p.W + it.tx * kTile + lxi;
   f32x2 ly[kPx / 2], A[kPx / 2], S[kPx / 2];
   lane_rows(lane, it.rows_in, ly);
-  load_entering(p, it.first, it.wpred, it.first ? 1u : __ldcg(p.pub_flag + it.wpred), lane, it.rows_in, A);
+  load_entering(p, link_slot, it.first, it.wpred, it.first ? 1u : __ldcg(p.pub_flag + it.wpred), lane, it.rows_in, A);
   // the product each ray leaves the segment with; one that ends in it gets its
   // product when the walk reaches the occluder it ended at (pending: those
   // rays, next: the largest such limit; kNoStop: it ran through the list)
   const uint32_t fl_out = it.last ? 2u : __ldcg(p.pub_flag + w);
   uint32_t pending = 0u, next = 0u;
+  const bool only = it.first && it.last;  // the tile's only segment
+  const size_t link = only ? 0 : link_slot(w);
 #pragma unroll
   for (int i = 0; i < kPx; ++i) {
     float a = i & 1 ? hi2(A[i / 2]) : lo2(A[i / 2]);
     if (a >= kShadowStop) {
-      a = fl_out == 2u ? 0.f : __ldcg(p.pub_a + (size_t)w * 256 + 32 * i + lane);
+      a = fl_out == 2u ? 0.f : __ldcg(p.pub_a + link + 32 * i + lane);
       if (a == 0.f) {
         const uint32_t lim = p.light_stop[pix0 + (size_t)2 * i * p.W];
         if (lim == kNoStop) {
@@ -307,7 +313,7 @@ __device__ __forceinline__ void bwd_item(const BwdParams& p, uint32_t w, BwdSmem
   }
 #pragma unroll
   for (int q = 0; q < kPx / 2; ++q)
-    S[q] = pk2(__ldcg(p.seg_sum + (size_t)w * 256 + 64 * q + lane), __ldcg(p.seg_sum + (size_t)w * 256 + 64 * q + 32 + lane));
+    S[q] = only ? 0ull : pk2(__ldcg(p.seg_sum + link + 64 * q + lane), __ldcg(p.seg_sum + link + 64 * q + 32 + lane));
 
   // the rows' sums over the 32 lanes: lane l < 24 takes term pair l >> 3 of
   // entry l & 7, in lane order
@@ -422,8 +428,8 @@ __device__ __forceinline__ void bwd_item(const BwdParams& p, uint32_t w, BwdSmem
   }
 }
 
-__device__ __noinline__ void bwd_item_masked(const BwdParams& p, uint32_t w, BwdSmem& B, int lane) {
-  bwd_item<true>(p, w, B, lane);
+__device__ __noinline__ void bwd_item_masked(const BwdParams& p, const Links& link_slot, uint32_t w, BwdSmem& B, int lane) {
+  bwd_item<true>(p, link_slot, w, B, lane);
 }
 
 __global__ void __launch_bounds__(kBwdWarps * 32, 4) k_shadow_bwd(const __grid_constant__ BwdParams p) {
@@ -433,9 +439,10 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 4) k_shadow_bwd(const __grid_c
   const uint32_t total = p.counts[0];
   uint32_t w;
   const bool mask = p.ticket[3] != 0u;
+  const Links links = frame_links(p.lvl_off);
   while (next_item(p.ticket + 1, total, lane, w)) {
-    if (mask) bwd_item_masked(p, p.open_list[w], smem[threadIdx.x >> 5], lane);
-    else bwd_item<false>(p, p.open_list[w], smem[threadIdx.x >> 5], lane);
+    if (mask) bwd_item_masked(p, links, p.open_list[w], smem[threadIdx.x >> 5], lane);
+    else bwd_item<false>(p, links, p.open_list[w], smem[threadIdx.x >> 5], lane);
   }
 }
 
@@ -583,7 +590,7 @@ void launch_shadow_backward(const FrameArgs& f, const ShadowBwdArgs& a, cudaStre
   p.light_final = at<float>(ws, L.light_final);
   p.light_stop = at<uint32_t>(ws, L.light_stop);
   p.ct = a.ct;
-  p.seg_sum = at<float>(ws, L.partial);  // the forward's partials are added up by now
+  p.seg_sum = at<float>(ws, L.seg_sum);
   p.ticket = a.ticket;
   p.light_geom = a.light_geom;
   p.W = L.width; p.H = L.height; p.gx = L.gx; p.ntiles = L.ntiles;

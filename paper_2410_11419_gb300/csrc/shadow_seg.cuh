@@ -87,16 +87,27 @@ __device__ __forceinline__ uint32_t live_halves(const f32x2 (&P)[kPx / 2]) {
   return (__any_sync(0xffffffffu, h0) ? 0x3u : 0u) | (__any_sync(0xffffffffu, h1) ? 0xCu : 0u);
 }
 
+// Where segment w's products for the next segment lie (256 floats each), and the
+// backward's sums of the segments after it.  Items are numbered level by level, a
+// level's tiles by decreasing segment count: the first segments of tiles with
+// no other, which have neither, are the last of level 0 and take no room.
+struct Links {
+  uint32_t more, gap;  // tiles with a second segment, and without
+  __device__ __forceinline__ size_t operator()(uint32_t w) const { return (size_t)(w < more ? w : w - gap) * 256; }
+};
+__device__ __forceinline__ Links frame_links(const uint32_t* lvl_off) {  // once per warp, not per item
+  const uint32_t tiles = lvl_off[1], more = lvl_off[2] - tiles;
+  return {more, tiles - more};
+}
+
 // A(C_s) of the lane's rays: 1 / 0 (in / outside the image) for a tile's
 // first segment, else the predecessor's publication (read from L2: it was
 // written on another SM); flag 2 publishes that every ray stopped.
 template <typename P>
-__device__ __forceinline__ void load_entering(const P& p, bool first, uint32_t wpred, uint32_t flag, int lane,
+__device__ __forceinline__ void load_entering(const P& p, const Links& link_slot, bool first, uint32_t wpred, uint32_t flag, int lane,
                                               int rows_in, f32x2 (&A)[kPx / 2]) {
-  auto one = [&](int i) {
-    return first ? (i < rows_in ? 1.f : 0.f)
-                 : (flag == 2u ? 0.f : __ldcg(p.pub_a + (size_t)wpred * 256 + 32 * i + lane));
-  };
+  const float* in = p.pub_a + (first ? 0 : link_slot(wpred)) + lane;
+  auto one = [&](int i) { return first ? (i < rows_in ? 1.f : 0.f) : (flag == 2u ? 0.f : __ldcg(in + 32 * i)); };
 #pragma unroll
   for (int q = 0; q < kPx / 2; ++q) A[q] = pk2(one(2 * q), one(2 * q + 1));
 }
