@@ -144,7 +144,9 @@ class Renderer:
         if getattr(self, "bws", None) is None:
             nb = N.gs3_backward_workspace_size(self.scene.handle)
             self.bws = torch.empty(nb, dtype=torch.uint8, device=self.ws.device)
-        grads = {f: torch.empty_like(self.scene.t[f]) for f in self.scene.ARRAYS_DEV}  # all overwritten
+        # all overwritten, but for the placeholders of a scene without lobes
+        grads = {f: torch.zeros_like(x) if self.scene.k == 0 and f.startswith("lobe_") else torch.empty_like(x)
+                 for f, x in ((f, self.scene.t[f]) for f in self.scene.ARRAYS_DEV)}
         N.gs3_render_backward(self.scene.handle, camera_struct(cam), light_struct(light), opts,
                               dl_drgb.contiguous(), self.ws, self.cap, self.bws, grads, s.cuda_stream)
         return grads
