@@ -558,7 +558,16 @@ void launch_tc(const TcParams& p, const MlpDev& m, int eb, bool after, int sms, 
   if (smem + reserve < floor_bytes) smem = floor_bytes - reserve;
   auto kern = eb == 2 ? (p.which == 0 ? k_mlp_tc<2, 0> : k_mlp_tc<2, 1>)
                       : (p.which == 0 ? k_mlp_tc<1, 0> : k_mlp_tc<1, 1>);
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the limit belongs to the kernel, not to this launch: set once, to the most any shape
+  // takes, so that another thread's smaller network never lowers it in between
+  static DeviceOnce once;
+  once.run([] {
+    bool ok = true;
+    for (const void* k : {(const void*)k_mlp_tc<2, 0>, (const void*)k_mlp_tc<2, 1>, (const void*)k_mlp_tc<1, 0>,
+                          (const void*)k_mlp_tc<1, 1>})
+      ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemCap) == cudaSuccess;
+    return ok;
+  });
   const int nsm = sms > 0 ? sms : device_sm_count();
   const int ntiles = (p.n * p.nl + kTcRows - 1) / kTcRows;
   const int ctas = (ntiles + groups - 1) / groups;
