@@ -430,7 +430,7 @@ gs3_status render_frame(gs3_scene* scene, const gs3_camera* cam, const gs3_light
     sl = side->s;
   }
   if ((stages & GS3_STAGE_LIGHT_BIN) && !no_shadow) {
-    launch_depth_sort(f, 1, sl);
+    launch_depth_sort(f, 1, sl, /*wait=*/fork);
     launch_binning(f, 1, sl);
   }
   if ((stages & GS3_STAGE_SHADOW_COMPOSITE) && !no_shadow) launch_shadow_composite(f, sl);
@@ -460,7 +460,7 @@ gs3_status render_frame(gs3_scene* scene, const gs3_camera* cam, const gs3_light
   if (fork) cudaEventRecord(side->join, sl);
   if (fork || beside) cudaStreamWaitEvent(s, side->join, 0);
   if ((stages & GS3_STAGE_MLP) && !beside) launch_networks(scene, f, early ? 1 : 3, 0, s);
-  if (stages & GS3_STAGE_CAMERA) launch_camera_composite(f, out_rgb, (stages & GS3_STAGE_MLP) && !beside, s);
+  if (stages & GS3_STAGE_CAMERA) launch_camera_composite(f, out_rgb, /*wait=*/beside || (fork && !(stages & GS3_STAGE_MLP)), s);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "gs3_render: launch");
   return GS3_OK;
@@ -558,7 +558,7 @@ gs3_status render_batch(const BatchFrame* frames, int n, cudaStream_t s, BatchSt
     cudaStream_t sr = bs.sub[r];
     cudaStreamWaitEvent(sr, bs.fork2, 0);
     if (f[r].opts.ablate & GS3_ABLATE_SHADOW_SPLAT) launch_fill_shadow_one(f[r], sr);
-    else launch_shadow_reduce(f[r], sr);
+    else launch_shadow_reduce(f[r], sr, /*wait=*/true);
     launch_networks(frames[r].scene, f[r], 1, 0, sr);
     cudaEventRecord(bs.join2[r], sr);
   }

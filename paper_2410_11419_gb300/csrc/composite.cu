@@ -1452,11 +1452,11 @@ void launch_shadow_composite_batch(const FrameArgs* const* f, int n, unsigned ch
   count_launch(2 + n + 1);
 }
 
-void launch_shadow_reduce(const FrameArgs& f, cudaStream_t s) {
+void launch_shadow_reduce(const FrameArgs& f, cudaStream_t s, bool wait) {
   const SplatBufs& b = f.L->sp[1];
   unsigned char* ws = f.ws;
   const int n = f.sc.n;
-  launch_after(k_shadow_reduce, (n * 8 + 255) / 256, 256, 0, s, n, at<uint32_t>(ws, b.off), at<uint32_t>(ws, b.cnt), at<float2>(ws, f.L->partial),
+  launch_behind(wait, k_shadow_reduce, (n * 8 + 255) / 256, 256, 0, s, n, at<uint32_t>(ws, b.off), at<uint32_t>(ws, b.cnt), at<float2>(ws, f.L->partial),
       at<uchar2>(ws, f.L->rank_flags), at<uint32_t>(ws, b.sv[1]), at<uint32_t>(ws, f.L->header), at<float>(ws, f.L->T),
       at<float>(ws, f.L->shadow_den));
   count_launch();
@@ -1470,10 +1470,8 @@ void launch_fill_shadow_one(const FrameArgs& f, cudaStream_t s) {
   count_launch();
 }
 
-void launch_camera_composite(const FrameArgs& f, float* out_rgb, bool after_mlp, cudaStream_t s) {
-  const CamParams p = camera_params(f, out_rgb);
-  if (after_mlp) launch_after(k_camera<false>, f.L->ntiles, kCamThreads, 0, s, p, nullptr, nullptr, 1);
-  else k_camera<false><<<f.L->ntiles, kCamThreads, 0, s>>>(p, nullptr, nullptr, 1);
+void launch_camera_composite(const FrameArgs& f, float* out_rgb, bool wait, cudaStream_t s) {
+  launch_behind(wait, k_camera<false>, f.L->ntiles, kCamThreads, 0, s, camera_params(f, out_rgb), nullptr, nullptr, 1);
   count_launch();
 }
 

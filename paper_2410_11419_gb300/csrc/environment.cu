@@ -160,7 +160,7 @@ gs3_status gs3_render_environment(gs3_scene* scene, const gs3_camera* cam, const
       // 2. once, on `stream` beside the light chains: the camera splat (after
       //    the first light's projections) and Psi
       cudaStreamWaitEvent(s, bs.cam, 0);
-      launch_depth_sort(f[0], 0, s);
+      launch_depth_sort(f[0], 0, s, /*wait=*/true);
       launch_binning(f[0], 0, s);
       launch_tile_order(f[0], 0, s);
       launch_mlp(f[0], s, /*identity_only=*/tc, /*which_mask=*/2);

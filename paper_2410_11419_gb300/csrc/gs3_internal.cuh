@@ -229,7 +229,7 @@ gs3_status run_backward(const FrameArgs& f, const float* dimg, void* bws, size_t
 
 // shading and both projections (K1); light_only: the shadow splat's projection only
 void launch_prep(const FrameArgs& f, cudaStream_t s, bool light_only = false);
-void launch_depth_sort(const FrameArgs& f, int splat, cudaStream_t s);
+void launch_depth_sort(const FrameArgs& f, int splat, cudaStream_t s, bool wait = false);
 void launch_binning(const FrameArgs& f, int splat, cudaStream_t s);
 void launch_shadow_composite(const FrameArgs& f, cudaStream_t s);
 // Batches of frames (up to kMaxBatch, each with its own workspace): the
@@ -274,7 +274,8 @@ __host__ __device__ inline uint32_t seg_count(uint32_t len, uint32_t seg) {
 }
 // a splat's tiles ordered longest list first (in length steps of 8), into L.tile_order[splat]
 void launch_tile_order(const FrameArgs& f, int splat, cudaStream_t s);
-void launch_shadow_reduce(const FrameArgs& f, cudaStream_t s);
+// wait (here and below): the stream's last operation is an event wait
+void launch_shadow_reduce(const FrameArgs& f, cudaStream_t s, bool wait = false);
 // Phi and Psi of one frame; which_mask bit 0 Phi, bit 1 Psi; identity_only:
 // only the networks an ablation replaces by the identity / zero
 // sms: the SMs that the tensor-core kernels may take (0: all)
@@ -298,8 +299,7 @@ void pack_mlp_tc(const MlpDev& m, int dtype, const SceneDev& sc, int which, unsi
 bool mlp_tc_supported(const MlpDev& m, int dtype);
 void launch_mlp_tc(const FrameArgs& f, const unsigned char* const blobs[2], cudaStream_t s, int which_mask = 3,
                    int sms = 0);
-// after_mlp: the stream's last operation is the networks' last kernel
-void launch_camera_composite(const FrameArgs& f, float* out_rgb, bool after_mlp, cudaStream_t s);
+void launch_camera_composite(const FrameArgs& f, float* out_rgb, bool wait, cudaStream_t s);
 // camera composite of nl <= kMaxBatch lights over f0's camera splat:
 // out (+)= sum_l w[l] (S_l Sh_l + R), (S_l, Sh_l) per camera rank from envcol
 void launch_camera_env(const FrameArgs& f0, const float4* envcol, int nl, const float* w, bool accumulate,
@@ -354,6 +354,11 @@ struct DeviceOnce {
 // is an ordinary launch).  Between two dependent kernels it takes 0.8 us instead of
 // 1.9.  Kernels that let their successor in at once (griddepcontrol.launch_dependents)
 // cost frames 2 to 5 %: the waiting blocks hold room that the other stream's need.
+// The rule: CUDA lets such a grid overlap with the previous kernel of its stream
+// alone, so it is used behind a kernel, a copy or a memset of that stream, and at the
+// start of an entry point, behind whatever the caller's stream holds; never directly
+// behind an event wait of this library's own, where there is nothing to overlap with
+// and the dependency is on another stream (launch_behind chooses).
 template <typename... P, typename... A>
 inline void launch_after(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A&&... args) {
   cudaLaunchAttribute attr;
@@ -367,6 +372,14 @@ inline void launch_after(void (*kernel)(P...), unsigned grid, unsigned block, si
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
   cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+// launch_after, or with `wait` (the stream's last operation is an event wait) an
+// ordinary launch
+template <typename... P, typename... A>
+inline void launch_behind(bool wait, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                          A&&... args) {
+  if (wait) kernel<<<grid, block, smem, s>>>(P(args)...);
+  else launch_after(kernel, grid, block, smem, s, args...);
 }
 __device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 

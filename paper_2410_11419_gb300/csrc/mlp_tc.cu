@@ -545,8 +545,8 @@ TcParams tc_params(const FrameArgs& f, int which, const unsigned char* blob) {
   return p;
 }
 
-// after: the stream's last operation is a kernel
-void launch_tc(const TcParams& p, const MlpDev& m, int eb, bool after, int sms, cudaStream_t s) {
+// wait: the stream's last operation may be an event wait
+void launch_tc(const TcParams& p, const MlpDev& m, int eb, bool wait, int sms, cudaStream_t s) {
   const int groups = tc_groups(m, eb);
   size_t smem = tc_smem_bytes(m, eb, groups);
   // CTAs of this kernel (of any launch) that share an SM must fit in its 512
@@ -572,8 +572,7 @@ void launch_tc(const TcParams& p, const MlpDev& m, int eb, bool after, int sms, 
   const int ntiles = (p.n * p.nl + kTcRows - 1) / kTcRows;
   const int ctas = (ntiles + groups - 1) / groups;
   const int grid = ctas < nsm ? ctas : nsm;
-  if (after) launch_after(kern, grid, kTcThreads * groups, smem, s, p);
-  else kern<<<grid, kTcThreads * groups, smem, s>>>(p);
+  launch_behind(wait, kern, grid, kTcThreads * groups, smem, s, p);
   count_launch();
 }
 
@@ -581,13 +580,13 @@ void launch_tc(const TcParams& p, const MlpDev& m, int eb, bool after, int sms, 
 
 void launch_mlp_tc(const FrameArgs& f, const unsigned char* const blobs[2], cudaStream_t s, int which_mask, int sms) {
   const int eb = elem_bytes(f.sc.mlp_dtype);
-  bool after = false;
+  bool wait = true;
   for (int which = 0; which < 2; ++which) {
     if (!(which_mask & (1 << which))) continue;
     const bool identity = (f.opts.ablate & (which == 0 ? GS3_ABLATE_PHI : GS3_ABLATE_PSI)) != 0;
     if (identity) continue;  // handled by the FP32 kernel's identity path
-    launch_tc(tc_params(f, which, blobs[which]), which == 0 ? f.sc.phi : f.sc.psi, eb, after, sms, s);
-    after = true;
+    launch_tc(tc_params(f, which, blobs[which]), which == 0 ? f.sc.phi : f.sc.psi, eb, wait, sms, s);
+    wait = false;
   }
 }
 
@@ -603,7 +602,7 @@ void launch_phi_lights_tc(const FrameArgs* const* f, int nl, float4* envcol, con
   }
   p.ccol = nullptr;
   p.envcol = envcol;
-  launch_tc(p, f[0]->sc.phi, elem_bytes(f[0]->sc.mlp_dtype), false, 0, s);
+  launch_tc(p, f[0]->sc.phi, elem_bytes(f[0]->sc.mlp_dtype), true, 0, s);
 }
 
 }  // namespace gs3

@@ -418,10 +418,10 @@ __global__ void __launch_bounds__(kBinBlock) k_reorder(int n, const uint32_t* __
 template <int ROUNDS, int PASSES>
 void onesweep_sort(const uint32_t* kin, const uint32_t* vin, uint32_t* k0, uint32_t* v0, uint32_t* k1,
                    uint32_t* v1, const uint32_t* n_ptr, uint32_t n_fixed, int nblocks, int passes,
-                   unsigned char* look_region, uint32_t* header, cudaStream_t s, bool own_status = false,
-                   int first_ticket = 0) {
+                   unsigned char* look_region, uint32_t* header, cudaStream_t s, bool wait = false,
+                   bool own_status = false, int first_ticket = 0) {
   if (!n_ptr && !vin && n_fixed <= kSmallSort && passes == 4) {
-    launch_after(k_sort_small, 1, kSmallThreads, 0, s, kin, k1, v1, n_fixed, own_status ? header : nullptr);
+    launch_behind(wait, k_sort_small, 1, kSmallThreads, 0, s, kin, k1, v1, n_fixed, own_status ? header : nullptr);
     count_launch();
     return;
   }
@@ -464,12 +464,12 @@ void depth_order(const uint32_t* keys, uint32_t n, uint32_t* k0, uint32_t* v0, u
   uint32_t* status = reinterpret_cast<uint32_t*>(front);
   auto blocks = [&](int rounds) { return (int)((n + kSortThreads * rounds - 1) / (kSortThreads * rounds)); };
   if (blocks(4) <= kDepthOrderBlocks)
-    onesweep_sort<4, 4>(keys, nullptr, k0, v0, k1, order, nullptr, n, blocks(4), 4, look, status, s, true, first_ticket);
+    onesweep_sort<4, 4>(keys, nullptr, k0, v0, k1, order, nullptr, n, blocks(4), 4, look, status, s, false, true, first_ticket);
   else
-    onesweep_sort<8, 4>(keys, nullptr, k0, v0, k1, order, nullptr, n, blocks(8), 4, look, status, s, true, first_ticket);
+    onesweep_sort<8, 4>(keys, nullptr, k0, v0, k1, order, nullptr, n, blocks(8), 4, look, status, s, false, true, first_ticket);
 }
 
-void launch_depth_sort(const FrameArgs& f, int sp, cudaStream_t s) {
+void launch_depth_sort(const FrameArgs& f, int sp, cudaStream_t s, bool wait) {
   const SplatBufs& b = f.L->sp[sp];
   unsigned char* ws = f.ws;
   const int n = f.sc.n;
@@ -478,7 +478,7 @@ void launch_depth_sort(const FrameArgs& f, int sp, cudaStream_t s) {
   onesweep_sort<kDepthSortRounds, 4>(at<uint32_t>(ws, b.key), nullptr, at<uint32_t>(ws, b.sk[0]),
                                      at<uint32_t>(ws, b.sv[0]), at<uint32_t>(ws, b.sk[1]), at<uint32_t>(ws, b.sv[1]),
                                      nullptr, (uint32_t)n, f.L->nb_n, 4, at<unsigned char>(ws, b.dlook),
-                                     at<uint32_t>(ws, f.L->header), s);
+                                     at<uint32_t>(ws, f.L->header), s, wait);
   // 4 passes end in buffer 1: sv[1] holds the index of each depth rank
   launch_after(k_reorder, f.L->nb_rows, kBinBlock, 0, s, n, at<uint32_t>(ws, b.sv[1]), at<SplatRec>(ws, b.rec), at<SplatRec>(ws, b.rrec),
       at<uint32_t>(ws, b.rank_of), at<uint32_t>(ws, b.cnt), at<float4>(ws, f.L->shade),
