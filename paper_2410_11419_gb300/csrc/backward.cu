@@ -143,10 +143,9 @@ __device__ __forceinline__ void cp_async4(void* dst, const void* src) {
 // zero weight does not cancel it: a pixel adds only the entries it takes.  Without
 // MASK, false if a pixel asks for it (nothing is added then).
 template <int NQ, bool MASK>
-__device__ __forceinline__ bool camera_bwd_strip(const CamBwdParams& p, CamBwdSmem& B, uint32_t unit) {
+__device__ __forceinline__ bool camera_bwd_strip(const CamBwdParams& p, CamBwdSmem& B, int tile, int part) {
   const int lane = threadIdx.x & 31;
-  constexpr uint32_t kParts = 4 / NQ;  // strips of 4 NQ rows
-  const int tile = (int)p.tile_order[unit / kParts], part = (int)(unit % kParts), half = part * NQ / 2;
+  const int half = part * NQ / 2;
   const int tx = tile % p.gx, ty = tile / p.gx;
   const uint32_t hbits = 3u << (2 * half);
   const float ox = (float)(tx * kTile), oy = (float)(ty * kTile);
@@ -366,8 +365,8 @@ __device__ __forceinline__ bool camera_bwd_strip(const CamBwdParams& p, CamBwdSm
 
 // (a call, which leaves the other form as it is without this one)
 template <int NQ>
-__device__ __noinline__ void camera_bwd_strip_masked(const CamBwdParams& p, CamBwdSmem& B, uint32_t unit) {
-  camera_bwd_strip<NQ, true>(p, B, unit);
+__device__ __noinline__ void camera_bwd_strip_masked(const CamBwdParams& p, CamBwdSmem& B, int tile, int part) {
+  camera_bwd_strip<NQ, true>(p, B, tile, part);
 }
 
 template <int NQ>
@@ -375,8 +374,10 @@ __global__ void __launch_bounds__(kCbWarps * 32, 4) k_camera_bwd(const __grid_co
   __shared__ CamBwdSmem smem[kCbWarps];
   CamBwdSmem& B = smem[threadIdx.x >> 5];
   const uint32_t unit = blockIdx.x * kCbWarps + (threadIdx.x >> 5);  // (tile in launch order, strip)
-  if (unit >= 4 / NQ * (uint32_t)p.ntiles) return;
-  if (*p.nonfinite || !camera_bwd_strip<NQ, false>(p, B, unit)) camera_bwd_strip_masked<NQ>(p, B, unit);
+  constexpr uint32_t kParts = 4 / NQ;  // strips of 4 NQ rows
+  if (unit >= kParts * (uint32_t)p.ntiles) return;
+  const int tile = (int)p.tile_order[unit / kParts], part = (int)(unit % kParts);
+  if (*p.nonfinite || !camera_bwd_strip<NQ, false>(p, B, tile, part)) camera_bwd_strip_masked<NQ>(p, B, tile, part);
 }
 
 __global__ void k_copy_strided(const float* src, int stride, int off, float* dst, int n) {

@@ -866,12 +866,11 @@ struct CamTile {
   int px, py0;
 };
 
-// Block blk of a frame: tile tile_order[blk] (longest list first).  128
-// threads, two pixels each: warp w covers quadrant w (the 8x8 block at
-// (8 (w & 1), 8 (w >> 1))), lane l column l & 7 and rows l >> 3 and
-// (l >> 3) + 4 of it, so the two pixels share the entry's dx terms.
-__device__ __forceinline__ CamTile camera_tile_of(const CamParams& p, int blk, CamPixels& x) {
-  const int tile = (int)p.tile_order[blk];
+// A block takes a tile (the longest lists first).  128 threads, two pixels
+// each: warp w covers quadrant w (the 8x8 block at (8 (w & 1), 8 (w >> 1))), lane
+// l column l & 7 and rows l >> 3 and (l >> 3) + 4 of it, so the two pixels share
+// the entry's dx terms.
+__device__ __forceinline__ CamTile camera_tile_of(const CamParams& p, int tile, CamPixels& x) {
   const int tx = tile % p.gx, ty = tile / p.gx;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int cx = 8 * (w & 1) + (lane & 7), cy = 8 * (w >> 1) + (lane >> 3);
@@ -983,9 +982,9 @@ using CamSmem = CamEntries<2, kCamGroup>;
 // MASK: the frame has colours that a zero weight does not cancel, so a pixel
 // adds only the entries it takes (their weights are positive).
 template <bool MASK>
-__device__ __forceinline__ void camera_tile(const CamParams& p, int blk, CamSmem (*smem)[2]) {
+__device__ __forceinline__ void camera_tile(const CamParams& p, int tile, CamSmem (*smem)[2]) {
   CamPixels x;
-  const CamTile t = camera_tile_of(p, blk, x);
+  const CamTile t = camera_tile_of(p, tile, x);
   f32x2 acc[2][4];  // per pixel: (S r, g), (S b, Sh), (R r, g), (R b, -)
 #pragma unroll
   for (int k = 0; k < 2; ++k)
@@ -1033,25 +1032,23 @@ __device__ __forceinline__ void camera_tile(const CamParams& p, int blk, CamSmem
 
 // One frame (p), or a batch of nreq frames (reqs in device memory) whose
 // tiles follow one another: frame r owns blocks [tile_prefix[r], tile_prefix[r + 1]).
-// (a call, which leaves the other form as it is without this one)
-__device__ __noinline__ void camera_tile_masked(const CamParams& p, int blk, CamSmem (*smem)[2]) {
-  camera_tile<true>(p, blk, smem);
-}
-
+// 6 blocks per SM whatever the second form takes.
 template <bool BATCH>
-__global__ void __launch_bounds__(kCamThreads) k_camera(const __grid_constant__ CamParams p, const CamParams* reqs, const uint32_t* tile_prefix,
+__global__ void __launch_bounds__(kCamThreads, 6) k_camera(const __grid_constant__ CamParams p, const CamParams* reqs, const uint32_t* tile_prefix,
                                                 int nreq) {
   after_previous();
   __shared__ CamSmem M[kCamThreads / 32][2];
   if (BATCH) {
     int r = 0;
     while (r < nreq - 1 && blockIdx.x >= tile_prefix[r + 1]) ++r;
-    const int blk = (int)(blockIdx.x - tile_prefix[r]);
-    if (*reqs[r].nonfinite) camera_tile_masked(reqs[r], blk, M);
-    else camera_tile<false>(reqs[r], blk, M);
+    const CamParams& q = reqs[r];
+    const int tile = (int)q.tile_order[blockIdx.x - tile_prefix[r]];  // (asked for together with the flag)
+    if (*q.nonfinite) camera_tile<true>(q, tile, M);
+    else camera_tile<false>(q, tile, M);
   } else {
-    if (*p.nonfinite) camera_tile_masked(p, (int)blockIdx.x, M);
-    else camera_tile<false>(p, (int)blockIdx.x, M);
+    const int tile = (int)p.tile_order[blockIdx.x];
+    if (*p.nonfinite) camera_tile<true>(p, tile, M);
+    else camera_tile<false>(p, tile, M);
   }
 }
 
@@ -1079,11 +1076,11 @@ using EnvSmem = CamEntries<kMaxBatch + 1, kEnvGroup>;  // colours: the lights', 
 // The thread layout and entry arithmetic of camera_tile, with 4 accumulators
 // per light and pixel plus 3 for R.
 template <bool MASK>
-__device__ __forceinline__ void camera_env_tile(const EnvCamParams& e, EnvSmem (*M)[2]) {
+__device__ __forceinline__ void camera_env_tile(const EnvCamParams& e, int tile, EnvSmem (*M)[2]) {
   const CamParams& p = e.c;
   const int nl = e.nl;
   CamPixels x;
-  const CamTile t = camera_tile_of(p, (int)blockIdx.x, x);
+  const CamTile t = camera_tile_of(p, tile, x);
   f32x2 R[2][2], S[2][kMaxBatch][2];  // per pixel: (R r, g), (R b, -); per light (S r, g), (S b, Sh)
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
@@ -1158,14 +1155,15 @@ __device__ __forceinline__ void camera_env_tile(const EnvCamParams& e, EnvSmem (
 }
 
 // (a call, which leaves the other form as it is without this one)
-__device__ __noinline__ void camera_env_tile_masked(const EnvCamParams& e, EnvSmem (*M)[2]) {
-  camera_env_tile<true>(e, M);
+__device__ __noinline__ void camera_env_tile_masked(const EnvCamParams& e, int tile, EnvSmem (*M)[2]) {
+  camera_env_tile<true>(e, tile, M);
 }
 
 __global__ void __launch_bounds__(kCamThreads) k_camera_env(const __grid_constant__ EnvCamParams e) {
   __shared__ EnvSmem M[kCamThreads / 32][2];
-  if (*e.c.nonfinite) camera_env_tile_masked(e, M);
-  else camera_env_tile<false>(e, M);
+  const int tile = (int)e.c.tile_order[blockIdx.x];
+  if (*e.c.nonfinite) camera_env_tile_masked(e, tile, M);
+  else camera_env_tile<false>(e, tile, M);
 }
 
 // Launch order of a splat's tiles: longest list first, so that the last
