@@ -292,7 +292,7 @@ __device__ __forceinline__ bool camera_bwd_strip(const CamBwdParams& p, CamBwdSm
 #pragma unroll
       for (int q = 0; q < NQ; ++q) {
         const f32x2 dy = add2(ly[q], yc.x);
-        const f32x2 pw = fma2(dy, fma2(yc.y, dy, v), sx);
+        const f32x2 pw = power2_pair(dy, yc.y, v, sx);
         f32x2 beta = pk2(lo2(pw) >= qx.w ? ex2(lo2(pw)) : 0.f, hi2(pw) >= qx.w ? ex2(hi2(pw)) : 0.f);
         f32x2 alpha = mul2(dup2(gi.x), beta);
         if (clampable) {  // the same for the warp: alpha = alpha_max passes no gradient to the geometry

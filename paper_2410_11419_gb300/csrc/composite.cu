@@ -77,7 +77,7 @@ struct ShadowParams {
   uint32_t* dead_list;         // items every ray enters stopped (K6c's)
   float* pub_a;                // [link_slot][256]: A(C_s+1) published by an item
   uint32_t* pub_flag;          // [item]: 0 not yet, 1 published, 2 published and every ray stopped
-  uint8_t* pass_mask;  // per list entry: halves with a passing pixel, 0x3 rows 0-7, 0xC rows 8-15
+  uint8_t* pass_mask;  // per list entry of a stopped segment: halves with a passing pixel, 0x3 rows 0-7, 0xC rows 8-15
   float2* partial;
   float* light_final;     // per light pixel: the product where the ray ended
   uint32_t* light_stop;   // per light pixel: 1 + index of the occluder that stopped it, or kNoStop
@@ -303,7 +303,7 @@ __device__ __forceinline__ float dead_half(const float4 e0, const float4 e1, int
     fx += 1.f;
     const f32x2 sx = dup2((e0.z * dx) * dx), v = dup2(e1.x * dx);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) den = add2(den, beta2_of(fma2(dy[q], fma2(c, dy[q], v), sx), e1.y));
+    for (int q = 0; q < 4; ++q) den = add2(den, beta2_of(power2_pair(dy[q], c, v, sx), e1.y));
   }
   return lo2(den) + hi2(den);
 }
@@ -532,10 +532,9 @@ __device__ __forceinline__ void live_item(const ShadowParams& p, const Links& li
       const uint32_t idx = is_recv ? j + mine : k + (lane - mine);
       rank = p.list[idx];
       const SplatRec q = p.rrec[rank];
-      const uint32_t bits = stage_entry(q, ox, oy, S.e, lane);
+      stage_entry(q, ox, oy, S.e, lane);
       if (is_recv) {
         slot = p.off[rank] + (uint32_t)((it.ty - q.r.y) * (q.r.z - q.r.x + 1) + (it.tx - q.r.x));
-        p.pass_mask[idx] = (uint8_t)bits;
       }
     }
     __syncwarp();
@@ -812,9 +811,8 @@ struct CamPixels {
 };
 
 // The weights alpha T with which entries t .. t + G - 1 enter the two pixels, 0
-// where they do not pass; T goes on behind them.  The alpha is gamma
-// 2^power2, the power's arithmetic that of the backward (power2_at).  A ray
-// stops before T would fall below tstop: it keeps its T, and its row moves
+// where they do not pass; T goes on behind them.  The alpha is gamma 2^power2.  A
+// ray stops before T would fall below tstop: it keeps its T, and its row moves
 // far away, so that nothing passes from there on.  The alphas of a group do
 // not depend on one another; only the product T is a chain.
 template <int COLS, int G>
@@ -828,7 +826,7 @@ __device__ __forceinline__ void camera_weights(const CamEntries<COLS, G>& E, int
     const float4 q = E.xart[t + i];
     const float dx = px.lx - q.x;
     const f32x2 dy = add2(px.ly, yc.x);
-    const f32x2 pw = fma2(dy, fma2(yc.y, dy, dup2(q.z * dx)), dup2((q.y * dx) * dx));
+    const f32x2 pw = power2_pair(dy, yc.y, dup2(q.z * dx), dup2((q.y * dx) * dx));
     const f32x2 ga = mul2(dup2(E.gi[t + i].x), beta2_of(pw, q.w));
     alpha[i] = pk2(fminf(amax, lo2(ga)), fminf(amax, hi2(ga)));
     T[i + 1] = mul2(T[i], fma2(alpha[i], dup2(-1.f), dup2(1.f)));
@@ -1178,8 +1176,7 @@ __global__ void __launch_bounds__(kCamThreads) k_camera_env(const __grid_constan
 // segments (a prefix of the order).  The order within a bucket may vary from run to run; no result
 // depends on it.
 __global__ void __launch_bounds__(1024) k_tile_order(const uint32_t* __restrict__ tile_start, int ntiles,
-                                                     uint32_t* __restrict__ order, uint32_t* __restrict__ lvl_off,
-                                                     uint32_t max_items) {
+                                                     uint32_t* __restrict__ order, uint32_t* __restrict__ lvl_off) {
   after_previous();
   constexpr int kBuckets = 1024;
   __shared__ uint32_t cnt[kBuckets];
@@ -1197,8 +1194,7 @@ __global__ void __launch_bounds__(1024) k_tile_order(const uint32_t* __restrict_
     __syncthreads();
     const uint32_t pairs = tile_start[ntiles];
     seg_len = kSegMin;
-    while (seg_len < kSegLen && (pairs / seg_len > kSegTarget || (uint32_t)ntiles + pairs / seg_len + 1u > max_items ||
-                                 longest > seg_len * (uint32_t)(kSegLevels - 1)))
+    while (seg_len < kSegLen && (pairs / seg_len > kSegTarget || longest > seg_len * (uint32_t)(kSegLevels - 1)))
       seg_len *= 2u;
     if (t == 0) lvl_off[kSegWord] = seg_len;
     if (t > 0 && t < (int)(kSegWord - kSegLevels)) lvl_off[kSegLevels + t] = 0u;  // the tickets and list counts
@@ -1254,7 +1250,7 @@ __global__ void __launch_bounds__(1024) k_tile_order(const uint32_t* __restrict_
 void launch_tile_order(const FrameArgs& f, int splat, cudaStream_t s) {
   const Workspace& L = *f.L;
   uint32_t* order = at<uint32_t>(f.ws, L.tile_order[splat]);
-  launch_after(k_tile_order, 1, 1024, 0, s, at<uint32_t>(f.ws, L.sp[splat].tile_start), L.ntiles, order, nullptr, 0u);
+  launch_after(k_tile_order, 1, 1024, 0, s, at<uint32_t>(f.ws, L.sp[splat].tile_start), L.ntiles, order, nullptr);
   count_launch();
 }
 
@@ -1380,8 +1376,7 @@ void prepare_shadow_composite(const FrameArgs& f, cudaStream_t s) {
   uint32_t* kb = at<uint32_t>(ws, b.tv[1 - fin]);
   // the light tiles by segment count, and the work items of each segment level
   uint32_t* lvl = at<uint32_t>(ws, f.L->seg_lvl);
-  launch_after(k_tile_order, 1, 1024, 0, s, at<uint32_t>(ws, b.tile_start), f.L->ntiles, at<uint32_t>(ws, f.L->tile_order[1]),
-                                  lvl, (uint32_t)shadow_seg_items(f.L->ntiles, f.L->cap));
+  launch_after(k_tile_order, 1, 1024, 0, s, at<uint32_t>(ws, b.tile_start), f.L->ntiles, at<uint32_t>(ws, f.L->tile_order[1]), lvl);
   // the occluder bounds the segment plan reads; the rest follow K6a
   const size_t items = shadow_seg_items(f.L->ntiles, f.L->cap);
   const int n = f.sc.n;

@@ -240,7 +240,7 @@ __device__ __forceinline__ void recv_bwd(const f32x2 (&ly)[kPx / 2], const f32x2
 #pragma unroll
   for (int q = 2 * H; q < 2 * H + 2; ++q) {
     const f32x2 dy = add2(ly[q], e.ny);
-    const f32x2 b = beta2_of(fma2(dy, fma2(e.c, dy, e.v), e.s), e.thr);
+    const f32x2 b = beta2_of(power2_pair(dy, e.c, e.v, e.s), e.thr);
     const f32x2 cb = where_passing<MASK>(b, mul2(coef, b));
     S[q] = fma2(cb, A[q], S[q]);
     const f32x2 w = mul2(cb, add2(A[q], nT)), wd = mul2(w, dy);
@@ -259,7 +259,7 @@ __device__ __forceinline__ void occ_bwd(const f32x2 (&ly)[kPx / 2], f32x2 (&A)[k
 #pragma unroll
   for (int q = 2 * H; q < 2 * H + 2; ++q) {
     const f32x2 dy = add2(ly[q], e.ny);
-    f32x2 b = beta2_of(fma2(dy, fma2(e.c, dy, e.v), e.s), e.thr);
+    f32x2 b = beta2_of(power2_pair(dy, e.c, e.v, e.s), e.thr);
     f32x2 f = fma2(dup2(ngamma), b, dup2(1.f));
     if (CLAMP) {
       f = pk2(fmaxf(lo2(f), 1.f - amax), fmaxf(hi2(f), 1.f - amax));
@@ -479,7 +479,7 @@ __device__ __forceinline__ void stopped_unit(const BwdParams& p, uint32_t idx, i
     Moments m{0ull, 0ull, 0ull};
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const f32x2 b = beta2_of(fma2(dy[q], fma2(c, dy[q], v), sx), e1.y), bd = mul2(b, dy[q]);
+      const f32x2 b = beta2_of(power2_pair(dy[q], c, v, sx), e1.y), bd = mul2(b, dy[q]);
       m.m0 = add2(m.m0, b);
       m.m1 = add2(m.m1, bd);
       m.m2 = fma2(bd, dy[q], m.m2);

@@ -55,7 +55,7 @@ __device__ __forceinline__ ColTerms col_terms(float lx, const StagedEntries& E, 
 }
 __device__ __forceinline__ f32x2 beta2_at(const ColTerms& e, f32x2 ly) {
   const f32x2 dy = add2(ly, e.ny);
-  return beta2_of(fma2(dy, fma2(e.c, dy, e.v), e.s), e.thr);
+  return beta2_of(power2_pair(dy, e.c, e.v, e.s), e.thr);
 }
 
 // An occluder on four rays of one half: P *= max(omin, 1 - gamma beta), which

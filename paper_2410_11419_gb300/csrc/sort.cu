@@ -19,10 +19,6 @@ namespace {
 // ---------------------------------------------------------------------------
 // Stable LSD radix sort pass, 8-bit digit, u32 key + u32 value.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t load_n(const uint32_t* n_ptr, uint32_t n_fixed) {
-  return n_ptr ? *n_ptr : n_fixed;
-}
-
 // ---------------------------------------------------------------------------
 // The depth sorts, one kernel per digit pass (decoupled look-back).  Each
 // block takes the next kSortThreads * ROUNDS items in order by a ticket, ranks
@@ -47,12 +43,11 @@ __device__ __forceinline__ uint32_t load_n(const uint32_t* n_ptr, uint32_t n_fix
 constexpr int kLookSpin = 1 << 20;
 constexpr int kLookWords = 4;
 
-// Every digit of every pass (PASSES <= 4 eight-bit digits), counted over the
-// n keys.  Warp-private counters; a warp whose 32 keys share a digit (usual
+// Every digit of every pass (PASSES eight-bit digits), counted over the n keys.  Warp-private counters; a warp whose 32 keys share a digit (usual
 // for the top digits of the depth keys) adds it once.
 template <int PASSES>
-__global__ void __launch_bounds__(256) k_digit_totals(const uint32_t* __restrict__ keys, const uint32_t* n_ptr,
-                                                      uint32_t n_fixed, int passes, uint32_t* __restrict__ totals) {
+__global__ void __launch_bounds__(256) k_digit_totals(const uint32_t* __restrict__ keys, uint32_t n,
+                                                      uint32_t* __restrict__ totals) {
   __shared__ uint32_t h[PASSES][kSortThreads / 32][256];
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
 #pragma unroll
@@ -60,7 +55,6 @@ __global__ void __launch_bounds__(256) k_digit_totals(const uint32_t* __restrict
 #pragma unroll
     for (int w = 0; w < kSortThreads / 32; ++w) h[p][w][t] = 0;
   __syncthreads();
-  const uint32_t n = load_n(n_ptr, n_fixed);
   // each warp takes 128 consecutive keys per step, four coalesced loads in flight per lane
   for (uint32_t wb = (blockIdx.x * (kSortThreads / 32) + warp) * 128u; wb < n; wb += gridDim.x * kSortThreads * 4u) {
     uint32_t k[4];
@@ -76,7 +70,6 @@ __global__ void __launch_bounds__(256) k_digit_totals(const uint32_t* __restrict
       if (!vm) break;
 #pragma unroll
       for (int p = 0; p < PASSES; ++p) {
-        if (p >= passes) break;
         const uint32_t d = (k[u] >> (8 * p)) & 255u;
         const uint32_t first = __shfl_sync(0xffffffffu, d, 0);
         if (__all_sync(0xffffffffu, !valid || d == first)) {
@@ -89,7 +82,7 @@ __global__ void __launch_bounds__(256) k_digit_totals(const uint32_t* __restrict
     }
   }
   __syncthreads();
-  for (int p = 0; p < passes; ++p) {
+  for (int p = 0; p < PASSES; ++p) {
     uint32_t c = 0;
 #pragma unroll
     for (int w = 0; w < kSortThreads / 32; ++w) c += h[p][w][t];
@@ -110,7 +103,7 @@ struct OnesweepSmem {
 template <int ROUNDS>
 __global__ void __launch_bounds__(kSortThreads, 3) k_onesweep(
     const uint32_t* __restrict__ kin, const uint32_t* __restrict__ vin, uint32_t* __restrict__ kout,
-    uint32_t* __restrict__ vout, const uint32_t* n_ptr, uint32_t n_fixed, int shift,
+    uint32_t* __restrict__ vout, uint32_t n, int shift,
     const uint32_t* __restrict__ totals, unsigned long long* look, uint32_t* ticket, uint32_t* header) {
   after_previous();
   constexpr int kItems = kSortThreads * ROUNDS;
@@ -118,7 +111,6 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_onesweep(
   extern __shared__ uint4 onesweep_raw[];
   OnesweepSmem<ROUNDS>& S = *reinterpret_cast<OnesweepSmem<ROUNDS>*>(onesweep_raw);
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const uint32_t n = load_n(n_ptr, n_fixed);
   if (t == 0) S.ticket = atomicAdd(ticket, 1u);
 #pragma unroll
   for (int w = 0; w < kWarps; ++w) S.cnt[w][t] = 0;
@@ -406,22 +398,21 @@ __global__ void __launch_bounds__(kBinBlock) k_reorder(int n, const uint32_t* __
   }
 }
 
-// Stable LSD sort of (key, value) pairs (vin null: values are the input
-// positions) on the low 8 * passes key bits (passes <= PASSES): one
+// Stable LSD sort of n keys with their positions on the low 8 * PASSES bits: one
 // k_digit_totals, then one k_onesweep per pass.  Even passes write (k0, v0),
 // odd passes (k1, v1), each reading the previous pass's output (pass 0 reads
-// (kin, vin)).  look_region: onesweep_bytes(nblocks, PASSES) bytes, zeroed here.
-// Up to kSmallSort keys: one launch of k_sort_small, whose output is (k1, v1).
+// kin and the positions).  look_region: onesweep_bytes(nblocks, PASSES) bytes, zeroed
+// here.  Up to kSmallSort keys: one launch of k_sort_small, whose output is (k1, v1).
 // own_status: the kOrderFront bytes before look_region belong to the sort and start
 // with `header`, the word for its status, which is cleared as well.  first_ticket: of
 // the first pass (past 0: a self-test, its waits run out).
-template <int ROUNDS, int PASSES>
-void onesweep_sort(const uint32_t* kin, const uint32_t* vin, uint32_t* k0, uint32_t* v0, uint32_t* k1,
-                   uint32_t* v1, const uint32_t* n_ptr, uint32_t n_fixed, int nblocks, int passes,
+template <int ROUNDS>
+void onesweep_sort(const uint32_t* kin, uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, uint32_t n, int nblocks,
                    unsigned char* look_region, uint32_t* header, cudaStream_t s, bool wait = false,
                    bool own_status = false, int first_ticket = 0) {
-  if (!n_ptr && !vin && n_fixed <= kSmallSort && passes == 4) {
-    launch_behind(wait, k_sort_small, 1, kSmallThreads, 0, s, kin, k1, v1, n_fixed, own_status ? header : nullptr);
+  constexpr int PASSES = 4;
+  if (n <= kSmallSort) {
+    launch_behind(wait, k_sort_small, 1, kSmallThreads, 0, s, kin, k1, v1, n, own_status ? header : nullptr);
     count_launch();
     return;
   }
@@ -436,21 +427,19 @@ void onesweep_sort(const uint32_t* kin, const uint32_t* vin, uint32_t* k0, uint3
   const size_t front = own_status ? kOrderFront : 0;
   cudaMemsetAsync(look_region - front, 0, front + onesweep_bytes(nblocks, PASSES), s);
   if (first_ticket) cudaMemsetAsync(tickets, first_ticket, 1, s);
-  const int tb_cap = device_sm_count() * 4;
-  int tb = n_ptr ? tb_cap : (int)((n_fixed + 1023) / 1024);
-  if (tb < 1) tb = 1;
-  if (tb > tb_cap) tb = tb_cap;
-  k_digit_totals<PASSES><<<tb, kSortThreads, 0, s>>>(kin, n_ptr, n_fixed, passes, totals);
+  const int tb_cap = device_sm_count() * 4, tb = (int)((n + 1023) / 1024);
+  k_digit_totals<PASSES><<<tb < tb_cap ? tb : tb_cap, kSortThreads, 0, s>>>(kin, n, totals);
   const uint32_t* ki = kin;
-  const uint32_t* vi = vin;
-  for (int p = 0; p < passes; ++p) {
+  const uint32_t* vi = nullptr;
+  for (int p = 0; p < PASSES; ++p) {
     uint32_t* ko = (p & 1) ? k1 : k0;
     uint32_t* vo = (p & 1) ? v1 : v0;
-    launch_after(k_onesweep<ROUNDS>, nblocks, kSortThreads, sizeof(OnesweepSmem<ROUNDS>), s, ki, vi, ko, vo, n_ptr, n_fixed, 8 * p, totals + 256 * p, look, tickets + p, header);
+    launch_after(k_onesweep<ROUNDS>, nblocks, kSortThreads, sizeof(OnesweepSmem<ROUNDS>), s, ki, vi, ko, vo, n, 8 * p,
+                 totals + 256 * p, look, tickets + p, header);
     ki = ko;
     vi = vo;
   }
-  count_launch(1 + passes);
+  count_launch(1 + PASSES);
 }
 
 }  // namespace
@@ -464,21 +453,19 @@ void depth_order(const uint32_t* keys, uint32_t n, uint32_t* k0, uint32_t* v0, u
   uint32_t* status = reinterpret_cast<uint32_t*>(front);
   auto blocks = [&](int rounds) { return (int)((n + kSortThreads * rounds - 1) / (kSortThreads * rounds)); };
   if (blocks(4) <= kDepthOrderBlocks)
-    onesweep_sort<4, 4>(keys, nullptr, k0, v0, k1, order, nullptr, n, blocks(4), 4, look, status, s, false, true, first_ticket);
+    onesweep_sort<4>(keys, k0, v0, k1, order, n, blocks(4), look, status, s, false, true, first_ticket);
   else
-    onesweep_sort<8, 4>(keys, nullptr, k0, v0, k1, order, nullptr, n, blocks(8), 4, look, status, s, false, true, first_ticket);
+    onesweep_sort<8>(keys, k0, v0, k1, order, n, blocks(8), look, status, s, false, true, first_ticket);
 }
 
 void launch_depth_sort(const FrameArgs& f, int sp, cudaStream_t s, bool wait) {
   const SplatBufs& b = f.L->sp[sp];
   unsigned char* ws = f.ws;
   const int n = f.sc.n;
-  // 1024 keys per block: four times the blocks of the pair sorts, for a
-  // sort of a few hundred thousand keys that would otherwise leave SMs idle
-  onesweep_sort<kDepthSortRounds, 4>(at<uint32_t>(ws, b.key), nullptr, at<uint32_t>(ws, b.sk[0]),
-                                     at<uint32_t>(ws, b.sv[0]), at<uint32_t>(ws, b.sk[1]), at<uint32_t>(ws, b.sv[1]),
-                                     nullptr, (uint32_t)n, f.L->nb_n, 4, at<unsigned char>(ws, b.dlook),
-                                     at<uint32_t>(ws, f.L->header), s, wait);
+  // 1024 keys per block, so that a few hundred thousand keys fill the SMs
+  onesweep_sort<kDepthSortRounds>(at<uint32_t>(ws, b.key), at<uint32_t>(ws, b.sk[0]), at<uint32_t>(ws, b.sv[0]),
+                                  at<uint32_t>(ws, b.sk[1]), at<uint32_t>(ws, b.sv[1]), (uint32_t)n, f.L->nb_n,
+                                  at<unsigned char>(ws, b.dlook), at<uint32_t>(ws, f.L->header), s, wait);
   // 4 passes end in buffer 1: sv[1] holds the index of each depth rank
   launch_after(k_reorder, f.L->nb_rows, kBinBlock, 0, s, n, at<uint32_t>(ws, b.sv[1]), at<SplatRec>(ws, b.rec), at<SplatRec>(ws, b.rrec),
       at<uint32_t>(ws, b.rank_of), at<uint32_t>(ws, b.cnt), at<float4>(ws, f.L->shade),
@@ -522,7 +509,7 @@ extern "C" gs3_status gs3_selftest_wait_timeout(uint32_t n, uint32_t* status_out
     cudaFuncSetAttribute(k_onesweep<kTileSortRounds>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)sizeof(OnesweepSmem<kTileSortRounds>));
     k_onesweep<kTileSortRounds><<<nblocks, kSortThreads, sizeof(OnesweepSmem<kTileSortRounds>)>>>(
-        kin, vin, kout, vout, nullptr, n, 0, totals, lk, tickets, status);
+        kin, vin, kout, vout, n, 0, totals, lk, tickets, status);
     count_launch();
     e = cudaGetLastError();
   }

@@ -5,6 +5,7 @@
 // whatever the thread layout.  Quadrant w of a 16x16 tile is the 8x8 block
 // at (8 (w & 1), 8 (w >> 1)).
 #pragma once
+#include "f32x2.cuh"
 #include "gs3_internal.cuh"
 
 namespace gs3 {
@@ -92,15 +93,10 @@ __device__ __forceinline__ bool ellipse_rows(const float4 e0, const float4 e1, f
   return best <= lim + 1e-4f * (1.f + size);
 }
 
-// power2 at one pixel (lx, ly) of the tile: the camera composite and its
-// backward evaluate an entry with this arithmetic, so both take every alpha
-// decision alike.
-__device__ __forceinline__ float power2_at(const float4 e0, float r, float lx, float ly) {
-  const float dx = lx - e0.x;
-  const float sx = (e0.z * dx) * dx, v = r * dx;
-  const float dy = ly - e0.y;
-  return fmaf(dy, fmaf(e0.w, dy, v), sx);
-}
+// power2 of two pixels of a column, dy apart from the centre (c twice; v = r dx and
+// sx = (a dx) dx twice): the composites and their backward use this form alone, so
+// they take every alpha decision alike.
+__device__ __forceinline__ f32x2 power2_pair(f32x2 dy, f32x2 c, f32x2 v, f32x2 sx) { return fma2(dy, fma2(c, dy, v), sx); }
 
 // The row of a pixel that takes no entry (outside the image, its ray stopped or
 // not yet reached): the power there is below every threshold, so the packed
