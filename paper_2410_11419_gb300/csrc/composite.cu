@@ -238,9 +238,10 @@ __device__ __forceinline__ int locate(const ShadowParams* reqs, int nreq, int ki
 
 // One frame (p) or a batch of nreq frames (reqs, in device memory; p is the
 // first, whose tickets the batch shares).  5 blocks per SM: 0.272 ms against
-// 0.279 at 4, 0.287 at 6 and 0.314 at 8.
+// 0.279 at 4, 0.287 at 6 and 0.314 at 8.  With 96 registers they leave too few for
+// another stream's blocks: eight lights side by side take 2,630 us, 2,623 with 88.
 template <bool BATCH>
-__global__ void __launch_bounds__(kSegWarps * 32, 5) k_shadow_chain(const ShadowParams p, const ShadowParams* reqs,
+__global__ void __maxnreg__(88) k_shadow_chain(const ShadowParams p, const ShadowParams* reqs,
                                                                     int nreq) {
   after_previous();
   __shared__ StagedEntries smem[kSegWarps];
