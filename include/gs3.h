@@ -298,7 +298,9 @@ size_t gs3_backward_workspace_size(const gs3_scene *scene);
  * final occluder product, then both projections and the shading.
  *   dL_drgb:   device float32 [height][width][3]
  *   workspace: the workspace of a gs3_render of the same scene, camera,
- *              light and options, unchanged since (it holds the forward state)
+ *              light and options, unchanged since (it holds the forward state;
+ *              the backward writes only to scratch in it, so that every stage
+ *              can be run again on what the frame left)
  *   bwd_ws:    device, >= gs3_backward_workspace_size bytes, caller-owned
  * The MLP gradients are those of the scene's FP32 networks evaluated at the
  * forward's inputs (their products on the tensor cores, the operands split

@@ -10,10 +10,12 @@
 // the forward kernel's arrangement: encoded inputs, the hidden layers forward,
 // the output layer and its gradient, the data gradients down to the inputs and
 // through the encoding.  The forward products are three-pass TF32 (x as its 10
-// leading mantissa bits and the rest, small' terms first, one accumulator): the
-// signs of h decide act', and a pre-activation within rounding of zero keeps the
-// side that a GEMM per layer in that form gives it.  On the way back only those
-// signs are needed; they stay in shared memory.  The activations (h_0 .. h_{L-1},
+// leading mantissa bits and the rest, small' terms first, one accumulator), as in a
+// GEMM per layer: the signs of h decide act', and a pre-activation within rounding
+// of zero keeps the side that form gives it.  BF16 triples would be nearer to
+// float64, and the frame's own networks use them (mlp_x3.cu), so for a few such
+// pre-activations this side is not the frame's.  On the way back only the signs are
+// needed; they stay in shared memory.  The activations (h_0 .. h_{L-1},
 // dz_L .. dz_1) go to global memory as the weight gradients contract them: h from
 // registers (eight lanes fill a 128-byte core matrix), dz, which lies in shared
 // memory in that form, by one warp's bulk copies under the next layer's MMAs.
@@ -26,9 +28,10 @@
 // ones.  CTAs own contiguous row ranges, k_mlp_x3_sum adds their partials in
 // order: no result depends on scheduling.
 //
-// The tiles pass in batches of kBatchTiles, which bounds the scratch memory (at
-// most 1.3 GB for 3 x 128).  Smaller batches, down to those that stay in L2, take
-// 4 to 20 % longer: a launch's last tiles leave SMs idle.
+// The tiles pass in batches of kBatchTiles, which bounds the stored activations (at
+// most 1.3 GB for 3 x 128, 1.8 GB for 4 x 128); the weight partials are kept per
+// batch (3 x 128: 25 MB per 311,296 Gaussians).  Smaller batches, down to those that
+// stay in L2, take 4 to 20 % longer: a launch's last tiles leave SMs idle.
 //
 // Bound: k_mlp_x3_rows by the chain of its 2 L products, one tile per SM at a time
 // (the hand-overs; a third of its MMAs less changes nothing), k_mlp_x3_wgrad by
