@@ -220,7 +220,8 @@ struct BwdSmem {  // one warp's
   uint8_t op[kRows];         // the rows' places in the batch
 };
 
-// 1 / f to within an ulp (f in [1 - alpha_max, 1]); exactly 1 for f = 1
+// 1 / f, rounded to nearest for every f in [0.01, 1] (compared with __frcp_rn over all
+// of them), so exactly 1 for f = 1
 __device__ __forceinline__ f32x2 rcp2(f32x2 f) {
   float a, b;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(a) : "f"(lo2(f)));
