@@ -41,7 +41,8 @@ __device__ __forceinline__ float ex2(float x) {
 __device__ __forceinline__ void make_entry(const SplatRec& q, float ox, float oy, float4& e0, float4& e1) {
   const float ux = (q.a.x - ox) + q.b.w, vy = (q.a.y - oy) + q.c.x;
   const uint32_t m = warp_mask8(ux, vy, q.c.y, q.c.z);
-  e0 = make_float4(ux, vy, -0.5f * kLog2e * q.b.x, -0.5f * kLog2e * q.b.z);
+  // a conic whose determinant overflowed is 0: kFarRow still has to lie outside
+  e0 = make_float4(ux, vy, -0.5f * kLog2e * q.b.x, fminf(-0.5f * kLog2e * q.b.z, -1.0e-30f));
   e1 = make_float4(-kLog2e * q.b.y, kLog2e * q.c.w, q.a.z, __uint_as_float(m));
 }
 
@@ -100,9 +101,9 @@ __device__ __forceinline__ f32x2 power2_pair(f32x2 dy, f32x2 c, f32x2 v, f32x2 s
 
 // The row of a pixel that takes no entry (outside the image, its ray stopped or
 // not yet reached): the power there is below every threshold, so the packed
-// walks need no test per pixel.  Far enough for deviations of up to 3e17 pixels
-// (at 1e6 rows a splat of 3e5 pixels passed); finite, as the backward's moments
-// multiply it by a zero weight.
+// walks need no test per pixel.  Far enough for every splat (make_entry keeps c at or
+// below -1e-30, which there is a power of -1e6; at 1e6 rows a splat of 3e5 pixels'
+// deviation passed), and finite, as the backward's moments multiply it by a zero weight.
 constexpr float kFarRow = 1.0e18f;
 
 // A shadow ray stops taking occluders once its product A falls below

@@ -29,7 +29,7 @@ def wide_scene(seed, n, scale, cam, light):
 
 
 @pytest.mark.parametrize("w,h", [(37, 51), (70, 41)])
-@pytest.mark.parametrize("scale", [1e3, 1e5, 1e7])
+@pytest.mark.parametrize("scale", [1e3, 1e5, 1e7, 4e8])
 def test_wide_splats(gs3, oracle, w, h, scale):
     from oracle import torch_ref as TR
     cam, light = synth.camera_light_pair(w, w, h)
