@@ -125,7 +125,8 @@ __device__ __forceinline__ uint32_t min_bits(const f32x2 (&P)[kPx / 2]) {
 }
 
 // K6a: A(C_s+1) of every segment but a tile's last, chained from A(C_s).
-__device__ __forceinline__ void chain_item(const ShadowParams& p, const Links& link_slot, uint32_t w, StagedEntries& S, int lane) {
+template <typename L>
+__device__ __forceinline__ void chain_item(const ShadowParams& p, const L& link_slot, uint32_t w, StagedEntries& S, int lane) {
   const float lx = (lane & 15) + 0.5f, omin = 1.f - p.amax;
   const SegItem it = seg_item(p, w, lane);
   if (it.last) return;  // nothing follows it
@@ -236,26 +237,36 @@ __device__ __forceinline__ int locate(const ShadowParams* reqs, int nreq, int ki
   return r;
 }
 
+// Links from shared memory where they are used, which leaves k_shadow_chain its registers
+struct SharedLinks {
+  const volatile Links* at;
+  __device__ __forceinline__ size_t operator()(uint32_t w) const {
+    return (size_t)(w < at->more ? w : w - at->gap) * 256;
+  }
+};
+
 // One frame (p) or a batch of nreq frames (reqs, in device memory; p is the
 // first, whose tickets the batch shares).  5 blocks per SM: 0.272 ms against
-// 0.279 at 4, 0.287 at 6 and 0.314 at 8.  With 96 registers they leave too few for
-// another stream's blocks: eight lights side by side take 2,630 us, 2,623 with 88.
+// 0.279 at 4, 0.287 at 6 and 0.314 at 8.  Past 88 registers they leave too few for
+// another stream's blocks (eight lights side by side: 2,630 us with 96, 2,615 with 88).
 template <bool BATCH>
-__global__ void __maxnreg__(88) k_shadow_chain(const ShadowParams p, const ShadowParams* reqs,
+__global__ void __launch_bounds__(kSegWarps * 32, 5) k_shadow_chain(const ShadowParams p, const ShadowParams* reqs,
                                                                     int nreq) {
   after_previous();
   __shared__ StagedEntries smem[kSegWarps];
-  StagedEntries& S = smem[threadIdx.x >> 5];
-  const int lane = threadIdx.x & 31;
+  __shared__ Links links[kSegWarps];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  StagedEntries& S = smem[warp];
   const uint32_t total = BATCH ? batch_items(reqs, nreq, kAllItems) : item_count(p, kAllItems);
-  const Links links = frame_links(p.lvl_off);
+  if (!BATCH && lane == 0) links[warp] = frame_links(p.lvl_off);
+  __syncwarp();
   uint32_t w;
   while (next_item(p.ticket, total, lane, w)) {
     if (BATCH) {
       const int r = locate(reqs, nreq, kAllItems, w);
       chain_item(reqs[r], frame_links(reqs[r].lvl_off), w, S, lane);
     } else {
-      chain_item(p, links, w, S, lane);
+      chain_item(p, SharedLinks{links + warp}, w, S, lane);
     }
   }
 }

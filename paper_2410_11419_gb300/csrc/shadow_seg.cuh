@@ -103,8 +103,8 @@ __device__ __forceinline__ Links frame_links(const uint32_t* lvl_off) {  // once
 // A(C_s) of the lane's rays: 1 / 0 (in / outside the image) for a tile's
 // first segment, else the predecessor's publication (read from L2: it was
 // written on another SM); flag 2 publishes that every ray stopped.
-template <typename P>
-__device__ __forceinline__ void load_entering(const P& p, const Links& link_slot, bool first, uint32_t wpred, uint32_t flag, int lane,
+template <typename P, typename L>
+__device__ __forceinline__ void load_entering(const P& p, const L& link_slot, bool first, uint32_t wpred, uint32_t flag, int lane,
                                               int rows_in, f32x2 (&A)[kPx / 2]) {
   const float* in = p.pub_a + (first ? 0 : link_slot(wpred)) + lane;
   auto one = [&](int i) { return first ? (i < rows_in ? 1.f : 0.f) : (flag == 2u ? 0.f : __ldcg(in + 32 * i)); };
