@@ -117,3 +117,24 @@ def test_infinite_pixel_gradient_stays_with_its_gaussians(gs3, ablate):
             meets = (one[f] != 0).any(axis=1)
             assert np.isfinite(got[f][~meets]).all(), f
             assert meets.sum() < 290 and not np.isfinite(got[f][meets]).all()
+
+
+def test_infinite_colour_in_a_batch(gs3):
+    """Frames of a batch keep their own form: each equals its frame rendered alone, bit for bit."""
+    import torch
+    from paper_2410_11419_gb300 import _native as N, render as R
+    scene, cam, light = scene_and_view(4)
+    scenes = [R.DeviceScene(scene)]
+    scene.albedo_d[250, :3] = np.inf
+    scenes.append(R.DeviceScene(scene))
+    server = R.Server(hbm_budget=1 << 30, max_inflight=1, max_batch=4)
+    ids = [server.add_scene(x) for x in scenes]
+    out = [torch.zeros((H, W, 3), device="cuda") for _ in range(8)]
+    torch.cuda.synchronize()
+    tickets = [server.submit(ids[i % 2], cam, light, x) for i, x in enumerate(out)]
+    assert all(server.wait(t)[0] == N.GS3_OK for t in tickets)
+    server.close()
+    for i, x in enumerate(out):
+        alone = R.Renderer(scenes[i % 2], W, H, 1 << 18).render(cam, light)
+        assert torch.equal(x.view(torch.int32), alone.view(torch.int32))
+        assert bool(torch.isfinite(x).all()) == (i % 2 == 0)
